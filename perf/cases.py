@@ -228,3 +228,91 @@ def run(state):
     if case["behind"]:
         cache.flush()
     return {"out": state["out"], "rows": state["rows"]}
+
+
+def _rotated(case, x, pos0):
+    """x [n, heads, d] rotated at positions pos0, pos0 + 1, ..., in 64 bits."""
+    d = case["head_dim"]
+    base = 10000.0 if d == 64 else 500000.0
+    inv = base ** (-2.0 * torch.arange(d // 2, device="cuda", dtype=torch.float64) / d)
+    theta = (pos0 + torch.arange(x.shape[0], device="cuda", dtype=torch.float64))[:, None, None] * inv
+    lo, hi = x.double().split(d // 2, dim=-1)
+    return torch.cat([lo * theta.cos() - hi * theta.sin(), hi * theta.cos() + lo * theta.sin()], dim=-1)
+
+
+def _stored(case, x):
+    """(rows [n, heads, d] as the attention reads them, their scales or None): what a quantised cache keeps of them."""
+    if case["cache"] == "plain":
+        return x.double(), None
+    levels = 127 if case["cache"] == "int8" else 7
+    top = x.double().abs().amax(-1, keepdim=True)
+    return (x.double() * (levels / top.clamp(min=1e-300))).round().clamp(-levels, levels) * (top / levels), (top / levels)[..., 0]
+
+
+class _Fold:
+    """One sequence's fold in 64 bits."""
+
+    def __init__(self, case, capacity):
+        shape = (case["kv_heads"], capacity, case["head_dim"])
+        self.case, self.len = case, 0
+        self.k, self.v = (torch.zeros(shape, dtype=torch.float64, device="cuda") for _ in range(2))
+        self.scales = [torch.zeros(shape[:2], dtype=torch.float64, device="cuda") for _ in range(2)]
+
+    def append(self, k, v):
+        new = slice(self.len, self.len + k.shape[0])
+        for plane, scales, rows in ((self.k, self.scales[0], _rotated(self.case, k, self.len)), (self.v, self.scales[1], v)):
+            rows, s = _stored(self.case, rows)
+            plane[:, new] = rows.transpose(0, 1)
+            if s is not None:
+                scales[:, new] = s.T
+        self.len = new.stop
+
+    def step(self, q, k, v):
+        case, first, n = self.case, self.len, q.shape[0]
+        self.append(k, v)
+        heads, d, group = case["kv_heads"], case["head_dim"], case["q_heads"] // case["kv_heads"]
+        keys = torch.arange(self.len, device="cuda")
+        lo = max(first - case["window"], 0) if case["window"] else 0
+        out = torch.empty((n, heads, group, d), dtype=torch.float64, device="cuda")
+        q = _rotated(case, q, first).view(n, heads, group, d) / math.sqrt(d)
+        some = max(1, (1 << 28) // (group * self.len))
+        for a in range(0, n, some):
+            b = min(n, a + some)
+            hidden = keys[None] > first + torch.arange(a, b, device="cuda")[:, None]
+            hidden |= (keys >= case["sinks"]) & (keys < lo)
+            hidden = hidden[:, None].expand(b - a, group, self.len).reshape(-1, self.len)
+            for h in range(heads):
+                p = (q[a:b, h].reshape(-1, d) @ self.k[h, :self.len].T).masked_fill_(hidden, -math.inf)
+                p = p.sub_(p.amax(-1, keepdim=True)).exp_()
+                out[a:b, h] = ((p @ self.v[h, :self.len]) / p.sum(-1, keepdim=True)).view(b - a, group, d)
+        return out.view(n, heads * group, d)
+
+
+def exact(case, seed):
+    """The outputs of run in 64 bits, from the statement of the fold alone; codes and pages of a pool are whole values and have none."""
+    if work(case)["flops"] > 6e13:
+        return None
+    gen = torch.Generator(device="cuda").manual_seed(seed)
+    chunks = _chunks(case)
+    end = case["prefix"] + sum(chunks)
+    if case["caches"]:
+        n, lens = case["caches"], _member_prefixes(case)
+        torch.randperm(n * -(-end // _PAGE), generator=gen, device="cuda")
+        held = [[_inputs(case, gen, min(1024, rows - at))[1:] for at in range(0, rows, 1024)] for rows in lens]
+        steps = [_inputs(case, gen, m, (n,)) for m in chunks]
+        outs = [torch.empty(s[0].shape, dtype=torch.float64, device="cuda") for s in steps]
+        for i in range(n):
+            fold = _Fold(case, end)
+            for k, v in held[i]:
+                fold.append(k, v)
+            for (q, k, v), out in zip(steps, outs):
+                out[i] = fold.step(q[i], k[i], v[i])
+        return {"out": outs, "pool": None}
+    fold = _Fold(case, end)
+    for at in range(0, case["prefix"], 2048):
+        fold.append(*_inputs(case, gen, min(2048, case["prefix"] - at))[1:])
+    steps = zip(*(x.split(chunks) for x in _inputs(case, gen, sum(chunks))))
+    out = torch.cat([fold.step(q, k, v) for q, k, v in steps])
+    new = slice(case["prefix"], end)
+    rows = [fold.k[:, new], fold.v[:, new]] if case["cache"] == "plain" else [None, None] + [s[:, new] for s in fold.scales]
+    return {"out": out.cpu() if case["host"] else out, "rows": rows}
