@@ -20,7 +20,7 @@
 // kernel below merges the slots of each KV head in order.
 //
 // Roles (384 threads): warps 0-3 / 4-7 softmax of row tile 0 / 1 (one thread per row; TMEM lane
-// = row), warp 8 TMA producer (Q per piece, then K(j), V(j), ... through a 5-slot ring), warps 9
+// = row), warp 8 TMA producer (Q per piece, then K(j), V(j), ... through a 4-slot ring), warps 9
 // and 10 tcgen05.mma issuers of row tile 0 and 1 (warp 9 owns the TMEM allocation); warp 11 only
 // completes the third warpgroup, which hands registers to the softmax warpgroups (setmaxnreg
 // 80 / 208) so that a whole 128-column score row stays in registers after one tensor-memory load.
@@ -38,9 +38,21 @@
 // a share of the exponentials to an FMA-pipe polynomial was measured and did not pay here: the
 // scheduler's issue port, not the special-function unit alone, is what the softmax saturates.)
 //
-// The exponential phases of the two row tiles are sequenced per scheduler (warp w of tile 0 and
-// warp w of tile 1 alternate strictly), which keeps the tiles in antiphase: one tile's softmax
-// runs under the other tile's MMAs.
+// What bounds the kernel is the chain of one row tile: softmax -> P V -> Q K^T (its scores land on the
+// probabilities) -> softmax.  Timelines of that chain (P V and Q K^T issued after the whole softmax): ~1750
+// cycles of softmax, then ~1550 from its last hand-over to the next scores, 768 of them tensor work and the rest
+// hand-over latency; two tiles in antiphase leave the tensor pipe 57 % busy.  Chunks of two row tiles on bf16
+// rows (kEarly) therefore put the probabilities of keys 64-127 into shared memory (swizzled as an A operand)
+// instead of tensor memory: once the first half's P V is issued nothing of the tile is left in the score columns,
+// and the next Q K^T runs under the softmax's second half.  The two issuers take turns on (first P V, Q K^T), which
+// keeps the tiles in antiphase.  Measured against the order above, cycles of a CTA: 256 tokens at prefix 61 K
+// 380 -> 341 thousand, 2048 tokens at prefix 14 K 424 -> 380 thousand; time 274 -> 257 us (at the power cap, the
+// clock settles 4 % lower) and 540 -> 505 us.  It takes a K/V slot of shared memory: quantised storage, which has
+// none to spare (two raw slots instead of three cost 10 %), and the two-stream mode keep the order above, and there
+// the exponential phases of the two tiles are sequenced per scheduler (warp w of tile 0 and warp w of tile 1
+// alternate strictly) to the same end.  Also measured: 64-key steps with two score buffers per tile (Q K^T of N = 64
+// reads shared memory at 128 bytes a cycle for 2/3 of the rate: no gain), and the maximum taken under the
+// exponentials with a second pass where it grew (5 % in cycles, but not on top of the early issue).
 //
 // Short chunks (at most 128 / G tokens: decode, question chunk) have one row tile only.  The two
 // tile slots then work on the same 128 rows and take alternate key tiles ("two streams"), each
@@ -72,6 +84,10 @@ constexpr int kSlots = 5;
 constexpr int kThreads = 384;
 constexpr uint32_t kOffQ = 0;                         // 2 tiles
 constexpr uint32_t kOffKV = 2 * kTileBytes;           // kSlots tiles
+// two row tiles on bf16 rows (kEarly): a ring of four slots, behind it one panel per row tile for the
+// probabilities of a tile's keys 64-127
+constexpr int kSlotsEarly = 4;
+constexpr uint32_t kOffP = kOffKV + kSlotsEarly * kTileBytes;
 constexpr uint32_t kOffCtl = kOffKV + kSlots * kTileBytes;
 constexpr uint32_t kSmemBytes = kOffCtl + 512 + 1024; // + control block + alignment slack
 // int8 cache storage (kQuant): 512 threads (warps 12-15 expand code tiles to bf16 tiles), three
@@ -90,7 +106,7 @@ constexpr float kRescaleThreshold = 8.0f;             // log2 units
 // barrier indices inside the control block
 constexpr int kRingBars = 6;                  // 5 slots of the shared ring, or 2 x 3 slots of the per-stream rings
 enum { B_QFULL = 0, B_QEMPTY = 1, B_FULL0 = 2, B_EMPTY0 = B_FULL0 + kRingBars, B_SFULL0 = B_EMPTY0 + kRingBars,
-       B_PA0 = B_SFULL0 + 2, B_PB0 = B_PA0 + 2, B_OFINAL0 = B_PB0 + 2, B_TURN0 = B_OFINAL0 + 2,
+       B_PA0 = B_SFULL0 + 2, B_PB0 = B_PA0 + 2, B_PVDONE0 = B_PB0 + 2, B_TURN0 = B_PVDONE0 + 2,
        B_DRAIN0 = B_TURN0 + 8, B_RAWFULL0 = B_DRAIN0 + 2, B_RAWEMPTY0 = B_RAWFULL0 + kRawSlots,
        B_COUNT = B_RAWEMPTY0 + kRawSlots };
 
@@ -142,11 +158,14 @@ __device__ __forceinline__ void exp_half(const uint32_t *v, uint32_t *p, float2 
 // completes on the partner's FULL barrier, into the partner's; a slot is free once the issuers of BOTH CTAs
 // have committed their reads of it.  Each SM then expands half the codes.  The host launches this variant only
 // when every row pair has two row tiles (a chunk of a multiple of 512 / G tokens).
-template <bool kWindow, int kQuant, bool kPair = false>
+// kEarly (bf16 rows, chunks of two row tiles): Q K^T of the next key tile is issued under the softmax of the
+// current one, see the issuer.
+template <bool kWindow, int kQuant, bool kPair, bool kEarly>
 __global__ void __launch_bounds__(kQuant ? kThreadsQ8 : kThreads, 1)
 attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                const __grid_constant__ CUtensorMap map_v) {
-    constexpr int NS = kQuant ? kSlotsQ8 : kSlots;        // slots of the shared ring
+    static_assert(!kEarly || kQuant == 0, "the early issue needs the space of a K/V slot for its probabilities");
+    constexpr int NS = kQuant ? kSlotsQ8 : kEarly ? kSlotsEarly : kSlots;        // slots of the shared ring
     constexpr int SR = kQuant ? 2 : 3;                     // slots of each stream's own ring
     constexpr uint32_t offCtl = kQuant ? kOffCtlQ8 : kOffCtl;
     constexpr uint32_t rawBytes = kQuant == 4 ? kRawBytes / 2 : kRawBytes;   // bytes of a 128-row code tile
@@ -172,7 +191,7 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
     // streams == 2 (chunks of at most 128 / G tokens, i.e. one row tile): the two tile slots work on
     // the SAME 128 rows and take alternate key tiles, so that one stream's softmax still runs under
     // the other stream's MMAs; each stream leaves its own partial result.
-    const int streams = a.streams;
+    const int streams = kEarly ? 1 : a.streams;
     const bool direct = a.ngroups == a.Hkv && streams == 1;
 
     // key tiles: this row pair needs tiles below nt_need; the group's share of the
@@ -214,7 +233,7 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
             mbar_init(bar(B_SFULL0 + i), 1);
             mbar_init(bar(B_PA0 + i), 4);
             mbar_init(bar(B_PB0 + i), 4);
-            mbar_init(bar(B_OFINAL0 + i), 1);
+            mbar_init(bar(B_PVDONE0 + i), 1);
         }
         for (int w = 0; w < 8; ++w) mbar_init(bar(B_TURN0 + w), 1);
         mbar_init(bar(B_DRAIN0), 1);
@@ -240,7 +259,7 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
         ctl->clk0 = clock64();
         ctl->ns0 = global_ns();
     }
-    // K/V tile slots.  Two row tiles: one ring of 5 that both issuers walk in step.  Two streams:
+    // K/V tile slots.  Two row tiles: one ring of 4 (quantised storage: 3) that both issuers walk in step.  Two streams:
     // each stream owns a ring of 3 (the sixth slot is the second Q tile, unused there), because a
     // parity wait is only sound for a thread that watches every use of its barrier in order.
     auto slot_addr = [&](int sl) { return base + (sl < NS ? kOffKV + (uint32_t)sl * kTileBytes : kOffQ + kTileBytes); };
@@ -448,12 +467,16 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
                 }
             };
             // 16 keys = 8 packed columns of P per MMA; half h covers keys 64h .. 64h+63
+            const uint64_t pdesc = desc_kmajor(base + kOffP + i * kPanel);
             auto issue_pv_half = [&](int slot, int h, bool accumulate) {
                 const uint64_t vdesc = desc_mnmajor(slot_addr(slot));
 #pragma unroll
-                for (int kk = 4 * h; kk < 4 * h + 4; ++kk)
-                    tc_mma_ts(t_o, t_s + kk * 8, vdesc + (uint64_t)((kk * 2048) >> 4), kIdescPV,
-                              (accumulate || kk > 4 * h) ? 1u : 0u);
+                for (int kk = 4 * h; kk < 4 * h + 4; ++kk) {
+                    if (kEarly && h == 1)
+                        tc_mma(t_o, pdesc + (uint64_t)(((kk - 4) * 32) >> 4), vdesc + (uint64_t)((kk * 2048) >> 4), kIdescPV, 1u);
+                    else
+                        tc_mma_ts(t_o, t_s + kk * 8, vdesc + (uint64_t)((kk * 2048) >> 4), kIdescPV, (accumulate || kk > 4 * h) ? 1u : 0u);
+                }
             };
             // a K/V slot is free once its readers have run: in the paired variant the partner's expansion warps
             // wait for my reads as well (they write my slot), so the commit goes to both CTAs' barriers
@@ -462,6 +485,7 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
                 else tc_commit(bar(B_EMPTY0 + slot));
             };
             int tg = 0, it = 0, pc = 0;   // ring loads before this piece, my key tiles issued, pieces so far
+            int turns = 0;                // (kEarly) my turns on the tensor pipe so far
             bool ok = true;
             // load number -> slot and parity: shared ring (number counts every load) or my own ring
             // (number counts my loads: K of my m-th tile is 2m, its V 2m + 1)
@@ -475,51 +499,58 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
                 ok = mbar_wait(bar(B_QFULL), pc & 1, ctl, a.status);
                 if (!ok) break;
                 tc_fence_after();
-                int jlast = -1;
-                for (int j = j0; j < ntiles && ok; j += jstep, ++it) {
+                // Per key tile: first half of P V (j - 1), second half, Q K^T (j).  The scores overwrite the
+                // probabilities, and this thread's MMAs run in order.  kEarly: Q K^T (j) goes between the halves and
+                // runs under the softmax's second half of tile j - 1, whose probabilities come through shared
+                // memory.  The two row tiles then take turns on (first half, Q K^T): if both were issued side by
+                // side both score tiles would come late, and the softmaxes of the two tiles would fall into step.
+                int jprev = -1;
+                for (int j = j0; ok; j += jstep) {
+                    const bool more = j < ntiles;
+                    if (!more) tc_commit(bar(B_QEMPTY));          // every Q K^T of mine in this piece has been issued
+                    if (!more && jprev < 0) break;
                     const int tk = streams == 2 ? 2 * it : tg + 2 * j;
-                    int kslot, vslot;
-                    uint32_t kpar, vpar;
-                    ring(tk, kslot, kpar);
-                    if (j > j0) {
-                        ring(tk - 1, vslot, vpar);                               // V of my previous tile
-                        ok = mbar_wait(bar(B_FULL0 + vslot), vpar, ctl, a.status);
-                        if (ok) ok = mbar_wait(bar(B_PA0 + i), (it - 1) & 1, ctl, a.status);
-                        if (!ok) break;
-                        tc_fence_after();
-                        issue_pv_half(vslot, 0, j - jstep > j0);
-                        ok = mbar_wait(bar(B_PB0 + i), (it - 1) & 1, ctl, a.status);
-                        if (!ok) break;
+                    int kslot = 0, vslot = 0;
+                    uint32_t kpar = 0, vpar = 0;
+                    if (more) ring(tk, kslot, kpar);
+                    auto second_half = [&]() -> bool {
+                        if (!mbar_wait(bar(B_PB0 + i), (it - 1) & 1, ctl, a.status)) return false;
                         tc_fence_after();
                         issue_pv_half(vslot, 1, true);
+                        if (kEarly || !more) tc_commit(bar(B_PVDONE0 + i));
                         commit_empty(vslot);
+                        return true;
+                    };
+                    if (jprev >= 0) {
+                        ring(streams == 2 ? 2 * it - 1 : tg + 2 * jprev + 1, vslot, vpar);
+                        ok = mbar_wait(bar(B_FULL0 + vslot), vpar, ctl, a.status);
+                        if (ok) ok = mbar_wait(bar(B_PA0 + i), (it - 1) & 1, ctl, a.status);
+                        if (kEarly && ok && tiles == 2 && (i == 1 || turns > 0))
+                            ok = mbar_wait(bar(B_TURN0 + i), (i == 0 ? turns - 1 : turns) & 1, ctl, a.status);
+                        if (!ok) break;
+                        tc_fence_after();
+                        issue_pv_half(vslot, 0, jprev > j0);
+                        if (!kEarly) ok = second_half();
+                        if (!ok) break;
                     }
-                    ok = mbar_wait(bar(B_FULL0 + kslot), kpar, ctl, a.status);
-                    if (!ok) break;
-                    tc_fence_after();
-                    issue_qk(kslot);
-                    tc_commit(bar(B_SFULL0 + i));
-                    commit_empty(kslot);
-                    jlast = j;
+                    if (more) {
+                        ok = mbar_wait(bar(B_FULL0 + kslot), kpar, ctl, a.status);
+                        if (!ok) break;
+                        tc_fence_after();
+                        issue_qk(kslot);
+                        tc_commit(bar(B_SFULL0 + i));
+                        commit_empty(kslot);
+                    }
+                    if (kEarly && jprev >= 0) {
+                        if (tiles == 2) mbar_arrive(bar(B_TURN0 + (i ^ 1)));
+                        ++turns;
+                        ok = second_half();
+                    }
+                    if (!more || !ok) break;
+                    jprev = j;
+                    ++it;
                 }
                 if (!ok) break;
-                tc_commit(bar(B_QEMPTY));          // every Q K^T of mine in this piece has been issued
-                if (jlast >= 0) {
-                    int vslot;
-                    uint32_t vpar;
-                    ring(streams == 2 ? 2 * it - 1 : tg + 2 * jlast + 1, vslot, vpar);
-                    ok = mbar_wait(bar(B_FULL0 + vslot), vpar, ctl, a.status);
-                    if (ok) ok = mbar_wait(bar(B_PA0 + i), (it - 1) & 1, ctl, a.status);
-                    if (!ok) break;
-                    tc_fence_after();
-                    issue_pv_half(vslot, 0, jlast > j0);
-                    ok = mbar_wait(bar(B_PB0 + i), (it - 1) & 1, ctl, a.status);
-                    if (!ok) break;
-                    tc_fence_after();
-                    issue_pv_half(vslot, 1, true);
-                    tc_commit(bar(B_OFINAL0 + i));
-                    commit_empty(vslot);
-                }
                 tg += 2 * ntiles;
                 ++pc;
             }
@@ -550,6 +581,7 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
         const float2 sl2v = make_float2(sl2, sl2);
         const int64_t nG = (int64_t)nmax * G;                 // rows of a partial slot
 
+        const uint32_t p_row = base + kOffP + i * kPanel + (uint32_t)r * 128u;     // (kEarly) my row of the probability panel
         int it = 0, oc = 0;            // my key tiles and my finished pieces so far
         int turn_base = 0;             // turns (see below) both tile slots have taken before this piece
         bool ok = i < tiles;
@@ -561,7 +593,8 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
             // happens with two streams, passes its spare turns without doing anything).  Strict
             // alternation is what a parity wait can follow: neither barrier is ever more than one
             // phase away from what its waiter expects.
-            const int nturns = ntiles <= 0 ? 0 : (streams == 2 ? (ntiles + 1) / 2 : ntiles);
+            // (kEarly: the issuers take the turns instead.)
+            const int nturns = (kEarly || ntiles <= 0) ? 0 : (streams == 2 ? (ntiles + 1) / 2 : ntiles);
             const int mine = ntiles > j0 ? (ntiles - j0 + jstep - 1) / jstep : 0;
             auto take_turn = [&](int g) -> bool {      // wait until turn g of this slot may start
                 bool got = true;
@@ -572,8 +605,13 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
                 }
                 return __all_sync(0xffffffffu, got);
             };
+            // (kEarly) every P V of mine so far has run
+            auto wait_pv = [&]() -> bool {
+                const bool got = mbar_wait(bar(B_PVDONE0 + i), (it - 1) & 1, ctl, a.status);
+                return __all_sync(0xffffffffu, got);
+            };
             auto pass_spare_turns = [&]() -> bool {
-                for (int t = mine; t < nturns && tiles == 2; ++t) {
+                for (int t = mine; !kEarly && t < nturns && tiles == 2; ++t) {
                     if (!take_turn(turn_base + t)) return false;
                     __syncwarp();
                     if (lane == 0) mbar_arrive(bar(B_TURN0 + (i == 0 ? 4 : 0) + (warp & 3)));
@@ -600,14 +638,15 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
                 if (!ok) break;
                 tc_fence_after();
                 if (!warp_live) {
-                    if (tiles == 2) ok = take_turn(turn_base + k);
+                    if (kEarly) { if (k > 0) ok = wait_pv(); }
+                    else if (tiles == 2) ok = take_turn(turn_base + k);
                     if (!ok) break;
                     tc_fence_before();
                     __syncwarp();
                     if (lane == 0) {
                         mbar_arrive(bar(B_PA0 + i));
                         mbar_arrive(bar(B_PB0 + i));
-                        mbar_arrive(bar(B_TURN0 + (i == 0 ? 4 : 0) + (warp & 3)));
+                        if (!kEarly) mbar_arrive(bar(B_TURN0 + (i == 0 ? 4 : 0) + (warp & 3)));
                     }
                     continue;
                 }
@@ -648,7 +687,13 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
                     l *= alpha;
                     m_ref = m_new;
                     if (k > 0) {
-                        // the commit that completed this S also covers my previous P V: O is quiescent here
+                        // O must be quiescent: the commit that completed this S also covers my previous P V
+                        // (kEarly: not its second half, which has a commit of its own)
+                        if (kEarly) {
+                            ok = wait_pv();
+                            if (!ok) break;
+                            tc_fence_after();
+                        }
                         const float2 av = make_float2(alpha, alpha);
 #pragma unroll 1
                         for (int c0 = 0; c0 < 128; c0 += 32) {
@@ -674,7 +719,7 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
                 // The two row tiles' warps that share a scheduler take turns on the exponentials:
                 // run side by side they halve each other's special-function rate and both tiles
                 // fall into step, leaving the tensor pipe idle while both are in their softmax.
-                if (tiles == 2) ok = take_turn(turn_base + k);
+                if (!kEarly && tiles == 2) ok = take_turn(turn_base + k);
                 if (!ok) break;
 
                 // probabilities; the first 64 keys are handed over before the rest is computed
@@ -686,13 +731,23 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
                 __syncwarp();
                 if (lane == 0) mbar_arrive(bar(B_PA0 + i));
                 exp_half(sc + 64, p, sl2v, negv, acc0, acc1);
-                KVF_TMEM_ST32(p, 0, t_s + 32);
-                tmem_wait_st();
-                tc_fence_before();
+                if (kEarly) {
+                    if (k > 0) ok = wait_pv();      // my previous P V read this panel (and every phase is waited for)
+                    if (!ok) break;
+#pragma unroll
+                    for (int c = 0; c < 8; ++c)
+                        asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(p_row + (uint32_t)((c ^ (r & 7)) << 4)),
+                                     "r"(p[4 * c]), "r"(p[4 * c + 1]), "r"(p[4 * c + 2]), "r"(p[4 * c + 3]) : "memory");
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the MMAs read through the async proxy
+                } else {
+                    KVF_TMEM_ST32(p, 0, t_s + 32);
+                    tmem_wait_st();
+                    tc_fence_before();
+                }
                 __syncwarp();
                 if (lane == 0) {
                     mbar_arrive(bar(B_PB0 + i));
-                    mbar_arrive(bar(B_TURN0 + (i == 0 ? 4 : 0) + (warp & 3)));   // the other tile's turn
+                    if (!kEarly) mbar_arrive(bar(B_TURN0 + (i == 0 ? 4 : 0) + (warp & 3)));   // the other tile's turn
                 }
                 const float2 acc = __fadd2_rn(acc0, acc1);
                 l += acc.x + acc.y;
@@ -701,7 +756,7 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
             ok = pass_spare_turns();
             if (!ok) break;
 
-            ok = mbar_wait(bar(B_OFINAL0 + i), oc & 1, ctl, a.status);
+            ok = mbar_wait(bar(B_PVDONE0 + i), (kEarly ? it - 1 : oc) & 1, ctl, a.status);
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
             ++oc;
@@ -710,6 +765,58 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
             const float inv = l > 0.f ? 1.f / l : 0.f;
             const float lse2 = l > 0.f ? m_ref * sl2 + log2f(l) : -INFINITY;
             const int64_t row = ((int64_t)cb * nmax + tok) * a.H + kvh * a.G + gi;
+            if (kEarly) {
+                // A thread holds a whole row, and rows lie 512 (256) bytes apart: stored as they are they would
+                // leave as 16-byte pieces (3.6 us for the 128 KiB of partial results of a CTA).  Each warp turns
+                // its 32 rows round in its part of the probability panel, whose last P V has run: 128 bytes of
+                // every row at a time, 16-byte chunks swizzled by the row, written out as whole 128-byte lines.
+                const uint32_t stage = base + kOffP + (uint32_t)warp * 4096u;
+                const int rw = row0 + i * kRows + (warp & 3) * 32;       // the warp's first row
+                auto emit = [&](const uint32_t (&w)[32], int byte0) {
+                    __syncwarp();                  // the segment before has been read
+#pragma unroll
+                    for (int c = 0; c < 8; ++c)
+                        asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(stage + (uint32_t)lane * 128u + (uint32_t)((c ^ (lane & 7)) << 4)),
+                                     "r"(w[4 * c]), "r"(w[4 * c + 1]), "r"(w[4 * c + 2]), "r"(w[4 * c + 3]) : "memory");
+                    __syncwarp();
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) {
+                        const int rr = 4 * q + (lane >> 3), c = lane & 7, R1 = rw + rr, tok1 = R1 / G, gi1 = R1 % G;
+                        uint4 v;
+                        asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+                                     : "r"(stage + (uint32_t)rr * 128u + (uint32_t)((c ^ (rr & 7)) << 4)) : "memory");
+                        if (tok1 >= n || gi1 >= a.G) continue;
+                        char *dst;
+                        if (!direct) dst = reinterpret_cast<char *>(a.part_o + (prow - R + R1) * kD);
+                        else dst = reinterpret_cast<char *>(a.out) + (((int64_t)cb * nmax + tok1) * a.H + kvh * a.G + gi1) * (kD * (a.out_f32 ? 4 : 2));
+                        *reinterpret_cast<uint4 *>(dst + byte0 + c * 16) = v;
+                    }
+                };
+                if (!direct || a.out_f32) {
+#pragma unroll
+                    for (int c0 = 0; c0 < 128; c0 += 32) {
+                        uint32_t w[32];
+                        KVF_TMEM_LD32(w, 0, t_o + c0);
+                        tmem_wait_ld();
+#pragma unroll
+                        for (int e = 0; e < 32; ++e) w[e] = __float_as_uint(__uint_as_float(w[e]) * inv);
+                        emit(w, c0 * 4);
+                    }
+                } else {
+#pragma unroll
+                    for (int c0 = 0; c0 < 128; c0 += 64) {
+                        uint32_t o[64], w[32];
+                        KVF_TMEM_LD32(o, 0, t_o + c0);
+                        KVF_TMEM_LD32(o, 32, t_o + c0 + 32);
+                        tmem_wait_ld();
+#pragma unroll
+                        for (int e = 0; e < 32; ++e) w[e] = pack_bf16(__uint_as_float(o[2 * e]) * inv, __uint_as_float(o[2 * e + 1]) * inv);
+                        emit(w, c0 * 2);
+                    }
+                }
+                // (the panel goes back to the probabilities; the next ones are stored after a wait_pv of every lane)
+                __syncwarp();
+            } else {
 #pragma unroll
             for (int c0 = 0; c0 < 128; c0 += 32) {
                 uint32_t o[32];
@@ -739,6 +846,7 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
                         dst[c] = make_uint4(w[0], w[1], w[2], w[3]);
                     }
                 }
+            }
             }
             if (valid) {
                 if (!direct) a.part_lse[prow] = lse2;
@@ -923,13 +1031,14 @@ cudaError_t launch_attn_tc(const AttnArgs &a, const TcMaps &maps, cudaStream_t s
     static_assert(kSmemBytes <= 232448, "shared memory budget of one CTA");
     static_assert(kSmemBytesQ8 <= 232448, "shared memory budget of one CTA (int8 storage)");
     const bool quant = a.quant_bits != 0;
-    auto kernel = a.quant_bits == 8 ? (a.win_lo > 0 ? attn_tc_kernel<true, 8> : attn_tc_kernel<false, 8>)
-                : a.quant_bits == 4 ? (a.win_lo > 0 ? attn_tc_kernel<true, 4> : attn_tc_kernel<false, 4>)
-                                    : (a.win_lo > 0 ? attn_tc_kernel<true, 0> : attn_tc_kernel<false, 0>);
+    auto kernel = a.quant_bits == 8 ? (a.win_lo > 0 ? attn_tc_kernel<true, 8, false, false> : attn_tc_kernel<false, 8, false, false>)
+                : a.quant_bits == 4 ? (a.win_lo > 0 ? attn_tc_kernel<true, 4, false, false> : attn_tc_kernel<false, 4, false, false>)
+                                    : a.streams == 1      ? (a.win_lo > 0 ? attn_tc_kernel<true, 0, false, true> : attn_tc_kernel<false, 0, false, true>)
+                                    : (a.win_lo > 0 ? attn_tc_kernel<true, 0, false, false> : attn_tc_kernel<false, 0, false, false>);
     const uint32_t smem = quant ? kSmemBytesQ8 : kSmemBytes;
     dim3 grid(attn_tc_row_pairs(a.n, a.Gp), a.ngroups, a.batch);
     if (pair_launch_ok(a)) {
-        auto paired = a.quant_bits == 8 ? attn_tc_kernel<false, 8, true> : attn_tc_kernel<false, 4, true>;
+        auto paired = a.quant_bits == 8 ? attn_tc_kernel<false, 8, true, false> : attn_tc_kernel<false, 4, true, false>;
         cudaError_t e = raise_smem_limit_once(reinterpret_cast<const void *>(paired), (int)smem);
         if (e != cudaSuccess) return e;
         if (pair_clusters_fit(reinterpret_cast<const void *>(paired), smem))
