@@ -319,6 +319,7 @@ kvf_status build_maps(kvf_cache *c) {
 
 struct Plan {
     bool qdec;     // a few query rows on a bf16 or quantised cache: the decode kernel that feeds MMAs from registers
+    bool small;    // head_dim 64, a small step: one launch does all of it (fold_small.cu)
     bool tc;
     int splits;    // CUDA-core path: splits of the key range; tensor-core path: ranges per KV head (rounded up)
     int ngroups;   // tensor-core path: ranges of the (KV head, key tile) line
@@ -334,10 +335,10 @@ int64_t window_lo(const kvf_cache *c, int64_t prefix) {
     return lo <= c->n_sink ? 0 : lo;       // the window reaches the sinks: nothing is hidden
 }
 
-Plan make_plan(const kvf_cache *c, int n, int64_t prefix, int batch = 1, int64_t part_rows_cap = -1) {
+Plan make_plan(const kvf_cache *c, int n, int64_t prefix, int batch = 1, int64_t part_rows_cap = -1, bool one_launch = true) {
     if (part_rows_cap < 0) part_rows_cap = c->part_rows_cap;
     Plan p;
-    p.qdec = false;
+    p.qdec = p.small = false;
     p.tc = c->tc || c->tc32;
     p.ngroups = 0;
     const int64_t L = prefix + n;
@@ -406,6 +407,20 @@ Plan make_plan(const kvf_cache *c, int n, int64_t prefix, int batch = 1, int64_t
         return p;
     }
     const int64_t nt = (L + 63) / 64 - WindowTiles(window_lo(c, prefix), c->n_sink, 64).skip;
+    if (one_launch && c->cfg.head_dim == 64 && c->force_splits <= 0 && !(c->cfg.flags & KVF_FORCE_SIMT)) {
+        // Small steps: rotate, append, attention and merge in one launch, up to 4.5 (32 query rows x 64 keys) per
+        // SM.  us per step through three launches and through one (fp32): 64 tokens of 4 / 1 heads at prefix 0: 13.0,
+        // 7.1; 448: 33.9, 8.8; 1984: 34.2, 19.2; 256 tokens at prefix 0: 33.2, 10.4; 1024 (640 such pieces): 35.7,
+        // 31.9; 3840 (2048): 51.1, 69.4.
+        const int tiles = fold_small_row_tiles(n, c->G) * Hkv;
+        if (2 * tiles * nt <= 9 * (int64_t)c->sm_count) {
+            p.small = true;
+            p.splits = fold_small_ranks(tiles, nt, c->sm_count);
+            p.ctas = tiles * p.splits;
+            p.kernels = 1;
+            return p;
+        }
+    }
     const int units = attn_simt_ctas(n, c->G, Hkv, 1);
     const int target = c->sm_count * 2;
     int64_t max_splits = part_rows_cap / ((int64_t)n * c->cfg.n_q_heads);
@@ -535,6 +550,25 @@ kvf_status join_combine(kvf_cache *c, cudaStream_t st) {
     return KVF_OK;
 }
 
+// A step in one launch reads its inputs while other CTAs write: its results and the cache may not overlap the inputs
+// (three launches read all inputs first), except the output rows lying exactly over the queries' (a row tile reads
+// its own queries before it writes).
+bool disjoint_step(const kvf_cache *c, const void *q, const void *k_new, const void *v_new, int n, const void *out, const float *lse) {
+    const kvf_config &f = c->cfg;
+    const size_t eb = elem_bytes(f.dtype), ob = (f.flags & KVF_OUT_F32) ? 4 : eb;
+    struct Range { const void *p; size_t bytes; };
+    const size_t qe = (size_t)n * f.n_q_heads * f.head_dim, ke = (size_t)n * f.n_kv_heads * f.head_dim;
+    const Range in[3] = {{q, qe * eb}, {k_new, ke * eb}, {v_new, ke * eb}};
+    const Range res[3] = {{out, qe * ob}, {lse, (size_t)n * f.n_q_heads * 4}, {c->storage, 2 * c->plane_bytes}};
+    for (int i = 0; i < 3; ++i)
+        for (int o = 0; o < 3; ++o) {
+            if (!in[i].p || !res[o].p || (i == 0 && o == 0 && q == out && ob == eb)) continue;
+            const uintptr_t a = reinterpret_cast<uintptr_t>(in[i].p), b = reinterpret_cast<uintptr_t>(res[o].p);
+            if (a < b + res[o].bytes && b < a + in[i].bytes) return false;
+        }
+    return true;
+}
+
 kvf_status step_impl(kvf_cache *c, const void *q, const void *k_new, const void *v_new, int32_t n,
                      int64_t pos0, void *out, float *lse, cudaStream_t st) {
     const kvf_config &f = c->cfg;
@@ -542,7 +576,7 @@ kvf_status step_impl(kvf_cache *c, const void *q, const void *k_new, const void 
     // k_new == null: queries only (kvf_attend) - nothing is appended, every query row sees the P rows held
     const bool attend = k_new == nullptr;
     const int64_t L = attend ? P : P + n;                     // rows the step's queries can see at most
-    const Plan plan = make_plan(c, n, L - n);
+    const Plan plan = make_plan(c, n, L - n, 1, -1, disjoint_step(c, q, k_new, v_new, n, out, lse));
     const bool behind = c->comb_stream != nullptr;
     unsigned long long capture = 0;
     if (behind) {
@@ -606,7 +640,9 @@ kvf_status step_impl(kvf_cache *c, const void *q, const void *k_new, const void 
     // plain launches for long tensor-bound steps, dependent launches for short ones (see g_pdl_allowed)
     const PdlScope pdl(!long_step(c, plan, aa.streams, L));
     cudaError_t e;
-    if (c->quant) {
+    if (plan.small) {
+        e = cudaSuccess;                   // (the attention launch rotates and appends)
+    } else if (c->quant) {
         // int8 storage: rotate + quantise + append (the attention kernel expands the code tiles itself)
         ProfScope ps(c, st, 0);
         e = launch_rope_append_q8(ra, c->qp, (f.flags & KVF_ROPE_INTERLEAVED) != 0, 1, st);
@@ -615,10 +651,11 @@ kvf_status step_impl(kvf_cache *c, const void *q, const void *k_new, const void 
         e = launch_rope_append(ra, f.dtype, (f.flags & KVF_ROPE_INTERLEAVED) != 0, 1, st);
     }
     if (e != cudaSuccess) return cuda_fail(e, "rope_append launch");
-    c->launches++;
+    if (!plan.small) c->launches++;
     {
         ProfScope ps(c, st, 1);
-        if (plan.qdec) e = launch_attn_q8_decode(aa, c->maps, st);
+        if (plan.small) e = launch_fold_small(ra, aa, f.dtype, (f.flags & KVF_ROPE_INTERLEAVED) != 0, st);
+        else if (plan.qdec) e = launch_attn_q8_decode(aa, c->maps, st);
         else if (c->tc) e = launch_attn_tc(aa, c->maps, st);
         else if (c->tc32) e = launch_attn_tc32(aa, st);
         else e = launch_attn_simt(aa, f.dtype, st, nullptr);

@@ -240,6 +240,11 @@ cudaError_t launch_attn_simt(const AttnArgs &a, int dtype, cudaStream_t s, int *
 cudaError_t launch_combine(const AttnArgs &a, int dtype, cudaStream_t s);
 int attn_simt_ctas(int n, int G, int Hkv, int splits);
 
+// Whole small step in one launch (head_dim 64; fold_small.cu): AttnArgs::splits = CTAs of a cluster.
+int fold_small_row_tiles(int n, int G);      // row tiles per KV head = grid.x
+int fold_small_ranks(int row_tiles, int64_t key_tiles, int sm_count);     // slices of the 64-row key tiles (row_tiles: of all KV heads)
+cudaError_t launch_fold_small(const RopeAppendArgs &r, const AttnArgs &a, int dtype, bool interleaved, cudaStream_t s);
+
 // Tensor-core path (bf16, head_dim 128).
 struct TcMaps {
     CUtensorMap q, k, v;

@@ -1,0 +1,88 @@
+"""Small steps of head_dim 64 take one launch (fold_small.cu): against the three-launch path (KVF_FORCE_SIMT) with every
+bit of the cache, and against the oracle through the chains of test_fold_gpu.py.
+
+Tolerance: both paths compute in fp32 and differ in the order of their sums: 64-term scores up to ~|s| = 8 (2^-21
+each), exponentials and output sums of unit size: a few 1e-6; a bf16 output may round the other way (one ulp, 2^-8
+relative, at |out| up to 4)."""
+import pytest
+import torch
+
+from paper_2605_12471_b200 import binding
+
+pytestmark = pytest.mark.gpu
+
+
+def _caches(h, kv, dtype, capacity, max_chunk, flags=0):
+    made = []
+    for extra in (0, binding.KVF_FORCE_SIMT):
+        c = binding.Cache(binding.make_config(h, kv, 64, dtype, capacity, max_chunk, rope_base=10000.0, flags=flags | extra))
+        c.storage.fill_(7)                 # (the value rows up to the tile boundary are cleared by both)
+        made.append(c)
+    return made
+
+
+def _inputs(h, kv, n, dtype, gen):
+    t = torch.float32 if dtype == "f32" else torch.bfloat16
+    return [torch.randn(n, heads, 64, generator=gen, device="cuda", dtype=t) for heads in (h, kv, kv)]
+
+
+def _compare(a, b, dtype):
+    (oa, la), (ob, lb) = a, b
+    tol = 1e-5 if dtype == "f32" else 2.0 ** -6
+    assert (oa.float() - ob.float()).abs().max().item() <= tol
+    assert (la - lb).abs().max().item() <= 1e-5
+
+
+# chunks at the edges of the 32-row tile, the 64-key tile and the slices; groups of 1, 3, 4, 7
+@pytest.mark.parametrize("h,kv", [(4, 1), (2, 2), (6, 2), (7, 1)])
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("flags", [0, binding.KVF_ROPE_INTERLEAVED], ids=["half", "interleaved"])
+def test_one_launch_against_three(h, kv, dtype, flags):
+    chunks = [1, 7, 8, 48, 63, 1, 64, 65, 3, 130, 250, 1, 33]
+    gen = torch.Generator(device="cuda").manual_seed(h * 10 + kv)
+    small, general = _caches(h, kv, dtype, 1000, 250, flags)
+    for n in chunks:
+        assert small.plan(n)[3] == 1 and general.plan(n)[3] >= 2
+        q, k, v = _inputs(h, kv, n, dtype, gen)
+        got = []
+        for c in (small, general):
+            lse = torch.empty(n, h, device="cuda")
+            got.append((c.fold_step(q, k, v, lse=lse), lse))
+        _compare(*got, dtype)
+        assert torch.equal(small.storage, general.storage), n
+        la, lb = torch.empty(n, h, device="cuda"), torch.empty(n, h, device="cuda")
+        _compare((small.attend(q, lse=la), la), (general.attend(q, lse=lb), lb), dtype)
+    assert small.status() == binding.KVF_OK
+
+
+def test_one_launch_under_a_window_and_with_wide_clusters():
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    for window, chunks in ((100, [64, 64, 50, 64, 1, 64]), (0, [250] * 4 + [8, 1, 32, 64])):
+        small, general = _caches(4, 1, "f32", 1500, 250)
+        if window:
+            small.set_window(4, window)
+            general.set_window(4, window)
+        for n in chunks:
+            q, k, v = _inputs(4, 1, n, "f32", gen)
+            got = []
+            for c in (small, general):
+                lse = torch.empty(n, 4, device="cuda")
+                got.append((c.fold_step(q, k, v, lse=lse), lse))
+            _compare(*got, "f32")
+            assert torch.equal(small.storage, general.storage)
+
+
+def test_results_over_the_inputs_take_the_three_launches():
+    """Output rows over the queries' own rows, and over the new keys' (2 / 2 heads: the same shape)."""
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    x = [_inputs(2, 2, 200, "f32", gen) for _ in range(2)]
+    for over in (0, 1, 2):
+        small, general = _caches(2, 2, "f32", 400, 200)
+        for ins in x:
+            want = general.fold_step(*ins)
+            mine = [t.clone() for t in ins]
+            launches = small.launch_count()
+            small.fold_step(*mine, out=mine[over])
+            assert (small.launch_count() - launches == 1) == (over == 0)
+            assert (mine[over] - want).abs().max().item() <= 1e-5
+        assert torch.equal(small.storage, general.storage)
