@@ -177,7 +177,9 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
 
     static_assert(!kPair || (kQuant != 0 && !kWindow), "the paired variant is for quantised caches without a window");
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int qpair = blockIdx.x, group = blockIdx.y;
+    // Grid (ranges, row pairs from the last to the first): the row pairs that see most keys start first and the
+    // shortest fill the tail.  (kPair: clusters along x, so x = row pair.)
+    const int qpair = kPair ? (int)blockIdx.x : (int)(gridDim.y - 1 - blockIdx.y), group = kPair ? blockIdx.y : blockIdx.x;
     const uint32_t rank = kPair ? cluster_cta_rank() : 0u;     // which of K (0) and V (1) this CTA expands
     const int cb = blockIdx.z;     // cache of a batch (0 when there is one cache)
     const int G = a.Gp;     // rows per token in the row layout (a power of two >= a.G, the query heads per KV head)
@@ -186,7 +188,7 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
     if (a.prefixes) pdl_wait();
     // tokens this cache folds; a.n is the longest chunk of the launch and the stride of the caches' blocks
     const int n = a.ns ? (int)a.ns[cb] : a.n, nmax = a.n;
-    if (blockIdx.x * 2 * kRows >= n * G) return;          // a shorter member of a batch: no row of this row pair exists
+    if (qpair * 2 * kRows >= n * G) return;          // a shorter member of a batch: no row of this row pair exists
     const int64_t P = a.prefixes ? a.prefixes[cb] : a.prefix, L = P + n * a.self_rows;
     // streams == 2 (chunks of at most 128 / G tokens, i.e. one row tile): the two tile slots work on
     // the SAME 128 rows and take alternate key tiles, so that one stream's softmax still runs under
@@ -254,7 +256,7 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
     const uint32_t tmem = *reinterpret_cast<volatile uint32_t *>(&ctl->tmem_base);
     // One CTA times itself in SM cycles and in nanoseconds: the ratio is the clock the launch ran at
     // (the last row pair: it sees the most keys of the chunk itself, so no CTA of the launch runs longer)
-    const bool clocked = blockIdx.x == gridDim.x - 1 && (blockIdx.y | blockIdx.z) == 0 && threadIdx.x == 0;
+    const bool clocked = qpair == (int)(kPair ? gridDim.x : gridDim.y) - 1 && group == 0 && blockIdx.z == 0 && threadIdx.x == 0;
     if (clocked) {
         ctl->clk0 = clock64();
         ctl->ns0 = global_ns();
@@ -1046,7 +1048,7 @@ cudaError_t launch_attn_tc(const AttnArgs &a, const TcMaps &maps, cudaStream_t s
     }
     cudaError_t e = raise_smem_limit_once(reinterpret_cast<const void *>(kernel), (int)smem);
     if (e != cudaSuccess) return e;
-    return launch_pdl(kernel, grid, dim3(quant ? kThreadsQ8 : kThreads), smem, s, a, maps.q, maps.k, maps.v);
+    return launch_pdl(kernel, dim3(grid.y, grid.x, grid.z), dim3(quant ? kThreadsQ8 : kThreads), smem, s, a, maps.q, maps.k, maps.v);
 }
 
 cudaError_t launch_combine_groups(const AttnArgs &a, cudaStream_t s) {

@@ -363,7 +363,7 @@ Plan make_plan(const kvf_cache *c, int n, int64_t prefix, int batch = 1, int64_t
     if (p.tc) {
         // one CTA per (row pair, group); the groups cut the Hkv * nt line of (KV head, key tile)
         // into equal ranges.  Whole KV heads if that fills the SMs, else as many groups as give
-        // one CTA per SM, with at least 4 key tiles each and within the partial area.
+        // one CTA per SM, with enough key tiles each and within the partial area.
         const int64_t nt = (L + kKvTile - 1) / kKvTile - WindowTiles(window_lo(c, prefix), c->n_sink, kKvTile).skip;
         // (row blocks of a KV head: 256-row pairs in the bf16 kernel, 128-row blocks in the fp32 one)
         const int pairs = c->tc32 ? attn_tc32_row_blocks(n, c->Gp) : attn_tc_row_pairs(n, c->Gp);
@@ -372,7 +372,18 @@ Plan make_plan(const kvf_cache *c, int n, int64_t prefix, int batch = 1, int64_t
             groups = (int64_t)Hkv * c->force_splits;
         } else if ((int64_t)pairs * Hkv * batch < c->sm_count) {
             groups = c->sm_count / (pairs * batch);
-            if (groups > Hkv * nt / 4) groups = Hkv * nt / 4;
+            // Fewest key tiles worth a CTA.  us per step (bf16, ranges per KV head: time), whole heads against
+            // finer cuts: 256 tokens of 32 / 8 heads, 4 key tiles: 1: 17.4, 4: 18.1; 8 tiles: 1: 24.6, 2: 23.2, 4:
+            // 20.1; 1020-row window (11 tiles) 2: 30.7, 4: 25.1; 64 tokens, 9 tiles: 2: 22.6, 4: 19.3, 6: 17.0; 200
+            // tokens of 16 / 16 heads, 14 tiles: 3: 26.1, 8: 20.3.  Two streams (a merge kernel in any case, two key
+            // tiles in flight per CTA): 32 tokens, 5 tiles: 1: 18.9, 3: 15.5; 9 tiles: 2: 18.7, 3: 16.6, 6: 18.9; 16
+            // tiles: 4: 17.3, 6: 20.2.
+            int64_t most = Hkv * nt / 4;
+            if (!c->tc32) {
+                if (attn_tc_streams(n, c->Gp) == 2) most = std::max<int64_t>(most, nt >= 5 ? 3 * Hkv : Hkv);
+                else most = nt <= 5 ? Hkv : Hkv * nt * 4 / 7;
+            }
+            if (groups > most) groups = most;
             // A group count that is a multiple of the KV heads keeps every CTA inside one KV head: one Q load
             // and one set of partial rows instead of two.  Measured at C = 256 (Llama shape): the second
             // piece costs a CTA about as long as 3.3 key tiles, so while the line is short - here below
@@ -384,16 +395,39 @@ Plan make_plan(const kvf_cache *c, int n, int64_t prefix, int batch = 1, int64_t
             }
         } else {
             // whole KV heads fill the SMs, but the last wave may be half empty (256 CTAs on 148 SMs):
-            // cut a little finer - up to twice the KV heads - if that fills the waves at least 5 %
-            // better; the price is the partial results of one chunk and the combine kernel
-            auto fill = [&](int64_t g) {
-                const int64_t ctas = (int64_t)pairs * g * batch;
-                const int64_t waves = (ctas + c->sm_count - 1) / c->sm_count;
-                return (double)ctas / (double)(waves * c->sm_count);
-            };
-            double best = fill(Hkv) + 0.05;
-            for (int64_t g = Hkv + 1; g <= 2 * Hkv && g * 4 <= Hkv * nt; ++g)
-                if (fill(g) > best) { best = fill(g); groups = g; }
+            // cut a little finer - up to twice the KV heads - if that saves more than it costs; the price is
+            // the partial results of one chunk and the merge kernel.
+            if (c->tc32) {
+                auto fill = [&](int64_t g) {
+                    const int64_t ctas = (int64_t)pairs * g * batch;
+                    const int64_t waves = (ctas + c->sm_count - 1) / c->sm_count;
+                    return (double)ctas / (double)(waves * c->sm_count);
+                };
+                double best = fill(Hkv) + 0.05;
+                for (int64_t g = Hkv + 1; g <= 2 * Hkv && g * 4 <= Hkv * nt; ++g)
+                    if (fill(g) > best) { best = fill(g); groups = g; }
+            } else {
+                // In key tiles of one CTA: the waves one after the other, each as long as its first row pair (they
+                // start longest first), and for partial results one tile per 2400 output rows: 2048 tokens of 32
+                // heads, 8 ranges (no merge) against 9: 55 / 90 us at prefix 0, 115 / 145 at 2 K, 234 / 257 at 6 K,
+                // 478 / 490 at 14 K, 1002 / 906 at 30 K - about 28 tiles of 1.9 us.
+                auto cost = [&](int64_t g) {
+                    double tiles = g > Hkv ? (double)n * c->cfg.n_q_heads * batch / 2400.0 : 0.0;
+                    const int64_t ctas = (int64_t)pairs * g * batch;
+                    for (int64_t at = 0; at < ctas; at += c->sm_count) {
+                        const int64_t pair = pairs - 1 - at / g % pairs;           // row pair of the wave's first CTA
+                        const int64_t tok = std::min<int64_t>(n, ((pair + 1) * 256 + c->Gp - 1) / c->Gp);
+                        const int64_t need = batch > 1 ? nt : nt - (L - (prefix + tok)) / kKvTile;
+                        tiles += (double)Hkv * (double)need / (double)g;
+                    }
+                    return tiles;
+                };
+                double best = cost(Hkv);
+                for (int64_t g = Hkv + 1; g <= 2 * Hkv && g * 4 <= Hkv * nt; ++g) {
+                    const double t = cost(g);
+                    if (t < best) { best = t; groups = g; }
+                }
+            }
         }
         const int streams = c->tc32 ? 1 : attn_tc_streams(n, c->Gp);
         const int64_t slots_cap = part_rows_cap / ((int64_t)n * c->Gp) / streams;   // slots = streams * (groups + Hkv - 1)
