@@ -210,7 +210,7 @@ kvf_status kvf_paged_cache_create(const kvf_config *cfg, void *dev_pool, size_t 
  * Effects, in stream order: rotate q into the workspace; write rotated k and v as rows
  * [len, len+n_tokens); attention; then the host-side length becomes len + n_tokens.
  * Errors: INVALID_ARG, CAPACITY (cache full), POS, CUDA (launch failure; length unchanged).
- * A step is two or three kernels on cuda_stream.  Short steps launch them with programmatic stream
+ * A step is two or three kernels on cuda_stream (a small one of head_dim 64 is one).  Short steps launch them with programmatic stream
  * serialisation (a kernel's set-up overlaps the tail of the one before); steps with long
  * tensor-bound attention kernels launch them plainly, which on a power-capped board is the faster
  * of the two.  KVF_DEPENDENT_LAUNCH=always or =never in the environment (read once) overrides the
@@ -337,7 +337,8 @@ float *kvf_cache_v_scales(const kvf_cache *c);
  *           need not end at KV-head boundaries; this is their number per KV head, rounded up
  *   plan[2] CTAs of the attention kernel
  *   plan[3] kernels launched by the step (3 = a combine kernel merges partial results; chunks of
- *           at most 128 / (H / Hkv) tokens always take that route on the tensor-core path)
+ *           at most 128 / (H / Hkv) tokens always take that route on the tensor-core path; 1 = a small
+ *           step of head_dim 64, unless its results overlap its inputs)
  */
 kvf_status kvf_cache_plan(const kvf_cache *c, int32_t n_tokens, int64_t prefix_len, int32_t plan[4]);
 
