@@ -47,7 +47,11 @@
 // and the next Q K^T runs under the softmax's second half.  The two issuers take turns on (first P V, Q K^T), which
 // keeps the tiles in antiphase.  Measured against the order above, cycles of a CTA: 256 tokens at prefix 61 K
 // 380 -> 341 thousand, 2048 tokens at prefix 14 K 424 -> 380 thousand; time 274 -> 257 us (at the power cap, the
-// clock settles 4 % lower) and 540 -> 505 us.  It takes a K/V slot of shared memory: quantised storage, which has
+// clock settles 4 % lower) and 540 -> 505 us.  Then 341 -> 309 thousand and 264 -> 250 us by taking latency out of the
+// softmax threads' chain: whether the panel is free is asked before the second half's arithmetic (a wait on a
+// barrier that is already complete takes ~250 cycles beside saturated shared memory), and whether a key tile
+// needs a mask is known from the tile number, without a vote.  (Leaving out the vote on the scores' wait as well: 312;
+// passing the turn ahead of the K slot's commit: no change.)  It takes a K/V slot of shared memory: quantised storage, which has
 // none to spare (two raw slots instead of three cost 10 %), and the two-stream mode keep the order above, and there
 // the exponential phases of the two tiles are sequenced per scheduler (warp w of tile 0 and warp w of tile 1
 // alternate strictly) to the same end.  Also measured: 64-key steps with two score buffers per tile (Q K^T of N = 64
@@ -579,6 +583,10 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
         // keys below `limit` are visible; a row past the chunk's end is never written, and each
         // row of S, P and O depends on that row alone, so such rows are left unmasked
         const int64_t limit = valid ? P + (tok + 1) * a.self_rows : ((int64_t)1 << 62);
+        // a key tile whose rows all lie below this needs no mask in any row of the warp (rows ascend, so the first
+        // row of the warp sees least)
+        const int tok_w = (row0 + (streams == 2 ? 0 : i * kRows) + (warp & 3) * 32) / G;
+        const int64_t clear = tok_w < n ? P + (tok_w + 1) * a.self_rows : ((int64_t)1 << 62);
         const float sl2 = a.scale_log2;
         const float2 sl2v = make_float2(sl2, sl2);
         const int64_t nG = (int64_t)nmax * G;                 // rows of a partial slot
@@ -655,7 +663,7 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
                 const int64_t key0 = (int64_t)wt.actual(kt0 + j) * kRows;
                 const int nvis = (int)max((int64_t)0, min((int64_t)kRows, limit - key0));
                 // a tile that starts before the window holds hidden columns (the sink tile, the window's first)
-                const bool masked = __any_sync(0xffffffffu, nvis < kRows) || (kWindow && key0 < a.win_lo);
+                const bool masked = key0 + kRows > clear || (kWindow && key0 < a.win_lo);
 
                 // the whole score row in registers after one load
                 uint32_t sc[128];
@@ -732,9 +740,13 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(bar(B_PA0 + i));
+                // (my previous P V read the panel the second half goes to; asked ahead of the arithmetic, for the answer
+                // takes ~200 cycles to come even if it is yes; every phase is waited for)
+                uint32_t panel_free = 1;
+                if (kEarly && k > 0) panel_free = mbar_test(bar(B_PVDONE0 + i), (it - 1) & 1);
                 exp_half(sc + 64, p, sl2v, negv, acc0, acc1);
                 if (kEarly) {
-                    if (k > 0) ok = wait_pv();      // my previous P V read this panel (and every phase is waited for)
+                    if (!__all_sync(0xffffffffu, panel_free)) ok = wait_pv();
                     if (!ok) break;
 #pragma unroll
                     for (int c = 0; c < 8; ++c)
