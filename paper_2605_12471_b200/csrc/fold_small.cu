@@ -3,7 +3,7 @@
 // The steps of a small model are a few microseconds of arithmetic behind three dependent launches (rotate +
 // append, attention, merge), and the attention kernel of attn_simt.cu, built for long key ranges, gives 256 query
 // rows to four to eight CTAs that walk their key tiles one after the other.  Here a CTA owns 32 query rows
-// (row = token * G + head-in-group) and one of up to eight slices of the key tiles; the CTAs of a row tile form a
+// (row = token * G + head-in-group) and one of up to 16 slices of the key tiles; the CTAs of a row tile form a
 // cluster and merge their (maximum, sum, output) through distributed shared memory, each finishing its share of
 // the rows.  A CTA rotates its own query rows, and the chunk's own keys where its slice holds them (no CTA reads
 // what another one writes); the CTAs of the last row tile, whose slices cover every row of the chunk, also write the
@@ -27,7 +27,7 @@ namespace {
 constexpr int BM = 32, BN = 64, D = 64, HALF = D / 2, kThreads = 256;
 constexpr int TR = 2;                // query rows per thread (x 4 keys, x 4 output columns)
 constexpr int QS = D + 4;            // padded row stride of the Q, K and probability tiles (floats)
-constexpr int kMaxRanks = 16;        // slices of the key tiles = CTAs of a cluster
+constexpr int kMaxRanks = 1 << (kFoldSmallWidths - 1);     // slices of the key tiles = CTAs of a cluster
 
 struct Smem {
     float q[BM * QS];
@@ -383,11 +383,11 @@ __global__ void __launch_bounds__(kThreads, 2) fold_small_kernel(const __grid_co
     if (ranks > 1) cluster_sync();                        // nobody leaves while a partner reads its shared memory
 }
 
-// Once per kernel and device: shared-memory limit, clusters of 16 CTAs (beyond the portable eight), and whether the
-// device can hold such a cluster.
+// Once per kernel and device: shared-memory limit, clusters of 16 CTAs (beyond the portable eight), and how many clusters
+// of each width the device holds at once.
 template <typename T, bool INTERLEAVED>
-cudaError_t prepare_once(bool *wide) {
-    struct Done { int dev; bool wide; };
+cudaError_t prepare_once(FoldSmallFit *fit) {
+    struct Done { int dev; FoldSmallFit fit; };
     static std::mutex mu;
     static std::vector<Done> done;
     int dev = 0;
@@ -396,38 +396,36 @@ cudaError_t prepare_once(bool *wide) {
     std::lock_guard<std::mutex> lock(mu);
     for (const Done &d : done)
         if (d.dev == dev) {
-            if (wide) *wide = d.wide;
+            if (fit) *fit = d.fit;
             return cudaSuccess;
         }
     auto kernel = fold_small_kernel<T, INTERLEAVED>;
     e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Smem));
     if (e != cudaSuccess) return e;
-    bool fits = false;
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
+    Done now = {dev, {}};
+    const bool wide = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+    bool refused = !wide;
+    for (int i = 0; i < kFoldSmallWidths; ++i) {
+        if ((1 << i) > 8 && !wide) break;
         cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(1, 1, kMaxRanks);
+        cfg.gridDim = dim3(1, 1, 1u << i);
         cfg.blockDim = dim3(kThreads);
         cfg.dynamicSmemBytes = sizeof(Smem);
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeClusterDimension;
         attr[0].val.clusterDim.x = 1;
         attr[0].val.clusterDim.y = 1;
-        attr[0].val.clusterDim.z = kMaxRanks;
+        attr[0].val.clusterDim.z = 1u << i;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
         int clusters = 0;
-        fits = cudaOccupancyMaxActiveClusters(&clusters, kernel, &cfg) == cudaSuccess && clusters > 0;
+        if (cudaOccupancyMaxActiveClusters(&clusters, kernel, &cfg) == cudaSuccess) now.fit.clusters[i] = clusters;
+        else refused = true;
     }
-    if (!fits) cudaGetLastError();
-    done.push_back({dev, fits});
-    if (wide) *wide = fits;
+    if (refused) cudaGetLastError();       // (a width the device refuses leaves its error behind)
+    done.push_back(now);
+    if (fit) *fit = now.fit;
     return cudaSuccess;
-}
-
-// (the four kernels differ in arithmetic only: what fits one fits all)
-bool wide_clusters() {
-    bool wide = false;
-    return prepare_once<float, false>(&wide) == cudaSuccess && wide;
 }
 
 template <typename T, bool INTERLEAVED>
@@ -455,14 +453,18 @@ cudaError_t launch_t(const RopeAppendArgs &r, const AttnArgs &a, int ranks, cuda
 
 int fold_small_row_tiles(int n, int G) { return (int)(((int64_t)n * G + BM - 1) / BM); }
 
-// Slices of the key tiles = CTAs of a cluster: a power of two, at least one key tile each, and no more than the
-// device holds at once (two CTAs per SM): a second wave costs more than longer slices (256 tokens, 4 / 1 heads, prefix
-// 1024: 8 slices 31.9 us, 16 slices - 512 CTAs - 53.9 us).
-int fold_small_ranks(int row_tiles, int64_t key_tiles, int sm_count) {
+// Slices of the key tiles = CTAs of a cluster: a power of two, at least one key tile each, and no more clusters than the
+// device holds at once: a second wave costs more than longer slices.  Two CTAs fit an SM, but a cluster stays within
+// one GPC: of 16 CTAs the device holds 14 clusters (16 row tiles, 24 key tiles: 16 slices 37.4 us, 8 slices 28.6), of 8 CTAs
+// 35 (36 row tiles, 16 key tiles: 8 slices 36.1 us, through three launches 34.4).
+int fold_small_ranks(int row_tiles, int64_t key_tiles, const FoldSmallFit &fit) {
     int ranks = 1;
-    while (ranks < kMaxRanks && 2 * ranks <= key_tiles && (int64_t)row_tiles * 2 * ranks <= 2 * sm_count) ranks *= 2;
-    return ranks == kMaxRanks && !wide_clusters() ? kMaxRanks / 2 : ranks;
+    for (int i = 1; i < kFoldSmallWidths && (1 << i) <= key_tiles && row_tiles <= fit.clusters[i]; ++i) ranks = 1 << i;
+    return ranks;
 }
+
+// (the four kernels differ in arithmetic only: what fits one fits all)
+cudaError_t fold_small_fit(FoldSmallFit *fit) { return prepare_once<float, false>(fit); }
 
 cudaError_t launch_fold_small(const RopeAppendArgs &r, const AttnArgs &a, int dtype, bool interleaved, cudaStream_t s) {
     if (a.d != D) return cudaErrorInvalidValue;

@@ -117,6 +117,7 @@ struct kvf_cache {
     bool tc;                 // bf16, head_dim 128: the tcgen05 kernel fed by TMA
     bool tc32;               // fp32, head_dim 128: the tcgen05 kernel on fp16 halves of the operands
     TcMaps maps;
+    FoldSmallFit small_fit = {};   // head_dim 64: clusters of the one-launch step the device holds
     int force_splits;
     int64_t part_rows_cap;   // rows of head_dim floats the partial area holds
     uint64_t launches;
@@ -441,20 +442,6 @@ Plan make_plan(const kvf_cache *c, int n, int64_t prefix, int batch = 1, int64_t
         return p;
     }
     const int64_t nt = (L + 63) / 64 - WindowTiles(window_lo(c, prefix), c->n_sink, 64).skip;
-    if (one_launch && c->cfg.head_dim == 64 && c->force_splits <= 0 && !(c->cfg.flags & KVF_FORCE_SIMT)) {
-        // Small steps: rotate, append, attention and merge in one launch, up to 4.5 (32 query rows x 64 keys) per
-        // SM.  us per step through three launches and through one (fp32): 64 tokens of 4 / 1 heads at prefix 0: 13.0,
-        // 7.1; 448: 33.9, 8.8; 1984: 34.2, 19.2; 256 tokens at prefix 0: 33.2, 10.4; 1024 (640 such pieces): 35.7,
-        // 31.9; 3840 (2048): 51.1, 69.4.
-        const int tiles = fold_small_row_tiles(n, c->G) * Hkv;
-        if (2 * tiles * nt <= 9 * (int64_t)c->sm_count) {
-            p.small = true;
-            p.splits = fold_small_ranks(tiles, nt, c->sm_count);
-            p.ctas = tiles * p.splits;
-            p.kernels = 1;
-            return p;
-        }
-    }
     const int units = attn_simt_ctas(n, c->G, Hkv, 1);
     const int target = c->sm_count * 2;
     int64_t max_splits = part_rows_cap / ((int64_t)n * c->cfg.n_q_heads);
@@ -474,6 +461,33 @@ Plan make_plan(const kvf_cache *c, int n, int64_t prefix, int batch = 1, int64_t
     if (splits > max_splits) splits = (int)max_splits;
     if ((int64_t)splits > nt) splits = (int)nt;
     if (splits < 1) splits = 1;
+    if (one_launch && c->cfg.head_dim == 64 && c->force_splits <= 0 && !(c->cfg.flags & KVF_FORCE_SIMT)) {
+        // Small steps: rotate, append, attention and merge in one launch, up to 4.5 (32 query rows x 64 keys) per
+        // SM.  us per step through three launches and through one (fp32): 64 tokens of 4 / 1 heads at prefix 0: 13.0,
+        // 7.1; 448: 33.9, 8.8; 1984: 34.2, 19.2; 256 tokens at prefix 0: 33.2, 10.4; 1024 (640 such pieces): 35.7,
+        // 31.9; 3840 (2048): 51.1, 69.4.
+        // A CTA walks its slice one key tile after another, while the three launches cut the key range into up to 64
+        // splits of four tiles: 31 - 38 us from a prefix of 1 K on, whatever its length, and ~8 us more where a split
+        // takes a fifth tile or their CTAs exceed the SMs.  A tile of a slice costs 3.9 us while a cluster's CTAs
+        // have an SM each and up to 6.6 where they share it, so the longest slice depends on the CTAs.  Key tiles per
+        // slice: us in one launch, in three (fp32): one token of 4 / 1 heads 7: 32.9, 35.7; 8: 36.9, 36.9; 11: 48.1, 38.0;
+        // 32: 129, 64; 48 tokens (6 row tiles) 5: 27.7, 37.2; 6: 31.6, 37.3, of 2 / 2 heads 36 - 42, 37.5; 64 tokens
+        // (8) 4: 33.0, 36.2; 5: 40.0, 37.5; 16 tokens of 32 / 8 heads (16, in clusters of 8) 3: 24.8, 35.0; 4: 31.9,
+        // 35.4 at 28 key tiles and 34.5 at 32; 160 tokens of 32 / 8 heads (uncut) 3: 30.3, 26.9.  Of 3350 steps within
+        // these limits (102 shapes, 1 - 512 key tiles, fp32 and bf16) nine measured 2 - 8 % slower than through three.
+        const int tiles = fold_small_row_tiles(n, c->G) * Hkv;
+        const int ranks = fold_small_ranks(tiles, nt, c->small_fit);
+        const int64_t at_once = (int64_t)tiles * ranks;
+        int64_t longest = at_once <= 48 ? 7 : at_once <= 80 ? 6 : at_once <= 96 ? 5 : ranks >= 16 ? 4 : ranks > 1 ? 3 : 2;
+        if (nt > 4 * (int64_t)splits || (int64_t)units * splits > c->sm_count) longest += ranks >= 16 ? 2 : 1;
+        if (2 * tiles * nt <= 9 * (int64_t)c->sm_count && nt <= longest * ranks) {
+            p.small = true;
+            p.splits = ranks;
+            p.ctas = tiles * ranks;
+            p.kernels = 1;
+            return p;
+        }
+    }
     p.splits = splits;
     p.ctas = units * splits;
     p.kernels = 2 + (splits > 1 ? 1 : 0);
@@ -759,6 +773,10 @@ kvf_status init_handle(kvf_cache *c, const kvf_config *cfg, void *storage, void 
     c->profile = false;
     c->tc = !(cfg->flags & KVF_FORCE_SIMT) && attn_tc_supported(cfg->dtype, cfg->head_dim, c->G);
     c->tc32 = !(cfg->flags & KVF_FORCE_SIMT) && attn_tc32_supported(cfg->dtype, cfg->head_dim, c->G);
+    if (cfg->head_dim == 64 && !(cfg->flags & KVF_FORCE_SIMT)) {
+        e = fold_small_fit(&c->small_fit);
+        if (e != cudaSuccess) return cuda_fail(e, "one-launch step setup");
+    }
     return KVF_OK;
 }
 

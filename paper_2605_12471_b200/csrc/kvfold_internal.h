@@ -242,7 +242,12 @@ int attn_simt_ctas(int n, int G, int Hkv, int splits);
 
 // Whole small step in one launch (head_dim 64; fold_small.cu): AttnArgs::splits = CTAs of a cluster.
 int fold_small_row_tiles(int n, int G);      // row tiles per KV head = grid.x
-int fold_small_ranks(int row_tiles, int64_t key_tiles, int sm_count);     // slices of the 64-row key tiles (row_tiles: of all KV heads)
+constexpr int kFoldSmallWidths = 5;          // clusters of 1, 2, 4, 8 and 16 CTAs
+struct FoldSmallFit {
+    int clusters[kFoldSmallWidths];          // how many of them the device holds at once (0: none)
+};
+cudaError_t fold_small_fit(FoldSmallFit *fit);     // of the current device
+int fold_small_ranks(int row_tiles, int64_t key_tiles, const FoldSmallFit &fit);     // slices of the 64-row key tiles (row_tiles: of all KV heads)
 cudaError_t launch_fold_small(const RopeAppendArgs &r, const AttnArgs &a, int dtype, bool interleaved, cudaStream_t s);
 
 // Tensor-core path (bf16, head_dim 128).

@@ -86,3 +86,27 @@ def test_results_over_the_inputs_take_the_three_launches():
             assert (small.launch_count() - launches == 1) == (over == 0)
             assert (mine[over] - want).abs().max().item() <= 1e-5
         assert torch.equal(small.storage, general.storage)
+
+
+# (n, heads, 64-row key tiles, kernels): slices of up to 7 (one row tile) and 4 (eight) key tiles take one launch, up to two
+# more where the three launches' splits take a fifth tile (no multiple of four); far beyond never
+@pytest.mark.parametrize("n,h,kv,tiles,kernels", [(1, 4, 1, 112, 1), (1, 4, 1, 113, 1), (1, 4, 1, 116, 3), (1, 4, 1, 513, 3),
+                                                  (8, 2, 2, 513, 3), (4, 14, 2, 132, 3), (64, 4, 1, 64, 1), (64, 4, 1, 68, 3)])
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_long_prefixes_take_the_launches_that_split_them(n, h, kv, tiles, kernels, dtype):
+    prefix = 64 * tiles - n
+    gen = torch.Generator(device="cuda").manual_seed(prefix)
+    small, general = _caches(h, kv, dtype, prefix + n, n)
+    held = torch.randn(small.storage.numel() // (4 if dtype == "f32" else 2), generator=gen, device="cuda", dtype=small.torch_dtype)
+    q, k, v = _inputs(h, kv, n, dtype, gen)
+    got = []
+    for c in (small, general):
+        c.storage.copy_(held.view(torch.uint8))
+        c.set_len(prefix)
+        lse = torch.empty(n, h, device="cuda")
+        before = c.launch_count()
+        got.append((c.fold_step(q, k, v, lse=lse), lse))
+        assert c.launch_count() - before == (kernels if c is small else 3)
+    assert small.plan(n, prefix)[3] == kernels
+    _compare(*got, dtype)
+    assert torch.equal(small.storage, general.storage)
