@@ -12,7 +12,7 @@
 // rows computed and never written), handled as two
 // 128-row tiles that take turns on the tensor pipe.  Keys come in 128-row tiles.  The (KV head,
 // key tile) pairs of a step are laid out on one line and cut into `ngroups` equal contiguous
-// ranges; CTA (x = row pair, y = group) runs its row pair against its group's range, which
+// ranges; CTA (row pair, group) runs its row pair against its group's range, which
 // touches at most two KV heads ("pieces").  The CTAs of a group stream the same tiles at the
 // same time, so a tile leaves HBM once and the other row pairs hit L2.  With ngroups == Hkv a
 // group is exactly one KV head and the CTA writes final outputs; otherwise every piece writes a
@@ -181,9 +181,12 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
 
     static_assert(!kPair || (kQuant != 0 && !kWindow), "the paired variant is for quantised caches without a window");
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    // Grid (ranges, row pairs from the last to the first): the row pairs that see most keys start first and the
-    // shortest fill the tail.  (kPair: clusters along x, so x = row pair.)
-    const int qpair = kPair ? (int)blockIdx.x : (int)(gridDim.y - 1 - blockIdx.y), group = kPair ? blockIdx.y : blockIdx.x;
+    // Ranges first, row pairs from the last to the first: the row pairs that see most keys start first and the shortest
+    // fill the tail.  Both in x, which has no limit a chunk could reach (y ends at 65 535: 262 140 tokens of 64 query heads
+    // per KV head).  (kPair: clusters along x, so x = row pair, y = range.)
+    const int pairs = kPair ? (int)gridDim.x : (int)gridDim.x / a.ngroups;
+    const int qpair = kPair ? (int)blockIdx.x : pairs - 1 - (int)blockIdx.x / a.ngroups;
+    const int group = kPair ? (int)blockIdx.y : (int)blockIdx.x % a.ngroups;
     const uint32_t rank = kPair ? cluster_cta_rank() : 0u;     // which of K (0) and V (1) this CTA expands
     const int cb = blockIdx.z;     // cache of a batch (0 when there is one cache)
     const int G = a.Gp;     // rows per token in the row layout (a power of two >= a.G, the query heads per KV head)
@@ -260,7 +263,7 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
     const uint32_t tmem = *reinterpret_cast<volatile uint32_t *>(&ctl->tmem_base);
     // One CTA times itself in SM cycles and in nanoseconds: the ratio is the clock the launch ran at
     // (the last row pair: it sees the most keys of the chunk itself, so no CTA of the launch runs longer)
-    const bool clocked = qpair == (int)(kPair ? gridDim.x : gridDim.y) - 1 && group == 0 && blockIdx.z == 0 && threadIdx.x == 0;
+    const bool clocked = qpair == pairs - 1 && group == 0 && blockIdx.z == 0 && threadIdx.x == 0;
     if (clocked) {
         ctl->clk0 = clock64();
         ctl->ns0 = global_ns();
@@ -1060,7 +1063,7 @@ cudaError_t launch_attn_tc(const AttnArgs &a, const TcMaps &maps, cudaStream_t s
     }
     cudaError_t e = raise_smem_limit_once(reinterpret_cast<const void *>(kernel), (int)smem);
     if (e != cudaSuccess) return e;
-    return launch_pdl(kernel, dim3(grid.y, grid.x, grid.z), dim3(quant ? kThreadsQ8 : kThreads), smem, s, a, maps.q, maps.k, maps.v);
+    return launch_pdl(kernel, dim3(grid.x * grid.y, 1, grid.z), dim3(quant ? kThreadsQ8 : kThreads), smem, s, a, maps.q, maps.k, maps.v);
 }
 
 cudaError_t launch_combine_groups(const AttnArgs &a, cudaStream_t s) {
