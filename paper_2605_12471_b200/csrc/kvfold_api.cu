@@ -368,23 +368,14 @@ Plan make_plan(const kvf_cache *c, int n, int64_t prefix, int batch = 1, int64_t
         const int64_t nt = (L + kKvTile - 1) / kKvTile - WindowTiles(window_lo(c, prefix), c->n_sink, kKvTile).skip;
         // (row blocks of a KV head: 256-row pairs in the bf16 kernel, 128-row blocks in the fp32 one)
         const int pairs = c->tc32 ? attn_tc32_row_blocks(n, c->Gp) : attn_tc_row_pairs(n, c->Gp);
+        const int streams = c->tc32 ? 1 : attn_tc_streams(n, c->Gp);
+        const int64_t slots_cap = part_rows_cap / ((int64_t)n * c->Gp) / streams;   // slots = streams * (groups + Hkv - 1)
         int64_t groups = Hkv;
         if (c->force_splits > 0) {
             groups = (int64_t)Hkv * c->force_splits;
-        } else if ((int64_t)pairs * Hkv * batch < c->sm_count) {
+        } else if ((int64_t)pairs * Hkv * batch < c->sm_count && c->tc32) {
             groups = c->sm_count / (pairs * batch);
-            // Fewest key tiles worth a CTA.  us per step (bf16, ranges per KV head: time), whole heads against
-            // finer cuts: 256 tokens of 32 / 8 heads, 4 key tiles: 1: 17.4, 4: 18.1; 8 tiles: 1: 24.6, 2: 23.2, 4:
-            // 20.1; 1020-row window (11 tiles) 2: 30.7, 4: 25.1; 64 tokens, 9 tiles: 2: 22.6, 4: 19.3, 6: 17.0; 200
-            // tokens of 16 / 16 heads, 14 tiles: 3: 26.1, 8: 20.3.  Two streams (a merge kernel in any case, two key
-            // tiles in flight per CTA): 32 tokens, 5 tiles: 1: 18.9, 3: 15.5; 9 tiles: 2: 18.7, 3: 16.6, 6: 18.9; 16
-            // tiles: 4: 17.3, 6: 20.2.
-            int64_t most = Hkv * nt / 4;
-            if (!c->tc32) {
-                if (attn_tc_streams(n, c->Gp) == 2) most = std::max<int64_t>(most, nt >= 5 ? 3 * Hkv : Hkv);
-                else most = nt <= 5 ? Hkv : Hkv * nt * 4 / 7;
-            }
-            if (groups > most) groups = most;
+            if (groups > Hkv * nt / 4) groups = Hkv * nt / 4;
             // A group count that is a multiple of the KV heads keeps every CTA inside one KV head: one Q load
             // and one set of partial rows instead of two.  Measured at C = 256 (Llama shape): the second
             // piece costs a CTA about as long as 3.3 key tiles, so while the line is short - here below
@@ -393,6 +384,41 @@ Plan make_plan(const kvf_cache *c, int n, int64_t prefix, int batch = 1, int64_t
             if (aligned >= Hkv && aligned < groups) {
                 const double line = (double)Hkv * (double)nt;
                 if (line / (double)aligned - line / (double)groups < 3.3) groups = aligned;
+            }
+        } else if ((int64_t)pairs * Hkv * batch < c->sm_count) {
+            // Ranges per KV head by what they cost, in us: the key tiles of the longest range (with two streams a
+            // stream has half of them) and the merge of the parts: its launch (a window's ends make an uncut head dearer by
+            // more than that), eight parts of a row in one trip to memory (a warp has Gp / 2 rows of its block's four
+            // tokens), beyond eight the merge kernel that holds any number, the parts written and read.  A range of one
+            // tile is no faster than one of two.  Fitted to 12 800 random steps timed under 2 to 18 cuts each (17 - 4096
+            // tokens, seven head shapes, 64 - 60 K rows, windows, batches, all storages): rms 5 % of a step; the cut
+            // chosen is 2.6 % above the best of them on average, where a fixed least of four tiles per CTA is 13 %.
+            // us per step (ranges per head: time): 256 tokens of 32 / 8 heads, bf16, 4 key tiles 1: 17.4, 4: 18.1; 8 tiles
+            // 1: 24.6, 2: 23.2, 4: 20.1; 64 tokens of 28 / 4 heads, 32 tiles 8: 22.2, 18: 31.2; 32 tokens of 12 / 2
+            // heads, 126 tiles 31: 35.2, 72: 55.7; 48 tokens of 8 / 2 heads, int8, 43 tiles 10: 28.0, 24: 22.6.
+            const double tile = (c->quant ? 2.4 : 1.55) * (streams == 2 ? 0.625 : 1.0);
+            const double rows = (double)n * c->cfg.n_q_heads * batch, launch = window_lo(c, prefix) > 0 ? -1.5 : 3.0;
+            auto merge = [&](int64_t parts) {
+                if (parts <= 1) return 0.0;
+                return launch + 0.7 * std::max(c->Gp / 2, 2) * (double)((parts + 7) / 8) + (parts > 8 ? 2.0 : 0.0) + 1.2e-4 * rows * (double)parts;
+            };
+            const int64_t room = std::min<int64_t>(c->sm_count / (pairs * batch), slots_cap - (Hkv - 1));
+            int64_t best = 1;
+            double least = 0.0;
+            for (int64_t r = 1; r == 1 || r <= room / Hkv;) {
+                const int64_t longest = (nt + r - 1) / r;
+                const double t = tile * (double)((longest + streams - 1) / streams * streams) + merge(streams * r);
+                if (r == 1 || t < least) { least = t; best = r; }
+                if (longest <= 3 - streams) break;
+                r = (nt + longest - 2) / (longest - 1);          // the fewest ranges with a shorter longest one
+            }
+            groups = best * Hkv;
+            // Ranges that run across KV heads fill the SMs the multiple of the heads leaves over.  A CTA's second piece
+            // (another Q load, another set of partial rows) costs it as long as ~3.3 key tiles, so only long lines
+            // (256 tokens of 32 / 8 heads: from ~12 K rows on).
+            if (room > groups && best == std::max<int64_t>(room / Hkv, 1)) {
+                const double saved = (double)nt / (double)best - (double)Hkv * (double)nt / (double)room;
+                if (saved >= 3.3 && tile * (saved - 3.3) > merge(streams * (best + 1)) - merge(streams * best)) groups = room;
             }
         } else {
             // whole KV heads fill the SMs, but the last wave may be half empty (256 CTAs on 148 SMs):
@@ -430,8 +456,6 @@ Plan make_plan(const kvf_cache *c, int n, int64_t prefix, int batch = 1, int64_t
                 }
             }
         }
-        const int streams = c->tc32 ? 1 : attn_tc_streams(n, c->Gp);
-        const int64_t slots_cap = part_rows_cap / ((int64_t)n * c->Gp) / streams;   // slots = streams * (groups + Hkv - 1)
         if (groups + Hkv - 1 > slots_cap) groups = slots_cap - (Hkv - 1);
         if (groups > Hkv * nt) groups = Hkv * nt;
         if (groups < Hkv) groups = Hkv;

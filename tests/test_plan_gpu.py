@@ -1,0 +1,34 @@
+"""The cuts of the (KV head, key tile) line at sizes where a finer or a coarser one is measurably slower (us per step in
+the comments: the cut asserted, the cut it must not be).  kvf_cache_plan launches nothing; the figures are of 148 SMs."""
+import pytest
+import torch
+
+from paper_2605_12471_b200 import binding
+
+pytestmark = pytest.mark.gpu
+
+
+def _plan(h, kv, n, rows, flags=0, window=0):
+    if torch.cuda.get_device_properties(0).multi_processor_count != 148:
+        pytest.skip("measured on 148 SMs")
+    c = binding.Cache(binding.make_config(h, kv, 128, "bf16", rows + n, n, rope_base=10000.0, flags=flags))
+    if window:
+        c.set_window(4, window)
+    return c.plan(n, rows)
+
+
+@pytest.mark.parametrize("h,kv,n,rows,flags,lo,hi", [
+    (28, 4, 64, 4000, 0, 2, 8),                             # 22 us with eight ranges per head, 31 with 18
+    (12, 2, 32, 16000, 0, 8, 32),                           # 35 with 31, 56 with 72
+    (16, 16, 96, 839, 0, 4, 4),                             # 15.9 with four, 17.5 with two and with three
+    (28, 4, 200, 500, 0, 1, 1),                             # 19.7 uncut, 21.6 with three
+    (32, 8, 512, 250, binding.KVF_CACHE_INT8, 1, 1),        # 30.3 uncut, 31.8 with two
+    (32, 8, 64, 700, binding.KVF_CACHE_INT8, 3, 8),         # 25.4 uncut, 20.3 with three
+    (32, 8, 256, 768, 0, 3, 4),                             # 20.1 with four, 24.6 uncut
+])
+def test_ranges_per_head_of_steps_that_leave_sms_idle(h, kv, n, rows, flags, lo, hi):
+    assert lo <= _plan(h, kv, n, rows, flags)[1] <= hi
+
+
+def test_ranges_under_a_window():
+    assert 3 <= _plan(32, 8, 256, 8192, window=1020)[1] <= 4       # 25.1 us with four, 30.7 with two
