@@ -422,39 +422,37 @@ Plan make_plan(const kvf_cache *c, int n, int64_t prefix, int batch = 1, int64_t
             }
         } else {
             // whole KV heads fill the SMs, but the last wave may be half empty (256 CTAs on 148 SMs):
-            // cut a little finer - up to twice the KV heads - if that saves more than it costs; the price is
-            // the partial results of one chunk and the merge kernel.
-            if (c->tc32) {
-                auto fill = [&](int64_t g) {
-                    const int64_t ctas = (int64_t)pairs * g * batch;
-                    const int64_t waves = (ctas + c->sm_count - 1) / c->sm_count;
-                    return (double)ctas / (double)(waves * c->sm_count);
-                };
-                double best = fill(Hkv) + 0.05;
-                for (int64_t g = Hkv + 1; g <= 2 * Hkv && g * 4 <= Hkv * nt; ++g)
-                    if (fill(g) > best) { best = fill(g); groups = g; }
-            } else {
-                // In key tiles of one CTA: the waves one after the other, each as long as its first row pair (they
-                // start longest first), and for partial results one tile per 2400 output rows: 2048 tokens of 32
-                // heads, 8 ranges (no merge) against 9: 55 / 90 us at prefix 0, 115 / 145 at 2 K, 234 / 257 at 6 K,
-                // 478 / 490 at 14 K, 1002 / 906 at 30 K - about 28 tiles of 1.9 us.
-                auto cost = [&](int64_t g) {
-                    double tiles = g > Hkv ? (double)n * c->cfg.n_q_heads * batch / 2400.0 : 0.0;
-                    const int64_t ctas = (int64_t)pairs * g * batch;
-                    for (int64_t at = 0; at < ctas; at += c->sm_count) {
-                        const int64_t pair = pairs - 1 - at / g % pairs;           // row pair of the wave's first CTA
-                        const int64_t tok = std::min<int64_t>(n, ((pair + 1) * 256 + c->Gp - 1) / c->Gp);
-                        const int64_t need = batch > 1 ? nt : nt - (L - (prefix + tok)) / kKvTile;
-                        tiles += (double)Hkv * (double)need / (double)g;
-                    }
-                    return tiles;
-                };
-                double best = cost(Hkv);
-                for (int64_t g = Hkv + 1; g <= 2 * Hkv && g * 4 <= Hkv * nt; ++g) {
-                    const double t = cost(g);
-                    if (t < best) { best = t; groups = g; }
+            // cut a little finer - up to twice the KV heads, where that fills the waves best - if it saves more than it
+            // costs; the price is the partial results of one chunk and the merge kernel.  (Only cuts the partial area
+            // holds, and no other than the best filling one: 1783 tokens of 32 / 8 heads at prefix 44 K, 28 row pairs: 10
+            // ranges 1052 us; 15 fill the waves as well, the area has room for 11, and those start a third wave: 1366.)
+            auto fill = [&](int64_t g) {
+                const int64_t ctas = (int64_t)pairs * g * batch;
+                const int64_t waves = (ctas + c->sm_count - 1) / c->sm_count;
+                return (double)ctas / (double)(waves * c->sm_count);
+            };
+            int64_t cut = Hkv;
+            double best = fill(Hkv) + 0.05;
+            for (int64_t g = Hkv + 1; g <= 2 * Hkv && g * 4 <= Hkv * nt && (c->tc32 || g + Hkv - 1 <= slots_cap); ++g)
+                if (fill(g) > best) { best = fill(g); cut = g; }
+            // In key tiles of one CTA: the waves one after the other, each as long as its first row pair (they
+            // start longest first; the paired quantised grid starts them shortest first, but counting it so chooses
+            // worse), and for partial results one tile per 2400 output rows: 2048 tokens of 32 heads, 8 ranges (no
+            // merge) against 9: 55 / 90 us at prefix 0, 115 / 145 at 2 K, 234 / 257 at 6 K, 478 / 490 at 14 K, 1002 / 906 at
+            // 30 K - about 28 tiles of 1.9 us; int8 102 / 135 at 0, 395 / 399 at 8 K, 537 / 529 at 12 K.  4326 random
+            // steps of all storages under both cuts: 20 took more than 1 % longer than under the other, 6 % at most.
+            auto cost = [&](int64_t g) {
+                double tiles = g > Hkv ? (double)n * c->cfg.n_q_heads * batch / 2400.0 : 0.0;
+                const int64_t ctas = (int64_t)pairs * g * batch;
+                for (int64_t at = 0; at < ctas; at += c->sm_count) {
+                    const int64_t pair = pairs - 1 - at / g % pairs;           // row pair of the wave's first CTA
+                    const int64_t tok = std::min<int64_t>(n, ((pair + 1) * 256 + c->Gp - 1) / c->Gp);
+                    const int64_t need = batch > 1 ? nt : nt - (L - (prefix + tok)) / kKvTile;
+                    tiles += (double)Hkv * (double)need / (double)g;
                 }
-            }
+                return tiles;
+            };
+            if (c->tc32 || (cut > Hkv && cost(cut) < cost(Hkv))) groups = cut;
         }
         if (groups + Hkv - 1 > slots_cap) groups = slots_cap - (Hkv - 1);
         if (groups > Hkv * nt) groups = Hkv * nt;

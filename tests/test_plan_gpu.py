@@ -32,3 +32,11 @@ def test_ranges_per_head_of_steps_that_leave_sms_idle(h, kv, n, rows, flags, lo,
 
 def test_ranges_under_a_window():
     assert 3 <= _plan(32, 8, 256, 8192, window=1020)[1] <= 4       # 25.1 us with four, 30.7 with two
+
+
+@pytest.mark.parametrize("n,rows,flags,groups", [(1783, 44202, 0, 10),                            # 1052 us; 11: 1366, uncut ~1190
+                                                 (1777, 20337, binding.KVF_CACHE_INT8, 10),       # 760; 11: 986
+                                                 (2048, 2000, 0, 8), (2048, 30000, 0, 9),         # 115 / 145 with 9; 906 / 1002 uncut
+                                                 (2048, 4000, binding.KVF_CACHE_INT8, 8)])        # 255 / 274 with 9
+def test_ranges_of_steps_that_fill_the_sms(n, rows, flags, groups):
+    assert _plan(32, 8, n, rows, flags)[2] == groups * -(-n // 64)
