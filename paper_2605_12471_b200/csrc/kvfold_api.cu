@@ -415,10 +415,10 @@ Plan make_plan(const kvf_cache *c, int n, int64_t prefix, int batch = 1, int64_t
             groups = best * Hkv;
             // Ranges that run across KV heads fill the SMs the multiple of the heads leaves over.  A CTA's second piece
             // (another Q load, another set of partial rows) costs it as long as ~3.3 key tiles, so only long lines
-            // (256 tokens of 32 / 8 heads: from ~12 K rows on).
+            // (256 tokens of 32 / 8 heads: from ~12 K rows on), and from whole heads only for the merge as well.
             if (room > groups && best == std::max<int64_t>(room / Hkv, 1)) {
                 const double saved = (double)nt / (double)best - (double)Hkv * (double)nt / (double)room;
-                if (saved >= 3.3 && tile * (saved - 3.3) > merge(streams * (best + 1)) - merge(streams * best)) groups = room;
+                if (saved >= 3.3 && (best > 1 || tile * (saved - 3.3) > merge(streams * 2) - merge(streams))) groups = room;
             }
         } else {
             // whole KV heads fill the SMs, but the last wave may be half empty (256 CTAs on 148 SMs):

@@ -32,6 +32,8 @@ def test_ranges_per_head_of_steps_that_leave_sms_idle(h, kv, n, rows, flags, lo,
 
 def test_ranges_under_a_window():
     assert 3 <= _plan(32, 8, 256, 8192, window=1020)[1] <= 4       # 25.1 us with four, 30.7 with two
+    # 13 row pairs, 11 ranges over four heads: 62.5 us; two per head: 70.8
+    assert _plan(28, 4, 416, 5860, binding.KVF_CACHE_INT8, window=2860)[2] == 13 * 11
 
 
 @pytest.mark.parametrize("n,rows,flags,groups", [(1783, 44202, 0, 10),                            # 1052 us; 11: 1366, uncut ~1190
