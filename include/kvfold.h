@@ -366,7 +366,8 @@ uint64_t kvf_cache_launch_count(const kvf_cache *c);
  * Per-kernel timing.  With enable != 0 every step records CUDA events around each of its
  * kernels on the step's stream.  kvf_cache_profile_read synchronises, then ADDS the elapsed
  * milliseconds and launch counts since the last read to
- *   ms[0]/launches[0] rotate+append, [1] attention, [2] split combine
+ *   ms[0]/launches[0] rotate+append, [1] attention, [2] split combine (a step of one launch counts
+ *   as attention)
  * and forgets the recorded events.  At most 65536 launches are kept between reads.
  */
 kvf_status kvf_cache_profile(kvf_cache *c, int32_t enable);

@@ -47,8 +47,8 @@
 // and the next Q K^T runs under the softmax's second half.  The two issuers take turns on (first P V, Q K^T), which
 // keeps the tiles in antiphase.  Measured against the order above, cycles of a CTA: 256 tokens at prefix 61 K
 // 380 -> 341 thousand, 2048 tokens at prefix 14 K 424 -> 380 thousand; time 274 -> 257 us (at the power cap, the
-// clock settles 4 % lower) and 540 -> 505 us.  Then 341 -> 309 thousand and 264 -> 250 us by taking latency out of the
-// softmax threads' chain: whether the panel is free is asked before the second half's arithmetic (a wait on a
+// clock settles 4 % lower) and 540 -> 505 us.  Then 341 -> 309 thousand (264 -> 250 us, another box's pair of runs) by taking
+// latency out of the softmax threads' chain: whether the panel is free is asked before the second half's arithmetic (a wait on a
 // barrier that is already complete takes ~250 cycles beside saturated shared memory), and whether a key tile
 // needs a mask is known from the tile number, without a vote.  (Leaving out the vote on the scores' wait as well: 312;
 // passing the turn ahead of the K slot's commit: no change.)  It takes a K/V slot of shared memory: quantised storage, which has
@@ -84,10 +84,10 @@ constexpr int kRows = 128;                    // rows of a Q tile = keys of a K/
 constexpr int kD = 128;                       // head_dim
 constexpr uint32_t kPanel = 128 * 128;        // bytes of a [128 rows][64 bf16] swizzled panel
 constexpr uint32_t kTileBytes = 2 * kPanel;   // a 128 x 128 bf16 tile = two panels
-constexpr int kSlots = 5;
+constexpr int kSlots = 5;                             // two streams on bf16 rows: behind the Q tiles, a sixth is the second of them
 constexpr int kThreads = 384;
 constexpr uint32_t kOffQ = 0;                         // 2 tiles
-constexpr uint32_t kOffKV = 2 * kTileBytes;           // kSlots tiles
+constexpr uint32_t kOffKV = 2 * kTileBytes;           // K/V tiles
 // two row tiles on bf16 rows (kEarly): a ring of four slots, behind it one panel per row tile for the
 // probabilities of a tile's keys 64-127
 constexpr int kSlotsEarly = 4;
@@ -108,7 +108,7 @@ constexpr uint32_t kTmemCols = 512;
 constexpr float kRescaleThreshold = 8.0f;             // log2 units
 
 // barrier indices inside the control block
-constexpr int kRingBars = 6;                  // 5 slots of the shared ring, or 2 x 3 slots of the per-stream rings
+constexpr int kRingBars = 6;                  // 2 x 3 slots of the per-stream rings (shared rings have 4, quantised storage 3)
 enum { B_QFULL = 0, B_QEMPTY = 1, B_FULL0 = 2, B_EMPTY0 = B_FULL0 + kRingBars, B_SFULL0 = B_EMPTY0 + kRingBars,
        B_PA0 = B_SFULL0 + 2, B_PB0 = B_PA0 + 2, B_PVDONE0 = B_PB0 + 2, B_TURN0 = B_PVDONE0 + 2,
        B_DRAIN0 = B_TURN0 + 8, B_RAWFULL0 = B_DRAIN0 + 2, B_RAWEMPTY0 = B_RAWFULL0 + kRawSlots,
@@ -169,7 +169,7 @@ __global__ void __launch_bounds__(kQuant ? kThreadsQ8 : kThreads, 1)
 attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                const __grid_constant__ CUtensorMap map_v) {
     static_assert(!kEarly || kQuant == 0, "the early issue needs the space of a K/V slot for its probabilities");
-    constexpr int NS = kQuant ? kSlotsQ8 : kEarly ? kSlotsEarly : kSlots;        // slots of the shared ring
+    constexpr int NS = kQuant ? kSlotsQ8 : kEarly ? kSlotsEarly : kSlots;        // slots behind the Q tiles: the shared ring's
     constexpr int SR = kQuant ? 2 : 3;                     // slots of each stream's own ring
     constexpr uint32_t offCtl = kQuant ? kOffCtlQ8 : kOffCtl;
     constexpr uint32_t rawBytes = kQuant == 4 ? kRawBytes / 2 : kRawBytes;   // bytes of a 128-row code tile
@@ -200,7 +200,8 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
     // streams == 2 (chunks of at most 128 / G tokens, i.e. one row tile): the two tile slots work on
     // the SAME 128 rows and take alternate key tiles, so that one stream's softmax still runs under
     // the other stream's MMAs; each stream leaves its own partial result.
-    const int streams = kEarly ? 1 : a.streams;
+    // (bf16 rows: the two modes are two kernels, kEarly for one and the two streams for the other)
+    const int streams = kEarly ? 1 : kQuant == 0 ? 2 : a.streams;
     const bool direct = a.ngroups == a.Hkv && streams == 1;
 
     // key tiles: this row pair needs tiles below nt_need; the group's share of the
@@ -744,7 +745,7 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
                 __syncwarp();
                 if (lane == 0) mbar_arrive(bar(B_PA0 + i));
                 // (my previous P V read the panel the second half goes to; asked ahead of the arithmetic, for the answer
-                // takes ~200 cycles to come even if it is yes; every phase is waited for)
+                // takes ~250 cycles to come even if it is yes; every phase is waited for)
                 uint32_t panel_free = 1;
                 if (kEarly && k > 0) panel_free = mbar_test(bar(B_PVDONE0 + i), (it - 1) & 1);
                 exp_half(sc + 64, p, sl2v, negv, acc0, acc1);
@@ -831,7 +832,8 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
                         emit(w, c0 * 2);
                     }
                 }
-                // (the panel goes back to the probabilities; the next ones are stored after a wait_pv of every lane)
+                // The panel goes back to the probabilities: the next piece's first tile stores them without a wait, so this is
+                // what keeps them behind the last reads of the staged rows (a warp stages and stores in its own 4 KiB).
                 __syncwarp();
             } else {
 #pragma unroll
