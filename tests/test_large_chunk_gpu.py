@@ -27,7 +27,7 @@ def test_more_row_pairs_than_a_grid_has_in_y():
     rot = torch.cat([lo * theta.cos() - hi * theta.sin(), hi * theta.cos() + lo * theta.sin()], dim=-1).bfloat16().float()
     p = torch.softmax(rot @ keys.T / math.sqrt(d), dim=-1)
     want = p @ values
-    # probabilities and outputs are rounded to bf16 (2^-9 of each, at worst 2^-8 in all of sum p |v| and of |out|), a query
-    # element of 64-bit angles may round the other way (2^-8 of one of 128 terms of a score)
+    # probabilities and outputs are rounded to bf16 (2^-8 of each: of sum p |v| and of |out|); a query element may round
+    # the other way from 64-bit angles (2^-8 of one of 128 terms of a score: 2e-3 of an output of unit size)
     bound = 2.0 ** -8 * (p @ values.abs() + want.abs()) + 2e-3
     assert ((out[toks].float() - want).abs() <= bound).all()

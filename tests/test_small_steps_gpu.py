@@ -110,3 +110,57 @@ def test_long_prefixes_take_the_launches_that_split_them(n, h, kv, tiles, kernel
     assert small.plan(n, prefix)[3] == kernels
     _compare(*got, dtype)
     assert torch.equal(small.storage, general.storage)
+
+
+@pytest.mark.parametrize("h,kv", [(4, 1), (7, 1), (2, 2)])
+def test_fp32_results_of_bf16_rows(h, kv):
+    gen = torch.Generator(device="cuda").manual_seed(h)
+    small, general = _caches(h, kv, "bf16", 400, 130, binding.KVF_OUT_F32)
+    for n in (1, 64, 130, 33):
+        q, k, v = _inputs(h, kv, n, "bf16", gen)
+        got = []
+        for c in (small, general):
+            lse = torch.empty(n, h, device="cuda")
+            got.append((c.fold_step(q, k, v, lse=lse), lse))
+            assert got[-1][0].dtype == torch.float32
+        assert small.plan(n, len(small) - n)[3] == 1
+        _compare(*got, "f32")                  # (nothing is rounded to bf16 behind the sums)
+        assert torch.equal(small.storage, general.storage)
+    # fp32 rows over bf16 queries are not "exactly over them": the three launches
+    buf = torch.empty(64 * h * 64, dtype=torch.float32, device="cuda")
+    over = buf.view(torch.bfloat16)[:64 * h * 64].view(64, h, 64)
+    q, k, v = _inputs(h, kv, 64, "bf16", gen)
+    over.copy_(q)
+    want, before = general.fold_step(q, k, v), small.launch_count()
+    got = small.fold_step(over, k, v, out=buf.view(64, h, 64))
+    assert small.launch_count() - before > 1
+    assert (got - want).abs().max().item() <= 1e-5
+
+
+def test_lse_and_cache_rows_over_the_inputs_take_the_three_launches():
+    gen = torch.Generator(device="cuda").manual_seed(9)
+    n, h = 64, 4
+    for over in (0, 1, 2):                     # the log-sum-exp over the first rows of the queries, keys and values
+        small, general = _caches(h, 1, "f32", 400, n)
+        ins = _inputs(h, 1, n, "f32", gen)
+        lse = torch.empty(n, h, device="cuda")
+        want = (general.fold_step(*ins, lse=lse), lse)
+        mine = [t.clone() for t in ins]
+        inside = mine[over].view(-1)[:n * h].view(n, h)
+        before = small.launch_count()
+        _compare((small.fold_step(*mine, lse=inside), inside), want, "f32")
+        assert small.launch_count() - before > 1
+        assert torch.equal(small.storage, general.storage)
+    for kv in (0, 1):                          # keys and values that lie in rows of the cache no one holds yet
+        small, general = _caches(h, 1, "f32", 400, n)
+        ins = _inputs(h, 1, n, "f32", gen)
+        want = general.fold_step(*ins)
+        inside = (small.v_plane() if kv else small.k_plane())[0, 200:200 + n].view(n, 1, 64)
+        inside.copy_(ins[1 + kv])
+        mine = [ins[0], inside, ins[2]] if kv == 0 else [ins[0], ins[1], inside]
+        before = small.launch_count()
+        got = small.fold_step(*mine)
+        assert small.launch_count() - before > 1
+        assert (got - want).abs().max().item() <= 1e-5
+        rows = slice(0, n)
+        assert torch.equal(small.k_plane()[:, rows], general.k_plane()[:, rows]) and torch.equal(small.v_plane()[:, rows], general.v_plane()[:, rows])
