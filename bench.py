@@ -37,9 +37,9 @@ FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustain
 # ncu capture of the last steps of a 65 536-token chain of 256-token chunks (too large to capture
 # at 131 072 tokens; traffic grows in proportion to the cache rows read, so the ratio carries
 # over).  Set to None whenever the attention kernel changes after the capture.
-NCU_TRAFFIC_BYTES_PER_CACHE_BYTE = 1.033
+NCU_TRAFFIC_BYTES_PER_CACHE_BYTE = 1.038
 NCU_TRAFFIC_SOURCE = ("ncu capture (dram__bytes_read.sum + dram__bytes_write.sum) of the attention kernel on the "
-                      "last steps of a 65 536-token chain of 256-token chunks: 1.033 DRAM bytes per algorithmic "
+                      "last steps of a 65 536-token chain of 256-token chunks: 1.038 DRAM bytes per algorithmic "
                       "cache byte, scaled by the cache rows a launch of this run reads")
 NOMINAL = {"bf16_tflops": 2250.0, "hbm_gbs": 7700.0}      # dense bf16 and HBM3e figures of the B200 data sheet
 TENSOR_FLOP_PER_SM_CLOCK = 8192.0                         # one 128 x 128 x 16 bf16 MMA (524 288 FLOP) per 64 clocks
@@ -903,13 +903,16 @@ def run_chain_bench(args, w, drift=False):
     attn_tflops = attn_flops / (kms[1] * 1e-3) / 1e12
     cache_bytes_read = sum(visible(P0 + t * C) + C for t in range(N)) * bytes_per_token
     hbm_gbs = cache_bytes_read / (kms[1] * 1e-3) / 1e9
+    plan_last = cache.plan(C, T - C)
+    one_wave = plan_last[2] <= N_SMS
     traffic = None
-    if NCU_TRAFFIC_BYTES_PER_CACHE_BYTE is not None and w.dtype == "bf16" and not (args.cache_int8 or args.cache_int4 or args.force_simt):
+    # (one wave of CTAs reads the cache once; a second wave walks it again, which the capture does not cover)
+    if NCU_TRAFFIC_BYTES_PER_CACHE_BYTE is not None and w.dtype == "bf16" and not (args.cache_int8 or args.cache_int4 or args.force_simt) \
+            and one_wave:
         traffic = NCU_TRAFFIC_BYTES_PER_CACHE_BYTE * cache_bytes_read / kcnt[1]
     # which roof binds: arithmetic intensity G*C FLOP per cache byte against the ridge of the measured peaks
     ridge = pk["bf16_tflops_sustained"] * 1e12 / (pk["hbm_gbs"] * 1e9)
     intensity = attn_flops / cache_bytes_read
-    plan_last = cache.plan(C, T - C)
     if w.dtype == "f32" and not plan_last[0]:
         # CUDA-core kernel (head_dim 64, or forced): the roof is the FFMA rate, 148 SMs x 128 lanes x 2 FLOP at
         # the 1965 MHz maximum clock
@@ -943,8 +946,9 @@ def run_chain_bench(args, w, drift=False):
         per_clock = TENSOR_FLOP_PER_SM_CLOCK / (3.0 if w.dtype == "f32" else 1.0)
         roofline["sm_mhz_during_profile"] = prof_mhz
         roofline["frac_of_tensor_rate_at_sampled_clock"] = attn_tflops * 1e12 / (prof_mhz * 1e6 * N_SMS * per_clock)
-    if ns_b > ns_a and roofline["bound"] == "tensor":
-        # (only the tcgen05 kernels for long chunks keep these counters: not reported for decode-shaped runs)
+    if ns_b > ns_a and roofline["bound"] == "tensor" and one_wave:
+        # (only the tcgen05 kernels for long chunks keep these counters: not reported for decode-shaped runs, nor where a launch
+        # is several waves, of which the counting CTA sees one)
         # the attention kernels inside the timed chains themselves (no events between the kernels there): time and
         # cycles one CTA of every launch (its last row block) was running, from the kernels' own counters
         in_ms = (ns_b - ns_a) * 1e-6 / steps_timed

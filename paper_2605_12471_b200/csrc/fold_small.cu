@@ -456,7 +456,7 @@ int fold_small_row_tiles(int n, int G) { return (int)(((int64_t)n * G + BM - 1) 
 // Slices of the key tiles = CTAs of a cluster: a power of two, at least one key tile each, and no more clusters than the
 // device holds at once: a second wave costs more than longer slices.  Two CTAs fit an SM, but a cluster stays within
 // one GPC: of 16 CTAs the device holds 14 clusters (16 row tiles, 24 key tiles: 16 slices 37.4 us, 8 slices 28.6), of 8 CTAs
-// 35 (36 row tiles, 16 key tiles: 8 slices 36.1 us, through three launches 34.4).
+// fewer than 36 (36 row tiles, 16 key tiles: 8 slices 36.1 us, through three launches 34.4).
 int fold_small_ranks(int row_tiles, int64_t key_tiles, const FoldSmallFit &fit) {
     int ranks = 1;
     for (int i = 1; i < kFoldSmallWidths && (1 << i) <= key_tiles && row_tiles <= fit.clusters[i]; ++i) ranks = 1 << i;
