@@ -495,13 +495,16 @@ Plan make_plan(const kvf_cache *c, int n, int64_t prefix, int batch = 1, int64_t
         // slice: us in one launch, in three (fp32): one token of 4 / 1 heads 7: 32.9, 35.7; 8: 36.9, 36.9; 11: 48.1, 38.0;
         // 32: 129, 64; 48 tokens (6 row tiles) 5: 27.7, 37.2; 6: 31.6, 37.3, of 2 / 2 heads 36 - 42, 37.5; 64 tokens
         // (8) 4: 33.0, 36.2; 5: 40.0, 37.5; 16 tokens of 32 / 8 heads (16, in clusters of 8) 3: 24.8, 35.0; 4: 31.9,
-        // 35.4 at 28 key tiles and 34.5 at 32; 160 tokens of 32 / 8 heads (uncut) 3: 30.3, 26.9.  Of 3350 steps within
-        // these limits (102 shapes, 1 - 512 key tiles, fp32 and bf16) nine measured 2 - 8 % slower than through three.
+        // 35.4 at 28 key tiles and 34.5 at 32; 160 tokens of 32 / 8 heads (uncut) 3: 30.3, 26.9.  One tile less on bf16
+        // rows, where the three launches are 2 us faster, for chunks that span two key tiles (a second table of sines): 72
+        // tokens of 2 / 2 heads 5: 38.6, 34.9; 160 tokens 4: 37.4, 34.5.  Of the 3322 steps within these limits among
+        // 3722 (102 shapes, 1 - 512 key tiles, fp32 and bf16) none measured more than 2 % slower than through three.
         const int tiles = fold_small_row_tiles(n, c->G) * Hkv;
         const int ranks = fold_small_ranks(tiles, nt, c->small_fit);
         const int64_t at_once = (int64_t)tiles * ranks;
         int64_t longest = at_once <= 48 ? 7 : at_once <= 80 ? 6 : at_once <= 96 ? 5 : ranks >= 16 ? 4 : ranks > 1 ? 3 : 2;
         if (nt > 4 * (int64_t)splits || (int64_t)units * splits > c->sm_count) longest += ranks >= 16 ? 2 : 1;
+        if (ranks >= 16 && n > 64 && c->cfg.dtype == KVF_BF16) longest -= 1;
         if (2 * tiles * nt <= 9 * (int64_t)c->sm_count && nt <= longest * ranks) {
             p.small = true;
             p.splits = ranks;

@@ -112,6 +112,12 @@ def test_long_prefixes_take_the_launches_that_split_them(n, h, kv, tiles, kernel
     assert torch.equal(small.storage, general.storage)
 
 
+def test_chunks_of_two_key_tiles_on_bf16_rows_have_shorter_slices():
+    for dtype, kernels in (("f32", 1), ("bf16", 3)):
+        c, _ = _caches(2, 2, dtype, 4096, 160)
+        assert c.plan(160, 4096 - 160)[3] == kernels          # bf16: 34.5 us in three launches, 37.4 in one
+
+
 @pytest.mark.parametrize("h,kv", [(4, 1), (7, 1), (2, 2)])
 def test_fp32_results_of_bf16_rows(h, kv):
     gen = torch.Generator(device="cuda").manual_seed(h)
