@@ -789,7 +789,13 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
                 // its 32 rows round in its part of the probability panel, whose last P V has run: 128 bytes of
                 // every row at a time, 16-byte chunks swizzled by the row, written out as whole 128-byte lines.
                 const uint32_t stage = base + kOffP + (uint32_t)warp * 4096u;
-                const int rw = row0 + i * kRows + (warp & 3) * 32;       // the warp's first row
+                const int R1 = row0 + i * kRows + (warp & 3) * 32 + (lane >> 3), lg = __ffs(G) - 1;      // first of the rows I write out
+                // (partial rows lie one after the other; G is a power of two: with a divide per row and line the
+                // index arithmetic took as long as the stores)
+                char *part = reinterpret_cast<char *>(a.part_o + (prow - R + R1) * kD) + (lane & 7) * 16;
+                char *fin = reinterpret_cast<char *>(a.out) + (lane & 7) * 16;
+                const int fin_row = kD * (a.out_f32 ? 4 : 2);
+                const int64_t fin0 = (int64_t)cb * nmax * a.H + kvh * a.G;
                 auto emit = [&](const uint32_t (&w)[32], int byte0) {
                     __syncwarp();                  // the segment before has been read
 #pragma unroll
@@ -799,15 +805,13 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
                     __syncwarp();
 #pragma unroll
                     for (int q = 0; q < 8; ++q) {
-                        const int rr = 4 * q + (lane >> 3), c = lane & 7, R1 = rw + rr, tok1 = R1 / G, gi1 = R1 % G;
+                        const int rr = 4 * q + (lane >> 3), Rq = R1 + 4 * q, tok1 = Rq >> lg, gi1 = Rq & (G - 1);
                         uint4 v;
                         asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-                                     : "r"(stage + (uint32_t)rr * 128u + (uint32_t)((c ^ (rr & 7)) << 4)) : "memory");
+                                     : "r"(stage + (uint32_t)rr * 128u + (uint32_t)(((lane & 7) ^ (rr & 7)) << 4)) : "memory");
                         if (tok1 >= n || gi1 >= a.G) continue;
-                        char *dst;
-                        if (!direct) dst = reinterpret_cast<char *>(a.part_o + (prow - R + R1) * kD);
-                        else dst = reinterpret_cast<char *>(a.out) + (((int64_t)cb * nmax + tok1) * a.H + kvh * a.G + gi1) * (kD * (a.out_f32 ? 4 : 2));
-                        *reinterpret_cast<uint4 *>(dst + byte0 + c * 16) = v;
+                        char *dst = direct ? fin + (fin0 + (int64_t)tok1 * a.H + gi1) * fin_row : part + q * (4 * kD * 4);
+                        *reinterpret_cast<uint4 *>(dst + byte0) = v;
                     }
                 };
                 if (!direct || a.out_f32) {
