@@ -17,10 +17,7 @@
 namespace kvf {
 namespace {
 
-// One token per CTA of 16 warps: a warp then has three of the token's 48 rows to do, one after the
-// other (each a load, a warp reduction and a store), instead of twelve.
-constexpr int kTok = 1;        // tokens per CTA
-constexpr int kThreads = 512;
+constexpr int kThreads = 512;  // 16 warps: a warp has three of a Llama-shaped token's 48 rows (each a load, a warp reduction and a store)
 
 __device__ __forceinline__ float bf16_lo(uint32_t w) { return __uint_as_float(w << 16); }
 __device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w & 0xFFFF0000u); }
@@ -51,8 +48,10 @@ __device__ __forceinline__ void quantise4(const float (&x)[4], int (&code)[4], f
 
 // One warp per row (d = 128: four elements per lane).  Query rows are rotated and written as bf16;
 // key rows are rotated in fp32, quantised and appended; value rows are quantised and appended.
-template <bool INTERLEAVED, int BITS>
-__global__ void __launch_bounds__(kThreads) rope_append_q8_kernel(const RopeAppendArgs a, const QuantPlanes qp) {
+// kTok = tokens per CTA (see tokens_per_cta); a warp takes the same rows of every token, so that up to four tokens' loads
+// and reductions are in flight together.
+template <bool INTERLEAVED, int BITS, int kTok>
+__global__ void __launch_bounds__(kThreads, 2) rope_append_q8_kernel(const RopeAppendArgs a, const QuantPlanes qp) {
     constexpr int RB = 128 * BITS / 8;          // bytes of a stored row
     __shared__ float2 cs[kTok][kMaxHalfDim];   // (cos, sin) per (token, pair)
     constexpr int d = 128, half = 64;
@@ -103,84 +102,88 @@ __global__ void __launch_bounds__(kThreads) rope_append_q8_kernel(const RopeAppe
     const __nv_bfloat16 *v = reinterpret_cast<const __nv_bfloat16 *>(a.v_new) + koff;
     __nv_bfloat16 *qr = reinterpret_cast<__nv_bfloat16 *>(a.q_rot) + qoff;
     const int heads = a.H + (a.k_new ? 2 * a.Hkv : 0);     // query rows, key rows, value rows (queries only: kvf_attend)
-    for (int row = warp; row < ntok * heads; row += kThreads / 32) {
-        const int t = row / heads, hh = row % heads;
-        const int64_t tok = tok0 + t;
-        const int64_t cache_row = prefix + tok;
-        if (hh >= a.H + a.Hkv) {
-            // ---- value row: elements 4 lane .. 4 lane + 3
-            const int g = hh - a.H - a.Hkv;
-            const uint2 w = *reinterpret_cast<const uint2 *>(v + (tok * a.Hkv + g) * d + 4 * lane);
-            const float x[4] = {bf16_lo(w.x), bf16_hi(w.x), bf16_lo(w.y), bf16_hi(w.y)};
-            int code[4];
-            float scale;
-            quantise4<BITS>(x, code, scale);
-            const int64_t r = code_off(g, cache_row);
-            if (BITS == 8) {
-                const uint32_t packed = (uint32_t)(code[0] & 0xFF) | ((uint32_t)(code[1] & 0xFF) << 8) |
-                                        ((uint32_t)(code[2] & 0xFF) << 16) | ((uint32_t)(code[3] & 0xFF) << 24);
-                *reinterpret_cast<uint32_t *>(qp.v_codes + r + 4 * lane) = packed;
-            } else {
-                *reinterpret_cast<uint16_t *>(qp.v_codes + r + 2 * lane) =
-                    (uint16_t)((code[0] + 8) | ((code[1] + 8) << 4) | ((code[2] + 8) << 8) | ((code[3] + 8) << 12));
+    constexpr int U = kTok < 4 ? kTok : 4;
+    for (int hh = warp; hh < heads; hh += kThreads / 32) {
+        const bool is_q = hh < a.H, is_v = hh >= a.H + a.Hkv;
+        const int g = is_q ? hh : is_v ? hh - a.H - a.Hkv : hh - a.H;        // query head, or KV head
+        const int row_heads = is_q ? a.H : a.Hkv;
+        const __nv_bfloat16 *src = (is_q ? q : is_v ? v : k) + ((int64_t)tok0 * row_heads + g) * d;
+        // where my four elements sit in the row: x[0..1] at e0, x[2..3] at e1.  Value rows and interleaved pairs: 4 lane
+        // .. 4 lane + 3; else the pairs (j, j + 64) for j = 2 lane, 2 lane + 1
+        const bool in_order = INTERLEAVED || is_v;
+        const int e0 = in_order ? 4 * lane : 2 * lane, e1 = in_order ? 4 * lane + 2 : half + 2 * lane;
+#pragma unroll 1
+        for (int t0 = 0; t0 < ntok; t0 += U) {
+            uint32_t w0[U], w1[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                w0[u] = w1[u] = 0u;
+                if (t0 + u < ntok) {
+                    const __nv_bfloat16 *p = src + (int64_t)(t0 + u) * row_heads * d;
+                    w0[u] = *reinterpret_cast<const uint32_t *>(p + e0);
+                    w1[u] = *reinterpret_cast<const uint32_t *>(p + e1);
+                }
             }
-            if (lane == 0) qp.v_scales[scale_idx(g, cache_row)] = scale;
-            continue;
-        }
-        const bool is_q = hh < a.H;
-        const __nv_bfloat16 *src = is_q ? q + (tok * a.H + hh) * d : k + (tok * a.Hkv + (hh - a.H)) * d;
-        float x[4];
-        int e0, e1;     // where x[0..1] and x[2..3] sit in the row
-        if (!INTERLEAVED) {
-            // pairs (j, j + 64) for j = 2 lane, 2 lane + 1
-            e0 = 2 * lane; e1 = half + 2 * lane;
-            const uint32_t lo = *reinterpret_cast<const uint32_t *>(src + e0);
-            const uint32_t hi = *reinterpret_cast<const uint32_t *>(src + e1);
-            const float2 w0 = cs[t][2 * lane], w1 = cs[t][2 * lane + 1];
-            rotate(bf16_lo(lo), bf16_lo(hi), w0.x, w0.y, x[0], x[2]);
-            rotate(bf16_hi(lo), bf16_hi(hi), w1.x, w1.y, x[1], x[3]);
-        } else {
-            // pairs (2 j, 2 j + 1) for j = 2 lane, 2 lane + 1
-            e0 = 4 * lane; e1 = 4 * lane + 2;
-            const uint2 w = *reinterpret_cast<const uint2 *>(src + e0);
-            const float2 w0 = cs[t][2 * lane], w1 = cs[t][2 * lane + 1];
-            rotate(bf16_lo(w.x), bf16_hi(w.x), w0.x, w0.y, x[0], x[1]);
-            rotate(bf16_lo(w.y), bf16_hi(w.y), w1.x, w1.y, x[2], x[3]);
-        }
-        if (is_q) {
-            __nv_bfloat16 *dst = qr + (tok * a.H + hh) * d;
-            __nv_bfloat162 p0 = __floats2bfloat162_rn(x[0], x[1]), p1 = __floats2bfloat162_rn(x[2], x[3]);
-            *reinterpret_cast<__nv_bfloat162 *>(dst + e0) = p0;
-            *reinterpret_cast<__nv_bfloat162 *>(dst + e1) = p1;
-        } else {
-            const int g = hh - a.H;
-            int code[4];
-            float scale;
-            quantise4<BITS>(x, code, scale);
-            const int64_t r = code_off(g, cache_row);
-            if (BITS == 8) {
-                *reinterpret_cast<uint16_t *>(qp.k_codes + r + e0) = (uint16_t)((code[0] & 0xFF) | ((code[1] & 0xFF) << 8));
-                *reinterpret_cast<uint16_t *>(qp.k_codes + r + e1) = (uint16_t)((code[2] & 0xFF) | ((code[3] & 0xFF) << 8));
-            } else {
-                // elements e0, e0 + 1 share byte e0 / 2 (e0 and e1 are even)
-                qp.k_codes[r + e0 / 2] = (int8_t)((code[0] + 8) | ((code[1] + 8) << 4));
-                qp.k_codes[r + e1 / 2] = (int8_t)((code[2] + 8) | ((code[3] + 8) << 4));
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int t = t0 + u;
+                if (t >= ntok) break;
+                const int64_t tok = tok0 + t, cache_row = prefix + tok;
+                float x[4];
+                if (is_v) {
+                    x[0] = bf16_lo(w0[u]); x[1] = bf16_hi(w0[u]); x[2] = bf16_lo(w1[u]); x[3] = bf16_hi(w1[u]);
+                } else {
+                    const float2 c0 = cs[t][2 * lane], c1 = cs[t][2 * lane + 1];
+                    if (!INTERLEAVED) {
+                        rotate(bf16_lo(w0[u]), bf16_lo(w1[u]), c0.x, c0.y, x[0], x[2]);
+                        rotate(bf16_hi(w0[u]), bf16_hi(w1[u]), c1.x, c1.y, x[1], x[3]);
+                    } else {
+                        rotate(bf16_lo(w0[u]), bf16_hi(w0[u]), c0.x, c0.y, x[0], x[1]);
+                        rotate(bf16_lo(w1[u]), bf16_hi(w1[u]), c1.x, c1.y, x[2], x[3]);
+                    }
+                }
+                if (is_q) {
+                    __nv_bfloat16 *dst = qr + (tok * a.H + g) * d;
+                    *reinterpret_cast<__nv_bfloat162 *>(dst + e0) = __floats2bfloat162_rn(x[0], x[1]);
+                    *reinterpret_cast<__nv_bfloat162 *>(dst + e1) = __floats2bfloat162_rn(x[2], x[3]);
+                    continue;
+                }
+                int code[4];
+                float scale;
+                quantise4<BITS>(x, code, scale);
+                int8_t *codes = (is_v ? qp.v_codes : qp.k_codes) + code_off(g, cache_row);
+                if (BITS == 8) {
+                    *reinterpret_cast<uint16_t *>(codes + e0) = (uint16_t)((code[0] & 0xFF) | ((code[1] & 0xFF) << 8));
+                    *reinterpret_cast<uint16_t *>(codes + e1) = (uint16_t)((code[2] & 0xFF) | ((code[3] & 0xFF) << 8));
+                } else {
+                    // elements e0, e0 + 1 share byte e0 / 2 (e0 and e1 are even)
+                    codes[e0 / 2] = (int8_t)((code[0] + 8) | ((code[1] + 8) << 4));
+                    codes[e1 / 2] = (int8_t)((code[2] + 8) | ((code[3] + 8) << 4));
+                }
+                if (lane == 0) (is_v ? qp.v_scales : qp.k_scales)[scale_idx(g, cache_row)] = scale;
             }
-            if (lane == 0) qp.k_scales[scale_idx(g, cache_row)] = scale;
         }
     }
+}
+
+// Tokens per CTA, as for bf16 rows (rope_append.cu): one while all CTAs are resident at once, then as many as share the
+// chain of one.  us between events (32 / 8 heads, int8, cold L2) with 1, 2, 4 tokens per CTA: 256 tokens 10.2, 10.2, 12.3; 512:
+// 14.3, 12.3, 12.3; 1024: 20.5, 16.4, 16.4; 2048: 32.8, 26.6, 24.6; 8192: 106.5, 77.8, 65.6; int4 the same.
+int tokens_per_cta(int64_t tokens) { return tokens < 512 ? 1 : tokens < 1024 ? 2 : 4; }
+
+template <int TOK>
+cudaError_t launch_tok(const RopeAppendArgs &a, const QuantPlanes &qp, bool interleaved, int batch, cudaStream_t s) {
+    auto kernel = qp.bits == 4 ? (interleaved ? rope_append_q8_kernel<true, 4, TOK> : rope_append_q8_kernel<false, 4, TOK>)
+                               : (interleaved ? rope_append_q8_kernel<true, 8, TOK> : rope_append_q8_kernel<false, 8, TOK>);
+    return launch_pdl(kernel, dim3((a.n + TOK - 1) / TOK, batch), dim3(kThreads), 0, s, a, qp);
 }
 
 }  // namespace
 
 cudaError_t launch_rope_append_q8(const RopeAppendArgs &a, const QuantPlanes &qp, bool interleaved, int batch, cudaStream_t s) {
-    const dim3 grid((a.n + kTok - 1) / kTok, batch);
-    if (qp.bits == 4) {
-        if (interleaved) return launch_pdl(rope_append_q8_kernel<true, 4>, grid, dim3(kThreads), 0, s, a, qp);
-        return launch_pdl(rope_append_q8_kernel<false, 4>, grid, dim3(kThreads), 0, s, a, qp);
-    }
-    if (interleaved) return launch_pdl(rope_append_q8_kernel<true, 8>, grid, dim3(kThreads), 0, s, a, qp);
-    return launch_pdl(rope_append_q8_kernel<false, 8>, grid, dim3(kThreads), 0, s, a, qp);
+    const int tok = tokens_per_cta((int64_t)a.n * batch);
+    return tok == 4 ? launch_tok<4>(a, qp, interleaved, batch, s) : tok == 2 ? launch_tok<2>(a, qp, interleaved, batch, s)
+                                                                             : launch_tok<1>(a, qp, interleaved, batch, s);
 }
 
 }  // namespace kvf

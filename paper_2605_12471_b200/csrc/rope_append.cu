@@ -14,15 +14,13 @@
 namespace kvf {
 namespace {
 
-constexpr int kTok = 1;        // tokens per CTA: with 512 threads every thread has one 16-byte item of a bf16
-constexpr int kThreads = 512;  // Llama-shaped token (320 rotated segments + 128 value segments), all loads in flight at once
+constexpr int kThreads = 512;  // every thread has one 16-byte item of a bf16 Llama-shaped token (320 rotated segments + 128 value segments)
 
 template <typename T> struct Vec16;
 template <> struct Vec16<float> {
     static constexpr int N = 4;
-    static __device__ __forceinline__ void load(const float *p, float (&x)[4]) {
-        float4 v = *reinterpret_cast<const float4 *>(p);
-        x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w;
+    static __device__ __forceinline__ void unpack(const uint4 &v, float (&x)[4]) {
+        x[0] = __uint_as_float(v.x); x[1] = __uint_as_float(v.y); x[2] = __uint_as_float(v.z); x[3] = __uint_as_float(v.w);
     }
     static __device__ __forceinline__ void store(float *p, const float (&x)[4]) {
         *reinterpret_cast<float4 *>(p) = make_float4(x[0], x[1], x[2], x[3]);
@@ -30,8 +28,7 @@ template <> struct Vec16<float> {
 };
 template <> struct Vec16<__nv_bfloat16> {
     static constexpr int N = 8;
-    static __device__ __forceinline__ void load(const __nv_bfloat16 *p, float (&x)[8]) {
-        uint4 v = *reinterpret_cast<const uint4 *>(p);
+    static __device__ __forceinline__ void unpack(const uint4 &v, float (&x)[8]) {
         const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
@@ -58,9 +55,11 @@ __device__ __forceinline__ void rotate(float a, float b, float c, float s, float
     rb = __fmaf_rn(b, c, cross_b);
 }
 
-template <typename T, bool INTERLEAVED>
-__global__ void __launch_bounds__(kThreads) rope_append_kernel(const RopeAppendArgs a) {
+// kTok = tokens per CTA (see tokens_per_cta).
+template <typename T, bool INTERLEAVED, int kTok>
+__global__ void __launch_bounds__(kThreads, 2) rope_append_kernel(const RopeAppendArgs a) {
     constexpr int VEC = Vec16<T>::N;
+    constexpr int U = kTok < 4 ? kTok : 4;     // tokens of an item whose loads are in flight together
     __shared__ float2 cs[kTok][kMaxHalfDim];   // (cos, sin) per (token, pair)
 
     const int d = a.d, half = d / 2;
@@ -119,67 +118,74 @@ __global__ void __launch_bounds__(kThreads) rope_append_kernel(const RopeAppendA
     T *vp = reinterpret_cast<T *>(a.v_plane);
     const int heads = a.H + (a.k_new ? a.Hkv : 0);     // (queries only when no keys are given: kvf_attend)
 
-    // One loop over the rotated segments of q and k and, behind them, the value segments (verbatim
-    // 16-byte copies): a thread's items are independent, so their loads go out back to back.
+    // A thread takes the same 16-byte item of every token of the CTA (rotated segments of q and k, behind them the
+    // value segments, verbatim copies): where it lies is worked out once, and the tokens' loads go out back to back.
     const int rot_chunks = INTERLEAVED ? d / VEC : half / VEC;       // vectors per row (interleaved) or per half row
-    const int rot_items = ntok * heads * rot_chunks;
+    const int rot_items = heads * rot_chunks;
     const int v_chunks = d / VEC;
-    const int items = rot_items + (a.v_new ? ntok * a.Hkv * v_chunks : 0);
+    const int items = rot_items + (a.v_new ? a.Hkv * v_chunks : 0);
     float amax = 0.f;               // largest magnitude written (tracked only under a range limit, fp32 caches)
     const bool ranged = sizeof(T) == 4 && a.range_limit > 0.f;
     for (int idx = threadIdx.x; idx < items; idx += kThreads) {
-        if (idx >= rot_items) {
-            const int i = idx - rot_items;
-            const int c = i % v_chunks;
-            const int g = (i / v_chunks) % a.Hkv;
-            const int t = i / (v_chunks * a.Hkv);
-            const uint4 val = *reinterpret_cast<const uint4 *>(v + ((int64_t)(tok0 + t) * a.Hkv + g) * d + c * VEC);
-            *reinterpret_cast<uint4 *>(vp + rows.offset(g, prefix + tok0 + t) + c * VEC) = val;
-            if (ranged)
-                amax = fmaxf(fmaxf(amax, fmaxf(fabsf(__uint_as_float(val.x)), fabsf(__uint_as_float(val.y)))),
-                             fmaxf(fabsf(__uint_as_float(val.z)), fabsf(__uint_as_float(val.w))));
-            continue;
-        }
-        const int c = idx % rot_chunks;
-        const int hh = (idx / rot_chunks) % heads;
-        const int t = idx / (rot_chunks * heads);
-        const T *src;
-        T *dst;
-        if (hh < a.H) {
-            src = q + ((int64_t)(tok0 + t) * a.H + hh) * d;
-            dst = qr + ((int64_t)(tok0 + t) * a.H + hh) * d;
-        } else {
-            const int g = hh - a.H;
-            src = k + ((int64_t)(tok0 + t) * a.Hkv + g) * d;
-            dst = kp + rows.offset(g, prefix + tok0 + t);
-        }
-        if (!INTERLEAVED) {
-            float lo[VEC], hi[VEC], rlo[VEC], rhi[VEC];
-            Vec16<T>::load(src + c * VEC, lo);
-            Vec16<T>::load(src + half + c * VEC, hi);
+        const bool value = idx >= rot_items;
+        const int it = value ? idx - rot_items : idx, chunks = value ? v_chunks : rot_chunks;
+        const int c = it % chunks, hh = it / chunks;
+        const bool query = !value && hh < a.H;
+        const int g = value || query ? hh : hh - a.H;           // query head, or KV head
+        const int row_heads = query ? a.H : a.Hkv;
+        const T *src = (query ? q : value ? v : k) + ((int64_t)tok0 * row_heads + g) * d + c * VEC;
+        const int64_t src_step = (int64_t)row_heads * d;
+        T *plane = value ? vp : kp;
+        auto dst = [&](int t) { return (query ? qr + ((int64_t)(tok0 + t) * a.H + g) * d : plane + rows.offset(g, prefix + tok0 + t)) + c * VEC; };
+#pragma unroll 1
+        for (int t0 = 0; t0 < ntok; t0 += U) {
+            uint4 lo[U], hi[U];
 #pragma unroll
-            for (int e = 0; e < VEC; ++e) {
-                const float2 w = cs[t][c * VEC + e];
-                rotate(lo[e], hi[e], w.x, w.y, rlo[e], rhi[e]);
-            }
-            Vec16<T>::store(dst + c * VEC, rlo);
-            Vec16<T>::store(dst + half + c * VEC, rhi);
-            if (ranged) {
+            for (int u = 0; u < U; ++u)
+                if (t0 + u < ntok) {
+                    lo[u] = *reinterpret_cast<const uint4 *>(src + (t0 + u) * src_step);
+                    if (!INTERLEAVED && !value) hi[u] = *reinterpret_cast<const uint4 *>(src + (t0 + u) * src_step + half);
+                }
 #pragma unroll
-                for (int e = 0; e < VEC; ++e) amax = fmaxf(amax, fmaxf(fabsf(rlo[e]), fabsf(rhi[e])));
-            }
-        } else {
-            float x[VEC], r[VEC];
-            Vec16<T>::load(src + c * VEC, x);
+            for (int u = 0; u < U; ++u) {
+                const int t = t0 + u;
+                if (t >= ntok) break;
+                T *to = dst(t);
+                if (value) {
+                    *reinterpret_cast<uint4 *>(to) = lo[u];
+                    if (ranged)
+                        amax = fmaxf(fmaxf(amax, fmaxf(fabsf(__uint_as_float(lo[u].x)), fabsf(__uint_as_float(lo[u].y)))),
+                                     fmaxf(fabsf(__uint_as_float(lo[u].z)), fabsf(__uint_as_float(lo[u].w))));
+                    continue;
+                }
+                float x[VEC], r[VEC];
+                Vec16<T>::unpack(lo[u], x);
+                if (!INTERLEAVED) {
+                    float y[VEC], ry[VEC];
+                    Vec16<T>::unpack(hi[u], y);
 #pragma unroll
-            for (int e = 0; e < VEC; e += 2) {
-                const float2 w = cs[t][(c * VEC + e) / 2];
-                rotate(x[e], x[e + 1], w.x, w.y, r[e], r[e + 1]);
-            }
-            Vec16<T>::store(dst + c * VEC, r);
-            if (ranged) {
+                    for (int e = 0; e < VEC; ++e) {
+                        const float2 w = cs[t][c * VEC + e];
+                        rotate(x[e], y[e], w.x, w.y, r[e], ry[e]);
+                    }
+                    Vec16<T>::store(to, r);
+                    Vec16<T>::store(to + half, ry);
+                    if (ranged) {
 #pragma unroll
-                for (int e = 0; e < VEC; ++e) amax = fmaxf(amax, fabsf(r[e]));
+                        for (int e = 0; e < VEC; ++e) amax = fmaxf(amax, fabsf(ry[e]));
+                    }
+                } else {
+#pragma unroll
+                    for (int e = 0; e < VEC; e += 2) {
+                        const float2 w = cs[t][(c * VEC + e) / 2];
+                        rotate(x[e], x[e + 1], w.x, w.y, r[e], r[e + 1]);
+                    }
+                    Vec16<T>::store(to, r);
+                }
+                if (ranged) {
+#pragma unroll
+                    for (int e = 0; e < VEC; ++e) amax = fmaxf(amax, fabsf(r[e]));
+                }
             }
         }
     }
@@ -188,20 +194,33 @@ __global__ void __launch_bounds__(kThreads) rope_append_kernel(const RopeAppendA
 
 }  // namespace
 
-cudaError_t launch_rope_append(const RopeAppendArgs &a, int dtype, bool interleaved, int batch, cudaStream_t s) {
-    int blocks = (a.n + kTok - 1) / kTok;
+// Tokens per CTA.  Few tokens: one each, their CTAs are all resident at once and the step waits for one token's chain (sines,
+// loads, stores).  More: that chain is paid for once per CTA instead of once per token, in waves; four tokens are as
+// many as have their loads in registers.  us between events (32 / 8 heads, cold L2) with 1, 2, 4 tokens per CTA, bf16: 256
+// tokens 8.2, 8.2, 10.2; 512: 12.3, 10.2, 10.2; 1024: 16.4, 14.4, 12.3; 2048: 24.6, 20.5, 18.4; 8192: 71.6, 55.3, 47.1
+// (201 MB: 31 us at the copy bandwidth); fp32: 512: 14.3, 12.3, 14.3; 2048: 32.8, 26.6, 27.6; 8192: 100.4, 75.8, 76.8.
+template <typename T> static int tokens_per_cta(int64_t tokens) { return tokens < 512 ? 1 : tokens < 1024 || sizeof(T) == 4 ? 2 : 4; }
+
+template <typename T, int TOK>
+static cudaError_t launch_tok(const RopeAppendArgs &a, bool interleaved, int batch, cudaStream_t s) {
+    int blocks = (a.n + TOK - 1) / TOK;
     if (a.zero_rows > 0) {
-        int64_t vecs = (int64_t)a.zero_rows * a.Hkv * (a.d / (dtype == 0 ? 8 : 4));
+        int64_t vecs = (int64_t)a.zero_rows * a.Hkv * (a.d / Vec16<T>::N);
         blocks += (int)((vecs + kThreads - 1) / kThreads);
     }
-    if (dtype == 0) {
-        if (interleaved) return launch_pdl(rope_append_kernel<__nv_bfloat16, true>, dim3(blocks, batch), dim3(kThreads), 0, s, a);
-        else return launch_pdl(rope_append_kernel<__nv_bfloat16, false>, dim3(blocks, batch), dim3(kThreads), 0, s, a);
-    } else {
-        if (interleaved) return launch_pdl(rope_append_kernel<float, true>, dim3(blocks, batch), dim3(kThreads), 0, s, a);
-        else return launch_pdl(rope_append_kernel<float, false>, dim3(blocks, batch), dim3(kThreads), 0, s, a);
-    }
-    return cudaGetLastError();
+    return launch_pdl(interleaved ? rope_append_kernel<T, true, TOK> : rope_append_kernel<T, false, TOK>, dim3(blocks, batch), dim3(kThreads), 0, s, a);
+}
+
+template <typename T>
+static cudaError_t launch_type(const RopeAppendArgs &a, bool interleaved, int batch, cudaStream_t s) {
+    const int tok = tokens_per_cta<T>((int64_t)a.n * batch);
+    if constexpr (sizeof(T) == 2)
+        if (tok == 4) return launch_tok<T, 4>(a, interleaved, batch, s);
+    return tok == 2 ? launch_tok<T, 2>(a, interleaved, batch, s) : launch_tok<T, 1>(a, interleaved, batch, s);
+}
+
+cudaError_t launch_rope_append(const RopeAppendArgs &a, int dtype, bool interleaved, int batch, cudaStream_t s) {
+    return dtype == 0 ? launch_type<__nv_bfloat16>(a, interleaved, batch, s) : launch_type<float>(a, interleaved, batch, s);
 }
 
 }  // namespace kvf

@@ -1,0 +1,67 @@
+"""Rotate + append with several tokens per CTA (512 tokens of a launch on): the cache bits are those of short chunks, which take
+one token per CTA, and the outputs those of the same rows folded in short chunks, within the bounds of tests/chain.py (a wrong
+rotation of a query would show: inputs are N(0, 1))."""
+import pytest
+import torch
+
+from paper_2605_12471_b200 import binding
+from tests.chain import TOL
+
+pytestmark = pytest.mark.gpu
+
+KINDS = {"bf16": ("bf16", 0), "bf16_interleaved": ("bf16", binding.KVF_ROPE_INTERLEAVED), "f32": ("f32", 0),
+         "f32_interleaved": ("f32", binding.KVF_ROPE_INTERLEAVED), "int8": ("bf16", binding.KVF_CACHE_INT8),
+         "int4_interleaved": ("bf16", binding.KVF_CACHE_INT4 | binding.KVF_ROPE_INTERLEAVED)}
+
+
+def _inputs(lead, n, h, kv, d, dtype):
+    return [torch.randn(*lead, n, heads, d, device="cuda").to(torch.float32 if dtype == "f32" else torch.bfloat16) for heads in (h, kv, kv)]
+
+
+# both sides of each line of the dispatch, remainders of 2 and 4 tokens; 7 / 1 heads leave threads of a CTA without an item
+@pytest.mark.parametrize("heads", [(8, 2), (7, 1)], ids=["8_2", "7_1"])
+@pytest.mark.parametrize("kind", KINDS)
+def test_long_chunks_append_the_bits_of_short_ones(kind, heads):
+    dtype, flags = KINDS[kind]
+    torch.manual_seed(len(kind))
+    for d in (128, 64) if not flags & (binding.KVF_CACHE_INT8 | binding.KVF_CACHE_INT4) else (128,):
+        for n in (511, 512, 513, 1023, 1024, 1027, 1030):
+            first = 77
+            x = _inputs((), first + n, *heads, d, dtype)
+            got = []
+            for cuts in ([first, n], [first] + [300] * (n // 300) + [n % 300]):
+                c = binding.Cache(binding.make_config(*heads, d, dtype, first + n + 50, n, rope_base=10000.0, flags=flags))
+                c.storage.fill_(0x5A)
+                out = torch.cat([c.fold_step(*(t.contiguous() for t in step)) for step in zip(*(t.split(cuts) for t in x))])
+                assert c.status() == binding.KVF_OK
+                got.append((out.float(), c.storage))
+            rows = slice(0, first + n)
+            assert torch.equal(*(_held(s, heads[1], first + n + 50, d, dtype, flags)[:, :, rows] for _, s in got))
+            assert (got[0][0] - got[1][0]).abs().max().item() <= 2 * TOL[dtype][0]
+
+
+def _held(storage, kv, capacity, d, dtype, flags):
+    """[K and V, KV head, row, bytes of codes or elements]"""
+    row = d // 2 if flags & binding.KVF_CACHE_INT4 else d if flags & binding.KVF_CACHE_INT8 else d * (4 if dtype == "f32" else 2)
+    return storage[:2 * kv * capacity * row].view(2, kv, capacity, row)
+
+
+@pytest.mark.parametrize("flags", [0, binding.KVF_CACHE_INT8], ids=["bf16", "int8"])
+def test_batches_append_the_bits_of_single_caches(flags):
+    torch.manual_seed(3)
+    for n in (57, 114, 129):                  # 9 members: 513, 1026 and 1161 tokens to a launch
+        cfg = binding.make_config(8, 2, 128, "bf16", 300, n, rope_base=10000.0, flags=flags)
+        pools = []
+        x = _inputs((9,), n, 8, 2, 128, "bf16")
+        for together in (True, False):
+            pool = torch.zeros(binding.paged_pool_bytes(cfg, 27), dtype=torch.uint8, device="cuda")
+            tables = torch.arange(27, device="cuda").flip(0).to(torch.int32).view(9, 3)
+            caches = [binding.PagedCache(cfg, pool, 27, tables[i]) for i in range(9)]
+            if together:
+                binding.Batch(caches).fold_step(*x)
+            else:
+                for c, step in zip(caches, zip(*x)):
+                    c.fold_step(*(t.contiguous() for t in step))
+            torch.cuda.synchronize()
+            pools.append(pool)
+        assert torch.equal(*pools)
