@@ -96,7 +96,8 @@ enum {
                                   the scheme open; here a row is quantised once, when it is appended:
                                   scale = max|x| / 127, code = clamp(rint(x * (127 / max|x|)), +-127) in
                                   fp32 (keys: on the rotated row before any rounding to bf16), and the
-                                  attention sees bf16(code * scale).  dtype KVF_BF16 and head_dim 128
+                                  attention sees bf16(code * scale) - steps of at most 16 query rows,
+                                  below, code * scale unrounded.  dtype KVF_BF16 and head_dim 128
                                   only (KVF_ERR_UNSUPPORTED otherwise, and for kvf_fold_step_static);
                                   the attention kernel expands code tiles to bf16 tiles in shared
                                   memory - or, for steps of at most 16 query rows (n_tokens * H/Hkv) on

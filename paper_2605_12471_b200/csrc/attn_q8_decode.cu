@@ -5,7 +5,7 @@
 // Section 2 of the paper: the chunk's queries attend to every row of the earlier chunks and,
 // causally, to the chunk itself; query head h reads KV head h / G.  The trials of Section 4 end
 // with 30 tokens decoded one at a time, each of them such a step.  The paper's Discussion stores
-// K/V through a round trip bf16 -> intN -> bf16: the attention sees bf16(code * row scale).
+// K/V through a round trip bf16 -> intN -> bf16; here the attention sees code * row scale itself.
 //
 // Such a step has almost no arithmetic and is bound by how fast the codes leave HBM.  The
 // tensor-core kernel for long chunks expands every code tile into a bf16 tile in shared memory,
@@ -15,8 +15,18 @@
 // stage for int8, 17 KiB for int4) filled by TMA, and two consumer warps per stage, each taking
 // 64 of the tile's keys (a warp always reads the same stage, so it sees every phase of that
 // stage's barriers, which is what a parity wait needs).  A warp expands codes straight into the
-// register fragments of mma.sync m16n8k16 (bf16 in, fp32 accumulate) and keeps its own running
-// softmax and output; the warps' results are merged at the end.
+// register fragments of mma.sync m16n8k16 (fp16 in, fp32 accumulate; bf16 rows: bf16 in) and keeps its own
+// running softmax and output; the warps' results are merged at the end.
+//
+// What bounds the quantised step is, behind the bytes, the instructions a code costs.  Codes are small whole
+// numbers, which fp16 holds exactly: the MMAs run on the codes, and a row's scale is applied where the row
+// is one number, to its scores (K) and to its probabilities (V).  A code ORed into the mantissa of 1024 and one
+// packed subtraction make two fp16 values: 1.25 instructions a code for K, 1.5 for V (pairs of keys), against 2.75 for
+// bf16(code * scale) by way of fp32.  What else enters the MMAs as fp16 is first scaled by powers of two, which
+// round nothing: a query row so that its largest element lies in [2^14, 2^15) (bf16 elements down to 2^-31 of it stay
+// exact), the V scales so that the largest seen so far lies there too (they move with it like the softmax's reference
+// maximum).  Probabilities then keep 11 significant bits instead of bf16's 8, and a key 2^-28 below the largest is still
+// a normal number.
 //
 // With so few query rows the KEYS take the 16-row side of the MMA and the query rows the 8-column
 // side (one or two column blocks), so no MMA row is wasted on padding and V needs no transpose:
@@ -35,6 +45,8 @@
 // normalised partial and its log2 denominator in slot (group + KV head), which
 // combine_groups_kernel merges (or writes the output itself when there is one range per head).
 // Every mbarrier wait is bounded and reports through the status word.
+#include <cuda_fp16.h>
+
 #include "kvfold_internal.h"
 #include "sm100_ptx.cuh"
 #include "quant_expand.cuh"
@@ -83,6 +95,47 @@ __device__ __forceinline__ uint32_t transpose8x8(uint32_t x) {
     asm("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(y) : "r"(x));
     return y;
 }
+// the same on fp16
+__device__ __forceinline__ void mma_f16(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+template <int BITS>
+__device__ __forceinline__ void mma_rows(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+    if constexpr (BITS == 16) mma_bf16(c, a, b0, b1);
+    else mma_f16(c, a, b0, b1);
+}
+__device__ __forceinline__ uint32_t pack_f16(float lo, float hi) {
+    __half2 h = __floats2half2_rn(lo, hi);
+    return *reinterpret_cast<uint32_t *>(&h);
+}
+// 2^(biased - 127), biased 1 .. 254
+__device__ __forceinline__ float pow2f(int biased) { return __int_as_float(biased << 23); }
+__device__ __forceinline__ int biased_exponent(float x) { return (__float_as_int(x) >> 23) & 0xFF; }
+
+// Codes to fp16 pairs, exactly.  int8: bytes 0 and 2 of x (the codes as stored, two's complement): 0x64xx with the sign bit
+// flipped is 1024 + 128 + code.  int4: the nibbles (code + 8) at bits 0 and 16 of x as 1024 + nibble, those at bits 4
+// and 20 as 1024 + 16 * nibble.
+__device__ __forceinline__ uint32_t codes_even_bytes(uint32_t x) {
+    const uint32_t y = (x & 0x00FF00FFu) ^ 0x64806480u;
+    const uint32_t off = 0x64806480u;
+    __half2 h = __hsub2(*reinterpret_cast<const __half2 *>(&y), *reinterpret_cast<const __half2 *>(&off));
+    return *reinterpret_cast<uint32_t *>(&h);
+}
+__device__ __forceinline__ uint32_t codes_low_nibbles(uint32_t x) {
+    const uint32_t y = (x & 0x000F000Fu) | 0x64006400u;
+    const uint32_t off = 0x64086408u;                                // 1032
+    __half2 h = __hsub2(*reinterpret_cast<const __half2 *>(&y), *reinterpret_cast<const __half2 *>(&off));
+    return *reinterpret_cast<uint32_t *>(&h);
+}
+__device__ __forceinline__ uint32_t codes_high_nibbles(uint32_t x) {
+    const uint32_t y = (x & 0x00F000F0u) | 0x64006400u;
+    const uint32_t sixteenth = 0x2C002C00u, off = 0xD480D480u;       // 1 / 16, -72
+    __half2 h = __hfma2(*reinterpret_cast<const __half2 *>(&y), *reinterpret_cast<const __half2 *>(&sixteenth), *reinterpret_cast<const __half2 *>(&off));
+    return *reinterpret_cast<uint32_t *>(&h);
+}
+
 // (volatile, here and below: the tiles are rewritten by later TMA copies)
 __device__ __forceinline__ void lds128(uint32_t addr, uint32_t (&w)[4]) {
     asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]) : "r"(addr));
@@ -94,9 +147,10 @@ __device__ __forceinline__ void lds64(uint32_t addr, uint32_t (&w)[2]) {
 // A fragments of S^T = K Q^T for one 16-key block: the 32 codes d = 32 t .. 32 t + 31 of key rows
 // `row` and `row + 8` of the code tile at shared address `tile` (rows swizzled over their 16-byte
 // chunks as the TMA left them).  k-step s covers d = 32 t + 4 s .. + 3: a0 / a2 from the first row,
-// a1 / a3 from the second, each bf16(code * scale) in element order.
+// a1 / a3 from the second.  Which of the elements sit in which half is as the expansion leaves them; query_order says
+// the same to Q: bf16 0 1 | 2 3, int8 0 2 | 1 3, int4 (two k-steps) 0 4 | 1 5, 2 6 | 3 7.
 template <int BITS>
-__device__ __forceinline__ void key_fragments(uint32_t tile, int row, int t, float sc_a, float sc_b, uint32_t (&ka)[8][4]) {
+__device__ __forceinline__ void key_fragments(uint32_t tile, int row, int t, uint32_t (&ka)[8][4]) {
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         const int r = row + 8 * h;
@@ -113,8 +167,6 @@ __device__ __forceinline__ void key_fragments(uint32_t tile, int row, int t, flo
             }
             continue;
         }
-        const float s1 = h ? sc_b : sc_a;
-        const float2 sc = make_float2(s1, s1);
         if (BITS == 8) {
             // 128-byte rows, 128-byte swizzle: chunk c of row r sits at c ^ (r & 7); my chunks are 2 t and 2 t + 1
             const uint32_t base = tile + (uint32_t)r * 128u, sw = (uint32_t)r & 7u;
@@ -123,7 +175,7 @@ __device__ __forceinline__ void key_fragments(uint32_t tile, int row, int t, flo
                 uint32_t w[4];
                 lds128(base + (((2u * (uint32_t)t + c) ^ sw) << 4), w);
 #pragma unroll
-                for (int i = 0; i < 4; ++i) expand4(w[i] ^ 0x80808080u, sc, ka[4 * c + i][h], ka[4 * c + i][2 + h]);
+                for (int i = 0; i < 4; ++i) { ka[4 * c + i][h] = codes_even_bytes(w[i]); ka[4 * c + i][2 + h] = codes_even_bytes(w[i] >> 8); }
             }
         } else {
             // 64-byte rows, 64-byte swizzle: chunk c of row r sits at c ^ ((r >> 1) & 3); my chunk is t
@@ -132,30 +184,24 @@ __device__ __forceinline__ void key_fragments(uint32_t tile, int row, int t, flo
             lds128(base + (((uint32_t)t ^ sw) << 4), w);
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                uint32_t o[4];
-                expand8(w[i], sc, o);
-                ka[2 * i][h] = o[0]; ka[2 * i][2 + h] = o[1];
-                ka[2 * i + 1][h] = o[2]; ka[2 * i + 1][2 + h] = o[3];
+                ka[2 * i][h] = codes_low_nibbles(w[i]); ka[2 * i][2 + h] = codes_high_nibbles(w[i]);
+                ka[2 * i + 1][h] = codes_low_nibbles(w[i] >> 8); ka[2 * i + 1][2 + h] = codes_high_nibbles(w[i] >> 8);
             }
         }
     }
 }
-
-// bf16 pair (x(wa), x(wb)) * sc of byte `byte` of two words whose bytes hold code + `bias`
-// (2^23 + byte is exact in fp32, as is the difference that follows)
-__device__ __forceinline__ uint32_t pair_of_rows(uint32_t wa, uint32_t wb, int byte, float2 off, float2 sc) {
-    float2 x = make_float2(__uint_as_float(__byte_perm(wa, 0x4B000000u, 0x7650 + byte)),
-                           __uint_as_float(__byte_perm(wb, 0x4B000000u, 0x7650 + byte)));
-    x = __fmul2_rn(__fadd2_rn(x, off), sc);
-    return pack_bf16_pair(x.x, x.y);
+// Element (of the thread's 32 of a query row) in half e & 1 of register e >> 1 of k-step ks.
+template <int BITS>
+__device__ __forceinline__ constexpr int query_order(int ks, int e) {
+    return BITS == 16 ? 4 * ks + e
+         : BITS == 8  ? 4 * ks + 2 * (e & 1) + (e >> 1)
+                      : 8 * (ks >> 1) + 2 * (ks & 1) + 4 * (e & 1) + (e >> 1);
 }
 
-// The codes d = 16 g .. 16 g + 15 of key rows row0 + 2 t + {0, 1, 8, 9} of the V code tile, ready
-// for pair_of_rows: int8 as four words of four codes (each byte code + 128), int4 as two words of
-// low nibbles (elements 16 g + 2 i) and two of high nibbles (elements 16 g + 2 i + 1), each code + 8.
-// (bf16 rows: the 16 values themselves, eight words of two.)
+// The codes d = 16 g .. 16 g + 15 of key rows row0 + 2 t + {0, 1, 8, 9} of the V code tile (bf16 rows: the 16 values, eight
+// words of two; int8: four words; int4: two).
 template <int BITS>
-__device__ __forceinline__ void value_codes(uint32_t tile, int row0, int g, int t, uint32_t (&w)[4][BITS == 16 ? 8 : 4]) {
+__device__ __forceinline__ void value_codes(uint32_t tile, int row0, int g, int t, uint32_t (&w)[4][BITS / 2]) {
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
         const int r = row0 + 2 * t + (i & 1) + 8 * (i >> 1);
@@ -171,39 +217,32 @@ __device__ __forceinline__ void value_codes(uint32_t tile, int row0, int g, int 
             }
         } else if constexpr (BITS == 8) {
             lds128(tile + (uint32_t)r * 128u + (((uint32_t)g ^ ((uint32_t)r & 7u)) << 4), w[i]);
-#pragma unroll
-            for (int k = 0; k < 4; ++k) w[i][k] ^= 0x80808080u;
         } else {
-            uint32_t x[2];
-            lds64(tile + (uint32_t)r * 64u + (((((uint32_t)g >> 1) ^ (((uint32_t)r >> 1) & 3u)) << 4) | (((uint32_t)g & 1u) << 3)), x);
-            w[i][0] = x[0] & 0x0F0F0F0Fu; w[i][1] = x[1] & 0x0F0F0F0Fu;
-            w[i][2] = (x[0] >> 4) & 0x0F0F0F0Fu; w[i][3] = (x[1] >> 4) & 0x0F0F0F0Fu;
+            lds64(tile + (uint32_t)r * 64u + (((((uint32_t)g >> 1) ^ (((uint32_t)r >> 1) & 3u)) << 4) | (((uint32_t)g & 1u) << 3)), w[i]);
         }
     }
 }
 // A fragment jp of O^T = V^T P^T: MMA rows g / g + 8 are d = 16 g + 2 jp / + 1, columns the 16 keys.
 template <int BITS>
-__device__ __forceinline__ void value_fragment(const uint32_t (&w)[4][BITS == 16 ? 8 : 4], int jp, float2 sc01, float2 sc89, uint32_t (&va)[4]) {
-    if constexpr (BITS == 16) {
-        // word jp of a row holds the row's values at d = 16 g + 2 jp (low half) and + 1 (high half)
-        va[0] = __byte_perm(w[0][jp], w[1][jp], 0x5410);
-        va[1] = __byte_perm(w[0][jp], w[1][jp], 0x7632);
-        va[2] = __byte_perm(w[2][jp], w[3][jp], 0x5410);
-        va[3] = __byte_perm(w[2][jp], w[3][jp], 0x7632);
-    } else if constexpr (BITS == 8) {
-        const float2 off = make_float2(-8388736.f, -8388736.f);          // 2^23 + 128
-        const int word = jp >> 1, b = 2 * (jp & 1);
-        va[0] = pair_of_rows(w[0][word], w[1][word], b, off, sc01);
-        va[1] = pair_of_rows(w[0][word], w[1][word], b + 1, off, sc01);
-        va[2] = pair_of_rows(w[2][word], w[3][word], b, off, sc89);
-        va[3] = pair_of_rows(w[2][word], w[3][word], b + 1, off, sc89);
-    } else {
-        const float2 off = make_float2(-8388616.f, -8388616.f);          // 2^23 + 8
-        const int word = jp >> 2, b = jp & 3;
-        va[0] = pair_of_rows(w[0][word], w[1][word], b, off, sc01);
-        va[1] = pair_of_rows(w[0][2 + word], w[1][2 + word], b, off, sc01);
-        va[2] = pair_of_rows(w[2][word], w[3][word], b, off, sc89);
-        va[3] = pair_of_rows(w[2][2 + word], w[3][2 + word], b, off, sc89);
+__device__ __forceinline__ void value_fragment(const uint32_t (&w)[4][BITS / 2], int jp, uint32_t (&va)[4]) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {              // keys + {0, 1}, keys + {8, 9}
+        const uint32_t *a = w[2 * h], *b = w[2 * h + 1];
+        if constexpr (BITS == 16) {
+            // word jp of a row holds the row's values at d = 16 g + 2 jp (low half) and + 1 (high half)
+            va[2 * h] = __byte_perm(a[jp], b[jp], 0x5410);
+            va[2 * h + 1] = __byte_perm(a[jp], b[jp], 0x7632);
+        } else if constexpr (BITS == 8) {
+            // bytes d, d + 1 of the first row below those of the second
+            const uint32_t x = __byte_perm(a[jp >> 1], b[jp >> 1], jp & 1 ? 0x7632 : 0x5410);
+            va[2 * h] = codes_even_bytes(x);
+            va[2 * h + 1] = codes_even_bytes(x >> 8);
+        } else {
+            // nibbles d & ~3 .. + 3 of the first row below those of the second
+            const uint32_t x = __byte_perm(a[jp >> 2], b[jp >> 2], jp & 2 ? 0x7632 : 0x5410) >> (jp & 1 ? 8 : 0);
+            va[2 * h] = codes_low_nibbles(x);
+            va[2 * h + 1] = codes_high_nibbles(x);
+        }
     }
 }
 
@@ -273,6 +312,7 @@ attn_q8_decode_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
     // ot[nb][jp][{0, 1}] (first d) and [{2, 3}] (second d); maxima and sums of rows 8 nb + 2 t + {0, 1}
     float ot[NB][8][4];
     float m_run[NB][2], l_run[NB][2];
+    int v_exp = 15;                // (quantised storage) exponent of the largest V scale so far: ot is in units of 2^(v_exp - 141)
 #pragma unroll
     for (int nb = 0; nb < NB; ++nb) {
         m_run[nb][0] = m_run[nb][1] = -INFINITY;
@@ -336,21 +376,47 @@ attn_q8_decode_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
     } else {
         // ------------------------------------------------------------------ consumers: 64 keys of every tile of one stage
         const int s = warp >> 1, half = warp & 1;
-        // Q^T's B fragments of the eight k-steps, in the order the key codes are taken: k-step ks of
-        // thread t covers d = 32 t + 4 ks .. + 3 of query row 8 nb + g
+        // Q^T's B fragments of the eight k-steps, in the order the key codes are taken (query_order), of query row
+        // 8 nb + g.  (Quantised storage: as fp16, times the power of two that brings the row's largest element into
+        // [2^14, 2^15); unscale[nb] undoes it.)
         uint32_t bq[NB][8][2];
+        float unscale[NB];
         {
             const __nv_bfloat16 *q_rot = reinterpret_cast<const __nv_bfloat16 *>(a.q_rot);
 #pragma unroll
             for (int nb = 0; nb < NB; ++nb) {
                 const int R = g + 8 * nb, tok = R / G, gi = R % G;
                 const __nv_bfloat16 *src = q_rot + (((int64_t)cb * nmax + tok) * a.H + kvh * G + gi) * kD + 32 * t4;
+                uint32_t raw[16];
 #pragma unroll
                 for (int ks = 0; ks < 8; ++ks) {
                     uint2 w = make_uint2(0u, 0u);
                     if (R < nG) w = *reinterpret_cast<const uint2 *>(src + 4 * ks);
-                    bq[nb][ks][0] = w.x;
-                    bq[nb][ks][1] = w.y;
+                    raw[2 * ks] = w.x;
+                    raw[2 * ks + 1] = w.y;
+                }
+                unscale[nb] = 1.f;
+                if constexpr (BITS == 16) {
+#pragma unroll
+                    for (int ks = 0; ks < 8; ++ks) { bq[nb][ks][0] = raw[2 * ks]; bq[nb][ks][1] = raw[2 * ks + 1]; }
+                } else {
+                    float x[32], top = 0.f;
+#pragma unroll
+                    for (int k = 0; k < 16; ++k) {
+                        x[2 * k] = __uint_as_float(raw[k] << 16);
+                        x[2 * k + 1] = __uint_as_float(raw[k] & 0xFFFF0000u);
+                        top = fmaxf(top, fmaxf(fabsf(x[2 * k]), fabsf(x[2 * k + 1])));
+                    }
+                    top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, 1));
+                    top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, 2));
+                    const int e = max(biased_exponent(top), 15);         // top < 2^(e - 126)
+                    const float up = pow2f(268 - e);
+                    unscale[nb] = pow2f(e - 14);
+#pragma unroll
+                    for (int ks = 0; ks < 8; ++ks)
+#pragma unroll
+                        for (int i = 0; i < 2; ++i)
+                            bq[nb][ks][i] = pack_f16(x[query_order<BITS>(ks, 2 * i)] * up, x[query_order<BITS>(ks, 2 * i + 1)] * up);
                 }
             }
         }
@@ -365,7 +431,12 @@ attn_q8_decode_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
                 const int R = 8 * nb + 2 * t4 + e;
                 limit[nb][e] = R < nG ? (R / G + 1) * a.self_rows : (1 << 30);
             }
-        const float sl2 = a.scale_log2;
+        // softmax scale * log2(e) of query rows 8 nb + 2 t + {0, 1} (whose scaling the threads of those g know)
+        float sl2[NB][2];
+#pragma unroll
+        for (int nb = 0; nb < NB; ++nb)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) sl2[nb][e] = a.scale_log2 * __shfl_sync(0xffffffffu, unscale[nb], (2 * t4 + e) * 4);
         bool ok = true;
         for (int t = s; t < ntiles && ok; t += NST) {
             ok = mbar_wait(bar_full + 8 * s, (t / NST) & 1, ctl, a.status);
@@ -381,12 +452,19 @@ attn_q8_decode_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
 
             // ---- scores of the 64 keys: four 16-key blocks, sacc[j][nb] = keys g / g + 8 of block j, rows 8 nb + 2 t + {0, 1}
             float sacc[4][NB][4];
+            float ks_row[4][2], vs_row[4][2], vs_top = 0.f;      // scales of those keys' rows (quantised storage)
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 const int rl = 16 * j + g;                       // my first key row within the 64
                 uint32_t ka[8][4];
-                key_fragments<BITS>(k_tile, half * 64 + rl, t4, BITS != 16 && rl < in_planes ? k_sc[half * 64 + rl] : 0.f,
-                                    BITS != 16 && rl + 8 < in_planes ? k_sc[half * 64 + rl + 8] : 0.f, ka);
+                key_fragments<BITS>(k_tile, half * 64 + rl, t4, ka);
+                if constexpr (BITS != 16) {
+                    ks_row[j][0] = rl < in_planes ? k_sc[half * 64 + rl] : 0.f;
+                    ks_row[j][1] = rl + 8 < in_planes ? k_sc[half * 64 + rl + 8] : 0.f;
+                    vs_row[j][0] = rl < in_planes ? v_sc[half * 64 + rl] : 0.f;
+                    vs_row[j][1] = rl + 8 < in_planes ? v_sc[half * 64 + rl + 8] : 0.f;
+                    vs_top = fmaxf(vs_top, fmaxf(vs_row[j][0], vs_row[j][1]));
+                }
 #pragma unroll
                 for (int nb = 0; nb < NB; ++nb) {
                     // a second accumulator for the odd k-steps: two chains of four MMAs instead of one of eight
@@ -395,8 +473,8 @@ attn_q8_decode_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
                     for (int e = 0; e < 4; ++e) { sacc[j][nb][e] = 0.f; odd[e] = 0.f; }
 #pragma unroll
                     for (int ks = 0; ks < 8; ks += 2) {
-                        mma_bf16(sacc[j][nb], ka[ks], bq[nb][ks][0], bq[nb][ks][1]);
-                        mma_bf16(odd, ka[ks + 1], bq[nb][ks + 1][0], bq[nb][ks + 1][1]);
+                        mma_rows<BITS>(sacc[j][nb], ka[ks], bq[nb][ks][0], bq[nb][ks][1]);
+                        mma_rows<BITS>(odd, ka[ks + 1], bq[nb][ks + 1][0], bq[nb][ks + 1][1]);
                     }
 #pragma unroll
                     for (int e = 0; e < 4; ++e) sacc[j][nb][e] += odd[e];
@@ -408,6 +486,21 @@ attn_q8_decode_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
             uint32_t pb[4][NB][2];         // P^T as B fragments of the four 16-key steps
             float alpha[NB][2];
             bool rescale = false;
+            float v_down = 1.f;            // what the output so far shrinks by when the V scales' reference moves
+            if constexpr (BITS != 16) {
+                vs_top = fmaxf(vs_top, __shfl_xor_sync(0xffffffffu, vs_top, 4));
+                vs_top = fmaxf(vs_top, __shfl_xor_sync(0xffffffffu, vs_top, 8));
+                vs_top = fmaxf(vs_top, __shfl_xor_sync(0xffffffffu, vs_top, 16));
+                const int e = biased_exponent(vs_top);
+                if (e > v_exp) {
+                    v_down = e - v_exp > 126 ? 0.f : pow2f(127 - (e - v_exp));
+                    v_exp = e;
+                    rescale = true;
+                }
+                const float up = pow2f(268 - v_exp);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) { vs_row[j][0] *= up; vs_row[j][1] *= up; }
+            }
 #pragma unroll
             for (int nb = 0; nb < NB; ++nb) {
                 float mx[2] = {-INFINITY, -INFINITY};
@@ -415,7 +508,7 @@ attn_q8_decode_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
                 for (int j = 0; j < 4; ++j)
 #pragma unroll
                     for (int e = 0; e < 4; ++e) {
-                        float v = sacc[j][nb][e] * sl2;
+                        float v = sacc[j][nb][e] * (BITS == 16 ? sl2[nb][e & 1] : ks_row[j][e >> 1] * sl2[nb][e & 1]);
                         if (masked && rel + 16 * j + 8 * (e >> 1) >= limit[nb][e & 1]) v = -INFINITY;
                         sacc[j][nb][e] = v;
                         mx[e & 1] = fmaxf(mx[e & 1], v);
@@ -432,6 +525,7 @@ attn_q8_decode_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
                     m_run[nb][e] = m_new;
                     l_run[nb][e] *= alpha[nb][e];
                     rescale = rescale || alpha[nb][e] != 1.f;
+                    if constexpr (BITS != 16) alpha[nb][e] *= v_down;
                 }
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
@@ -440,8 +534,13 @@ attn_q8_decode_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
                     l_run[nb][0] += p0 + p2;
                     l_run[nb][1] += p1 + p3;
                     // (key g, rows 2 t, 2 t + 1) transposed: (keys 2 t, 2 t + 1; row g) - P^T's b0; keys + 8: b1
-                    pb[j][nb][0] = transpose8x8(pack_bf16_pair(p0, p1));
-                    pb[j][nb][1] = transpose8x8(pack_bf16_pair(p2, p3));
+                    if constexpr (BITS == 16) {
+                        pb[j][nb][0] = transpose8x8(pack_bf16_pair(p0, p1));
+                        pb[j][nb][1] = transpose8x8(pack_bf16_pair(p2, p3));
+                    } else {
+                        pb[j][nb][0] = transpose8x8(pack_f16(p0 * vs_row[j][0], p1 * vs_row[j][0]));
+                        pb[j][nb][1] = transpose8x8(pack_f16(p2 * vs_row[j][1], p3 * vs_row[j][1]));
+                    }
                 }
             }
             if (__any_sync(0xffffffffu, rescale)) {
@@ -456,20 +555,14 @@ attn_q8_decode_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
             // ---- O^T += V^T P^T, 16 keys at a time
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-                const int r0 = 16 * j + 2 * t4;                  // my first key row within the 64
-                float2 sc01, sc89;
-                sc01.x = BITS != 16 && r0 < in_planes ? v_sc[half * 64 + r0] : 0.f;
-                sc01.y = BITS != 16 && r0 + 1 < in_planes ? v_sc[half * 64 + r0 + 1] : 0.f;
-                sc89.x = BITS != 16 && r0 + 8 < in_planes ? v_sc[half * 64 + r0 + 8] : 0.f;
-                sc89.y = BITS != 16 && r0 + 9 < in_planes ? v_sc[half * 64 + r0 + 9] : 0.f;
-                uint32_t w[4][BITS == 16 ? 8 : 4];
+                uint32_t w[4][BITS / 2];
                 value_codes<BITS>(v_tile, half * 64 + 16 * j, g, t4, w);
 #pragma unroll
                 for (int jp = 0; jp < 8; ++jp) {
                     uint32_t va[4];
-                    value_fragment<BITS>(w, jp, sc01, sc89, va);
+                    value_fragment<BITS>(w, jp, va);
 #pragma unroll
-                    for (int nb = 0; nb < NB; ++nb) mma_bf16(ot[nb][jp], va, pb[j][nb][0], pb[j][nb][1]);
+                    for (int nb = 0; nb < NB; ++nb) mma_rows<BITS>(ot[nb][jp], va, pb[j][nb][0], pb[j][nb][1]);
                 }
             }
             __syncwarp();
@@ -485,6 +578,7 @@ attn_q8_decode_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
     if (warp < kWarps) {
         float *mo = mrg + (size_t)warp * (kMergeWarp / 4);
         float *mm = mo + kMaxRows * kD;
+        const float v_unit = pow2f(v_exp - 14);
 #pragma unroll
         for (int nb = 0; nb < NB; ++nb)
 #pragma unroll
@@ -496,7 +590,8 @@ attn_q8_decode_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
                 const int r = 8 * nb + 2 * t4 + e;
 #pragma unroll
                 for (int jp = 0; jp < 8; ++jp)
-                    *reinterpret_cast<float2 *>(mo + r * kD + 16 * g + 2 * jp) = make_float2(ot[nb][jp][e], ot[nb][jp][2 + e]);
+                    *reinterpret_cast<float2 *>(mo + r * kD + 16 * g + 2 * jp) =
+                        BITS == 16 ? make_float2(ot[nb][jp][e], ot[nb][jp][2 + e]) : make_float2(ot[nb][jp][e] * v_unit, ot[nb][jp][2 + e] * v_unit);
                 if (g == 0) {
                     mm[2 * r] = m_run[nb][e];
                     mm[2 * r + 1] = l;

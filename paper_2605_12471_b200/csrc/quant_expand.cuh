@@ -1,6 +1,6 @@
 // Expansion of quantised cache codes to the bf16 values the attention sees: bf16(code * row scale),
 // the product taken in fp32 and rounded once to bf16 (the paper's Discussion: a round trip
-// bf16 -> intN -> bf16 of the stored rows).  Shared by the kernels that read code tiles.
+// bf16 -> intN -> bf16 of the stored rows), for the kernel that needs tiles of bf16 in shared memory.
 #pragma once
 #include <cuda_bf16.h>
 #include <stdint.h>
