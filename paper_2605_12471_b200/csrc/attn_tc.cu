@@ -51,8 +51,13 @@
 // latency out of the softmax threads' chain: whether the panel is free is asked before the second half's arithmetic (a wait on a
 // barrier that is already complete takes ~250 cycles beside saturated shared memory), and whether a key tile
 // needs a mask is known from the tile number, without a vote.  (Leaving out the vote on the scores' wait as well: 312;
-// passing the turn ahead of the K slot's commit: no change.)  It takes a K/V slot of shared memory: quantised storage, which has
-// none to spare (two raw slots instead of three cost 10 %), and the two-stream mode keep the order above, and there
+// passing the turn ahead of the K slot's commit: no change.)  It takes a K/V slot of shared memory.  On quantised storage only
+// pairs of CTAs have that to spare (each keeps raw codes of the 64 rows it expands, no more), and three tile slots
+// instead of four: 439 -> 413 thousand cycles at prefix 61 K (int8, 256 tokens; int4 452 -> 422), 551 -> 512 for 2048 tokens at
+// 14 K.  What bounds them then is shared memory (MMA operands, the tile stored, sent and received: ~90 % of the
+// cycles bf16 rows take) and the turn-round of the K slot.  Tried on the way: codes from global memory into registers and
+// four slots (470 thousand: the loads queue behind the stores), the copies to the partner from a warp of their own (430).
+// CTAs on their own (quantised) and the two-stream mode keep the order above, and there
 // the exponential phases of the two tiles are sequenced per scheduler (warp w of tile 0 and warp w of tile 1
 // alternate strictly) to the same end.  Also measured: 64-key steps with two score buffers per tile (Q K^T of N = 64
 // reads shared memory at 128 bytes a cycle for 2/3 of the rate: no gain), and the maximum taken under the
@@ -104,6 +109,16 @@ constexpr uint32_t kOffRawQ8 = kOffKV + kSlotsQ8 * kTileBytes;
 constexpr uint32_t kOffScaleQ8 = kOffRawQ8 + kRawSlots * kRawBytes;      // 128 fp32 row scales per raw slot
 constexpr uint32_t kOffCtlQ8 = (kOffScaleQ8 + kRawSlots * 512 + 1023) / 1024 * 1024;
 constexpr uint32_t kSmemBytesQ8 = kOffCtlQ8 + 512 + 1024;
+// Pairs of CTAs on quantised storage (kPair): a K tile slot, two V tile slots, one panel per row tile for the probabilities
+// of keys 64-127, and a ring of four raw slots, each the 64 rows of a tile (and their scales) that this CTA expands
+constexpr int kRawSlotsPair = 4;
+constexpr int kRowsPair = 64;
+constexpr uint32_t kRawBytesPair = kRowsPair * 128;
+constexpr uint32_t kOffPPair = kOffKV + 3 * kTileBytes;
+constexpr uint32_t kOffRawPair = kOffPPair + 2 * kPanel;
+constexpr uint32_t kOffScalePair = kOffRawPair + kRawSlotsPair * kRawBytesPair;
+constexpr uint32_t kOffCtlPair = kOffScalePair + kRawSlotsPair * kRowsPair * 4;
+constexpr uint32_t kSmemBytesPair = kOffCtlPair + 512 + 1024;
 constexpr uint32_t kTmemCols = 512;
 constexpr float kRescaleThreshold = 8.0f;             // log2 units
 
@@ -111,8 +126,8 @@ constexpr float kRescaleThreshold = 8.0f;             // log2 units
 constexpr int kRingBars = 6;                  // 2 x 3 slots of the per-stream rings (shared rings have 4, quantised storage 3)
 enum { B_QFULL = 0, B_QEMPTY = 1, B_FULL0 = 2, B_EMPTY0 = B_FULL0 + kRingBars, B_SFULL0 = B_EMPTY0 + kRingBars,
        B_PA0 = B_SFULL0 + 2, B_PB0 = B_PA0 + 2, B_PVDONE0 = B_PB0 + 2, B_TURN0 = B_PVDONE0 + 2,
-       B_DRAIN0 = B_TURN0 + 8, B_RAWFULL0 = B_DRAIN0 + 2, B_RAWEMPTY0 = B_RAWFULL0 + kRawSlots,
-       B_COUNT = B_RAWEMPTY0 + kRawSlots };
+       B_DRAIN0 = B_TURN0 + 8, B_RAWFULL0 = B_DRAIN0 + 2, B_RAWEMPTY0 = B_RAWFULL0 + kRawSlotsPair,
+       B_COUNT = B_RAWEMPTY0 + kRawSlotsPair };
 
 struct Ctl {
     unsigned long long bars[40];
@@ -168,18 +183,21 @@ template <bool kWindow, int kQuant, bool kPair, bool kEarly>
 __global__ void __launch_bounds__(kQuant ? kThreadsQ8 : kThreads, 1)
 attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                const __grid_constant__ CUtensorMap map_v) {
-    static_assert(!kEarly || kQuant == 0, "the early issue needs the space of a K/V slot for its probabilities");
+    static_assert(!kEarly || kQuant == 0 || kPair, "the early issue needs the space of a K/V slot for its probabilities");
     constexpr int NS = kQuant ? kSlotsQ8 : kEarly ? kSlotsEarly : kSlots;        // slots behind the Q tiles: the shared ring's
     constexpr int SR = kQuant ? 2 : 3;                     // slots of each stream's own ring
-    constexpr uint32_t offCtl = kQuant ? kOffCtlQ8 : kOffCtl;
-    constexpr uint32_t rawBytes = kQuant == 4 ? kRawBytes / 2 : kRawBytes;   // bytes of a 128-row code tile
+    constexpr uint32_t offCtl = kPair ? kOffCtlPair : kQuant ? kOffCtlQ8 : kOffCtl;
+    constexpr uint32_t offP = kPair ? kOffPPair : kOffP;
+    constexpr int rawSlots = kPair ? kRawSlotsPair : kRawSlots, rawRows = kPair ? kRowsPair : kRows;   // ring of raw tiles, rows of one
+    constexpr uint32_t offRaw = kPair ? kOffRawPair : kOffRawQ8, offScale = kPair ? kOffScalePair : kOffScaleQ8;
+    constexpr uint32_t rawStride = rawRows * 128u, rawBytes = kQuant == 4 ? rawStride / 2 : rawStride;   // bytes of a slot, of the codes in it
     extern __shared__ uint8_t smem_raw[];
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     Ctl *ctl = reinterpret_cast<Ctl *>(smem_raw + (base - smem_u32(smem_raw)) + offCtl);
     const uint32_t bar0 = base + offCtl;
     auto bar = [&](int i) { return bar0 + 8u * (uint32_t)i; };
 
-    static_assert(!kPair || (kQuant != 0 && !kWindow), "the paired variant is for quantised caches without a window");
+    static_assert(!kPair || (kQuant != 0 && !kWindow && kEarly), "the paired variant is for quantised caches without a window, with the early issue");
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // Ranges first, row pairs from the last to the first: the row pairs that see most keys start first and the shortest
     // fill the tail.  Both in x, which has no limit a chunk could reach (y ends at 65 535: 262 140 tokens of 64 query heads
@@ -187,7 +205,7 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
     const int pairs = kPair ? (int)gridDim.x : (int)gridDim.x / a.ngroups;
     const int qpair = kPair ? (int)blockIdx.x : pairs - 1 - (int)blockIdx.x / a.ngroups;
     const int group = kPair ? (int)blockIdx.y : (int)blockIdx.x % a.ngroups;
-    const uint32_t rank = kPair ? cluster_cta_rank() : 0u;     // which of K (0) and V (1) this CTA expands
+    const uint32_t rank = kPair ? cluster_cta_rank() : 0u;     // which half of a tile's key rows this CTA expands
     const int cb = blockIdx.z;     // cache of a batch (0 when there is one cache)
     const int G = a.Gp;     // rows per token in the row layout (a power of two >= a.G, the query heads per KV head)
     // (a ragged batch keeps its members' row counts in device memory, written by an earlier kernel
@@ -238,7 +256,7 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
         mbar_init(bar(B_QEMPTY), tiles);                                  // both issuers read Q
         for (int s = 0; s < kRingBars; ++s) { mbar_init(bar(B_FULL0 + s), kQuant ? 4 : 1); mbar_init(bar(B_EMPTY0 + s), kPair ? 2 * tiles : streams == 2 ? 1 : tiles); }   // consumers of a K/V tile
         if (kQuant)
-            for (int s = 0; s < kRawSlots; ++s) { mbar_init(bar(B_RAWFULL0 + s), 1); mbar_init(bar(B_RAWEMPTY0 + s), 4); }
+            for (int s = 0; s < rawSlots; ++s) { mbar_init(bar(B_RAWFULL0 + s), 1); mbar_init(bar(B_RAWEMPTY0 + s), 4); }
         for (int i = 0; i < 2; ++i) {
             mbar_init(bar(B_SFULL0 + i), 1);
             mbar_init(bar(B_PA0 + i), 4);
@@ -272,11 +290,20 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
     // K/V tile slots.  Two row tiles: one ring of 4 (quantised storage: 3) that both issuers walk in step.  Two streams:
     // each stream owns a ring of 3 (the sixth slot is the second Q tile, unused there), because a
     // parity wait is only sound for a thread that watches every use of its barrier in order.
+    // Pairs of CTAs: K tiles share slot 0, V tiles alternate between 1 and 2.  A tile is expanded into registers before its
+    // slot is free, so filling one takes a fifth of the time two row tiles take over a key tile: K, read for 0.7 of it, has
+    // that long left; V, read for 0.8 of it but needed the moment its K is done, has not.
+    auto pair_slot = [](int num, int &slot, int &use) {
+        const int m = num >> 1;
+        slot = num & 1 ? 1 + (m & 1) : 0;
+        use = num & 1 ? m >> 1 : m;
+    };
     auto slot_addr = [&](int sl) { return base + (sl < NS ? kOffKV + (uint32_t)sl * kTileBytes : kOffQ + kTileBytes); };
 
     if (kQuant && warp >= 12) {
         // ------------------------------------------------------------------ int8 -> bf16 tile expansion
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
+        if (kPair) asm volatile("setmaxnreg.dec.sync.aligned.u32 80;");
+        else asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
         // One thread per key row; in the paired variant two threads per row (64 codes each: the thread's
         // half of d is one panel of the bf16 tile) and this CTA's 64 of the tile's 128 rows.
         const int t = kPair ? (int)rank * 64 + (warp - 12) * 16 + (lane >> 1) : (warp - 12) * 32 + lane;   // key row of the tile
@@ -296,57 +323,64 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
                     use = rc[st] / SR;
                     ++rc[st];
                 }
-                const int r = rg % kRawSlots;
+                if (kPair) pair_slot(tg, slot, use);
+                const int r = rg % rawSlots;
                 const int64_t key = (int64_t)wt.actual(kt0 + (tt >> 1)) * kRows + t;
-                ok = mbar_wait(bar(B_RAWFULL0 + r), (rg / kRawSlots) & 1, ctl, a.status);
-                if (ok) ok = mbar_wait(bar(B_EMPTY0 + slot), (use & 1) ^ 1, ctl, a.status);
+                const int rt = kPair ? t - (int)rank * kRowsPair : t;        // row in the raw slot
+                ok = mbar_wait(bar(B_RAWFULL0 + r), (rg / rawSlots) & 1, ctl, a.status);
+                if (!kPair && ok) ok = mbar_wait(bar(B_EMPTY0 + slot), (use & 1) ^ 1, ctl, a.status);
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
                 // the row's scale arrived with the tile (rows past the end of the planes were not copied)
                 float scale = 0.f;
                 if (key < a.capacity)
-                    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(scale) : "r"(base + kOffScaleQ8 + (uint32_t)r * 512u + (uint32_t)t * 4u));
+                    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(scale) : "r"(base + offScale + (uint32_t)r * (rawRows * 4u) + (uint32_t)rt * 4u));
                 const uint32_t dst = slot_addr(slot) + (uint32_t)t * 128u + hd * kPanel;
                 const float2 sc = make_float2(scale, scale);
-                if (kQuant == 4) {
-                    // 64-byte code rows, 64-byte swizzle: chunk c of row t sits at c ^ ((t >> 1) & 3)
-                    constexpr uint32_t NC = kPair ? 2 : 4;               // 16-byte chunks of codes I expand
-                    const uint32_t src = base + kOffRawQ8 + (uint32_t)r * kRawBytes + (uint32_t)t * 64u;
-                    const uint32_t sw4 = (uint32_t)((t >> 1) & 3);
-                    uint32_t w[4 * NC];
+                constexpr uint32_t NC = (kPair ? 4 : 8) / (kQuant == 4 ? 2 : 1);     // 16-byte chunks of codes I expand
+                // int8: 128-byte code rows, 128-byte swizzle, chunk c of row t sits at c ^ (t & 7); int4: 64-byte rows, 64-byte
+                // swizzle, c ^ ((t >> 1) & 3)
+                const uint32_t src = base + offRaw + (uint32_t)r * rawStride + (uint32_t)rt * (kQuant == 4 ? 64u : 128u);
+                const uint32_t swc = kQuant == 4 ? (uint32_t)((t >> 1) & 3) : sw;
+                // all 16-byte chunks of the code row first, then the arithmetic: the chunks are
+                // independent, which is what gives one thread enough work in flight
+                uint32_t w[4 * NC];
 #pragma unroll
-                    for (uint32_t c = 0; c < NC; ++c)
-                        asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
-                                     : "=r"(w[4 * c]), "=r"(w[4 * c + 1]), "=r"(w[4 * c + 2]), "=r"(w[4 * c + 3]) : "r"(src + (((c + NC * hd) ^ sw4) << 4)));
-#pragma unroll
-                    for (uint32_t k = 0; k < 4 * NC; ++k) {        // word k = 8 codes = one 16-byte chunk of the bf16 row
-                        uint32_t o[4];
+                for (uint32_t c = 0; c < NC; ++c)
+                    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+                                 : "=r"(w[4 * c]), "=r"(w[4 * c + 1]), "=r"(w[4 * c + 2]), "=r"(w[4 * c + 3]) : "r"(src + (((c + NC * hd) ^ swc) << 4)));
+                // 16-byte chunk k of the bf16 row (of my panel, when paired): eight elements
+                constexpr int NK = kPair ? 8 : 16;
+                auto expand_chunk = [&](int k, uint32_t (&o)[4]) {
+                    if (kQuant == 4) {
                         expand8(w[k], sc, o);
-                        asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(dst + (k >> 3) * kPanel + (((k & 7) ^ sw) << 4)),
-                                     "r"(o[0]), "r"(o[1]), "r"(o[2]), "r"(o[3]) : "memory");
+                    } else {
+                        expand4(w[2 * k] ^ 0x80808080u, sc, o[0], o[1]);
+                        expand4(w[2 * k + 1] ^ 0x80808080u, sc, o[2], o[3]);
                     }
+                };
+                auto store_chunk = [&](int k, const uint32_t (&o)[4]) {
+                    asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(dst + (uint32_t)(k >> 3) * kPanel + ((((uint32_t)k & 7u) ^ sw) << 4)),
+                                 "r"(o[0]), "r"(o[1]), "r"(o[2]), "r"(o[3]) : "memory");
+                };
+                if (kPair) {
+                    // expanded ahead of the slot: only the stores and the copy to the partner wait for it
+                    uint32_t o[NK][4];
+#pragma unroll
+                    for (int k = 0; k < NK; ++k) expand_chunk(k, o[k]);
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(bar(B_RAWEMPTY0 + r));
+                    ok = mbar_wait(bar(B_EMPTY0 + slot), (use & 1) ^ 1, ctl, a.status);
+                    ok = __all_sync(0xffffffffu, ok);
+                    if (!ok) break;
+#pragma unroll
+                    for (int k = 0; k < NK; ++k) store_chunk(k, o[k]);
                 } else {
-                    constexpr uint32_t NC = kPair ? 4 : 8;               // 16-byte chunks of codes I expand
-                    const uint32_t src = base + kOffRawQ8 + (uint32_t)r * kRawBytes + (uint32_t)t * 128u;
-                    // all 16-byte chunks of the code row first, then the arithmetic: the chunks are
-                    // independent, which is what gives one thread enough work in flight
-                    uint32_t w[4 * NC];
 #pragma unroll
-                    for (uint32_t c = 0; c < NC; ++c)
-                        asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
-                                     : "=r"(w[4 * c]), "=r"(w[4 * c + 1]), "=r"(w[4 * c + 2]), "=r"(w[4 * c + 3]) : "r"(src + (((c + NC * hd) ^ sw) << 4)));
-#pragma unroll
-                    for (uint32_t c = 0; c < NC; ++c) {
-                        uint32_t o[8];
-                        expand4(w[4 * c] ^ 0x80808080u, sc, o[0], o[1]);
-                        expand4(w[4 * c + 1] ^ 0x80808080u, sc, o[2], o[3]);
-                        expand4(w[4 * c + 2] ^ 0x80808080u, sc, o[4], o[5]);
-                        expand4(w[4 * c + 3] ^ 0x80808080u, sc, o[6], o[7]);
-                        const uint32_t k0 = 2 * c, k1 = 2 * c + 1;     // 16-byte chunks of the bf16 row (of my panel, when paired)
-                        asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(dst + (k0 >> 3) * kPanel + (((k0 & 7) ^ sw) << 4)),
-                                     "r"(o[0]), "r"(o[1]), "r"(o[2]), "r"(o[3]) : "memory");
-                        asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(dst + (k1 >> 3) * kPanel + (((k1 & 7) ^ sw) << 4)),
-                                     "r"(o[4]), "r"(o[5]), "r"(o[6]), "r"(o[7]) : "memory");
+                    for (int k = 0; k < NK; ++k) {
+                        uint32_t o[4];
+                        expand_chunk(k, o);
+                        store_chunk(k, o);
                     }
                 }
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the MMAs (and the copy below) read through the async proxy
@@ -368,13 +402,13 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
                         }
                     } else {
                         mbar_arrive(bar(B_FULL0 + slot));
+                        mbar_arrive(bar(B_RAWEMPTY0 + r));
                     }
-                    mbar_arrive(bar(B_RAWEMPTY0 + r));
                 }
             }
         }
     } else if (warp >= 8) {
-        if (kQuant) asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
+        if (kQuant && !kPair) asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
         else asm volatile("setmaxnreg.dec.sync.aligned.u32 80;");
         if (warp == 8 && lane == 0) {
             // ------------------------------------------------------------------ TMA producer
@@ -401,27 +435,30 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
                     const int ktile = wt.actual(kt0 + (t >> 1));
                     const int key0 = ktile * kRows;
                     if (kQuant) {
-                        // a raw code tile (128 rows of 128 bytes, 128-byte swizzle) into the next raw slot
-                        const int r = rg % kRawSlots;
-                        ok = mbar_wait(bar(B_RAWEMPTY0 + r), ((rg / kRawSlots) & 1) ^ 1, ctl, a.status);
+                        // a raw code tile (128-byte rows, 128-byte swizzle; int4 half of that) into the next raw slot: its 128
+                        // rows, or when paired the 64 of them that this CTA expands
+                        const int r = rg % rawSlots;
+                        const int first = kPair ? (int)rank * kRowsPair : 0;
+                        ok = mbar_wait(bar(B_RAWEMPTY0 + r), ((rg / rawSlots) & 1) ^ 1, ctl, a.status);
                         if (!ok) break;
+                        const uint32_t raw = base + offRaw + (uint32_t)r * rawStride, raw_scale = base + offScale + (uint32_t)r * (rawRows * 4u);
                         // ... and the rows' scales behind it (as many as the plane still holds)
                         if (page_table) {
                             // paged cache: a key tile is one page, which always holds its 128 rows and their scales
                             if (kPair || !(t & 1)) page = page_table[ktile];       // K then V of the same tile
-                            const float *scales = ((t & 1) ? a.v_scales : a.k_scales) + (int64_t)page * a.scale_page_stride + kvh * kRows;
-                            mbar_expect_tx(bar(B_RAWFULL0 + r), rawBytes + kRows * 4u);
-                            tma_load_4d(base + kOffRawQ8 + (uint32_t)r * kRawBytes, m, bar(B_RAWFULL0 + r), 0, 0, kvh, page);
-                            bulk_load(base + kOffScaleQ8 + (uint32_t)r * 512u, scales, kRows * 4u, bar(B_RAWFULL0 + r));
+                            const float *scales = ((t & 1) ? a.v_scales : a.k_scales) + (int64_t)page * a.scale_page_stride + kvh * kRows + first;
+                            mbar_expect_tx(bar(B_RAWFULL0 + r), rawBytes + rawRows * 4u);
+                            tma_load_4d(raw, m, bar(B_RAWFULL0 + r), 0, first, kvh, page);
+                            bulk_load(raw_scale, scales, rawRows * 4u, bar(B_RAWFULL0 + r));
                             ++rg;
                             continue;
                         }
-                        const int64_t left = a.scale_stride - key0;
-                        const uint32_t sbytes = (uint32_t)(left < kRows ? left : kRows) * 4u;
-                        const float *scales = ((t & 1) ? a.v_scales : a.k_scales) + (int64_t)kvh * a.scale_stride + key0;
+                        const int64_t left = a.scale_stride - (key0 + first);
+                        const uint32_t sbytes = (uint32_t)(left < 0 ? 0 : left < rawRows ? left : rawRows) * 4u;
+                        const float *scales = ((t & 1) ? a.v_scales : a.k_scales) + (int64_t)kvh * a.scale_stride + key0 + first;
                         mbar_expect_tx(bar(B_RAWFULL0 + r), rawBytes + sbytes);
-                        tma_load_3d(base + kOffRawQ8 + (uint32_t)r * kRawBytes, m, bar(B_RAWFULL0 + r), 0, key0, kvh);
-                        bulk_load(base + kOffScaleQ8 + (uint32_t)r * 512u, scales, sbytes, bar(B_RAWFULL0 + r));
+                        tma_load_3d(raw, m, bar(B_RAWFULL0 + r), 0, key0 + first, kvh);
+                        if (sbytes) bulk_load(raw_scale, scales, sbytes, bar(B_RAWFULL0 + r));
                         ++rg;
                         continue;
                     }
@@ -449,8 +486,8 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
             // do not leave while a copy may still be writing into this CTA's shared memory
             if (pc > 0) mbar_wait_drain(bar(B_QFULL), (pc - 1) & 1, a.status);
             if (kQuant) {
-                for (int c = max(0, rg - kRawSlots); c < rg; ++c)
-                    mbar_wait_drain(bar(B_RAWFULL0 + c % kRawSlots), (c / kRawSlots) & 1, a.status);
+                for (int c = max(0, rg - rawSlots); c < rg; ++c)
+                    mbar_wait_drain(bar(B_RAWFULL0 + c % rawSlots), (c / rawSlots) & 1, a.status);
             } else if (streams == 2) {
                 for (int st = 0; st < 2; ++st)
                     for (int c = max(0, rc[st] - SR); c < rc[st]; ++c)
@@ -477,7 +514,7 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
                 }
             };
             // 16 keys = 8 packed columns of P per MMA; half h covers keys 64h .. 64h+63
-            const uint64_t pdesc = desc_kmajor(base + kOffP + i * kPanel);
+            const uint64_t pdesc = desc_kmajor(base + offP + i * kPanel);
             auto issue_pv_half = [&](int slot, int h, bool accumulate) {
                 const uint64_t vdesc = desc_mnmajor(slot_addr(slot));
 #pragma unroll
@@ -500,7 +537,8 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
             // load number -> slot and parity: shared ring (number counts every load) or my own ring
             // (number counts my loads: K of my m-th tile is 2m, its V 2m + 1)
             auto ring = [&](int num, int &slot, uint32_t &par) {
-                if (streams == 2) { slot = i * SR + num % SR; par = (num / SR) & 1; }
+                if (kPair) { int use; pair_slot(num, slot, use); par = use & 1; }
+                else if (streams == 2) { slot = i * SR + num % SR; par = (num / SR) & 1; }
                 else { slot = num % NS; par = (num / NS) & 1; }
             };
             int kt0, ntiles;
@@ -571,7 +609,10 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
         }
     } else {
         // ------------------------------------------------------------------ softmax, one thread per row
-        if (kQuant) asm volatile("setmaxnreg.inc.sync.aligned.u32 192;");
+        // (the shares of the three kinds of warps add up to the launch's 64 K registers; pairs of CTAs: what 176 spill here costs less
+        // than what 56 and 72 spill there, 1.2 % of the CTA's cycles)
+        if (kPair) asm volatile("setmaxnreg.inc.sync.aligned.u32 176;");
+        else if (kQuant) asm volatile("setmaxnreg.inc.sync.aligned.u32 192;");
         else asm volatile("setmaxnreg.inc.sync.aligned.u32 208;");
         const int i = warp >> 2;                        // row tile
         const int r = (warp & 3) * 32 + lane;           // row in the tile = TMEM lane
@@ -595,7 +636,7 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
         const float2 sl2v = make_float2(sl2, sl2);
         const int64_t nG = (int64_t)nmax * G;                 // rows of a partial slot
 
-        const uint32_t p_row = base + kOffP + i * kPanel + (uint32_t)r * 128u;     // (kEarly) my row of the probability panel
+        const uint32_t p_row = base + offP + i * kPanel + (uint32_t)r * 128u;     // (kEarly) my row of the probability panel
         int it = 0, oc = 0;            // my key tiles and my finished pieces so far
         int turn_base = 0;             // turns (see below) both tile slots have taken before this piece
         bool ok = i < tiles;
@@ -788,7 +829,7 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
                 // leave as 16-byte pieces (3.6 us for the 128 KiB of partial results of a CTA).  Each warp turns
                 // its 32 rows round in its part of the probability panel, whose last P V has run: 128 bytes of
                 // every row at a time, 16-byte chunks swizzled by the row, written out as whole 128-byte lines.
-                const uint32_t stage = base + kOffP + (uint32_t)warp * 4096u;
+                const uint32_t stage = base + offP + (uint32_t)warp * 4096u;
                 const int R1 = row0 + i * kRows + (warp & 3) * 32 + (lane >> 3), lg = __ffs(G) - 1;      // first of the rows I write out
                 // (partial rows lie one after the other; G is a power of two: with a divide per row and line the
                 // index arithmetic took as long as the stores)
@@ -1053,6 +1094,7 @@ cudaError_t launch_attn_tc(const AttnArgs &a, const TcMaps &maps, cudaStream_t s
     static_assert(sizeof(Ctl) <= 512, "control block");
     static_assert(kSmemBytes <= 232448, "shared memory budget of one CTA");
     static_assert(kSmemBytesQ8 <= 232448, "shared memory budget of one CTA (int8 storage)");
+    static_assert(kSmemBytesPair <= 232448 && kOffCtlPair % 1024 == 0, "shared memory budget of one CTA (pairs of CTAs)");
     const bool quant = a.quant_bits != 0;
     auto kernel = a.quant_bits == 8 ? (a.win_lo > 0 ? attn_tc_kernel<true, 8, false, false> : attn_tc_kernel<false, 8, false, false>)
                 : a.quant_bits == 4 ? (a.win_lo > 0 ? attn_tc_kernel<true, 4, false, false> : attn_tc_kernel<false, 4, false, false>)
@@ -1061,11 +1103,11 @@ cudaError_t launch_attn_tc(const AttnArgs &a, const TcMaps &maps, cudaStream_t s
     const uint32_t smem = quant ? kSmemBytesQ8 : kSmemBytes;
     dim3 grid(attn_tc_row_pairs(a.n, a.Gp), a.ngroups, a.batch);
     if (pair_launch_ok(a)) {
-        auto paired = a.quant_bits == 8 ? attn_tc_kernel<false, 8, true, false> : attn_tc_kernel<false, 4, true, false>;
-        cudaError_t e = raise_smem_limit_once(reinterpret_cast<const void *>(paired), (int)smem);
+        auto paired = a.quant_bits == 8 ? attn_tc_kernel<false, 8, true, true> : attn_tc_kernel<false, 4, true, true>;
+        cudaError_t e = raise_smem_limit_once(reinterpret_cast<const void *>(paired), (int)kSmemBytesPair);
         if (e != cudaSuccess) return e;
-        if (pair_clusters_fit(reinterpret_cast<const void *>(paired), smem))
-            return launch_pdl_cluster2(paired, grid, dim3(kThreadsQ8), smem, s, a, maps.q, maps.k, maps.v);
+        if (pair_clusters_fit(reinterpret_cast<const void *>(paired), kSmemBytesPair))
+            return launch_pdl_cluster2(paired, grid, dim3(kThreadsQ8), kSmemBytesPair, s, a, maps.q, maps.k_half, maps.v_half);
     }
     cudaError_t e = raise_smem_limit_once(reinterpret_cast<const void *>(kernel), (int)smem);
     if (e != cudaSuccess) return e;

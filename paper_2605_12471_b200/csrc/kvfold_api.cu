@@ -262,20 +262,24 @@ kvf_status build_maps(kvf_cache *c) {
                             (uint64_t)f.max_chunk, row, row * f.n_q_heads, d, (uint32_t)c->Gp,
                             (uint32_t)(128 / c->Gp));
     if (s != KVF_OK) return s;
-    if (c->page_table && c->quant) {
-        // pages of codes: (row bytes, row in page, KV head, page), the K and the V block of a page apart
+    if (c->quant) {
+        // Codes of a box of rows of one head, 128 (int8) or 64 (int4) bytes each, swizzled over the row's 16-byte chunks: a
+        // key tile of 128 rows, and the half of one that a CTA of a pair expands.  Planes are [Hkv][capacity][row bytes];
+        // pages (row bytes, row in page, KV head, page), the K and the V block of a page apart.
         const cuuint64_t rb = (cuuint64_t)d * c->qp.bits / 8;
-        for (int kv = 0; kv < 2; ++kv) {
-            cuuint64_t dims[4] = {rb, (cuuint64_t)kKvTile, (cuuint64_t)f.n_kv_heads, (cuuint64_t)c->n_pool_pages};
-            cuuint64_t strides[3] = {rb, rb * kKvTile, (cuuint64_t)c->qp.page_bytes};
-            cuuint32_t box[4] = {(cuuint32_t)rb, (cuuint32_t)kKvTile, 1u, 1u};
-            cuuint32_t estr[4] = {1u, 1u, 1u, 1u};
-            CUresult r = fn(kv ? &c->maps.v : &c->maps.k, CU_TENSOR_MAP_DATA_TYPE_UINT8, 4, kv ? (void *)c->qp.v_codes : (void *)c->qp.k_codes,
+        const bool paged = c->page_table != nullptr;
+        const cuuint64_t dims[4] = {rb, paged ? (cuuint64_t)kKvTile : (cuuint64_t)f.capacity, (cuuint64_t)f.n_kv_heads, (cuuint64_t)c->n_pool_pages};
+        const cuuint64_t strides[3] = {rb, rb * dims[1], (cuuint64_t)c->qp.page_bytes};
+        const cuuint32_t estr[4] = {1u, 1u, 1u, 1u};
+        CUtensorMap *maps[4] = {&c->maps.k, &c->maps.v, &c->maps.k_half, &c->maps.v_half};
+        for (int i = 0; i < 4; ++i) {
+            const cuuint32_t box[4] = {(cuuint32_t)rb, (cuuint32_t)(i < 2 ? kKvTile : kKvTile / 2), 1u, 1u};
+            CUresult r = fn(maps[i], CU_TENSOR_MAP_DATA_TYPE_UINT8, paged ? 4 : 3, i & 1 ? (void *)c->qp.v_codes : (void *)c->qp.k_codes,
                             dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                             c->qp.bits == 4 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
                             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
             if (r != CUDA_SUCCESS) {
-                snprintf(g_cuda_err, sizeof(g_cuda_err), "cuTensorMapEncodeTiled (paged codes) failed with CUresult %d", (int)r);
+                snprintf(g_cuda_err, sizeof(g_cuda_err), "cuTensorMapEncodeTiled (%s) failed with CUresult %d", paged ? "paged codes" : "codes", (int)r);
                 return KVF_ERR_CUDA;
             }
         }
@@ -287,26 +291,6 @@ kvf_status build_maps(kvf_cache *c) {
         if (s != KVF_OK) return s;
         return make_page_map(fn, &c->maps.v, c->storage + c->plane_bytes, d, f.n_kv_heads, (uint64_t)c->n_pool_pages,
                              page_bytes);
-    }
-    if (c->quant) {
-        // code planes [Hkv][capacity][row bytes]: one box = 128 rows of one head x 128 (int8) or 64 (int4)
-        // bytes, swizzled over the row's 16-byte chunks
-        const cuuint64_t rb = (cuuint64_t)d * c->qp.bits / 8;
-        for (int kv = 0; kv < 2; ++kv) {
-            cuuint64_t dims[3] = {rb, (cuuint64_t)f.capacity, (cuuint64_t)f.n_kv_heads};
-            cuuint64_t strides[2] = {rb, rb * f.capacity};
-            cuuint32_t box[3] = {(cuuint32_t)rb, (cuuint32_t)kKvTile, 1u};
-            cuuint32_t estr[3] = {1u, 1u, 1u};
-            CUresult r = fn(kv ? &c->maps.v : &c->maps.k, CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, kv ? (void *)c->qp.v_codes : (void *)c->qp.k_codes,
-                            dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                            c->qp.bits == 4 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
-                            CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-            if (r != CUDA_SUCCESS) {
-                snprintf(g_cuda_err, sizeof(g_cuda_err), "cuTensorMapEncodeTiled (int8 codes) failed with CUresult %d", (int)r);
-                return KVF_ERR_CUDA;
-            }
-        }
-        return KVF_OK;
     }
     // planes [Hkv][capacity][d]: one box = 128 rows of one head x 64
     char *kbase = c->storage;

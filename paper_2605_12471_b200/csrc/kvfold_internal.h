@@ -253,6 +253,7 @@ cudaError_t launch_fold_small(const RopeAppendArgs &r, const AttnArgs &a, int dt
 // Tensor-core path (bf16, head_dim 128).
 struct TcMaps {
     CUtensorMap q, k, v;
+    CUtensorMap k_half, v_half;      // quantised storage: boxes of half a key tile's rows, for the pairs of CTAs
 };
 bool attn_tc_supported(int dtype, int d, int G);
 int attn_tc_padded_group(int G);       // G rounded up to a power of two: rows a token takes in the tcgen05 kernels' row layout

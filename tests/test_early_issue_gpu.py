@@ -53,3 +53,22 @@ def test_two_row_tiles_against_the_cuda_core_kernel(prefix, growing, out_f32):
     for n in (33, 64, 65, 190):
         for splits in (0, 1, 3):
             _run(prefix, n, splits, growing, out_f32, gen)
+
+
+# pairs of CTAs on quantised rows: the last key tile ends in the half of either CTA, at its edge, or before the second half
+@pytest.mark.parametrize("flags", [binding.KVF_CACHE_INT8, binding.KVF_CACHE_INT4], ids=["int8", "int4"])
+def test_pairs_of_ctas_at_the_end_of_the_planes(flags):
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    for n in (128, 256):
+        for prefix in (0, 44, 64, 65, 100, 172, 1000):
+            rows = prefix + n
+            x = [torch.randn(rows, heads, 128, generator=gen, device="cuda").bfloat16() for heads in (8, 2, 2)]
+            outs = []
+            for capacity in (rows, rows + 777):
+                c = binding.Cache(binding.make_config(8, 2, 128, "bf16", capacity, rows, rope_base=10000.0, flags=flags))
+                c.storage.fill_(0xFF)                # scales of rows nobody wrote: NaN
+                if prefix:
+                    c.fold_step(*(t[:prefix].contiguous() for t in x))
+                outs.append(c.fold_step(*(t[prefix:].contiguous() for t in x)))
+                assert c.status() == binding.KVF_OK
+            assert torch.isfinite(outs[0]).all() and torch.equal(*outs)
