@@ -459,11 +459,10 @@ attn_q8_decode_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
                 uint32_t ka[8][4];
                 key_fragments<BITS>(k_tile, half * 64 + rl, t4, ka);
                 if constexpr (BITS != 16) {
-                    ks_row[j][0] = rl < in_planes ? k_sc[half * 64 + rl] : 0.f;
-                    ks_row[j][1] = rl + 8 < in_planes ? k_sc[half * 64 + rl + 8] : 0.f;
-                    vs_row[j][0] = rl < in_planes ? v_sc[half * 64 + rl] : 0.f;
-                    vs_row[j][1] = rl + 8 < in_planes ? v_sc[half * 64 + rl + 8] : 0.f;
-                    vs_top = fmaxf(vs_top, fmaxf(vs_row[j][0], vs_row[j][1]));
+                    ks_row[j][0] = k_sc[half * 64 + rl];
+                    ks_row[j][1] = k_sc[half * 64 + rl + 8];
+                    vs_row[j][0] = v_sc[half * 64 + rl];
+                    vs_row[j][1] = v_sc[half * 64 + rl + 8];
                 }
 #pragma unroll
                 for (int nb = 0; nb < NB; ++nb) {
@@ -480,14 +479,37 @@ attn_q8_decode_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
                     for (int e = 0; e < 4; ++e) sacc[j][nb][e] += odd[e];
                 }
             }
-            // ---- mask (only where the chunk's own keys are near), running maximum, probabilities
-            const bool masked = key_h + 64 > P;
-            const int rel = masked ? (int)(key_h - P) + g : 0;      // my first key, counted from P (> -64 where it matters)
+            // ---- scores in log2 units, mask (only where the chunk's own keys are near: whole warps branch), running
+            // maximum, probabilities
+            if (BITS != 16 && in_planes < 64)
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+#pragma unroll
+                    for (int h = 0; h < 2; ++h)
+                        if (16 * j + 8 * h + g >= in_planes) ks_row[j][h] = vs_row[j][h] = 0.f;
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+#pragma unroll
+                for (int nb = 0; nb < NB; ++nb)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) sacc[j][nb][e] *= BITS == 16 ? sl2[nb][e & 1] : ks_row[j][e >> 1] * sl2[nb][e & 1];
+            if (key_h + 64 > P) {
+                const int rel = (int)(key_h - P) + g;               // my first key, counted from P (> -64)
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+#pragma unroll
+                    for (int nb = 0; nb < NB; ++nb)
+#pragma unroll
+                        for (int e = 0; e < 4; ++e)
+                            if (rel + 16 * j + 8 * (e >> 1) >= limit[nb][e & 1]) sacc[j][nb][e] = -INFINITY;
+            }
             uint32_t pb[4][NB][2];         // P^T as B fragments of the four 16-key steps
             float alpha[NB][2];
             bool rescale = false;
             float v_down = 1.f;            // what the output so far shrinks by when the V scales' reference moves
             if constexpr (BITS != 16) {
+#pragma unroll
+                for (int j = 0; j < 4; ++j) vs_top = fmaxf(vs_top, fmaxf(vs_row[j][0], vs_row[j][1]));
                 vs_top = fmaxf(vs_top, __shfl_xor_sync(0xffffffffu, vs_top, 4));
                 vs_top = fmaxf(vs_top, __shfl_xor_sync(0xffffffffu, vs_top, 8));
                 vs_top = fmaxf(vs_top, __shfl_xor_sync(0xffffffffu, vs_top, 16));
@@ -507,12 +529,7 @@ attn_q8_decode_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
 #pragma unroll
                 for (int j = 0; j < 4; ++j)
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        float v = sacc[j][nb][e] * (BITS == 16 ? sl2[nb][e & 1] : ks_row[j][e >> 1] * sl2[nb][e & 1]);
-                        if (masked && rel + 16 * j + 8 * (e >> 1) >= limit[nb][e & 1]) v = -INFINITY;
-                        sacc[j][nb][e] = v;
-                        mx[e & 1] = fmaxf(mx[e & 1], v);
-                    }
+                    for (int e = 0; e < 4; ++e) mx[e & 1] = fmaxf(mx[e & 1], sacc[j][nb][e]);
                 float m_safe[2];
 #pragma unroll
                 for (int e = 0; e < 2; ++e) {
