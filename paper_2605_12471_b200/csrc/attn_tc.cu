@@ -78,6 +78,8 @@
 // The kernel may be launched while the kernel before it in the stream is finishing (programmatic
 // dependent launch): everything up to pdl_wait() touches only launch arguments and the CTA's own
 // shared and tensor memory (a ragged batch, whose row counts live in device memory, waits first).
+#include <algorithm>
+
 #include "kvfold_internal.h"
 #include "sm100_ptx.cuh"
 #include "quant_expand.cuh"
@@ -932,6 +934,22 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
     if (clocked) add_clock_counters(a.status, clock64() - ctl->clk0, global_ns() - ctl->ns0);
 }
 
+// One merged row: lane = float4 column, `den` and `M` as below.
+__device__ __forceinline__ void write_merged(const AttnArgs &a, int cb, int kvh, int tok, int gi, int lane, float4 acc, float den, float M) {
+    const int64_t row = ((int64_t)cb * a.n + tok) * a.H + kvh * a.G + gi;
+    const float inv = den > 0.f ? 1.f / den : 0.f;
+    acc.x *= inv; acc.y *= inv; acc.z *= inv; acc.w *= inv;
+    if (a.out_f32) {
+        *reinterpret_cast<float4 *>(reinterpret_cast<float *>(a.out) + row * kD + lane * 4) = acc;
+    } else {
+        uint2 pk;
+        pk.x = pack_bf16(acc.x, acc.y);
+        pk.y = pack_bf16(acc.z, acc.w);
+        *reinterpret_cast<uint2 *>(reinterpret_cast<__nv_bfloat16 *>(a.out) + row * kD + lane * 4) = pk;
+    }
+    if (lane == 0 && a.lse) a.lse[row] = (M + log2f(den)) * 0.6931471805599453f;
+}
+
 // Merge the pieces of each KV head.  Group g owns [g * line / ngroups, (g+1) * line / ngroups) of
 // the (KV head, key tile) line, its piece for KV head h sits in slot g + h.  With lse_s = log2 of
 // a piece's softmax denominator and O_s its normalised output,
@@ -987,7 +1005,6 @@ __global__ void __launch_bounds__(256, kFew ? 4 : 2) combine_groups_kernel(const
         if (tok >= n) break;
         if (gi >= G) continue;
         const int64_t R = (int64_t)tok * Gp + gi;
-        const int64_t row = ((int64_t)cb * a.n + tok) * a.H + kvh * G + gi;
         const float *po = part_o + R * kD;                    // part s: po + s * nG * kD
         const float *pl = part_lse + R;                       //         pl + s * nG
         // the first eight pieces (usually all of them) are fetched together with the denominators,
@@ -1023,18 +1040,105 @@ __global__ void __launch_bounds__(256, kFew ? 4 : 2) combine_groups_kernel(const
                 }
             }
         }
-        const float inv = den > 0.f ? 1.f / den : 0.f;
-        acc.x *= inv; acc.y *= inv; acc.z *= inv; acc.w *= inv;
-        if (a.out_f32) {
-            *reinterpret_cast<float4 *>(reinterpret_cast<float *>(a.out) + row * kD + lane * 4) = acc;
-        } else {
-            uint2 pk;
-            pk.x = pack_bf16(acc.x, acc.y);
-            pk.y = pack_bf16(acc.z, acc.w);
-            *reinterpret_cast<uint2 *>(reinterpret_cast<__nv_bfloat16 *>(a.out) + row * kD + lane * 4) = pk;
-        }
-        if (lane == 0 && a.lse) a.lse[row] = (M + log2f(den)) * 0.6931471805599453f;
+        write_merged(a, cb, kvh, tok, gi, lane, acc, den, M);
     }
+}
+
+// The same merge for at most four parts (short prefixes, windows): a warp has the parts of both its rows in flight at once, so
+// a chunk whose blocks are all resident costs one trip to memory instead of one per row (four with groups of 7, whose
+// tokens take eight rows).  The same bits.
+constexpr int kSmallParts = 4, kSmallRows = 2;
+__global__ void __launch_bounds__(256, 4) combine_small_kernel(const __grid_constant__ AttnArgs a) {
+    const int kvh = blockIdx.y, cb = blockIdx.z;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, lgp = __ffs(a.Gp) - 1;
+    pdl_launch_dependents();
+    const int g0 = a.g_first[kvh], np = (a.g_last[kvh] - g0 + 1) * a.streams;
+    const int64_t nG = (int64_t)a.n * a.Gp, R0 = ((int64_t)blockIdx.x * 8 + warp) * kSmallRows;
+    const int64_t at = cb * a.part_rows + (int64_t)(g0 + kvh) * a.streams * nG + R0;      // my first row; the next part's nG further
+    const float4 *po = reinterpret_cast<const float4 *>(a.part_o + at * kD) + lane;
+    const float *pl = a.part_lse + at;
+    pdl_wait();
+    float4 pv[kSmallRows][kSmallParts];
+    float ls[kSmallRows];
+    bool live[kSmallRows];
+#pragma unroll
+    for (int u = 0; u < kSmallRows; ++u) {
+        live[u] = R0 + u < nG && ((int)(R0 + u) & (a.Gp - 1)) < a.G;          // (padding rows are computed, never merged)
+#pragma unroll
+        for (int s = 0; s < kSmallParts; ++s)
+            if (live[u] && s < np) pv[u][s] = po[(s * nG + u) * (kD / 4)];
+        ls[u] = live[u] && lane < np ? pl[lane * nG + u] : -INFINITY;
+    }
+#pragma unroll
+    for (int u = 0; u < kSmallRows; ++u) {
+        if (!live[u]) continue;
+        float M = ls[u];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+        const float wl = ls[u] == -INFINITY ? 0.f : exp2f(ls[u] - M);
+        float den = 0.f;
+        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int s = 0; s < kSmallParts; ++s)
+            if (s < np) {
+                const float w = __shfl_sync(0xffffffffu, wl, s);
+                den += w;
+                acc.x = fmaf(w, pv[u][s].x, acc.x); acc.y = fmaf(w, pv[u][s].y, acc.y);
+                acc.z = fmaf(w, pv[u][s].z, acc.z); acc.w = fmaf(w, pv[u][s].w, acc.w);
+            }
+        write_merged(a, cb, kvh, (int)((R0 + u) >> lgp), (int)(R0 + u) & (a.Gp - 1), lane, acc, den, M);
+    }
+}
+
+// The same merge where there are few rows of many parts (decode and question chunks: one to 128 rows per KV head, 18 to 36
+// parts, 74 with two KV heads): a block per row, whose eight warps fetch the parts side by side into shared memory, and one
+// of them sums them up in the order above - the same bits with one trip to memory instead of one per eight parts.
+constexpr int kRowMergeParts = 96;
+__global__ void __launch_bounds__(256) combine_rows_kernel(const __grid_constant__ AttnArgs a) {
+    extern __shared__ float4 part[];                  // [parts][32]
+    const int kvh = blockIdx.y, cb = blockIdx.z;
+    const int tok = blockIdx.x / a.G, gi = blockIdx.x % a.G;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    pdl_launch_dependents();
+    const int g0 = a.g_first[kvh], st = a.streams, np = (a.g_last[kvh] - g0 + 1) * st;
+    const int64_t nG = (int64_t)a.n * a.Gp, R = (int64_t)tok * a.Gp + gi;
+    const int64_t at = cb * a.part_rows + (int64_t)(g0 + kvh) * st * nG + R;      // part s: nG rows further
+    const float4 *po = reinterpret_cast<const float4 *>(a.part_o + at * kD) + lane;
+    const float *pl = a.part_lse + at;
+    pdl_wait();
+    float ls[kRowMergeParts / 32];                   // (warp 0) lane s: denominators of parts s, s + 32, ...
+#pragma unroll
+    for (int h = 0; h < kRowMergeParts / 32; ++h) ls[h] = warp == 0 && lane + 32 * h < np ? pl[(lane + 32 * h) * nG] : -INFINITY;
+    float4 v[kRowMergeParts / 8];
+#pragma unroll
+    for (int k = 0; k < kRowMergeParts / 8; ++k)
+        if (warp + 8 * k < np) v[k] = po[(warp + 8 * k) * nG * (kD / 4)];
+#pragma unroll
+    for (int k = 0; k < kRowMergeParts / 8; ++k)
+        if (warp + 8 * k < np) part[(warp + 8 * k) * 32 + lane] = v[k];
+    __syncthreads();
+    if (warp > 0) return;
+    float M = ls[0];
+#pragma unroll
+    for (int h = 1; h < kRowMergeParts / 32; ++h) M = fmaxf(M, ls[h]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+    float wl[kRowMergeParts / 32];
+#pragma unroll
+    for (int h = 0; h < kRowMergeParts / 32; ++h) wl[h] = ls[h] == -INFINITY ? 0.f : exp2f(ls[h] - M);
+    float den = 0.f;
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int h = 0; h < kRowMergeParts / 32; ++h)
+#pragma unroll 8
+        for (int s = 32 * h; s < min(np, 32 * h + 32); ++s) {
+            const float w = __shfl_sync(0xffffffffu, wl[h], s & 31);
+            const float4 x = part[s * 32 + lane];
+            den += w;
+            acc.x = fmaf(w, x.x, acc.x); acc.y = fmaf(w, x.y, acc.y);
+            acc.z = fmaf(w, x.z, acc.z); acc.w = fmaf(w, x.w, acc.w);
+        }
+    write_merged(a, cb, kvh, tok, gi, lane, acc, den, M);
 }
 
 }  // namespace
@@ -1118,8 +1222,21 @@ cudaError_t launch_combine_groups(const AttnArgs &a, cudaStream_t s) {
     dim3 grid((a.n + kCombineTokens - 1) / kCombineTokens, a.Hkv, a.batch);
     // at most eight parts per KV head (two streams x four pieces, or eight pieces)?  The host knows when it
     // worked out the groups of each head.
-    bool few = a.range_valid != 0 && a.Hkv <= kRangeHeads;
-    for (int h = 0; few && h < a.Hkv; ++h) few = (a.g_last[h] - a.g_first[h] + 1) * a.streams <= 8;
+    const bool known = a.range_valid != 0 && a.Hkv <= kRangeHeads;
+    int most = 0;
+    for (int h = 0; known && h < a.Hkv; ++h) most = std::max(most, (a.g_last[h] - a.g_first[h] + 1) * a.streams);
+    // Four parts at most, two rows to a warp in flight: 256 tokens of 28 / 4 heads 10.5 -> 8.5 us between events, 512 tokens of
+    // 32 / 8 heads 11.5 -> 10.6, 256 tokens 8.5 both ways (window_32k, 128 such steps back to back: 3073 -> 2992 us).
+    if (known && most <= kSmallParts) {
+        const int64_t rows = (int64_t)a.n * a.Gp;
+        return launch_pdl(combine_small_kernel, dim3((unsigned)((rows + 8 * kSmallRows - 1) / (8 * kSmallRows)), a.Hkv, a.batch), dim3(256), 0, s, a);
+    }
+    const bool few = known && most <= 8;
+    // Nine parts and more, a block per row while all of them are resident at once (eight to an SM): one token of 32 / 8
+    // heads, 18 parts, 8.5 -> 6.5 us, four tokens 12.7 -> 6.6, 32 tokens (36 parts) 16.8 -> 10.6; one of 12 / 2 heads, 74 parts,
+    // 16.7 -> 8.5.
+    if (known && !few && most <= kRowMergeParts && (int64_t)a.n * a.H * a.batch <= 8 * 148)
+        return launch_pdl(combine_rows_kernel, dim3(a.n * a.G, a.Hkv, a.batch), dim3(256), (size_t)most * 512, s, a);
     if (few) return launch_pdl(combine_groups_kernel<true>, grid, dim3(256), 0, s, a);
     return launch_pdl(combine_groups_kernel<false>, grid, dim3(256), 0, s, a);
 }
