@@ -15,7 +15,7 @@
 // visible, rows of the chunk causally.
 //
 // Measured (fp32, 64 tokens of 4 / 1 heads at prefix 448, replayed back to back): 33.9 us per step through the three
-// kernels, 8.8 us here, ~7 of them the same at prefix 0 (launch, one trip to memory, one key tile, the merge). A key
+// kernels, 8.7 us here, 5.6 at prefix 0 (launch, one trip to memory, one key tile of 32, the merge). A key
 // tile more in a slice costs 3.7 - 5 us: latency of dependent shared-memory loads at two warps per scheduler (IPC
 // 0.34, half of the stall cycles on them), so slices are as short as the device has room for.  Tried: 4 x 4 blocks
 // per thread on half the threads (a third less shared-memory traffic, fewer warps: 6.3 us a tile).
@@ -24,18 +24,18 @@
 namespace kvf {
 namespace {
 
-constexpr int BM = 32, BN = 64, D = 64, HALF = D / 2, kThreads = 256;
-constexpr int TR = 2;                // query rows per thread (x 4 keys, x 4 output columns)
+constexpr int BM = 32, kMaxBN = 64, D = 64, HALF = D / 2, kThreads = 256;
+constexpr int TR = 2;                // query rows per thread (x BN / 16 keys, x 4 output columns)
 constexpr int QS = D + 4;            // padded row stride of the Q, K and probability tiles (floats)
 constexpr int kMaxRanks = 1 << (kFoldSmallWidths - 1);     // slices of the key tiles = CTAs of a cluster
 
 struct Smem {
     float q[BM * QS];
-    float k[BN * QS];                // behind the last key tile: this CTA's unnormalised output [BM][D]
-    float v[BN * D];
+    float k[kMaxBN * QS];                // behind the last key tile: this CTA's unnormalised output [BM][D]
+    float v[kMaxBN * D];
     float p[BM * QS];
     float2 cs_q[BM][HALF];           // (cos, sin) per (token of the row tile, pair)
-    float2 cs_k[BN][HALF];           // ... per (key of the tile that belongs to the chunk, pair)
+    float2 cs_k[kMaxBN][HALF];           // ... per (key of the tile that belongs to the chunk, pair)
     float m[BM], l[BM];
 };
 
@@ -120,11 +120,13 @@ __device__ __forceinline__ void cluster_sync() {
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-template <typename T, bool INTERLEAVED>
+// BN = keys of a tile: 64, or 32 (see fold_small_ranks).
+template <typename T, bool INTERLEAVED, int BN>
 __global__ void __launch_bounds__(kThreads, 2) fold_small_kernel(const __grid_constant__ RopeAppendArgs r, const __grid_constant__ AttnArgs a) {
     constexpr int VEC = 16 / (int)sizeof(T);
     constexpr int RC = HALF / VEC;                       // vectors of half a row
-    constexpr int KI = BN * RC / kThreads;               // (first half, second half) vector pairs of a key tile per thread
+    constexpr int NK = BN / 16;                          // keys of a thread
+    constexpr int KI = (BN * RC + kThreads - 1) / kThreads;               // (first half, second half) vector pairs of a key tile per thread
     constexpr int VI = BN * 2 * RC / kThreads;           // vectors of a value tile per thread
     extern __shared__ __align__(16) uint8_t smem_raw[];
     Smem &sm = *reinterpret_cast<Smem *>(smem_raw);
@@ -178,6 +180,7 @@ __global__ void __launch_bounds__(kThreads, 2) fold_small_kernel(const __grid_co
 #pragma unroll
         for (int u = 0; u < KI; ++u) {
             const int i = tid + u * kThreads;
+            if (BN * RC < kThreads && i >= BN * RC) break;
             const T *src = row_of(kp, k_new, key0 + i / RC);
             klo[u] = src ? *reinterpret_cast<const uint4 *>(src + i % RC * VEC) : zero;
             khi[u] = src ? *reinterpret_cast<const uint4 *>(src + HALF + i % RC * VEC) : zero;
@@ -239,6 +242,7 @@ __global__ void __launch_bounds__(kThreads, 2) fold_small_kernel(const __grid_co
 #pragma unroll
         for (int u = 0; u < KI; ++u) {
             const int i = tid + u * kThreads, row = i / RC, c = i % RC;
+            if (BN * RC < kThreads && i >= BN * RC) break;
             const int64_t key = key0 + row;
             float lo[VEC], hi[VEC];
             unpack(klo[u], lo);
@@ -267,28 +271,28 @@ __global__ void __launch_bounds__(kThreads, 2) fold_small_kernel(const __grid_co
         if (kt + 1 < kt_end) fetch(kt + 1);               // in flight under this tile's arithmetic
 
         // (packed multiply-adds: two sums per score, over even and odd elements)
-        float2 s2[TR][4] = {};
+        float2 s2[TR][NK] = {};
 #pragma unroll 4
         for (int k4 = 0; k4 < D / 4; ++k4) {
-            float4 qa[TR], kb[4];
+            float4 qa[TR], kb[NK];
 #pragma unroll
             for (int i = 0; i < TR; ++i) qa[i] = *reinterpret_cast<const float4 *>(sm.q + (TR * ty + i) * QS + k4 * 4);
 #pragma unroll
-            for (int j = 0; j < 4; ++j) kb[j] = *reinterpret_cast<const float4 *>(sm.k + (tx + 16 * j) * QS + k4 * 4);
+            for (int j = 0; j < NK; ++j) kb[j] = *reinterpret_cast<const float4 *>(sm.k + (tx + 16 * j) * QS + k4 * 4);
 #pragma unroll
             for (int i = 0; i < TR; ++i)
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
+                for (int j = 0; j < NK; ++j) {
                     s2[i][j] = __ffma2_rn(make_float2(qa[i].x, qa[i].y), make_float2(kb[j].x, kb[j].y), s2[i][j]);
                     s2[i][j] = __ffma2_rn(make_float2(qa[i].z, qa[i].w), make_float2(kb[j].z, kb[j].w), s2[i][j]);
                 }
         }
-        float s[TR][4];
+        float s[TR][NK];
 #pragma unroll
         for (int i = 0; i < TR; ++i) {
             float mx = -INFINITY;
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
+            for (int j = 0; j < NK; ++j) {
                 const int64_t key = key0 + tx + 16 * j;
                 const bool vis = key < limit[i] && (key >= a.win_lo || key < a.n_sink);
                 s[i][j] = vis ? (s2[i][j].x + s2[i][j].y) * a.scale_log2 : -INFINITY;
@@ -300,7 +304,7 @@ __global__ void __launch_bounds__(kThreads, 2) fold_small_kernel(const __grid_co
             const float alpha = exp2f(m[i] - m_safe);
             float sum = 0.f;
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
+            for (int j = 0; j < NK; ++j) {
                 const float p = exp2f(s[i][j] - m_safe);
                 sum += p;
                 sm.p[(TR * ty + i) * QS + tx + 16 * j] = p;
@@ -385,7 +389,7 @@ __global__ void __launch_bounds__(kThreads, 2) fold_small_kernel(const __grid_co
 
 // Once per kernel and device: shared-memory limit, clusters of 16 CTAs (beyond the portable eight), and how many clusters
 // of each width the device holds at once.
-template <typename T, bool INTERLEAVED>
+template <typename T, bool INTERLEAVED, int BN>
 cudaError_t prepare_once(FoldSmallFit *fit) {
     struct Done { int dev; FoldSmallFit fit; };
     static std::mutex mu;
@@ -399,7 +403,7 @@ cudaError_t prepare_once(FoldSmallFit *fit) {
             if (fit) *fit = d.fit;
             return cudaSuccess;
         }
-    auto kernel = fold_small_kernel<T, INTERLEAVED>;
+    auto kernel = fold_small_kernel<T, INTERLEAVED, BN>;
     e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Smem));
     if (e != cudaSuccess) return e;
     Done now = {dev, {}};
@@ -428,9 +432,9 @@ cudaError_t prepare_once(FoldSmallFit *fit) {
     return cudaSuccess;
 }
 
-template <typename T, bool INTERLEAVED>
-cudaError_t launch_t(const RopeAppendArgs &r, const AttnArgs &a, int ranks, cudaStream_t s) {
-    cudaError_t e = prepare_once<T, INTERLEAVED>(nullptr);
+template <typename T, bool INTERLEAVED, int BN>
+cudaError_t launch_bn(const RopeAppendArgs &r, const AttnArgs &a, int ranks, cudaStream_t s) {
+    cudaError_t e = prepare_once<T, INTERLEAVED, BN>(nullptr);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(fold_small_row_tiles(a.n, a.G), a.Hkv, ranks);
@@ -446,30 +450,59 @@ cudaError_t launch_t(const RopeAppendArgs &r, const AttnArgs &a, int ranks, cuda
     attr[1].val.clusterDim.z = (unsigned)ranks;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, fold_small_kernel<T, INTERLEAVED>, r, a);
+    return cudaLaunchKernelEx(&cfg, fold_small_kernel<T, INTERLEAVED, BN>, r, a);
+}
+
+template <typename T, bool INTERLEAVED>
+cudaError_t launch_t(const RopeAppendArgs &r, const AttnArgs &a, const FoldSmallCut &cut, cudaStream_t s) {
+    return cut.keys == 32 ? launch_bn<T, INTERLEAVED, 32>(r, a, cut.ranks, s) : launch_bn<T, INTERLEAVED, 64>(r, a, cut.ranks, s);
 }
 
 }  // namespace
 
 int fold_small_row_tiles(int n, int G) { return (int)(((int64_t)n * G + BM - 1) / BM); }
 
-// Slices of the key tiles = CTAs of a cluster: a power of two, at least one key tile each, and no more clusters than the
-// device holds at once: a second wave costs more than longer slices.  Two CTAs fit an SM, but a cluster stays within
-// one GPC: of 16 CTAs the device holds 14 clusters (16 row tiles, 24 key tiles: 16 slices 37.4 us, 8 slices 28.6), of 8 CTAs
-// fewer than 36 (36 row tiles, 16 key tiles: 8 slices 36.1 us, through three launches 34.4).
+// Slices of the key tiles = CTAs of a cluster: a power of two, and no more clusters than the device holds at once: a second
+// wave costs more than longer slices.  Two CTAs fit an SM, but a cluster stays within one GPC: of 16 CTAs the device holds 14
+// clusters (16 row tiles, 24 key tiles: 16 slices 37.4 us, 8 slices 28.6), of 8 CTAs fewer than 36 (36 row tiles, 16 key
+// tiles: 8 slices 36.1 us, through three launches 34.4).
 int fold_small_ranks(int row_tiles, int64_t key_tiles, const FoldSmallFit &fit) {
     int ranks = 1;
     for (int i = 1; i < kFoldSmallWidths && (1 << i) <= key_tiles && row_tiles <= fit.clusters[i]; ++i) ranks = 1 << i;
     return ranks;
 }
 
-// (the four kernels differ in arithmetic only: what fits one fits all)
-cudaError_t fold_small_fit(FoldSmallFit *fit) { return prepare_once<float, false>(fit); }
+// The cut a small step runs with: as many slices as that or more, in tiles of 64 or 32 keys, by what the longest slice costs
+// (us per tile: 3.9 while a cluster's CTAs have an SM each, 6.6 where they share it; 32 keys 2.2).  More slices than whole
+// tiles fit into (the last ones empty) where that makes the longest one shorter: 64 tokens of 4 / 1 heads, three key tiles
+// in two slices 14.3 us, in four 7.8; five in four 14.5, in eight 8.6.  Tiles of 32 keys up to 64 CTAs: the same step in
+// eight slices 6.7, 64 tokens at prefix 0 7.0 -> 5.6, one token 5.8 -> 4.3 (bf16 6.1 -> 4.8); with more CTAs what a slice saves goes
+// into the larger merge (eight row tiles, 16 slices: 8.7 -> 9.2) and long slices gain nothing.  (A window's first tile
+// holds its sinks, up to 64: no tiles of 32.)
+FoldSmallCut fold_small_cut(int row_tiles, int64_t keys, bool window, const FoldSmallFit &fit) {
+    auto cost = [&](const FoldSmallCut &c) {
+        const int64_t tiles = (keys + c.keys - 1) / c.keys, slice = (tiles + c.ranks - 1) / c.ranks;
+        const bool alone = 2 * (int64_t)row_tiles * c.ranks <= fit.clusters[0];
+        return (double)slice * (c.keys == 32 ? 2.2 : alone ? 3.9 : 6.6) + 0.05 * c.ranks;
+    };
+    FoldSmallCut best = {64, fold_small_ranks(row_tiles, (keys + 63) / 64, fit)};
+    for (int bn = 64; bn >= (window ? 64 : 32); bn -= 32)
+        for (int i = 0; i < kFoldSmallWidths; ++i) {
+            const FoldSmallCut c = {bn, 1 << i};
+            if (row_tiles > fit.clusters[i] || (i > 0 && (int64_t)(c.ranks / 2) * bn >= keys)) break;
+            if (bn == 32 && (int64_t)row_tiles * c.ranks > 64) break;
+            if (c.ranks >= best.ranks && cost(c) < cost(best)) best = c;
+        }
+    return best;
+}
 
-cudaError_t launch_fold_small(const RopeAppendArgs &r, const AttnArgs &a, int dtype, bool interleaved, cudaStream_t s) {
+// (the four kernels differ in arithmetic only: what fits one fits all)
+cudaError_t fold_small_fit(FoldSmallFit *fit) { return prepare_once<float, false, 64>(fit); }
+
+cudaError_t launch_fold_small(const RopeAppendArgs &r, const AttnArgs &a, const FoldSmallCut &cut, int dtype, bool interleaved, cudaStream_t s) {
     if (a.d != D) return cudaErrorInvalidValue;
-    if (dtype == 0) return interleaved ? launch_t<__nv_bfloat16, true>(r, a, a.splits, s) : launch_t<__nv_bfloat16, false>(r, a, a.splits, s);
-    return interleaved ? launch_t<float, true>(r, a, a.splits, s) : launch_t<float, false>(r, a, a.splits, s);
+    if (dtype == 0) return interleaved ? launch_t<__nv_bfloat16, true>(r, a, cut, s) : launch_t<__nv_bfloat16, false>(r, a, cut, s);
+    return interleaved ? launch_t<float, true>(r, a, cut, s) : launch_t<float, false>(r, a, cut, s);
 }
 
 }  // namespace kvf

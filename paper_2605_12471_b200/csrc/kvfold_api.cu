@@ -309,6 +309,7 @@ struct Plan {
     int splits;    // CUDA-core path: splits of the key range; tensor-core path: ranges per KV head (rounded up)
     int ngroups;   // tensor-core path: ranges of the (KV head, key tile) line
     int ctas, kernels;
+    FoldSmallCut cut;   // of a small step
 };
 
 // `batch` caches share the launch (their CTAs fill the SMs together) and `part_rows_cap` is the
@@ -491,8 +492,10 @@ Plan make_plan(const kvf_cache *c, int n, int64_t prefix, int batch = 1, int64_t
         if (ranks >= 16 && n > 64 && c->cfg.dtype == KVF_BF16) longest -= 1;
         if (2 * tiles * nt <= 9 * (int64_t)c->sm_count && nt <= longest * ranks) {
             p.small = true;
-            p.splits = ranks;
-            p.ctas = tiles * ranks;
+            const bool window = window_lo(c, prefix) > 0;
+            p.cut = fold_small_cut(tiles, window ? nt * 64 : L, window, c->small_fit);
+            p.splits = p.cut.ranks;
+            p.ctas = tiles * p.cut.ranks;
             p.kernels = 1;
             return p;
         }
@@ -711,7 +714,7 @@ kvf_status step_impl(kvf_cache *c, const void *q, const void *k_new, const void 
     if (!plan.small) c->launches++;
     {
         ProfScope ps(c, st, 1);
-        if (plan.small) e = launch_fold_small(ra, aa, f.dtype, (f.flags & KVF_ROPE_INTERLEAVED) != 0, st);
+        if (plan.small) e = launch_fold_small(ra, aa, plan.cut, f.dtype, (f.flags & KVF_ROPE_INTERLEAVED) != 0, st);
         else if (plan.qdec) e = launch_attn_q8_decode(aa, c->maps, st);
         else if (c->tc) e = launch_attn_tc(aa, c->maps, st);
         else if (c->tc32) e = launch_attn_tc32(aa, st);

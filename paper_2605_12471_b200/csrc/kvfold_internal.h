@@ -240,7 +240,7 @@ cudaError_t launch_attn_simt(const AttnArgs &a, int dtype, cudaStream_t s, int *
 cudaError_t launch_combine(const AttnArgs &a, int dtype, cudaStream_t s);
 int attn_simt_ctas(int n, int G, int Hkv, int splits);
 
-// Whole small step in one launch (head_dim 64; fold_small.cu): AttnArgs::splits = CTAs of a cluster.
+// Whole small step in one launch (head_dim 64; fold_small.cu).
 int fold_small_row_tiles(int n, int G);      // row tiles per KV head = grid.x
 constexpr int kFoldSmallWidths = 5;          // clusters of 1, 2, 4, 8 and 16 CTAs
 struct FoldSmallFit {
@@ -248,7 +248,11 @@ struct FoldSmallFit {
 };
 cudaError_t fold_small_fit(FoldSmallFit *fit);     // of the current device
 int fold_small_ranks(int row_tiles, int64_t key_tiles, const FoldSmallFit &fit);     // slices of the 64-row key tiles (row_tiles: of all KV heads)
-cudaError_t launch_fold_small(const RopeAppendArgs &r, const AttnArgs &a, int dtype, bool interleaved, cudaStream_t s);
+struct FoldSmallCut {
+    int keys, ranks;                         // keys of a tile (64 or 32), slices
+};
+FoldSmallCut fold_small_cut(int row_tiles, int64_t keys, bool window, const FoldSmallFit &fit);      // (keys: that the step sees)
+cudaError_t launch_fold_small(const RopeAppendArgs &r, const AttnArgs &a, const FoldSmallCut &cut, int dtype, bool interleaved, cudaStream_t s);
 
 // Tensor-core path (bf16, head_dim 128).
 struct TcMaps {

@@ -112,6 +112,33 @@ def test_long_prefixes_take_the_launches_that_split_them(n, h, kv, tiles, kernel
     assert torch.equal(small.storage, general.storage)
 
 
+# tiles of 32 keys: prefixes around their edges and around every number of slices, chunks within one and across two of them
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("flags", [0, binding.KVF_ROPE_INTERLEAVED], ids=["half", "interleaved"])
+def test_short_slices(dtype, flags):
+    gen = torch.Generator(device="cuda").manual_seed(7)
+    slices = set()
+    for prefix in (0, 1, 31, 32, 33, 63, 64, 97, 128, 130, 191, 255, 256, 400, 480):
+        for n in (1, 5, 32, 33, 64):
+            small, general = _caches(4, 1, dtype, prefix + n, prefix + n, flags)
+            got = []
+            held, new = _inputs(4, 1, max(prefix, 1), dtype, gen), _inputs(4, 1, n, dtype, gen)
+            for c in (small, general):
+                c.storage.fill_(0x5A)
+                if prefix:
+                    general.set_len(0)
+                    general.fold_step(*held)
+                    c.storage.copy_(general.storage)
+                c.set_len(prefix)
+                lse = torch.empty(n, 4, device="cuda")
+                got.append((c.fold_step(*new, lse=lse), lse))
+            slices.add(small.plan(n, prefix)[1])
+            assert small.plan(n, prefix)[3] == 1 and small.status() == binding.KVF_OK
+            _compare(*got, dtype)
+            assert torch.equal(small.storage, general.storage)
+    assert slices == {1, 2, 4, 8, 16}
+
+
 def test_chunks_of_two_key_tiles_on_bf16_rows_have_shorter_slices():
     for dtype, kernels in (("f32", 1), ("bf16", 3)):
         c, _ = _caches(2, 2, dtype, 4096, 160)
