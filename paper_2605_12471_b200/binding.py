@@ -174,7 +174,14 @@ def workspace_bytes(cfg: kvf_config) -> int:
     return int(load().kvf_workspace_bytes(ctypes.byref(cfg)))
 
 
+# The current stream's handle without a Stream object around it (3.3 us): steps of a few microseconds wait for it.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
 def _stream_ptr(stream: Optional[torch.cuda.Stream]) -> int:
+    if stream is None and _raw_stream is not None and _device is not None and torch.cuda.is_initialized():
+        return _raw_stream(_device())
     return (stream or torch.cuda.current_stream()).cuda_stream
 
 
@@ -229,16 +236,17 @@ class Cache:
                   pos0: Optional[int] = None, out: Optional[torch.Tensor] = None,
                   lse: Optional[torch.Tensor] = None, stream: Optional[torch.cuda.Stream] = None) -> torch.Tensor:
         """kvf_fold_step on device tensors; returns the chunk's attention output."""
+        # (a step of a toy model is a few microseconds on the GPU: the call does no more than it needs)
+        lib, h, dtype = _lib or load(), self._h, self.torch_dtype
+        assert q.is_cuda and q.is_contiguous() and q.dtype is dtype
+        assert k_new.is_cuda and k_new.is_contiguous() and k_new.dtype is dtype
+        assert v_new.is_cuda and v_new.is_contiguous() and v_new.dtype is dtype
         n = q.shape[0]
-        for t in (q, k_new, v_new):
-            assert t.is_cuda and t.is_contiguous() and t.dtype == self.torch_dtype
         if out is None:
             out = torch.empty((n, self.cfg.n_q_heads, self.cfg.head_dim), dtype=self.out_dtype, device=q.device)
-        if pos0 is None:
-            pos0 = len(self)
-        rc = load().kvf_fold_step(self._h, q.data_ptr(), k_new.data_ptr(), v_new.data_ptr(), n, int(pos0),
-                                  out.data_ptr(), lse.data_ptr() if lse is not None else None,
-                                  _stream_ptr(stream))
+        rc = lib.kvf_fold_step(h, q.data_ptr(), k_new.data_ptr(), v_new.data_ptr(), n,
+                               lib.kvf_cache_len(h) if pos0 is None else int(pos0), out.data_ptr(),
+                               None if lse is None else lse.data_ptr(), _stream_ptr(stream))
         if rc != KVF_OK:
             raise KvfError(rc, "kvf_fold_step")
         return out
