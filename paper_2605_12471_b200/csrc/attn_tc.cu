@@ -370,8 +370,8 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
                     uint32_t o[NK][4];
 #pragma unroll
                     for (int k = 0; k < NK; ++k) expand_chunk(k, o[k]);
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(bar(B_RAWEMPTY0 + r));
+                    // (The raw slot is given back behind the stores, below, not here: nothing but they makes sure that the loads
+                    // of the codes have returned, and a load held up behind the MMAs' operands could read the next tile.)
                     ok = mbar_wait(bar(B_EMPTY0 + slot), (use & 1) ^ 1, ctl, a.status);
                     ok = __all_sync(0xffffffffu, ok);
                     if (!ok) break;
@@ -404,8 +404,8 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
                         }
                     } else {
                         mbar_arrive(bar(B_FULL0 + slot));
-                        mbar_arrive(bar(B_RAWEMPTY0 + r));
                     }
+                    mbar_arrive(bar(B_RAWEMPTY0 + r));
                 }
             }
         }

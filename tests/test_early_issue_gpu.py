@@ -72,3 +72,23 @@ def test_pairs_of_ctas_at_the_end_of_the_planes(flags):
                 outs.append(c.fold_step(*(t[prefix:].contiguous() for t in x)))
                 assert c.status() == binding.KVF_OK
             assert torch.isfinite(outs[0]).all() and torch.equal(*outs)
+
+
+@pytest.mark.parametrize("flags", [binding.KVF_CACHE_INT8, binding.KVF_CACHE_INT4], ids=["int8", "int4"])
+def test_pairs_of_ctas_repeat_their_bits(flags):
+    """A raw tile given back before its codes were read would show as another tile's codes now and then."""
+    gen = torch.Generator(device="cuda").manual_seed(6)
+    n = 256
+    for prefix in (2048, 8448, 20000):
+        c = binding.Cache(binding.make_config(32, 8, 128, "bf16", prefix + n, 2048, rope_base=10000.0, flags=flags))
+        for at in range(0, prefix, 2048):
+            c.fold_step(*(torch.randn(min(2048, prefix - at), heads, 128, generator=gen, device="cuda").bfloat16() for heads in (32, 8, 8)))
+        x = [torch.randn(n, heads, 128, generator=gen, device="cuda").bfloat16() for heads in (32, 8, 8)]
+        first = c.fold_step(*x)
+        outs = [torch.empty_like(first) for _ in range(50)]
+        for _ in range(8):
+            for out in outs:
+                c.set_len(prefix)
+                c.fold_step(*x, out=out)
+            assert all(torch.equal(first, out) for out in outs)
+        assert c.status() == binding.KVF_OK
