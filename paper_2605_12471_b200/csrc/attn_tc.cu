@@ -54,7 +54,7 @@
 // passing the turn ahead of the K slot's commit: no change.)  It takes a K/V slot of shared memory.  On quantised storage only
 // pairs of CTAs have that to spare (each keeps raw codes of the 64 rows it expands, no more), and three tile slots
 // instead of four: 439 -> 413 thousand cycles at prefix 61 K (int8, 256 tokens; int4 452 -> 422), 551 -> 512 for 2048 tokens at
-// 14 K.  What bounds them then is shared memory (MMA operands, the tile stored, sent and received: ~90 % of the
+// 14 K, 65 536 tokens in chunks of 256 43.2 -> 41.5 ms; 41.9 since a raw slot is given back behind the stores.  What bounds them then is shared memory (MMA operands, the tile stored, sent and received: ~90 % of the
 // cycles bf16 rows take) and the turn-round of the K slot.  Tried on the way: codes from global memory into registers and
 // four slots (470 thousand: the loads queue behind the stores), the copies to the partner from a warp of their own (430).
 // CTAs on their own (quantised) and the two-stream mode keep the order above, and there
