@@ -169,7 +169,7 @@ __global__ void __launch_bounds__(kThreads, 2) rope_append_q8_kernel(const RopeA
 // Tokens per CTA, as for bf16 rows (rope_append.cu): one while all CTAs are resident at once, then as many as share the
 // chain of one.  us between events (32 / 8 heads, int8, cold L2) with 1, 2, 4 tokens per CTA: 256 tokens 10.2, 10.2, 12.3; 512:
 // 14.3, 12.3, 12.3; 1024: 20.5, 16.4, 16.4; 2048: 32.8, 26.6, 24.6; 8192: 106.5, 77.8, 65.6; int4 the same.
-int tokens_per_cta(int64_t tokens) { return tokens < 512 ? 1 : tokens < 1024 ? 2 : 4; }
+int tokens_per_cta(int64_t tokens) { return tokens <= 2 * 148 ? 1 : tokens < 1024 ? 2 : 4; }
 
 template <int TOK>
 cudaError_t launch_tok(const RopeAppendArgs &a, const QuantPlanes &qp, bool interleaved, int batch, cudaStream_t s) {

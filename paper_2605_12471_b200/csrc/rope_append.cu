@@ -194,12 +194,13 @@ __global__ void __launch_bounds__(kThreads, 2) rope_append_kernel(const RopeAppe
 
 }  // namespace
 
-// Tokens per CTA.  Few tokens: one each, their CTAs are all resident at once and the step waits for one token's chain (sines,
+// Tokens per CTA.  Few tokens: one each, their CTAs are all resident at once (two to an SM) and the step waits for one token's chain (sines,
 // loads, stores).  More: that chain is paid for once per CTA instead of once per token, in waves; four tokens are as
 // many as have their loads in registers.  us between events (32 / 8 heads, cold L2) with 1, 2, 4 tokens per CTA, bf16: 256
 // tokens 8.2, 8.2, 10.2; 512: 12.3, 10.2, 10.2; 1024: 16.4, 14.4, 12.3; 2048: 24.6, 20.5, 18.4; 8192: 71.6, 55.3, 47.1
-// (201 MB: 31 us at the copy bandwidth); fp32: 512: 14.3, 12.3, 14.3; 2048: 32.8, 26.6, 27.6; 8192: 100.4, 75.8, 76.8.
-template <typename T> static int tokens_per_cta(int64_t tokens) { return tokens < 512 ? 1 : tokens < 1024 || sizeof(T) == 4 ? 2 : 4; }
+// (201 MB: 31 us at the copy bandwidth); 436 tokens of 28 / 4 heads, fp32, one each are a second wave: 66.2 us for the two
+// steps of a chain, two each 64.3; fp32: 512: 14.3, 12.3, 14.3; 2048: 32.8, 26.6, 27.6; 8192: 100.4, 75.8, 76.8.
+template <typename T> static int tokens_per_cta(int64_t tokens) { return tokens <= 2 * 148 ? 1 : tokens < 1024 || sizeof(T) == 4 ? 2 : 4; }
 
 template <typename T, int TOK>
 static cudaError_t launch_tok(const RopeAppendArgs &a, bool interleaved, int batch, cudaStream_t s) {

@@ -1,4 +1,4 @@
-"""Rotate + append with several tokens per CTA (512 tokens of a launch on): the cache bits are those of short chunks, which take
+"""Rotate + append with several tokens per CTA (297 tokens of a launch on): the cache bits are those of short chunks, which take
 one token per CTA, and the outputs those of the same rows folded in short chunks, within the bounds of tests/chain.py (a wrong
 rotation of a query would show: inputs are N(0, 1))."""
 import pytest
@@ -25,11 +25,11 @@ def test_long_chunks_append_the_bits_of_short_ones(kind, heads):
     dtype, flags = KINDS[kind]
     torch.manual_seed(len(kind))
     for d in (128, 64) if not flags & (binding.KVF_CACHE_INT8 | binding.KVF_CACHE_INT4) else (128,):
-        for n in (511, 512, 513, 1023, 1024, 1027, 1030):
+        for n in (296, 297, 300, 513, 1023, 1024, 1027, 1030):
             first = 77
             x = _inputs((), first + n, *heads, d, dtype)
             got = []
-            for cuts in ([first, n], [first] + [300] * (n // 300) + [n % 300]):
+            for cuts in ([first, n], [first] + [250] * (n // 250) + [n % 250]):
                 c = binding.Cache(binding.make_config(*heads, d, dtype, first + n + 50, n, rope_base=10000.0, flags=flags))
                 c.storage.fill_(0x5A)
                 out = torch.cat([c.fold_step(*(t.contiguous() for t in step)) for step in zip(*(t.split(cuts) for t in x))])
@@ -49,7 +49,7 @@ def _held(storage, kv, capacity, d, dtype, flags):
 @pytest.mark.parametrize("flags", [0, binding.KVF_CACHE_INT8], ids=["bf16", "int8"])
 def test_batches_append_the_bits_of_single_caches(flags):
     torch.manual_seed(3)
-    for n in (57, 114, 129):                  # 9 members: 513, 1026 and 1161 tokens to a launch
+    for n in (33, 57, 114, 129):              # 9 members: 297, 513, 1026 and 1161 tokens to a launch
         cfg = binding.make_config(8, 2, 128, "bf16", 300, n, rope_base=10000.0, flags=flags)
         pools = []
         x = _inputs((9,), n, 8, 2, 128, "bf16")
