@@ -97,7 +97,12 @@ enum {
                                   scale = max|x| / 127, code = clamp(rint(x * (127 / max|x|)), +-127) in
                                   fp32 (keys: on the rotated row before any rounding to bf16), and the
                                   attention sees bf16(code * scale) - steps of at most 16 query rows,
-                                  below, code * scale unrounded.  dtype KVF_BF16 and head_dim 128
+                                  below, code * scale unrounded (in a batch the longest chunk of the
+                                  launch decides for all members; under a window every step sees the
+                                  rounded value).  Such a step rounds the product of a probability and
+                                  a V row's scale once: to 11 bits, 8 bits from 2^-30 of the largest
+                                  product among the keys that the query row sees, to zero below 2^-39
+                                  of it.  dtype KVF_BF16 and head_dim 128
                                   only (KVF_ERR_UNSUPPORTED otherwise, and for kvf_fold_step_static);
                                   the attention kernel expands code tiles to bf16 tiles in shared
                                   memory - or, for steps of at most 16 query rows (n_tokens * H/Hkv) on

@@ -52,6 +52,8 @@ def _load():
     lib.okvf_cache_reset.restype = None
     lib.okvf_cache_set_quant.argtypes = [ctypes.c_void_p, ctypes.c_int]
     lib.okvf_cache_set_quant.restype = ctypes.c_int
+    lib.okvf_cache_set_unrounded.argtypes = [ctypes.c_void_p, ctypes.c_int]
+    lib.okvf_cache_set_unrounded.restype = None
     lib.okvf_quant_row.argtypes = [fp, ctypes.c_int, ctypes.c_int, ip, fp, fp]
     lib.okvf_quant_row.restype = None
     lib.okvf_cache_set_window.argtypes = [ctypes.c_void_p, ctypes.c_int64, ctypes.c_int64]
@@ -175,6 +177,10 @@ class OracleCache:
         """Quantised storage: rows go through an int8 / int4 round trip when appended (bits = 8 / 4; 0 = off)."""
         if _load().okvf_cache_set_quant(self._h, int(bits)) != 0:
             raise ValueError("only 0, 8 or 4 bits")
+
+    def set_unrounded(self, on: bool):
+        """How the steps that follow read quantised rows: code * scale, or (the default) that rounded to bf16."""
+        _load().okvf_cache_set_unrounded(self._h, int(on))
 
     def set_window(self, n_sink: int, window: int):
         """Sink + window variant: earlier chunks' rows are visible only if among the first n_sink

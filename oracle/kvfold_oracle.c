@@ -50,7 +50,10 @@
  * and a value row goes through the same three lines unrotated; amax = 0 gives
  * codes 0 and scale 0.  The decision that produces an integer is taken in
  * fp32, the precision the CUDA library takes it in; the attention over the
- * stored values stays in fp64.
+ * stored values stays in fp64.  Steps of a few query rows multiply the codes
+ * themselves and see code_j * scale without the rounding to bf16: with
+ * okvf_cache_set_unrounded(c, 1) the steps that follow read every row, earlier
+ * ones too, that way (the rows held are the same).
  *
  * Readings taken where the paper is silent (each is a build-wide reading):
  *   - RoPE pairs element j with element j + d/2 (rotate-half); the
@@ -76,10 +79,12 @@ typedef struct okvf_cache {
     int64_t capacity, len;
     int64_t n_sink, window; /* window <= 0: every earlier row is visible */
     int quant_bits;         /* 0: rows are stored as given; 8 / 4: int8 / int4 round trip at append */
+    int unrounded;          /* quantised rows are read as code * scale */
     double scale;
     double *inv_freq; /* [head_dim/2] */
     double *K;        /* [n_kv_heads][capacity][head_dim], rotated keys */
     double *V;        /* [n_kv_heads][capacity][head_dim] */
+    double *K_prod, *V_prod; /* quantised rows as code * scale (NULL without quantised storage) */
 } okvf_cache;
 
 /* inv_freq[j] = base^(-2j/d)  (RoFormer's frequencies, cited by Section 2). */
@@ -117,7 +122,7 @@ okvf_cache *okvf_cache_create(int n_q_heads, int n_kv_heads, int head_dim, int64
 
 void okvf_cache_destroy(okvf_cache *c) {
     if (!c) return;
-    free(c->inv_freq); free(c->K); free(c->V); free(c);
+    free(c->inv_freq); free(c->K); free(c->V); free(c->K_prod); free(c->V_prod); free(c);
 }
 
 int64_t okvf_cache_len(const okvf_cache *c) { return c->len; }
@@ -125,9 +130,17 @@ void okvf_cache_reset(okvf_cache *c) { c->len = 0; }
 /* Quantised storage (see the header): bits = 0, 8 or 4.  Returns 0, or 1 for other values. */
 int okvf_cache_set_quant(okvf_cache *c, int bits) {
     if (bits != 0 && bits != 8 && bits != 4) return 1;
+    if (bits != 0 && !c->K_prod) {
+        size_t plane = (size_t)c->n_kv_heads * (size_t)c->capacity * (size_t)c->head_dim;
+        c->K_prod = (double *)malloc(sizeof(double) * plane);
+        c->V_prod = (double *)malloc(sizeof(double) * plane);
+        if (!c->K_prod || !c->V_prod) return 1;
+    }
     c->quant_bits = bits;
     return 0;
 }
+/* Quantised rows as the steps that follow read them: code * scale (on), or that rounded to bf16. */
+void okvf_cache_set_unrounded(okvf_cache *c, int on) { c->unrounded = on != 0; }
 /* Sink + window variant (see the header); window <= 0 switches it off. */
 void okvf_cache_set_window(okvf_cache *c, int64_t n_sink, int64_t window) {
     c->n_sink = n_sink < 0 ? 0 : n_sink;
@@ -266,15 +279,22 @@ int okvf_fold_step(okvf_cache *c, const double *q, const double *k_new, const do
             if (c->quant_bits != 0) {
                 /* the row as the library holds it: fp32 rotation in the faithful order, int8 round
                  * or int4 round trip, bf16; the value row likewise without the rotation */
-                float xf[512], rot[512], st[512];
+                float xf[512], rot[512], st[512], scale;
+                int32_t code[512];
                 if (d > 512) return 1;
                 for (int e = 0; e < d; ++e) xf[e] = (float)k_new[src + e];
                 okvf_rope_faithful(xf, 1, 1, d, pos0 + i, c->inv_freq, c->interleaved, 0, rot);
-                okvf_quant_row(rot, d, c->quant_bits, NULL, NULL, st);
-                for (int e = 0; e < d; ++e) c->K[dst + e] = (double)st[e];
+                okvf_quant_row(rot, d, c->quant_bits, code, &scale, st);
+                for (int e = 0; e < d; ++e) {
+                    c->K[dst + e] = (double)st[e];
+                    c->K_prod[dst + e] = (double)code[e] * (double)scale;
+                }
                 for (int e = 0; e < d; ++e) xf[e] = (float)v_new[src + e];
-                okvf_quant_row(xf, d, c->quant_bits, NULL, NULL, st);
-                for (int e = 0; e < d; ++e) c->V[dst + e] = (double)st[e];
+                okvf_quant_row(xf, d, c->quant_bits, code, &scale, st);
+                for (int e = 0; e < d; ++e) {
+                    c->V[dst + e] = (double)st[e];
+                    c->V_prod[dst + e] = (double)code[e] * (double)scale;
+                }
                 continue;
             }
             rope_vec(k_new + src, c->K + dst, d, pos0 + i, c->inv_freq, c->interleaved);
@@ -292,8 +312,9 @@ int okvf_fold_step(okvf_cache *c, const double *q, const double *k_new, const do
             double *qr = (double *)malloc(sizeof(double) * (size_t)d);
             double *s = (double *)malloc(sizeof(double) * (size_t)visible);
             rope_vec(q + ((size_t)i * H + h) * d, qr, d, pos0 + i, c->inv_freq, c->interleaved);
-            const double *Kg = c->K + (size_t)g * cap * d;
-            const double *Vg = c->V + (size_t)g * cap * d;
+            const int prod = c->quant_bits != 0 && c->unrounded;
+            const double *Kg = (prod ? c->K_prod : c->K) + (size_t)g * cap * d;
+            const double *Vg = (prod ? c->V_prod : c->V) + (size_t)g * cap * d;
             double m = -INFINITY;
             for (int64_t r = 0; r < visible; ++r) {
                 /* sink + window: an earlier chunk's row survives eviction only as a sink or

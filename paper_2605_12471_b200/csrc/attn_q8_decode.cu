@@ -23,10 +23,17 @@
 // is one number, to its scores (K) and to its probabilities (V).  A code ORed into the mantissa of 1024 and one
 // packed subtraction make two fp16 values: 1.25 instructions a code for K, 1.5 for V (pairs of keys), against 2.75 for
 // bf16(code * scale) by way of fp32.  What else enters the MMAs as fp16 is first scaled by powers of two, which
-// round nothing: a query row so that its largest element lies in [2^14, 2^15) (bf16 elements down to 2^-31 of it stay
-// exact), the V scales so that the largest seen so far lies there too (they move with it like the softmax's reference
-// maximum).  Probabilities then keep 11 significant bits instead of bf16's 8, and a key 2^-28 below the largest is still
-// a normal number.
+// round nothing:
+//  - a query row so that its largest element lies in [2^14, 2^15), which keeps bf16 elements down to 2^-31 of it exact.  Where
+//    a row has nonzero elements below that, the MMAs of Q K^T take queries and codes as bf16 instead (codes then
+//    cost 1.75 instructions), so that scores are always sums of exact products;
+//  - the products of probability and V scale so that the largest that the row has seen lies in [2^14, 2^16): per query row,
+//    over the keys that it sees, because a row that is hidden from it, or that hardly counts, must not
+//    decide what is left of the others.  Products keep 11 significant bits (bf16 probabilities had 8), 8 of them down to
+//    2^-30 of the row's largest; what vanishes is 2^-39 of it and less, far below the fp32 sums.
+// (One reference per warp, the largest V scale loaded so far, lost rows 2^33 below a hidden one.  Without references: products
+// as bf16 with V codes as bf16, 8 bits, cost 2 us of 54 at one token of int8 and 5.5 of 73 at four; in two bf16 parts 5 and 16.  As it is:
+// one token as before, four tokens of int8 73.5 -> 76.8 us, of int4 65.5 -> 66: two blocks of query rows have no registers to spare.)
 //
 // With so few query rows the KEYS take the 16-row side of the MMA and the query rows the 8-column
 // side (one or two column blocks), so no MMA row is wasted on padding and V needs no transpose:
@@ -46,6 +53,8 @@
 // combine_groups_kernel merges (or writes the output itself when there is one range per head).
 // Every mbarrier wait is bounded and reports through the status word.
 #include <cuda_fp16.h>
+
+#include <type_traits>
 
 #include "kvfold_internal.h"
 #include "sm100_ptx.cuh"
@@ -101,10 +110,10 @@ __device__ __forceinline__ void mma_f16(float (&c)[4], const uint32_t (&a)[4], u
                  : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
                  : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
-template <int BITS>
+template <bool F16>
 __device__ __forceinline__ void mma_rows(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-    if constexpr (BITS == 16) mma_bf16(c, a, b0, b1);
-    else mma_f16(c, a, b0, b1);
+    if constexpr (F16) mma_f16(c, a, b0, b1);
+    else mma_bf16(c, a, b0, b1);
 }
 __device__ __forceinline__ uint32_t pack_f16(float lo, float hi) {
     __half2 h = __floats2half2_rn(lo, hi);
@@ -136,6 +145,15 @@ __device__ __forceinline__ uint32_t codes_high_nibbles(uint32_t x) {
     return *reinterpret_cast<uint32_t *>(&h);
 }
 
+// Codes to bf16 pairs, exactly (for queries that fp16 does not hold).  int8: seven bits in the mantissa of 128, less 128 or,
+// with the sign bit as the lowest bit of the exponent, 256.  int4: the nibbles at bits 0 and 16 as 128 + nibble.
+__device__ __forceinline__ uint32_t sub_bf16(uint32_t x, uint32_t y) {
+    __nv_bfloat162 d = __hsub2(*reinterpret_cast<const __nv_bfloat162 *>(&x), *reinterpret_cast<const __nv_bfloat162 *>(&y));
+    return *reinterpret_cast<uint32_t *>(&d);
+}
+__device__ __forceinline__ uint32_t bf16_even_bytes(uint32_t x) { return sub_bf16((x & 0x007F007Fu) | 0x43004300u, (x & 0x00800080u) | 0x43004300u); }
+__device__ __forceinline__ uint32_t bf16_low_nibbles(uint32_t x) { return sub_bf16((x & 0x000F000Fu) | 0x43004300u, 0x43084308u); }
+
 // (volatile, here and below: the tiles are rewritten by later TMA copies)
 __device__ __forceinline__ void lds128(uint32_t addr, uint32_t (&w)[4]) {
     asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]) : "r"(addr));
@@ -148,8 +166,8 @@ __device__ __forceinline__ void lds64(uint32_t addr, uint32_t (&w)[2]) {
 // `row` and `row + 8` of the code tile at shared address `tile` (rows swizzled over their 16-byte
 // chunks as the TMA left them).  k-step s covers d = 32 t + 4 s .. + 3: a0 / a2 from the first row,
 // a1 / a3 from the second.  Which of the elements sit in which half is as the expansion leaves them; query_order says
-// the same to Q: bf16 0 1 | 2 3, int8 0 2 | 1 3, int4 (two k-steps) 0 4 | 1 5, 2 6 | 3 7.
-template <int BITS>
+// the same to Q: bf16 0 1 | 2 3, int8 0 2 | 1 3, int4 (two k-steps) 0 4 | 1 5, 2 6 | 3 7.  F16: codes as fp16, else as bf16.
+template <int BITS, bool F16>
 __device__ __forceinline__ void key_fragments(uint32_t tile, int row, int t, uint32_t (&ka)[8][4]) {
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
@@ -175,7 +193,10 @@ __device__ __forceinline__ void key_fragments(uint32_t tile, int row, int t, uin
                 uint32_t w[4];
                 lds128(base + (((2u * (uint32_t)t + c) ^ sw) << 4), w);
 #pragma unroll
-                for (int i = 0; i < 4; ++i) { ka[4 * c + i][h] = codes_even_bytes(w[i]); ka[4 * c + i][2 + h] = codes_even_bytes(w[i] >> 8); }
+                for (int i = 0; i < 4; ++i) {
+                    ka[4 * c + i][h] = F16 ? codes_even_bytes(w[i]) : bf16_even_bytes(w[i]);
+                    ka[4 * c + i][2 + h] = F16 ? codes_even_bytes(w[i] >> 8) : bf16_even_bytes(w[i] >> 8);
+                }
             }
         } else {
             // 64-byte rows, 64-byte swizzle: chunk c of row r sits at c ^ ((r >> 1) & 3); my chunk is t
@@ -184,12 +205,21 @@ __device__ __forceinline__ void key_fragments(uint32_t tile, int row, int t, uin
             lds128(base + (((uint32_t)t ^ sw) << 4), w);
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                ka[2 * i][h] = codes_low_nibbles(w[i]); ka[2 * i][2 + h] = codes_high_nibbles(w[i]);
-                ka[2 * i + 1][h] = codes_low_nibbles(w[i] >> 8); ka[2 * i + 1][2 + h] = codes_high_nibbles(w[i] >> 8);
+                ka[2 * i][h] = F16 ? codes_low_nibbles(w[i]) : bf16_low_nibbles(w[i]);
+                ka[2 * i][2 + h] = F16 ? codes_high_nibbles(w[i]) : bf16_low_nibbles(w[i] >> 4);
+                ka[2 * i + 1][h] = F16 ? codes_low_nibbles(w[i] >> 8) : bf16_low_nibbles(w[i] >> 8);
+                ka[2 * i + 1][2 + h] = F16 ? codes_high_nibbles(w[i] >> 8) : bf16_low_nibbles(w[i] >> 12);
             }
         }
     }
 }
+// Largest of the values that the eight threads of a query row hold (they differ in the keys).
+__device__ __forceinline__ float max_of_keys(float x) {
+    x = fmaxf(x, __shfl_xor_sync(0xffffffffu, x, 4));
+    x = fmaxf(x, __shfl_xor_sync(0xffffffffu, x, 8));
+    return fmaxf(x, __shfl_xor_sync(0xffffffffu, x, 16));
+}
+
 // Element (of the thread's 32 of a query row) in half e & 1 of register e >> 1 of k-step ks.
 template <int BITS>
 __device__ __forceinline__ constexpr int query_order(int ks, int e) {
@@ -312,11 +342,14 @@ attn_q8_decode_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
     // ot[nb][jp][{0, 1}] (first d) and [{2, 3}] (second d); maxima and sums of rows 8 nb + 2 t + {0, 1}
     float ot[NB][8][4];
     float m_run[NB][2], l_run[NB][2];
-    int v_exp = 15;                // (quantised storage) exponent of the largest V scale so far: ot is in units of 2^(v_exp - 141)
+    // (quantised storage) probabilities times V scales enter the MMAs, and ot, times 2^(up - 127): each row's largest product
+    // is then 2^14 or more and below fp16's end
+    int up[NB][2];
 #pragma unroll
     for (int nb = 0; nb < NB; ++nb) {
         m_run[nb][0] = m_run[nb][1] = -INFINITY;
         l_run[nb][0] = l_run[nb][1] = 0.f;
+        up[nb][0] = up[nb][1] = 127;
 #pragma unroll
         for (int jp = 0; jp < 8; ++jp)
 #pragma unroll
@@ -377,17 +410,17 @@ attn_q8_decode_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
         // ------------------------------------------------------------------ consumers: 64 keys of every tile of one stage
         const int s = warp >> 1, half = warp & 1;
         // Q^T's B fragments of the eight k-steps, in the order the key codes are taken (query_order), of query row
-        // 8 nb + g.  (Quantised storage: as fp16, times the power of two that brings the row's largest element into
-        // [2^14, 2^15); unscale[nb] undoes it.)
+        // 8 nb + g.  Quantised storage: as fp16, times the power of two that brings the row's largest element into
+        // [2^14, 2^15).  fp16 then holds bf16 elements down to 2^-31 of it exactly; rows with nonzero elements below that
+        // go into bf16 MMAs as they are (times 2^-64 above 2^64: a sum over codes must not overflow).  unscale[nb] undoes it.
         uint32_t bq[NB][8][2];
         float unscale[NB];
+        bool f16_q = BITS != 16;
         {
             const __nv_bfloat16 *q_rot = reinterpret_cast<const __nv_bfloat16 *>(a.q_rot);
-#pragma unroll
-            for (int nb = 0; nb < NB; ++nb) {
+            auto load_row = [&](int nb, uint32_t (&raw)[16]) {
                 const int R = g + 8 * nb, tok = R / G, gi = R % G;
                 const __nv_bfloat16 *src = q_rot + (((int64_t)cb * nmax + tok) * a.H + kvh * G + gi) * kD + 32 * t4;
-                uint32_t raw[16];
 #pragma unroll
                 for (int ks = 0; ks < 8; ++ks) {
                     uint2 w = make_uint2(0u, 0u);
@@ -395,42 +428,55 @@ attn_q8_decode_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
                     raw[2 * ks] = w.x;
                     raw[2 * ks + 1] = w.y;
                 }
+            };
+            // pack(element 2 i, element 2 i + 1 of k-step ks) of a row scaled by `by`
+            auto scaled_row = [&](int nb, const uint32_t (&raw)[16], float by, auto pack) {
+                auto x = [&](int k) { return __uint_as_float(k & 1 ? raw[k >> 1] & 0xFFFF0000u : raw[k >> 1] << 16) * by; };
+#pragma unroll
+                for (int ks = 0; ks < 8; ++ks)
+#pragma unroll
+                    for (int i = 0; i < 2; ++i) bq[nb][ks][i] = pack(x(query_order<BITS>(ks, 2 * i)), x(query_order<BITS>(ks, 2 * i + 1)));
+            };
+            bool lossy = false;
+            int top_exp[NB];
+#pragma unroll
+            for (int nb = 0; nb < NB; ++nb) {
+                uint32_t raw[16];
+                load_row(nb, raw);
                 unscale[nb] = 1.f;
                 if constexpr (BITS == 16) {
 #pragma unroll
                     for (int ks = 0; ks < 8; ++ks) { bq[nb][ks][0] = raw[2 * ks]; bq[nb][ks][1] = raw[2 * ks + 1]; }
                 } else {
-                    float x[32], top = 0.f;
+                    float top = 0.f;
 #pragma unroll
-                    for (int k = 0; k < 16; ++k) {
-                        x[2 * k] = __uint_as_float(raw[k] << 16);
-                        x[2 * k + 1] = __uint_as_float(raw[k] & 0xFFFF0000u);
-                        top = fmaxf(top, fmaxf(fabsf(x[2 * k]), fabsf(x[2 * k + 1])));
-                    }
+                    for (int k = 0; k < 16; ++k)
+                        top = fmaxf(top, fmaxf(fabsf(__uint_as_float(raw[k] << 16)), fabsf(__uint_as_float(raw[k] & 0xFFFF0000u))));
                     top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, 1));
                     top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, 2));
                     const int e = max(biased_exponent(top), 15);         // top < 2^(e - 126)
-                    const float up = pow2f(268 - e);
+                    top_exp[nb] = e;
                     unscale[nb] = pow2f(e - 14);
+                    scaled_row(nb, raw, pow2f(268 - e), [&](float lo, float hi) {
+                        const uint32_t h = pack_f16(lo, hi);
+                        const float2 back = __half22float2(*reinterpret_cast<const __half2 *>(&h));
+                        lossy = lossy || back.x != lo || back.y != hi;
+                        return h;
+                    });
+                }
+            }
+            if (BITS != 16 && __any_sync(0xffffffffu, lossy)) {          // (every warp of the CTA has the same rows)
+                f16_q = false;
 #pragma unroll
-                    for (int ks = 0; ks < 8; ++ks)
-#pragma unroll
-                        for (int i = 0; i < 2; ++i)
-                            bq[nb][ks][i] = pack_f16(x[query_order<BITS>(ks, 2 * i)] * up, x[query_order<BITS>(ks, 2 * i + 1)] * up);
+                for (int nb = 0; nb < NB; ++nb) {
+                    uint32_t raw[16];
+                    load_row(nb, raw);
+                    const bool large = top_exp[nb] > 191;
+                    unscale[nb] = large ? 0x1p64f : 1.f;
+                    scaled_row(nb, raw, large ? 0x1p-64f : 1.f, [](float lo, float hi) { return pack_bf16_pair(lo, hi); });
                 }
             }
         }
-        // keys below the limit are visible (rows past the chunk's end are never written; each row of S, P
-        // and O depends on that row alone, so they are left unmasked)
-        // (counted from the chunk's first key, P)
-        int limit[NB][2];
-#pragma unroll
-        for (int nb = 0; nb < NB; ++nb)
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                const int R = 8 * nb + 2 * t4 + e;
-                limit[nb][e] = R < nG ? (R / G + 1) * a.self_rows : (1 << 30);
-            }
         // softmax scale * log2(e) of query rows 8 nb + 2 t + {0, 1} (whose scaling the threads of those g know)
         float sl2[NB][2];
 #pragma unroll
@@ -452,122 +498,180 @@ attn_q8_decode_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
 
             // ---- scores of the 64 keys: four 16-key blocks, sacc[j][nb] = keys g / g + 8 of block j, rows 8 nb + 2 t + {0, 1}
             float sacc[4][NB][4];
-            float ks_row[4][2], vs_row[4][2], vs_top = 0.f;      // scales of those keys' rows (quantised storage)
+            auto score_blocks = [&](auto f16) {
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int rl = 16 * j + g;                       // my first key row within the 64
-                uint32_t ka[8][4];
-                key_fragments<BITS>(k_tile, half * 64 + rl, t4, ka);
-                if constexpr (BITS != 16) {
-                    ks_row[j][0] = k_sc[half * 64 + rl];
-                    ks_row[j][1] = k_sc[half * 64 + rl + 8];
-                    vs_row[j][0] = v_sc[half * 64 + rl];
-                    vs_row[j][1] = v_sc[half * 64 + rl + 8];
-                }
+                for (int j = 0; j < 4; ++j) {
+                    const int rl = 16 * j + g;                       // my first key row within the 64
+                    uint32_t ka[8][4];
+                    key_fragments<BITS, decltype(f16)::value>(k_tile, half * 64 + rl, t4, ka);
 #pragma unroll
-                for (int nb = 0; nb < NB; ++nb) {
-                    // a second accumulator for the odd k-steps: two chains of four MMAs instead of one of eight
-                    float odd[4];
+                    for (int nb = 0; nb < NB; ++nb) {
+                        // a second accumulator for the odd k-steps: two chains of four MMAs instead of one of eight
+                        float odd[4];
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) { sacc[j][nb][e] = 0.f; odd[e] = 0.f; }
+                        for (int e = 0; e < 4; ++e) { sacc[j][nb][e] = 0.f; odd[e] = 0.f; }
 #pragma unroll
-                    for (int ks = 0; ks < 8; ks += 2) {
-                        mma_rows<BITS>(sacc[j][nb], ka[ks], bq[nb][ks][0], bq[nb][ks][1]);
-                        mma_rows<BITS>(odd, ka[ks + 1], bq[nb][ks + 1][0], bq[nb][ks + 1][1]);
+                        for (int ks = 0; ks < 8; ks += 2) {
+                            mma_rows<decltype(f16)::value>(sacc[j][nb], ka[ks], bq[nb][ks][0], bq[nb][ks][1]);
+                            mma_rows<decltype(f16)::value>(odd, ka[ks + 1], bq[nb][ks + 1][0], bq[nb][ks + 1][1]);
+                        }
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) sacc[j][nb][e] += odd[e];
                     }
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) sacc[j][nb][e] += odd[e];
                 }
-            }
+            };
+            if (BITS != 16 && f16_q) score_blocks(std::true_type{});
+            else score_blocks(std::false_type{});
             // ---- scores in log2 units, mask (only where the chunk's own keys are near: whole warps branch), running
             // maximum, probabilities
-            if (BITS != 16 && in_planes < 64)
+            // (quantised storage: the scales of the rows of my keys are fetched where they are used - registers)
+            float row_scale[4][2];
+            auto fetch_scales = [&](const float *sc) {
 #pragma unroll
                 for (int j = 0; j < 4; ++j)
 #pragma unroll
-                    for (int h = 0; h < 2; ++h)
-                        if (16 * j + 8 * h + g >= in_planes) ks_row[j][h] = vs_row[j][h] = 0.f;
+                    for (int h = 0; h < 2; ++h) row_scale[j][h] = sc[half * 64 + 16 * j + 8 * h + g];
+                if (in_planes < 64)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+#pragma unroll
+                        for (int h = 0; h < 2; ++h)
+                            if (16 * j + 8 * h + g >= in_planes) row_scale[j][h] = 0.f;
+            };
+            if (BITS != 16) fetch_scales(k_sc);
 #pragma unroll
             for (int j = 0; j < 4; ++j)
 #pragma unroll
                 for (int nb = 0; nb < NB; ++nb)
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) sacc[j][nb][e] *= BITS == 16 ? sl2[nb][e & 1] : ks_row[j][e >> 1] * sl2[nb][e & 1];
+                    for (int e = 0; e < 4; ++e) sacc[j][nb][e] *= BITS == 16 ? sl2[nb][e & 1] : row_scale[j][e >> 1] * sl2[nb][e & 1];
             if (key_h + 64 > P) {
+                // keys below a row's limit are visible (rows past the chunk's end are never written; each row of S, P
+                // and O depends on that row alone, so they are left unmasked)
                 const int rel = (int)(key_h - P) + g;               // my first key, counted from P (> -64)
-#pragma unroll
-                for (int j = 0; j < 4; ++j)
-#pragma unroll
-                    for (int nb = 0; nb < NB; ++nb)
-#pragma unroll
-                        for (int e = 0; e < 4; ++e)
-                            if (rel + 16 * j + 8 * (e >> 1) >= limit[nb][e & 1]) sacc[j][nb][e] = -INFINITY;
-            }
-            uint32_t pb[4][NB][2];         // P^T as B fragments of the four 16-key steps
-            float alpha[NB][2];
-            bool rescale = false;
-            float v_down = 1.f;            // what the output so far shrinks by when the V scales' reference moves
-            if constexpr (BITS != 16) {
-#pragma unroll
-                for (int j = 0; j < 4; ++j) vs_top = fmaxf(vs_top, fmaxf(vs_row[j][0], vs_row[j][1]));
-                vs_top = fmaxf(vs_top, __shfl_xor_sync(0xffffffffu, vs_top, 4));
-                vs_top = fmaxf(vs_top, __shfl_xor_sync(0xffffffffu, vs_top, 8));
-                vs_top = fmaxf(vs_top, __shfl_xor_sync(0xffffffffu, vs_top, 16));
-                const int e = biased_exponent(vs_top);
-                if (e > v_exp) {
-                    v_down = e - v_exp > 126 ? 0.f : pow2f(127 - (e - v_exp));
-                    v_exp = e;
-                    rescale = true;
-                }
-                const float up = pow2f(268 - v_exp);
-#pragma unroll
-                for (int j = 0; j < 4; ++j) { vs_row[j][0] *= up; vs_row[j][1] *= up; }
-            }
-#pragma unroll
-            for (int nb = 0; nb < NB; ++nb) {
-                float mx[2] = {-INFINITY, -INFINITY};
-#pragma unroll
-                for (int j = 0; j < 4; ++j)
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) mx[e & 1] = fmaxf(mx[e & 1], sacc[j][nb][e]);
-                float m_safe[2];
-#pragma unroll
-                for (int e = 0; e < 2; ++e) {
-                    mx[e] = fmaxf(mx[e], __shfl_xor_sync(0xffffffffu, mx[e], 4));
-                    mx[e] = fmaxf(mx[e], __shfl_xor_sync(0xffffffffu, mx[e], 8));
-                    mx[e] = fmaxf(mx[e], __shfl_xor_sync(0xffffffffu, mx[e], 16));
-                    const float m_new = fmaxf(m_run[nb][e], mx[e]);
-                    m_safe[e] = m_new == -INFINITY ? 0.f : m_new;
-                    alpha[nb][e] = ex2(m_run[nb][e] - m_safe[e]);                   // m_run = -inf -> 0
-                    m_run[nb][e] = m_new;
-                    l_run[nb][e] *= alpha[nb][e];
-                    rescale = rescale || alpha[nb][e] != 1.f;
-                    if constexpr (BITS != 16) alpha[nb][e] *= v_down;
-                }
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const float p0 = ex2(sacc[j][nb][0] - m_safe[0]), p1 = ex2(sacc[j][nb][1] - m_safe[1]);
-                    const float p2 = ex2(sacc[j][nb][2] - m_safe[0]), p3 = ex2(sacc[j][nb][3] - m_safe[1]);
-                    l_run[nb][0] += p0 + p2;
-                    l_run[nb][1] += p1 + p3;
-                    // (key g, rows 2 t, 2 t + 1) transposed: (keys 2 t, 2 t + 1; row g) - P^T's b0; keys + 8: b1
-                    if constexpr (BITS == 16) {
-                        pb[j][nb][0] = transpose8x8(pack_bf16_pair(p0, p1));
-                        pb[j][nb][1] = transpose8x8(pack_bf16_pair(p2, p3));
-                    } else {
-                        pb[j][nb][0] = transpose8x8(pack_f16(p0 * vs_row[j][0], p1 * vs_row[j][0]));
-                        pb[j][nb][1] = transpose8x8(pack_f16(p2 * vs_row[j][1], p3 * vs_row[j][1]));
-                    }
-                }
-            }
-            if (__any_sync(0xffffffffu, rescale)) {
 #pragma unroll
                 for (int nb = 0; nb < NB; ++nb)
 #pragma unroll
-                    for (int jp = 0; jp < 8; ++jp) {
-                        ot[nb][jp][0] *= alpha[nb][0]; ot[nb][jp][1] *= alpha[nb][1];
-                        ot[nb][jp][2] *= alpha[nb][0]; ot[nb][jp][3] *= alpha[nb][1];
+                    for (int e = 0; e < 2; ++e) {
+                        const int R = 8 * nb + 2 * t4 + e, limit = R < nG ? (R / G + 1) * a.self_rows : (1 << 30);
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            if (rel + 16 * j >= limit) sacc[j][nb][e] = -INFINITY;
+                            if (rel + 16 * j + 8 >= limit) sacc[j][nb][2 + e] = -INFINITY;
+                        }
                     }
+            }
+            uint32_t pb[4][NB][2];         // P^T as B fragments of the four 16-key steps
+            if constexpr (BITS == 16) {
+                float alpha[NB][2];
+                bool rescale = false;
+#pragma unroll
+                for (int nb = 0; nb < NB; ++nb) {
+                    float mx[2] = {-INFINITY, -INFINITY};
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) mx[e & 1] = fmaxf(mx[e & 1], sacc[j][nb][e]);
+                    float m_safe[2];
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        mx[e] = max_of_keys(mx[e]);
+                        const float m_new = fmaxf(m_run[nb][e], mx[e]);
+                        m_safe[e] = m_new == -INFINITY ? 0.f : m_new;
+                        alpha[nb][e] = ex2(m_run[nb][e] - m_safe[e]);                   // m_run = -inf -> 0
+                        m_run[nb][e] = m_new;
+                        l_run[nb][e] *= alpha[nb][e];
+                        rescale = rescale || alpha[nb][e] != 1.f;
+                    }
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const float p0 = ex2(sacc[j][nb][0] - m_safe[0]), p1 = ex2(sacc[j][nb][1] - m_safe[1]);
+                        const float p2 = ex2(sacc[j][nb][2] - m_safe[0]), p3 = ex2(sacc[j][nb][3] - m_safe[1]);
+                        l_run[nb][0] += p0 + p2;
+                        l_run[nb][1] += p1 + p3;
+                        // (key g, rows 2 t, 2 t + 1) transposed: (keys 2 t, 2 t + 1; row g) - P^T's b0; keys + 8: b1
+                        pb[j][nb][0] = transpose8x8(pack_bf16_pair(p0, p1));
+                        pb[j][nb][1] = transpose8x8(pack_bf16_pair(p2, p3));
+                    }
+                }
+                if (__any_sync(0xffffffffu, rescale)) {
+#pragma unroll
+                    for (int nb = 0; nb < NB; ++nb)
+#pragma unroll
+                        for (int jp = 0; jp < 8; ++jp) {
+                            ot[nb][jp][0] *= alpha[nb][0]; ot[nb][jp][1] *= alpha[nb][1];
+                            ot[nb][jp][2] *= alpha[nb][0]; ot[nb][jp][3] *= alpha[nb][1];
+                        }
+                }
+            } else {
+                // The reference m_run of a row's softmax moves when a score is more than 2 above it (a probability is at most
+                // 4), `up` when the reference has moved or a product would leave fp16: then the largest product of the row
+                // seen so far - keys that the row does not see have none - is brought back into [2^14, 2^15).
+                // (my largest score or product of row 8 nb + 2 t + e: worked out again where it is needed - registers)
+                auto largest = [&](int nb, int e) {
+                    float x = fmaxf(sacc[0][nb][e], sacc[0][nb][2 + e]);
+#pragma unroll
+                    for (int j = 1; j < 4; ++j) x = fmaxf(x, fmaxf(sacc[j][nb][e], sacc[j][nb][2 + e]));
+                    return x;
+                };
+                float alpha[NB][2];
+                bool above = false;
+#pragma unroll
+                for (int nb = 0; nb < NB; ++nb)
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        above = above || largest(nb, e) > m_run[nb][e] + 2.f;
+                        alpha[nb][e] = 1.f;
+                    }
+                above = __any_sync(0xffffffffu, above);
+                if (above)
+#pragma unroll
+                    for (int nb = 0; nb < NB; ++nb)
+#pragma unroll
+                        for (int e = 0; e < 2; ++e) {
+                            const float m_new = fmaxf(m_run[nb][e], max_of_keys(largest(nb, e)));
+                            alpha[nb][e] = m_new == -INFINITY ? 0.f : ex2(m_run[nb][e] - m_new);      // m_run = -inf -> 0
+                            m_run[nb][e] = m_new;
+                            l_run[nb][e] *= alpha[nb][e];
+                        }
+                bool beyond = false;
+                fetch_scales(v_sc);
+#pragma unroll
+                for (int nb = 0; nb < NB; ++nb) {
+                    const float m0 = m_run[nb][0] == -INFINITY ? 0.f : m_run[nb][0], m1 = m_run[nb][1] == -INFINITY ? 0.f : m_run[nb][1];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const float p0 = ex2(sacc[j][nb][0] - m0), p1 = ex2(sacc[j][nb][1] - m1);
+                        const float p2 = ex2(sacc[j][nb][2] - m0), p3 = ex2(sacc[j][nb][3] - m1);
+                        l_run[nb][0] += p0 + p2;
+                        l_run[nb][1] += p1 + p3;
+                        sacc[j][nb][0] = p0 * row_scale[j][0]; sacc[j][nb][1] = p1 * row_scale[j][0];
+                        sacc[j][nb][2] = p2 * row_scale[j][1]; sacc[j][nb][3] = p3 * row_scale[j][1];
+                    }
+                    beyond = beyond || largest(nb, 0) * pow2f(up[nb][0]) >= 65504.f || largest(nb, 1) * pow2f(up[nb][1]) >= 65504.f;
+                }
+                if (above || __any_sync(0xffffffffu, beyond))
+#pragma unroll
+                    for (int nb = 0; nb < NB; ++nb)
+#pragma unroll
+                        for (int e = 0; e < 2; ++e) {
+                            // (the earlier keys' largest product was 2^14 of their units or more)
+                            const float x = fmaxf(max_of_keys(largest(nb, e)), alpha[nb][e] * pow2f(268 - up[nb][e]));
+                            const int to = min(max(268 - biased_exponent(x), 14), 253);
+                            const float by = alpha[nb][e] * pow2f(127 + min(max(to - up[nb][e], -126), 126));
+                            up[nb][e] = to;
+#pragma unroll
+                            for (int jp = 0; jp < 8; ++jp) { ot[nb][jp][e] *= by; ot[nb][jp][2 + e] *= by; }
+                        }
+#pragma unroll
+                for (int nb = 0; nb < NB; ++nb) {
+                    const float f0 = pow2f(up[nb][0]), f1 = pow2f(up[nb][1]);
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        pb[j][nb][0] = transpose8x8(pack_f16(sacc[j][nb][0] * f0, sacc[j][nb][1] * f1));
+                        pb[j][nb][1] = transpose8x8(pack_f16(sacc[j][nb][2] * f0, sacc[j][nb][3] * f1));
+                    }
+                }
             }
             // ---- O^T += V^T P^T, 16 keys at a time
 #pragma unroll
@@ -579,7 +683,7 @@ attn_q8_decode_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
                     uint32_t va[4];
                     value_fragment<BITS>(w, jp, va);
 #pragma unroll
-                    for (int nb = 0; nb < NB; ++nb) mma_rows<BITS>(ot[nb][jp], va, pb[j][nb][0], pb[j][nb][1]);
+                    for (int nb = 0; nb < NB; ++nb) mma_rows<BITS != 16>(ot[nb][jp], va, pb[j][nb][0], pb[j][nb][1]);
                 }
             }
             __syncwarp();
@@ -595,7 +699,6 @@ attn_q8_decode_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
     if (warp < kWarps) {
         float *mo = mrg + (size_t)warp * (kMergeWarp / 4);
         float *mm = mo + kMaxRows * kD;
-        const float v_unit = pow2f(v_exp - 14);
 #pragma unroll
         for (int nb = 0; nb < NB; ++nb)
 #pragma unroll
@@ -605,10 +708,11 @@ attn_q8_decode_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
                 l += __shfl_xor_sync(0xffffffffu, l, 8);
                 l += __shfl_xor_sync(0xffffffffu, l, 16);
                 const int r = 8 * nb + 2 * t4 + e;
+                const float down = pow2f(254 - up[nb][e]);
 #pragma unroll
                 for (int jp = 0; jp < 8; ++jp)
                     *reinterpret_cast<float2 *>(mo + r * kD + 16 * g + 2 * jp) =
-                        BITS == 16 ? make_float2(ot[nb][jp][e], ot[nb][jp][2 + e]) : make_float2(ot[nb][jp][e] * v_unit, ot[nb][jp][2 + e] * v_unit);
+                        BITS == 16 ? make_float2(ot[nb][jp][e], ot[nb][jp][2 + e]) : make_float2(ot[nb][jp][e] * down, ot[nb][jp][2 + e] * down);
                 if (g == 0) {
                     mm[2 * r] = m_run[nb][e];
                     mm[2 * r + 1] = l;

@@ -5,12 +5,13 @@
 // or int4 (Q = 7) with one fp32 scale, decided once when the row is appended:
 //     amax = max |x_j|     inv = Q / amax       scale = amax / Q          (fp32, round to nearest)
 //     code_j = clamp(rint(x_j * inv), -Q, Q)                               (ties to even)
-//     value seen by the attention = bf16(code_j * scale)                   (fp32 product, one rounding)
+//     value seen by the attention = bf16(code_j * scale)                   (fp32 product, one rounding;
+//                                   code_j * scale itself in the decode kernel, attn_q8_decode.cu)
 // For a key row x is the rotated row in fp32 (same operation order as the bf16 path, before any
 // rounding to bf16); a value row is quantised as given.  amax = 0 gives codes 0 and scale 0.
 // The cache then holds d + 4 (int8) or d / 2 + 4 (int4: code + 8, two to a byte, element 2i in the low
-// nibble of byte i) bytes per row instead of 2 d; the attention kernel expands code tiles to bf16 tiles
-// in shared memory.  Paged caches keep codes and scales of 128 tokens of every KV head in one page
+// nibble of byte i) bytes per row instead of 2 d; the attention kernel for long chunks expands code tiles to
+// bf16 tiles in shared memory.  Paged caches keep codes and scales of 128 tokens of every KV head in one page
 // (see QuantPlanes); a batch of paged caches is one launch (blockIdx.y = cache).
 #include "kvfold_internal.h"
 

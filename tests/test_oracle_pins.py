@@ -361,6 +361,26 @@ def test_quantised_fold_is_the_plain_fold_on_rows_that_went_through_the_round_tr
     assert lo < rel < hi, rel                                 # int4 moves the outputs an order of magnitude more
 
 
+@pytest.mark.parametrize("bits", [8, 4])
+def test_unrounded_quantised_rows_are_read_as_code_times_scale(bits):
+    T, H, Hkv, d = 40, 4, 2, 16
+    q, k, v = (a.astype(np.float32).astype(np.float64) for a in _qkv(RNG(44), T, H, Hkv, d))
+    k_codes, k_scales, _ = oracle.quant_rows(oracle.rope_faithful(k.astype(np.float32), 0, oracle.inv_freq(10000.0, d)), bits)
+    v_codes, v_scales, _ = oracle.quant_rows(v.astype(np.float32), bits)
+    kp, vp = k_codes * k_scales[..., None].astype(np.float64), v_codes * v_scales[..., None].astype(np.float64)
+    qr = bf.rope_complex(q, np.arange(T), 10000.0)
+    c = oracle.OracleCache(H, Hkv, d, capacity=T)
+    c.set_quant(bits)
+    c.fold_step(q[:25], k[:25], v[:25])                       # the switch covers rows appended before it
+    c.set_unrounded(True)
+    got = c.fold_step(q[25:], k[25:], v[25:])
+    for h in range(H):
+        s = (qr[25:, h] @ kp[:, h // 2].T) / np.sqrt(d)
+        s = np.where(np.arange(T)[None, :] <= np.arange(25, T)[:, None], s, -np.inf)
+        p = np.exp(s - s.max(axis=1, keepdims=True))
+        assert np.abs(got[:, h] - (p / p.sum(axis=1, keepdims=True)) @ vp[:, h // 2]).max() <= 1e-12
+
+
 def test_append_only_prefix_rows_are_bit_unchanged():
     T, H, Hkv, d = 30, 2, 2, 8
     q, k, v = _qkv(RNG(18), T, H, Hkv, d)
