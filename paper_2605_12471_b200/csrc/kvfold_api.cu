@@ -663,6 +663,7 @@ kvf_status step_impl(kvf_cache *c, const void *q, const void *k_new, const void 
     ra.prefixes = nullptr; ra.pos0s = nullptr; ra.ns = nullptr;
     ra.status = reinterpret_cast<int *>(c->workspace + c->lay.status);
     ra.range_limit = c->tc32 ? 65504.f : 0.f;      // the fp32 tensor-core kernel computes on fp16 halves
+    ra.sms = c->sm_count;
     ra.table = c->table;
 
     AttnArgs aa;
@@ -1353,6 +1354,7 @@ kvf_status batch_step(kvf_batch *b, const void *q, const void *k_new, const void
     ra.pos0s = ragged ? dev_pos0s : nullptr;
     ra.ns = ns ? dev_ns : nullptr;
     ra.status = nullptr; ra.range_limit = 0.f;
+    ra.sms = c0->sm_count;
     ra.table = c0->table;
 
     AttnArgs aa;

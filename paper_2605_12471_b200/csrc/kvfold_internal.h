@@ -134,6 +134,7 @@ struct RopeAppendArgs {
     // above range_limit in magnitude sets code 7 in *status (range_limit = 0: no check)
     int *status;
     float range_limit;
+    int32_t sms;                     // of the device
     RopeTable table;
 };
 

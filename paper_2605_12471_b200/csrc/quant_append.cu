@@ -49,10 +49,10 @@ __device__ __forceinline__ void quantise4(const float (&x)[4], int (&code)[4], f
 
 // One warp per row (d = 128: four elements per lane).  Query rows are rotated and written as bf16;
 // key rows are rotated in fp32, quantised and appended; value rows are quantised and appended.
-// kTok = tokens per CTA (see tokens_per_cta); a warp takes the same rows of every token, so that up to four tokens' loads
+// kTok = tokens per CTA, kResident = CTAs of an SM (see launch_bits); a warp takes the same rows of every token, so that up to four tokens' loads
 // and reductions are in flight together.
-template <bool INTERLEAVED, int BITS, int kTok>
-__global__ void __launch_bounds__(kThreads, 2) rope_append_q8_kernel(const RopeAppendArgs a, const QuantPlanes qp) {
+template <bool INTERLEAVED, int BITS, int kTok, int kResident>
+__global__ void __launch_bounds__(kThreads, kResident) rope_append_q8_kernel(const RopeAppendArgs a, const QuantPlanes qp) {
     constexpr int RB = 128 * BITS / 8;          // bytes of a stored row
     __shared__ float2 cs[kTok][kMaxHalfDim];   // (cos, sin) per (token, pair)
     constexpr int d = 128, half = 64;
@@ -103,7 +103,6 @@ __global__ void __launch_bounds__(kThreads, 2) rope_append_q8_kernel(const RopeA
     const __nv_bfloat16 *v = reinterpret_cast<const __nv_bfloat16 *>(a.v_new) + koff;
     __nv_bfloat16 *qr = reinterpret_cast<__nv_bfloat16 *>(a.q_rot) + qoff;
     const int heads = a.H + (a.k_new ? 2 * a.Hkv : 0);     // query rows, key rows, value rows (queries only: kvf_attend)
-    constexpr int U = kTok < 4 ? kTok : 4;
     for (int hh = warp; hh < heads; hh += kThreads / 32) {
         const bool is_q = hh < a.H, is_v = hh >= a.H + a.Hkv;
         const int g = is_q ? hh : is_v ? hh - a.H - a.Hkv : hh - a.H;        // query head, or KV head
@@ -113,11 +112,12 @@ __global__ void __launch_bounds__(kThreads, 2) rope_append_q8_kernel(const RopeA
         // .. 4 lane + 3; else the pairs (j, j + 64) for j = 2 lane, 2 lane + 1
         const bool in_order = INTERLEAVED || is_v;
         const int e0 = in_order ? 4 * lane : 2 * lane, e1 = in_order ? 4 * lane + 2 : half + 2 * lane;
+        // (one turn; without the loop the compiler's order costs two and four tokens 2 - 4 % of a launch)
 #pragma unroll 1
-        for (int t0 = 0; t0 < ntok; t0 += U) {
-            uint32_t w0[U], w1[U];
+        for (int t0 = 0; t0 < ntok; t0 += kTok) {
+            uint32_t w0[kTok], w1[kTok];
 #pragma unroll
-            for (int u = 0; u < U; ++u) {
+            for (int u = 0; u < kTok; ++u) {
                 w0[u] = w1[u] = 0u;
                 if (t0 + u < ntok) {
                     const __nv_bfloat16 *p = src + (int64_t)(t0 + u) * row_heads * d;
@@ -126,7 +126,7 @@ __global__ void __launch_bounds__(kThreads, 2) rope_append_q8_kernel(const RopeA
                 }
             }
 #pragma unroll
-            for (int u = 0; u < U; ++u) {
+            for (int u = 0; u < kTok; ++u) {
                 const int t = t0 + u;
                 if (t >= ntok) break;
                 const int64_t tok = tok0 + t, cache_row = prefix + tok;
@@ -167,24 +167,30 @@ __global__ void __launch_bounds__(kThreads, 2) rope_append_q8_kernel(const RopeA
     }
 }
 
-// Tokens per CTA, as for bf16 rows (rope_append.cu): one while all CTAs are resident at once, then as many as share the
-// chain of one.  us between events (32 / 8 heads, int8, cold L2) with 1, 2, 4 tokens per CTA: 256 tokens 10.2, 10.2, 12.3; 512:
-// 14.3, 12.3, 12.3; 1024: 20.5, 16.4, 16.4; 2048: 32.8, 26.6, 24.6; 8192: 106.5, 77.8, 65.6; int4 the same.
-int tokens_per_cta(int64_t tokens) { return tokens <= 2 * 148 ? 1 : tokens < 1024 ? 2 : 4; }
-
-template <int TOK>
+template <int BITS, int TOK, int RESIDENT>
 cudaError_t launch_tok(const RopeAppendArgs &a, const QuantPlanes &qp, bool interleaved, int batch, cudaStream_t s) {
-    auto kernel = qp.bits == 4 ? (interleaved ? rope_append_q8_kernel<true, 4, TOK> : rope_append_q8_kernel<false, 4, TOK>)
-                               : (interleaved ? rope_append_q8_kernel<true, 8, TOK> : rope_append_q8_kernel<false, 8, TOK>);
+    auto kernel = interleaved ? rope_append_q8_kernel<true, BITS, TOK, RESIDENT> : rope_append_q8_kernel<false, BITS, TOK, RESIDENT>;
     return launch_pdl(kernel, dim3((a.n + TOK - 1) / TOK, batch), dim3(kThreads), 0, s, a, qp);
+}
+
+// As for bf16 rows (rope_append.cu): one token per CTA while two CTAs on an SM hold the launch, and where the members of a batch
+// have one each (then four on an SM: 32 registers); else two tokens, from six tokens an SM on four.  us per launch, cold inputs, plain
+// launches back to back, int8, 32 / 8 heads, one token with two / four CTAs on an SM, two, four tokens: 256 tokens 5.1 / 5.5 / 5.8 / 8.0; 360:
+// 8.6 / 6.7 / 6.5 / 8.1; 512: 9.1 / 8.1 / 6.7 / 8.3; 640: 11.9 / 9.9 / 10.4 / 10.0; 900: 15.0 / 12.1 / 11.7 / 10.3; 2048: 28.0 / 22.3 / 21.7 / 19.7;
+// 8192: 104 / 79 / 75 / 64; members of one token, 297: 7.7 / 7.3 / 8.2 / 9.1; 360 of 28 / 4 heads: 8.2 / 7.3 / 8.9 / 9.9; 1024: 17.4 / 18.1 /
+// 18.3 / 20.0.
+template <int BITS>
+cudaError_t launch_bits(const RopeAppendArgs &a, const QuantPlanes &qp, bool interleaved, int batch, cudaStream_t s) {
+    const int64_t tokens = (int64_t)a.n * batch, sms = a.sms;
+    if (tokens <= 2 * sms) return launch_tok<BITS, 1, 2>(a, qp, interleaved, batch, s);
+    if (a.n < 2) return launch_tok<BITS, 1, 4>(a, qp, interleaved, batch, s);
+    return tokens < 6 * sms || a.n < 4 ? launch_tok<BITS, 2, 2>(a, qp, interleaved, batch, s) : launch_tok<BITS, 4, 2>(a, qp, interleaved, batch, s);
 }
 
 }  // namespace
 
 cudaError_t launch_rope_append_q8(const RopeAppendArgs &a, const QuantPlanes &qp, bool interleaved, int batch, cudaStream_t s) {
-    const int tok = tokens_per_cta((int64_t)a.n * batch);
-    return tok == 4 ? launch_tok<4>(a, qp, interleaved, batch, s) : tok == 2 ? launch_tok<2>(a, qp, interleaved, batch, s)
-                                                                             : launch_tok<1>(a, qp, interleaved, batch, s);
+    return qp.bits == 4 ? launch_bits<4>(a, qp, interleaved, batch, s) : launch_bits<8>(a, qp, interleaved, batch, s);
 }
 
 }  // namespace kvf

@@ -55,11 +55,10 @@ __device__ __forceinline__ void rotate(float a, float b, float c, float s, float
     rb = __fmaf_rn(b, c, cross_b);
 }
 
-// kTok = tokens per CTA (see tokens_per_cta).
-template <typename T, bool INTERLEAVED, int kTok>
-__global__ void __launch_bounds__(kThreads, 2) rope_append_kernel(const RopeAppendArgs a) {
+// kTok = tokens per CTA, kResident = CTAs of an SM (see launch_type).
+template <typename T, bool INTERLEAVED, int kTok, int kResident>
+__global__ void __launch_bounds__(kThreads, kResident) rope_append_kernel(const RopeAppendArgs a) {
     constexpr int VEC = Vec16<T>::N;
-    constexpr int U = kTok < 4 ? kTok : 4;     // tokens of an item whose loads are in flight together
     __shared__ float2 cs[kTok][kMaxHalfDim];   // (cos, sin) per (token, pair)
 
     const int d = a.d, half = d / 2;
@@ -137,55 +136,51 @@ __global__ void __launch_bounds__(kThreads, 2) rope_append_kernel(const RopeAppe
         const int64_t src_step = (int64_t)row_heads * d;
         T *plane = value ? vp : kp;
         auto dst = [&](int t) { return (query ? qr + ((int64_t)(tok0 + t) * a.H + g) * d : plane + rows.offset(g, prefix + tok0 + t)) + c * VEC; };
-#pragma unroll 1
-        for (int t0 = 0; t0 < ntok; t0 += U) {
-            uint4 lo[U], hi[U];
+        uint4 lo[kTok], hi[kTok];
 #pragma unroll
-            for (int u = 0; u < U; ++u)
-                if (t0 + u < ntok) {
-                    lo[u] = *reinterpret_cast<const uint4 *>(src + (t0 + u) * src_step);
-                    if (!INTERLEAVED && !value) hi[u] = *reinterpret_cast<const uint4 *>(src + (t0 + u) * src_step + half);
+        for (int t = 0; t < kTok; ++t)
+            if (t < ntok) {
+                lo[t] = *reinterpret_cast<const uint4 *>(src + t * src_step);
+                if (!INTERLEAVED && !value) hi[t] = *reinterpret_cast<const uint4 *>(src + t * src_step + half);
+            }
+#pragma unroll
+        for (int t = 0; t < kTok; ++t) {
+            if (t >= ntok) break;
+            T *to = dst(t);
+            if (value) {
+                *reinterpret_cast<uint4 *>(to) = lo[t];
+                if (ranged)
+                    amax = fmaxf(fmaxf(amax, fmaxf(fabsf(__uint_as_float(lo[t].x)), fabsf(__uint_as_float(lo[t].y)))),
+                                 fmaxf(fabsf(__uint_as_float(lo[t].z)), fabsf(__uint_as_float(lo[t].w))));
+                continue;
+            }
+            float x[VEC], r[VEC];
+            Vec16<T>::unpack(lo[t], x);
+            if (!INTERLEAVED) {
+                float y[VEC], ry[VEC];
+                Vec16<T>::unpack(hi[t], y);
+#pragma unroll
+                for (int e = 0; e < VEC; ++e) {
+                    const float2 w = cs[t][c * VEC + e];
+                    rotate(x[e], y[e], w.x, w.y, r[e], ry[e]);
                 }
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const int t = t0 + u;
-                if (t >= ntok) break;
-                T *to = dst(t);
-                if (value) {
-                    *reinterpret_cast<uint4 *>(to) = lo[u];
-                    if (ranged)
-                        amax = fmaxf(fmaxf(amax, fmaxf(fabsf(__uint_as_float(lo[u].x)), fabsf(__uint_as_float(lo[u].y)))),
-                                     fmaxf(fabsf(__uint_as_float(lo[u].z)), fabsf(__uint_as_float(lo[u].w))));
-                    continue;
-                }
-                float x[VEC], r[VEC];
-                Vec16<T>::unpack(lo[u], x);
-                if (!INTERLEAVED) {
-                    float y[VEC], ry[VEC];
-                    Vec16<T>::unpack(hi[u], y);
-#pragma unroll
-                    for (int e = 0; e < VEC; ++e) {
-                        const float2 w = cs[t][c * VEC + e];
-                        rotate(x[e], y[e], w.x, w.y, r[e], ry[e]);
-                    }
-                    Vec16<T>::store(to, r);
-                    Vec16<T>::store(to + half, ry);
-                    if (ranged) {
-#pragma unroll
-                        for (int e = 0; e < VEC; ++e) amax = fmaxf(amax, fabsf(ry[e]));
-                    }
-                } else {
-#pragma unroll
-                    for (int e = 0; e < VEC; e += 2) {
-                        const float2 w = cs[t][(c * VEC + e) / 2];
-                        rotate(x[e], x[e + 1], w.x, w.y, r[e], r[e + 1]);
-                    }
-                    Vec16<T>::store(to, r);
-                }
+                Vec16<T>::store(to, r);
+                Vec16<T>::store(to + half, ry);
                 if (ranged) {
 #pragma unroll
-                    for (int e = 0; e < VEC; ++e) amax = fmaxf(amax, fabsf(r[e]));
+                    for (int e = 0; e < VEC; ++e) amax = fmaxf(amax, fabsf(ry[e]));
                 }
+            } else {
+#pragma unroll
+                for (int e = 0; e < VEC; e += 2) {
+                    const float2 w = cs[t][(c * VEC + e) / 2];
+                    rotate(x[e], x[e + 1], w.x, w.y, r[e], r[e + 1]);
+                }
+                Vec16<T>::store(to, r);
+            }
+            if (ranged) {
+#pragma unroll
+                for (int e = 0; e < VEC; ++e) amax = fmaxf(amax, fabsf(r[e]));
             }
         }
     }
@@ -194,30 +189,33 @@ __global__ void __launch_bounds__(kThreads, 2) rope_append_kernel(const RopeAppe
 
 }  // namespace
 
-// Tokens per CTA.  Few tokens: one each, their CTAs are all resident at once (two to an SM) and the step waits for one token's chain (sines,
-// loads, stores).  More: that chain is paid for once per CTA instead of once per token, in waves; four tokens are as
-// many as have their loads in registers.  us between events (32 / 8 heads, cold L2) with 1, 2, 4 tokens per CTA, bf16: 256
-// tokens 8.2, 8.2, 10.2; 512: 12.3, 10.2, 10.2; 1024: 16.4, 14.4, 12.3; 2048: 24.6, 20.5, 18.4; 8192: 71.6, 55.3, 47.1
-// (201 MB: 31 us at the copy bandwidth); 436 tokens of 28 / 4 heads, fp32, one each are a second wave: 66.2 us for the two
-// steps of a chain, two each 64.3; fp32: 512: 14.3, 12.3, 14.3; 2048: 32.8, 26.6, 27.6; 8192: 100.4, 75.8, 76.8.
-template <typename T> static int tokens_per_cta(int64_t tokens) { return tokens <= 2 * 148 ? 1 : tokens < 1024 || sizeof(T) == 4 ? 2 : 4; }
-
-template <typename T, int TOK>
+template <typename T, int TOK, int RESIDENT>
 static cudaError_t launch_tok(const RopeAppendArgs &a, bool interleaved, int batch, cudaStream_t s) {
     int blocks = (a.n + TOK - 1) / TOK;
     if (a.zero_rows > 0) {
         int64_t vecs = (int64_t)a.zero_rows * a.Hkv * (a.d / Vec16<T>::N);
         blocks += (int)((vecs + kThreads - 1) / kThreads);
     }
-    return launch_pdl(interleaved ? rope_append_kernel<T, true, TOK> : rope_append_kernel<T, false, TOK>, dim3(blocks, batch), dim3(kThreads), 0, s, a);
+    auto kernel = interleaved ? rope_append_kernel<T, true, TOK, RESIDENT> : rope_append_kernel<T, false, TOK, RESIDENT>;
+    return launch_pdl(kernel, dim3(blocks, batch), dim3(kThreads), 0, s, a);
 }
 
+// One token per CTA while two CTAs on an SM hold the launch: a step waits for a token's chain (sines, loads, stores), and as a
+// dependent launch no more than two to an SM are better than the four that 32 registers allow - they start while SMs are still taken
+// and would crowd on the others (128 steps of 256 tokens under a window: 2994 us with two, 3077 with four).  More tokens: bf16
+// four CTAs of one token on an SM, from seven tokens an SM on four tokens per CTA, which pay for the chain once; fp32
+// two.  Members of a batch with fewer tokens than that keep one per CTA.  us per launch, cold inputs, plain launches back to
+// back: bf16, 32 / 8 heads, one token with two / four CTAs on an SM, two, four tokens: 256 tokens 4.0 / 3.9 / 4.2 / 5.3; 360: 6.2 / 4.4 /
+// 5.2 / 5.6; 512: 6.7 / 5.0 / 5.3 / 5.9; 640: 8.0 / 6.0 / 7.4 / 8.2; 1024: 10.9 / 8.0 / 9.1 / 8.3; 2048: 18.9 / 13.3 / 15.5 / 14.3; 3584: 30.7 / 21.6 / 23.8 /
+// 21.1; 8192: 66.3 / 45.9 / 49.1 / 41.0 (201 MB: 31 at the copy bandwidth); 592 members of one token 7.6 / 7.4 / 7.9 / 8.3.  (From 1036 to
+// 3300 tokens one per CTA is faster by itself, but not in a step: 2048 tokens of 28 / 4 heads 90.9 us with one, 89.2 with four.)
+// fp32, one token with two CTAs on an SM and two tokens: 256 tokens 5.3 / 5.3; 360: 8.1 / 6.1; 512: 8.9 / 7.0; 1024: 15.4 / 12.1; 8192: 95 / 70.5.
 template <typename T>
 static cudaError_t launch_type(const RopeAppendArgs &a, bool interleaved, int batch, cudaStream_t s) {
-    const int tok = tokens_per_cta<T>((int64_t)a.n * batch);
-    if constexpr (sizeof(T) == 2)
-        if (tok == 4) return launch_tok<T, 4>(a, interleaved, batch, s);
-    return tok == 2 ? launch_tok<T, 2>(a, interleaved, batch, s) : launch_tok<T, 1>(a, interleaved, batch, s);
+    const int64_t tokens = (int64_t)a.n * batch, sms = a.sms;
+    if (tokens <= 2 * sms) return launch_tok<T, 1, 2>(a, interleaved, batch, s);
+    if constexpr (sizeof(T) == 4) return launch_tok<T, 2, 2>(a, interleaved, batch, s);      // (no batches of fp32 caches)
+    else return tokens < 7 * sms || a.n < 4 ? launch_tok<T, 1, 4>(a, interleaved, batch, s) : launch_tok<T, 4, 2>(a, interleaved, batch, s);
 }
 
 cudaError_t launch_rope_append(const RopeAppendArgs &a, int dtype, bool interleaved, int batch, cudaStream_t s) {

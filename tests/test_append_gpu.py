@@ -40,6 +40,52 @@ def test_long_chunks_append_the_bits_of_short_ones(kind, heads):
             assert (got[0][0] - got[1][0]).abs().max().item() <= 2 * TOL[dtype][0]
 
 
+# the lines of the dispatch in tokens per SM: one CTA of one token becomes four to an SM (fp32, quantised rows: two tokens) behind 2,
+# four tokens from 7 (quantised: 6) on; remainders behind them
+@pytest.mark.parametrize("kind", KINDS)
+def test_the_lines_between_one_and_several_tokens_per_cta(kind):
+    dtype, flags = KINDS[kind]
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    quant = flags & (binding.KVF_CACHE_INT8 | binding.KVF_CACHE_INT4)
+    lines = [2 * sms] + ([6 * sms - 1] if quant else [7 * sms - 1] if dtype == "bf16" else [])
+    torch.manual_seed(len(kind))
+    for n in (line + more for line in lines for more in (0, 1, 2, 3)):
+        x = _inputs((), n, 8, 2, 128, dtype)
+        got = []
+        for cuts in ([n], [250] * (n // 250) + [n % 250]):
+            c = binding.Cache(binding.make_config(8, 2, 128, dtype, n, n, rope_base=10000.0, flags=flags))
+            out = torch.cat([c.fold_step(*(t.contiguous() for t in step)) for step in zip(*(t.split(cuts) for t in x))])
+            assert c.status() == binding.KVF_OK
+            got.append((out.float(), c.k_plane(), c.v_plane(), *((c.scales(0), c.scales(1)) if quant else ())))
+        assert (got[0][0] - got[1][0]).abs().max().item() <= 2 * TOL[dtype][0]
+        assert all(torch.equal(*pair) for pair in list(zip(*got))[1:])
+
+
+@pytest.mark.parametrize("flags", [0, binding.KVF_CACHE_INT8, binding.KVF_CACHE_INT4], ids=["bf16", "int8", "int4"])
+@pytest.mark.parametrize("members,n", [(300, 1), (310, 2), (200, 3), (160, 4), (1100, 3)])
+def test_many_members_of_a_few_tokens(members, n, flags):
+    """A CTA takes tokens of one member only."""
+    torch.manual_seed(members)
+    cfg = binding.make_config(4, 1, 128, "bf16", 128, 20, rope_base=10000.0, flags=flags)
+    x, first = _inputs((members,), n, 4, 1, 128, "bf16"), _inputs((members,), 20, 4, 1, 128, "bf16")
+    ws = torch.empty(binding.workspace_bytes(cfg), dtype=torch.uint8, device="cuda")
+    pools, outs = [], []
+    for together in (True, False):
+        pool = torch.zeros(binding.paged_pool_bytes(cfg, members), dtype=torch.uint8, device="cuda")
+        tables = torch.arange(members, device="cuda").flip(0).to(torch.int32).view(members, 1)
+        caches = [binding.PagedCache(cfg, pool, members, tables[i], workspace=ws) for i in range(members)]
+        for c, step in zip(caches, zip(*first)):
+            c.fold_step(*(t.contiguous() for t in step))
+        if together:
+            outs.append(binding.Batch(caches).fold_step(*x))
+        else:
+            outs.append(torch.stack([c.fold_step(*(t.contiguous() for t in step)) for c, step in zip(caches, zip(*x))]))
+        torch.cuda.synchronize()
+        pools.append(pool)
+    assert torch.equal(*pools)
+    assert (outs[0].float() - outs[1].float()).abs().max().item() <= 2 * TOL["bf16"][0]
+
+
 def _held(storage, kv, capacity, d, dtype, flags):
     """[K and V, KV head, row, bytes of codes or elements]"""
     row = d // 2 if flags & binding.KVF_CACHE_INT4 else d if flags & binding.KVF_CACHE_INT8 else d * (4 if dtype == "f32" else 2)
