@@ -1218,7 +1218,7 @@ cudaError_t launch_attn_tc(const AttnArgs &a, const TcMaps &maps, cudaStream_t s
     return launch_pdl(kernel, dim3(grid.x * grid.y, 1, grid.z), dim3(quant ? kThreadsQ8 : kThreads), smem, s, a, maps.q, maps.k, maps.v);
 }
 
-cudaError_t launch_combine_groups(const AttnArgs &a, cudaStream_t s) {
+cudaError_t launch_combine_groups(const AttnArgs &a, int sms, cudaStream_t s) {
     dim3 grid((a.n + kCombineTokens - 1) / kCombineTokens, a.Hkv, a.batch);
     // at most eight parts per KV head (two streams x four pieces, or eight pieces)?  The host knows when it
     // worked out the groups of each head.
@@ -1232,10 +1232,13 @@ cudaError_t launch_combine_groups(const AttnArgs &a, cudaStream_t s) {
         return launch_pdl(combine_small_kernel, dim3((unsigned)((rows + 8 * kSmallRows - 1) / (8 * kSmallRows)), a.Hkv, a.batch), dim3(256), 0, s, a);
     }
     const bool few = known && most <= 8;
-    // Nine parts and more, a block per row while all of them are resident at once (eight to an SM): one token of 32 / 8
-    // heads, 18 parts, 8.5 -> 6.5 us, four tokens 12.7 -> 6.6, 32 tokens (36 parts) 16.8 -> 10.6; one of 12 / 2 heads, 74 parts,
-    // 16.7 -> 8.5.
-    if (known && !few && most <= kRowMergeParts && (int64_t)a.n * a.H * a.batch <= 8 * 148)
+    // Nine parts and more, a block per row as long as there are two waves of them at most (64 registers: four blocks on an SM;
+    // 96 parts of shared memory as well), where they still beat the general kernel.  us per launch back to back, general / per
+    // row: 32 / 8 heads, 9 parts, 64 rows 3.0 / 1.9, 512: 4.5 / 2.7, 768: 4.5 / 3.5, 1024: 4.5 / 3.9, 1184: 4.6 / 4.3, 1536: 4.6 / 5.2; 18
+    // parts 1184: 6.1 / 4.6; 36 parts 1024: 9.8 / 5.3; 96 parts 64: 11.1 / 3.2, 1184: 20.7 / 9.1; groups of six to eight, whose tokens take
+    // eight rows of a block, more: 12 / 2 heads, 74 parts, 48 rows 30.8 / 2.9, 768: 30.9 / 7.1.  More than 96 parts (one KV head on every
+    // SM) would need more registers and shared memory.
+    if (known && !few && most <= kRowMergeParts && (int64_t)a.n * a.H * a.batch <= 8 * (int64_t)sms)
         return launch_pdl(combine_rows_kernel, dim3(a.n * a.G, a.Hkv, a.batch), dim3(256), (size_t)most * 512, s, a);
     if (few) return launch_pdl(combine_groups_kernel<true>, grid, dim3(256), 0, s, a);
     return launch_pdl(combine_groups_kernel<false>, grid, dim3(256), 0, s, a);

@@ -741,7 +741,7 @@ kvf_status step_impl(kvf_cache *c, const void *q, const void *k_new, const void 
         }
         {
             ProfScope ps(c, cs, 2);
-            e = plan.tc ? launch_combine_groups(aa, cs) : launch_combine(aa, f.dtype, cs);
+            e = plan.tc ? launch_combine_groups(aa, c->sm_count, cs) : launch_combine(aa, f.dtype, cs);
         }
         if (e != cudaSuccess) return cuda_fail(e, "combine launch");
         c->launches++;
@@ -1399,7 +1399,7 @@ kvf_status batch_step(kvf_batch *b, const void *q, const void *k_new, const void
     if (e != cudaSuccess) return cuda_fail(e, "attention launch (batch)");
     b->launches++;
     if (plan.kernels > 2) {
-        e = launch_combine_groups(aa, st);
+        e = launch_combine_groups(aa, c0->sm_count, st);
         if (e != cudaSuccess) return cuda_fail(e, "combine launch (batch)");
         b->launches++;
     }

@@ -265,7 +265,7 @@ int attn_tc_padded_group(int G);       // G rounded up to a power of two: rows a
 int attn_tc_row_pairs(int n, int G);   // 256-row pairs per KV head (G: the padded group, as below)
 int attn_tc_streams(int n, int G);     // 2 when the chunk fits one 128-row tile
 cudaError_t launch_attn_tc(const AttnArgs &a, const TcMaps &maps, cudaStream_t s);   // grid (ngroups x row pairs); pairs of CTAs: (row pairs, ngroups)
-cudaError_t launch_combine_groups(const AttnArgs &a, cudaStream_t s);                // needed when ngroups != Hkv
+cudaError_t launch_combine_groups(const AttnArgs &a, int sms, cudaStream_t s);                // needed when ngroups != Hkv
 
 // Decode-shaped steps (at most attn_q8_decode_max_rows() query rows) on a quantised cache: codes are
 // expanded into mma.sync register fragments, shared memory is all ring.  Grid = ngroups CTAs, ngroups a
