@@ -1,6 +1,6 @@
-"""Rotate + append with several tokens per CTA (297 tokens of a launch on): the cache bits are those of short chunks, which take
-one token per CTA, and the outputs those of the same rows folded in short chunks, within the bounds of tests/chain.py (a wrong
-rotation of a query would show: inputs are N(0, 1))."""
+"""Rotate + append of long chunks, several tokens per CTA or four CTAs on an SM (297 tokens of a launch on): the cache bits, row
+scales included, are those of short chunks, which take one token per CTA and two CTAs on an SM, and the outputs those of the same
+rows folded in short chunks, within the bounds of tests/chain.py (a wrong rotation of a query would show: inputs are N(0, 1))."""
 import pytest
 import torch
 
@@ -28,14 +28,18 @@ def test_long_chunks_append_the_bits_of_short_ones(kind, heads):
         for n in (296, 297, 300, 513, 1023, 1024, 1027, 1030):
             first = 77
             x = _inputs((), first + n, *heads, d, dtype)
-            got = []
+            got, scales = [], []
             for cuts in ([first, n], [first] + [250] * (n // 250) + [n % 250]):
                 c = binding.Cache(binding.make_config(*heads, d, dtype, first + n + 50, n, rope_base=10000.0, flags=flags))
                 c.storage.fill_(0x5A)
                 out = torch.cat([c.fold_step(*(t.contiguous() for t in step)) for step in zip(*(t.split(cuts) for t in x))])
                 assert c.status() == binding.KVF_OK
                 got.append((out.float(), c.storage))
+                if flags & (binding.KVF_CACHE_INT8 | binding.KVF_CACHE_INT4):
+                    scales.append([c.scales(kv) for kv in (0, 1)])
             rows = slice(0, first + n)
+            if flags & (binding.KVF_CACHE_INT8 | binding.KVF_CACHE_INT4):
+                assert all(torch.equal(*(s[:, rows] for s in pair)) for pair in zip(scales[-2], scales[-1]))
             assert torch.equal(*(_held(s, heads[1], first + n + 50, d, dtype, flags)[:, :, rows] for _, s in got))
             assert (got[0][0] - got[1][0]).abs().max().item() <= 2 * TOL[dtype][0]
 
@@ -92,7 +96,7 @@ def _held(storage, kv, capacity, d, dtype, flags):
     return storage[:2 * kv * capacity * row].view(2, kv, capacity, row)
 
 
-@pytest.mark.parametrize("flags", [0, binding.KVF_CACHE_INT8], ids=["bf16", "int8"])
+@pytest.mark.parametrize("flags", [0, binding.KVF_CACHE_INT8, binding.KVF_CACHE_INT4], ids=["bf16", "int8", "int4"])
 def test_batches_append_the_bits_of_single_caches(flags):
     torch.manual_seed(3)
     for n in (33, 57, 114, 129):              # 9 members: 297, 513, 1026 and 1161 tokens to a launch
