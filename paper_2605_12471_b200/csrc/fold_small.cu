@@ -120,7 +120,7 @@ __device__ __forceinline__ void cluster_sync() {
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-// BN = keys of a tile: 64, or 32 (see fold_small_ranks).
+// BN = keys of a tile: 64, or 32 (see fold_small_cut).
 template <typename T, bool INTERLEAVED, int BN>
 __global__ void __launch_bounds__(kThreads, 2) fold_small_kernel(const __grid_constant__ RopeAppendArgs r, const __grid_constant__ AttnArgs a) {
     constexpr int VEC = 16 / (int)sizeof(T);
@@ -496,7 +496,8 @@ FoldSmallCut fold_small_cut(int row_tiles, int64_t keys, bool window, const Fold
     return best;
 }
 
-// (the four kernels differ in arithmetic only: what fits one fits all)
+// (the eight kernels differ in arithmetic and tile width only, in neither threads, shared memory nor the limit on registers: what
+// fits one fits all)
 cudaError_t fold_small_fit(FoldSmallFit *fit) { return prepare_once<float, false, 64>(fit); }
 
 cudaError_t launch_fold_small(const RopeAppendArgs &r, const AttnArgs &a, const FoldSmallCut &cut, int dtype, bool interleaved, cudaStream_t s) {

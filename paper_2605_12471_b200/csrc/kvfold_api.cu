@@ -377,7 +377,10 @@ Plan make_plan(const kvf_cache *c, int n, int64_t prefix, int batch = 1, int64_t
             // tokens), beyond eight the merge kernel that holds any number, the parts written and read.  A range of one
             // tile is no faster than one of two.  Fitted to 12 800 random steps timed under 2 to 18 cuts each (17 - 4096
             // tokens, seven head shapes, 64 - 60 K rows, windows, batches, all storages): rms 5 % of a step; the cut
-            // chosen is 2.6 % above the best of them on average, where a fixed least of four tiles per CTA is 13 %.
+            // chosen is 2.6 % above the best of them on average, where a fixed least of four tiles per CTA is 13 %.  (The fit is
+            // from before up to four parts, and nine and more of few rows, had merge kernels of their own, 1 - 5 us cheaper
+            // (launch_combine_groups has figures), and before pairs of CTAs on quantised rows issued Q K^T early; not
+            // fitted again since: more cuts than it chooses may pay.)
             // us per step (ranges per head: time): 256 tokens of 32 / 8 heads, bf16, 4 key tiles 1: 17.4, 4: 18.1; 8 tiles
             // 1: 24.6, 2: 23.2, 4: 20.1; 64 tokens of 28 / 4 heads, 32 tiles 8: 22.2, 18: 31.2; 32 tokens of 12 / 2
             // heads, 126 tiles 31: 35.2, 72: 55.7; 48 tokens of 8 / 2 heads, int8, 43 tiles 10: 28.0, 24: 22.6.
@@ -426,6 +429,8 @@ Plan make_plan(const kvf_cache *c, int n, int64_t prefix, int batch = 1, int64_t
             // merge) against 9: 55 / 90 us at prefix 0, 115 / 145 at 2 K, 234 / 257 at 6 K, 478 / 490 at 14 K, 1002 / 906 at
             // 30 K - about 28 tiles of 1.9 us; int8 102 / 135 at 0, 395 / 399 at 8 K, 537 / 529 at 12 K.  4326 random
             // steps of all storages under both cuts: 20 took more than 1 % longer than under the other, 6 % at most.
+            // (From before the merge kernel for four parts at most, which these cuts now take - a KV head has three; not
+            // measured again since.)
             auto cost = [&](int64_t g) {
                 double tiles = g > Hkv ? (double)n * c->cfg.n_q_heads * batch / 2400.0 : 0.0;
                 const int64_t ctas = (int64_t)pairs * g * batch;
@@ -484,6 +489,8 @@ Plan make_plan(const kvf_cache *c, int n, int64_t prefix, int batch = 1, int64_t
         // rows, where the three launches are 2 us faster, for chunks that span two key tiles (a second table of sines): 72
         // tokens of 2 / 2 heads 5: 38.6, 34.9; 160 tokens 4: 37.4, 34.5.  Of the 3322 steps within these limits among
         // 3722 (102 shapes, 1 - 512 key tiles, fp32 and bf16) none measured more than 2 % slower than through three.
+        // (All of this with tiles of 64 keys in the slices of fold_small_ranks; what is launched is fold_small_cut's,
+        // which is never slower, so that the limits hold; steps beyond them may have become faster in one launch.)
         const int tiles = fold_small_row_tiles(n, c->G) * Hkv;
         const int ranks = fold_small_ranks(tiles, nt, c->small_fit);
         const int64_t at_once = (int64_t)tiles * ranks;
