@@ -33,7 +33,9 @@
 //    2^-30 of the row's largest; what vanishes is 2^-39 of it and less, far below the fp32 sums.
 // (One reference per warp, the largest V scale loaded so far, lost rows 2^33 below a hidden one.  Without references: products
 // as bf16 with V codes as bf16, 8 bits, cost 2 us of 54 at one token of int8 and 5.5 of 73 at four; in two bf16 parts 5 and 16.  As it is:
-// one token as before, four tokens of int8 73.5 -> 76.8 us, of int4 65.5 -> 66: two blocks of query rows have no registers to spare.)
+// one token 54 us as before, four tokens of int8 73.5 -> 76.8, of int4 65.5 -> 66.5: two blocks of query rows have no registers to
+// spare; behind short prefixes 0.15 - 0.2 us of 9 - 11 (the look at the queries, one more trip between the threads in a warp's
+// first tile), two blocks 0.1 - 0.5.)
 //
 // With so few query rows the KEYS take the 16-row side of the MMA and the query rows the 8-column
 // side (one or two column blocks), so no MMA row is wasted on padding and V needs no transpose:
@@ -477,6 +479,18 @@ attn_q8_decode_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
                 }
             }
         }
+        // Keys below a row's limit, counted from the chunk's first key, P, are visible (rows past the chunk's end are never
+        // written; each row of S, P and O depends on that row alone, so they are left unmasked).  bf16 rows have it at hand:
+        // the divide, in the last tile of a short step, is 0.1 us of 10; quantised rows have no registers for it and take longer with.
+        auto limit_of = [&](int nb, int e) {
+            const int R = 8 * nb + 2 * t4 + e;
+            return R < nG ? (R / G + 1) * a.self_rows : 1 << 30;
+        };
+        int limit[NB][2];
+#pragma unroll
+        for (int nb = 0; nb < NB; ++nb)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) limit[nb][e] = BITS == 16 ? limit_of(nb, e) : 0;
         // softmax scale * log2(e) of query rows 8 nb + 2 t + {0, 1} (whose scaling the threads of those g know)
         float sl2[NB][2];
 #pragma unroll
@@ -546,18 +560,16 @@ attn_q8_decode_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
 #pragma unroll
                     for (int e = 0; e < 4; ++e) sacc[j][nb][e] *= BITS == 16 ? sl2[nb][e & 1] : row_scale[j][e >> 1] * sl2[nb][e & 1];
             if (key_h + 64 > P) {
-                // keys below a row's limit are visible (rows past the chunk's end are never written; each row of S, P
-                // and O depends on that row alone, so they are left unmasked)
                 const int rel = (int)(key_h - P) + g;               // my first key, counted from P (> -64)
 #pragma unroll
                 for (int nb = 0; nb < NB; ++nb)
 #pragma unroll
                     for (int e = 0; e < 2; ++e) {
-                        const int R = 8 * nb + 2 * t4 + e, limit = R < nG ? (R / G + 1) * a.self_rows : (1 << 30);
+                        const int end = BITS == 16 ? limit[nb][e] : limit_of(nb, e);
 #pragma unroll
                         for (int j = 0; j < 4; ++j) {
-                            if (rel + 16 * j >= limit) sacc[j][nb][e] = -INFINITY;
-                            if (rel + 16 * j + 8 >= limit) sacc[j][nb][2 + e] = -INFINITY;
+                            if (rel + 16 * j >= end) sacc[j][nb][e] = -INFINITY;
+                            if (rel + 16 * j + 8 >= end) sacc[j][nb][2 + e] = -INFINITY;
                         }
                     }
             }
