@@ -112,6 +112,8 @@ __global__ void __launch_bounds__(kThreads, kResident) rope_append_q8_kernel(con
         // .. 4 lane + 3; else the pairs (j, j + 64) for j = 2 lane, 2 lane + 1
         const bool in_order = INTERLEAVED || is_v;
         const int e0 = in_order ? 4 * lane : 2 * lane, e1 = in_order ? 4 * lane + 2 : half + 2 * lane;
+        // (Rows in order are loaded and stored in two pieces as well: one piece behind a branch of the warp took as long, 2048
+        // tokens 20.5 / 20.7 us.)
         // (one turn; without the loop the compiler's order costs two and four tokens 2 - 4 % of a launch)
 #pragma unroll 1
         for (int t0 = 0; t0 < ntok; t0 += kTok) {
