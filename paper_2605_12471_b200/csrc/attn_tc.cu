@@ -28,8 +28,8 @@
 // overwrite the first 64 columns of their own S tile, in two halves that are handed to the
 // second MMA separately, and feed it straight from tensor memory; the tensor pipe runs one
 // thread's MMAs in issue order, so the next Q K^T of a row tile cannot overtake the P V that
-// still reads those columns.  A single issuing thread for both tiles spends ~126 cycles per MMA
-// (measured) against 64 cycles of tensor work, hence one issuer per row tile.
+// still reads those columns.  A single issuing thread for both tiles spent ~126 cycles per MMA
+// against 64 cycles of tensor work (measured in a branch of one lane, see the issuer), hence one issuer per row tile.
 //
 // Softmax arithmetic.  p = 2^(s * scale * log2(e) - m) with the reference maximum m moved only
 // when the tile maximum exceeds it by more than 2^8 (then the accumulator is rescaled), packed
@@ -51,7 +51,9 @@
 // latency out of the softmax threads' chain: whether the panel is free is asked before the second half's arithmetic (a wait on a
 // barrier that is already complete takes ~250 cycles beside saturated shared memory), and whether a key tile
 // needs a mask is known from the tile number, without a vote.  (Leaving out the vote on the scores' wait as well: 312;
-// passing the turn ahead of the K slot's commit: no change.)  It takes a K/V slot of shared memory.  On quantised storage only
+// passing the turn ahead of the K slot's commit: no change on bf16 rows, 1 % on pairs of CTAs.)  With issuing warps that
+// walk their loops as a whole it is 2690 cycles for a pair of tiles, of which shared memory is busy 2560 (operands of the MMAs
+// 1792, tiles coming in 512, probabilities 256).  It takes a K/V slot of shared memory.  On quantised storage only
 // pairs of CTAs have that to spare (each keeps raw codes of the 64 rows it expands, no more), and three tile slots
 // instead of four: 439 -> 413 thousand cycles at prefix 61 K (int8, 256 tokens; int4 452 -> 422), 551 -> 512 for 2048 tokens at
 // 14 K, 65 536 tokens in chunks of 256 43.2 -> 41.5 ms; 41.9 since a raw slot is given back behind the stores.  What bounds them then is shared memory (MMA operands, the tile stored, sent and received: ~90 % of the
@@ -152,6 +154,36 @@ __device__ __forceinline__ uint64_t desc_mnmajor(uint32_t addr) {
     return (uint64_t)((addr >> 4) & 0x3FFFu) | ((uint64_t)(kPanel >> 4) << 16) | ((uint64_t)(1024 >> 4) << 32) |
            ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
 }
+
+// One go at several barriers: the answers are asked for back to back and looked at together (an answer takes 150 - 200 cycles to
+// come even when it is yes).
+struct Phase {
+    uint32_t bar, parity;
+};
+__device__ __forceinline__ bool mbar_try_wait4(const Phase (&w)[4]) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p, q, r, s;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %9;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 q, [%3], %4, %9;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 r, [%5], %6, %9;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 s, [%7], %8, %9;\n\t"
+        "and.pred p, p, q;\n\t"
+        "and.pred r, r, s;\n\t"
+        "and.pred p, p, r;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok) : "r"(w[0].bar), "r"(w[0].parity), "r"(w[1].bar), "r"(w[1].parity), "r"(w[2].bar), "r"(w[2].parity),
+          "r"(w[3].bar), "r"(w[3].parity), "r"(kSuspendHintNs) : "memory");
+    return ok;
+}
+__device__ __forceinline__ bool mbar_wait4(const Phase (&w)[4], Ctl *ctl, int *status) {
+    if (mbar_try_wait4(w)) return true;
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        if (!mbar_wait(w[k].bar, w[k].parity, ctl, status)) return false;
+    return true;
+}
+
 // Instruction descriptor: D fp32, A and B bf16, M = 128, N = 128; bit 16 = B is MN-major.
 constexpr uint32_t kIdescQK = (1u << 4) | (1u << 7) | (1u << 10) | ((128u >> 3) << 17) | ((128u >> 4) << 24);
 constexpr uint32_t kIdescPV = kIdescQK | (1u << 16);
@@ -498,11 +530,18 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
                 for (int t = max(0, tg - NS); t < tg; ++t)
                     mbar_wait_drain(bar(B_FULL0 + t % NS), (t / NS) & 1, a.status);
             }
-        } else if ((warp == 9 || (warp == 10 && tiles == 2)) && lane == 0) {
+        } else if (warp == 9 || (warp == 10 && tiles == 2)) {
             // ------------------------------------------------------------------ MMA issuer of row tile i
             // One issuing thread per row tile: each thread's MMAs run in its issue order (P V (j)
             // before the Q K^T (j+1) that overwrites the probabilities), the two tiles' streams
             // interleave freely on the tensor pipe, and neither waits on the other's softmax.
+            // The whole warp walks the loop and one thread of it issues: the addresses are then the same in all lanes as far as
+            // the compiler knows, and descriptors stay in uniform registers.  In a branch of one lane every MMA moved its
+            // own there first, and these ~350 instructions a tile, in a warp that shares its scheduler with two of the softmax,
+            // were what the kernel waited for.  Cycles of a CTA, 256 tokens in 131 072: 167 -> 152 million, deep chain 135.6 -> 131.5 ms;
+            // 2048 tokens in 16 384: 1.76 -> 1.61 million, 1933 -> 1826 us; int8, 256 tokens in 65 536: 58.6 -> 53.0 million, 42.0 ->
+            // 39.6 ms.  (Of it 3 % of the cycles of bf16 rows: what a tile waits for ahead of its first MMAs asked in one go.)
+            const bool leader = elect_one();
             const int i = warp - 9;
             const uint32_t t_s = tmem + i * 128, t_o = tmem + 256 + i * 128;
             const uint64_t qdesc = desc_kmajor(base + kOffQ + (streams == 2 ? 0 : i) * kTileBytes);
@@ -512,7 +551,7 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
 #pragma unroll
                 for (int kk = 0; kk < 8; ++kk) {
                     const uint64_t off = (uint64_t)(((kk >> 2) * kPanel + (kk & 3) * 32) >> 4);   // start-address field
-                    tc_mma(t_s, qdesc + off, kdesc + off, kIdescQK, kk > 0);
+                    if (leader) tc_mma(t_s, qdesc + off, kdesc + off, kIdescQK, kk > 0);
                 }
             };
             // 16 keys = 8 packed columns of P per MMA; half h covers keys 64h .. 64h+63
@@ -521,6 +560,7 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
                 const uint64_t vdesc = desc_mnmajor(slot_addr(slot));
 #pragma unroll
                 for (int kk = 4 * h; kk < 4 * h + 4; ++kk) {
+                    if (!leader) continue;
                     if (kEarly && h == 1)
                         tc_mma(t_o, pdesc + (uint64_t)(((kk - 4) * 32) >> 4), vdesc + (uint64_t)((kk * 2048) >> 4), kIdescPV, 1u);
                     else
@@ -530,6 +570,7 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
             // a K/V slot is free once its readers have run: in the paired variant the partner's expansion warps
             // wait for my reads as well (they write my slot), so the commit goes to both CTAs' barriers
             auto commit_empty = [&](int slot) {
+                if (!leader) return;
                 if (kPair) tc_commit_pair(bar(B_EMPTY0 + slot));
                 else tc_commit(bar(B_EMPTY0 + slot));
             };
@@ -557,7 +598,7 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
                 int jprev = -1;
                 for (int j = j0; ok; j += jstep) {
                     const bool more = j < ntiles;
-                    if (!more) tc_commit(bar(B_QEMPTY));          // every Q K^T of mine in this piece has been issued
+                    if (!more && leader) tc_commit(bar(B_QEMPTY));          // every Q K^T of mine in this piece has been issued
                     if (!more && jprev < 0) break;
                     const int tk = streams == 2 ? 2 * it : tg + 2 * j;
                     int kslot = 0, vslot = 0;
@@ -567,16 +608,19 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
                         if (!mbar_wait(bar(B_PB0 + i), (it - 1) & 1, ctl, a.status)) return false;
                         tc_fence_after();
                         issue_pv_half(vslot, 1, true);
-                        if (kEarly || !more) tc_commit(bar(B_PVDONE0 + i));
+                        if ((kEarly || !more) && leader) tc_commit(bar(B_PVDONE0 + i));
                         commit_empty(vslot);
                         return true;
                     };
                     if (jprev >= 0) {
                         ring(streams == 2 ? 2 * it - 1 : tg + 2 * jprev + 1, vslot, vpar);
-                        ok = mbar_wait(bar(B_FULL0 + vslot), vpar, ctl, a.status);
-                        if (ok) ok = mbar_wait(bar(B_PA0 + i), (it - 1) & 1, ctl, a.status);
-                        if (kEarly && ok && tiles == 2 && (i == 1 || turns > 0))
-                            ok = mbar_wait(bar(B_TURN0 + i), (i == 0 ? turns - 1 : turns) & 1, ctl, a.status);
+                        const Phase v_full = {bar(B_FULL0 + vslot), vpar}, p_half = {bar(B_PA0 + i), (uint32_t)(it - 1) & 1u};
+                        const bool turn = kEarly && tiles == 2 && (i == 1 || turns > 0);
+                        const Phase my_turn = turn ? Phase{bar(B_TURN0 + i), (uint32_t)(i == 0 ? turns - 1 : turns) & 1u} : p_half;
+                        // (what is not there to be waited for is asked for twice; pairs of CTAs: a K tile is the last to come, and P V
+                        // need not wait for it)
+                        const Phase all[4] = {v_full, kEarly && !kPair && more ? Phase{bar(B_FULL0 + kslot), kpar} : v_full, p_half, my_turn};
+                        ok = mbar_wait4(all, ctl, a.status);
                         if (!ok) break;
                         tc_fence_after();
                         issue_pv_half(vslot, 0, jprev > j0);
@@ -584,18 +628,19 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
                         if (!ok) break;
                     }
                     if (more) {
-                        ok = mbar_wait(bar(B_FULL0 + kslot), kpar, ctl, a.status);
+                        // (bf16 rows: waited for above, but for a piece's first)
+                        if (!kEarly || kPair || jprev < 0) ok = mbar_wait(bar(B_FULL0 + kslot), kpar, ctl, a.status);
                         if (!ok) break;
                         tc_fence_after();
                         issue_qk(kslot);
-                        tc_commit(bar(B_SFULL0 + i));
-                        commit_empty(kslot);
+                        if (leader) tc_commit(bar(B_SFULL0 + i));
                     }
                     if (kEarly && jprev >= 0) {
-                        if (tiles == 2) mbar_arrive(bar(B_TURN0 + (i ^ 1)));
+                        if (tiles == 2 && leader) mbar_arrive(bar(B_TURN0 + (i ^ 1)));
                         ++turns;
-                        ok = second_half();
                     }
+                    if (more) commit_empty(kslot);
+                    if (kEarly && jprev >= 0) ok = second_half();
                     if (!more || !ok) break;
                     jprev = j;
                     ++it;
@@ -604,10 +649,12 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
                 tg += 2 * ntiles;
                 ++pc;
             }
-            // whatever made this thread leave its loop, tensor memory is released only after every
+            // whatever made this warp leave its loop, tensor memory is released only after every
             // MMA it issued has run
-            tc_commit(bar(B_DRAIN0 + i));
-            mbar_wait_drain(bar(B_DRAIN0 + i), 0, a.status);
+            if (leader) {
+                tc_commit(bar(B_DRAIN0 + i));
+                mbar_wait_drain(bar(B_DRAIN0 + i), 0, a.status);
+            }
         }
     } else {
         // ------------------------------------------------------------------ softmax, one thread per row

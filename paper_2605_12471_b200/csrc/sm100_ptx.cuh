@@ -143,6 +143,13 @@ __device__ __forceinline__ void bulk_push(uint32_t dst_cluster, uint32_t src, ui
                  ::"r"(dst_cluster), "r"(src), "r"(bytes), "r"(bar_cluster) : "memory");
 }
 
+// one thread of a converged warp
+__device__ __forceinline__ bool elect_one() {
+    uint32_t one;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(one));
+    return one != 0;
+}
+
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_commit(uint32_t bar) {
