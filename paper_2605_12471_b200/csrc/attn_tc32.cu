@@ -27,29 +27,33 @@
 // writes final outputs, otherwise each piece leaves a normalised partial and its log2
 // denominator in slot (group + KV head) for combine_groups_kernel.
 //
-// Roles (512 threads, one CTA per SM):
-//   warps 0-3   softmax, one thread per row (TMEM lane = row): scores of a step from tensor memory
-//               (read twice: maximum, then exponentials), probabilities split into fp16 hi / lo and
-//               written back to tensor memory, the step's P V added to the 128 output registers
-//   warps 4-7   K converters: 16 rows of the step's K tile per warp, fp32 from global memory (one
+// Roles (640 threads, one CTA per SM):
+//   warps 0-3   softmax, one thread per row (TMEM lane = row): a piece's query row split into tensor memory; scores of a
+//               step from tensor memory into registers, probabilities split into fp16 hi / lo and written back
+//   warps 4-7   output, one thread per row: each step's P V added to 128 registers in round-to-nearest fp32
+//   warps 8-11  K converters: 16 rows of the step's K tile per warp (8 in a pair of CTAs), fp32 from global memory (one
 //               coalesced 512-byte row per warp instruction), split, written as 128-byte-swizzled
-//               K-major fp16 tiles into a ring of three slots; in a slot the 64 rows of K_lo follow
+//               K-major fp16 tiles into a ring of four slots; in a slot the 64 rows of K_lo follow
 //               the 64 rows of K_hi inside each 64-column panel, so [K_hi; K_lo] is ONE 128-row operand
-//   warps 8-11  V converters: the same for V (ring of two slots, V_hi then V_lo; a V tile is read
-//               MN-major, so its rows are laid out as a K tile's); both converter groups also split
-//               the piece's 128 x 128 Q tile
-//   warp 12     issuer of the score MMAs (one thread) and owner of the tensor-memory allocation
-//   warp 13     issuer of the output MMAs (one thread)
-// One tcgen05.mma costs its issuing thread about as long as a 128 x 128 x 16 MMA runs, whatever its
-// N, so the kernel is built to issue few, wide MMAs from two threads: per 64-key step and 16
-// elements of d, Q_hi [K_hi; K_lo]^T is one MMA with N = 128 (its columns 0-63 are Q_hi K_hi, 64-127
-// the small term Q_hi K_lo) and Q_lo K_hi^T one with N = 64 added onto columns 0-63; the softmax
+//   warps 12-15 V converters: the same for V (ring of three slots, V_hi then V_lo; a V tile is read
+//               MN-major, so its rows are laid out as a K tile's)
+//   warp 16     issuer of the score MMAs and owner of the tensor-memory allocation
+//   warp 17     issuer of the output MMAs
+// Few, wide MMAs: per 64-key step and 16 elements of d, Q_hi [K_hi; K_lo]^T is one MMA with N = 128 (its columns 0-63 are
+// Q_hi K_hi, 64-127 the small term Q_hi K_lo) and Q_lo K_hi^T one with N = 64 added onto columns 0-63; the softmax
 // adds the two halves of a score.  16 score MMAs and 12 output MMAs per step (a first version with
 // 24 + 12 from one thread spent ~120 cycles per MMA on issue alone and left the tensor pipe 70 % idle).
-// Tensor memory: S0 | S1 (128 fp32 columns each: 64 scores + 64 small terms) | P0 | P1 (hi: 32
-// columns, lo: 32 columns) | O (128).  The score issuer runs ahead of the softmax by one step (S is
-// double-buffered), the output issuer starts a step's P V as soon as its probabilities are
-// written and the previous P V has been added to the registers.
+// Tensor memory: S (128 fp32 columns: 64 scores + 64 small terms) | P0 | P1 (hi: 32 columns, lo: 32 columns) | O (128) |
+// Q_hi | Q_lo (64 columns each, two elements to a column).  The scores of the next step are issued as soon as the softmax
+// has this step's in registers, and run under its exponentials: one S is enough.  The output issuer starts a step's P V as
+// soon as its probabilities are written and the previous P V has been added to the registers.
+//
+// What bounds it: the chain of the softmax thread (~2300 cycles a step, one softmax warp per scheduler), beside 1664 of tensor work
+// and 1536 of shared memory (operands of the MMAs 96 KB a step, tiles stored, sent and received 96 KB), and the power cap. Until
+// the output rows had warps of their own and the queries lay in tensor memory, the softmax thread added P V as well
+// (800 cycles of its 2700) and the MMAs read Q from shared memory (64 KB a step more; with the output warps alone the MMAs
+// took that time instead: 159 -> 162 million cycles of a CTA).  65 536 tokens in chunks of 512: 159 -> 134 million cycles, 111 ->
+// 102 ms (1.48 -> 1.38 GHz).
 //
 // Every wait on an mbarrier is bounded and reports through the status word, as in the bf16 kernel.
 #include "kvfold_internal.h"
@@ -64,26 +68,26 @@ constexpr int kRows = 128;                     // query rows of a CTA
 constexpr int kD = 128;                        // head_dim
 constexpr int kKeys = 64;                      // keys of one step
 constexpr int kTileKeys = 128;                 // keys of one tile of the plan's line = two steps
-constexpr int kThreads = 512;
-constexpr uint32_t kQPanel = kRows * 128;      // [128 rows][64 fp16], 128-byte swizzle
-constexpr uint32_t kQPart = 2 * kQPanel;       // hi or lo of the Q tile
+constexpr int kThreads = 640;
 constexpr uint32_t kKPanel = kKeys * 128;      // [64 keys][64 fp16]
 constexpr uint32_t kKPart = 2 * kKPanel;       // hi or lo of a K (or V) step tile
 constexpr uint32_t kKSlot = 2 * kKPart;        // hi + lo
-constexpr int kKSlots = 3, kVSlots = 2;
-constexpr uint32_t kOffQ = 0;                                  // Q hi, Q lo
-constexpr uint32_t kOffK = 2 * kQPart;
+constexpr int kKSlots = 4, kVSlots = 3;
+constexpr uint32_t kOffK = 0;
 constexpr uint32_t kOffV = kOffK + kKSlots * kKSlot;
 constexpr uint32_t kOffCtl = kOffV + kVSlots * kKSlot;
-constexpr uint32_t kSmemBytes = kOffCtl + 512 + 1024;          // + control block + alignment slack
+constexpr uint32_t kOffRow = kOffCtl + 512;                    // three times one float per row: see the output warps
+constexpr int kRowSlots = 3;
+constexpr uint32_t kSmemBytes = kOffRow + kRowSlots * kRows * 4 + 1024;          // + alignment slack
 constexpr uint32_t kTmemCols = 512;
-constexpr uint32_t kColS = 0, kColP = 256, kColO = 384;        // S0|S1 at 0, 128; P0|P1 at 256, 320; O at 384
+constexpr uint32_t kColS = 0, kColP = 128, kColO = 256, kColQ = 384;        // P0|P1 at 128, 192; Q_hi|Q_lo at 384, 448
 constexpr uint32_t kKOperand = 2 * kKPanel;                    // one 64-column panel of [K_hi; K_lo]: 128 rows
 constexpr float kRescaleThreshold = 8.0f;                      // log2 units
 
 enum { B_QFULL = 0, B_QEMPTY = 1, B_KFULL0 = 2, B_KEMPTY0 = B_KFULL0 + kKSlots, B_VFULL0 = B_KEMPTY0 + kKSlots,
-       B_VEMPTY0 = B_VFULL0 + kVSlots, B_SFULL0 = B_VEMPTY0 + kVSlots, B_SFREE0 = B_SFULL0 + 2, B_PFULL0 = B_SFREE0 + 2,
-       B_OFULL = B_PFULL0 + 2, B_OFREE = B_OFULL + 1, B_DRAIN0 = B_OFREE + 1, B_COUNT = B_DRAIN0 + 2 };
+       B_VEMPTY0 = B_VFULL0 + kVSlots, B_SFULL = B_VEMPTY0 + kVSlots, B_SFREE = B_SFULL + 1, B_PFULL0 = B_SFREE + 1,
+       B_PFREE0 = B_PFULL0 + 2, B_OFULL = B_PFREE0 + 2, B_OFREE = B_OFULL + 1, B_ROWDONE = B_OFREE + 1, B_DRAIN0 = B_ROWDONE + 1,
+       B_COUNT = B_DRAIN0 + 2 };
 
 struct Ctl {
     unsigned long long bars[32];
@@ -142,9 +146,10 @@ __device__ __forceinline__ void store_split4(uint8_t *part_hi, uint8_t *part_lo,
                  : "=r"(a[o + 0]), "=r"(a[o + 1]), "=r"(a[o + 2]), "=r"(a[o + 3]), "=r"(a[o + 4]), "=r"(a[o + 5]), "=r"(a[o + 6]), "=r"(a[o + 7]), \
                    "=r"(a[o + 8]), "=r"(a[o + 9]), "=r"(a[o + 10]), "=r"(a[o + 11]), "=r"(a[o + 12]), "=r"(a[o + 13]), "=r"(a[o + 14]), "=r"(a[o + 15]) \
                  : "r"(taddr) : "memory")
-#define KVF_TMEM_ST8(a, o, taddr)                                                               \
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%8], {%0, %1, %2, %3, %4, %5, %6, %7};" \
+#define KVF_TMEM_ST16(a, o, taddr)                                                              \
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%16], {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15};" \
                  ::"r"(a[o + 0]), "r"(a[o + 1]), "r"(a[o + 2]), "r"(a[o + 3]), "r"(a[o + 4]), "r"(a[o + 5]), "r"(a[o + 6]), "r"(a[o + 7]), \
+                   "r"(a[o + 8]), "r"(a[o + 9]), "r"(a[o + 10]), "r"(a[o + 11]), "r"(a[o + 12]), "r"(a[o + 13]), "r"(a[o + 14]), "r"(a[o + 15]), \
                    "r"(taddr) : "memory")
 
 // kPair: the CTAs of row blocks 2k and 2k + 1 form a cluster of two that walks the same 64-key steps.  Each
@@ -196,23 +201,25 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc32_kernel(const AttnArgs a
     auto step_key0 = [&](int kt0, int s) { return (int64_t)wt.actual(kt0 + (s >> 1)) * kTileKeys + (s & 1) * kKeys; };
 
     if (threadIdx.x == 0) {
-        mbar_init(bar(B_QFULL), 8);
+        mbar_init(bar(B_QFULL), 4);
         mbar_init(bar(B_QEMPTY), 1);
         for (int s = 0; s < kKSlots; ++s) { mbar_init(bar(B_KFULL0 + s), 4); mbar_init(bar(B_KEMPTY0 + s), kPair ? 2 : 1); }
         for (int s = 0; s < kVSlots; ++s) { mbar_init(bar(B_VFULL0 + s), 4); mbar_init(bar(B_VEMPTY0 + s), kPair ? 2 : 1); }
+        mbar_init(bar(B_SFULL), 1);
+        mbar_init(bar(B_SFREE), 4);
         for (int i = 0; i < 2; ++i) {
-            mbar_init(bar(B_SFULL0 + i), 1);
-            mbar_init(bar(B_SFREE0 + i), 4);
             mbar_init(bar(B_PFULL0 + i), 4);
+            mbar_init(bar(B_PFREE0 + i), 1);
         }
         mbar_init(bar(B_OFULL), 1);
         mbar_init(bar(B_OFREE), 4);
+        mbar_init(bar(B_ROWDONE), 4);
         mbar_init(bar(B_DRAIN0), 1);
         mbar_init(bar(B_DRAIN0 + 1), 1);
         ctl->abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == 12) {
+    if (warp == 16) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&ctl->tmem_base)), "r"(kTmemCols) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
@@ -231,14 +238,15 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc32_kernel(const AttnArgs a
         ctl->ns0 = global_ns();
     }
 
-    if (warp >= 12) {
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 48;");
+    // The shares of registers: softmax 128 x 128, output 128 x 168, converters 256 x 72, issuers 128 x 40 = the launch's 640 x 96.
+    if (warp >= 16) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");
         // (whole warps walk the issuers' loops and one thread issues: the descriptors stay in uniform registers.  In branches of one
         // lane the chain of 65 536 tokens, 512 at a time, took 119.9 ms instead of 110.6, 176 million cycles of a CTA instead of 159)
         const bool leader = elect_one();
-        if (warp == 12) {
+        if (warp == 16) {
             // ------------------------------------------------------------------ issuer of the score MMAs
-            const uint64_t dqh = desc_kmajor(base + kOffQ), dql = desc_kmajor(base + kOffQ + kQPart);
+            const uint32_t t_s = tmem + kColS, q_hi = tmem + kColQ, q_lo = q_hi + 64u;
             int g = 0;                   // steps so far, all pieces = load number of the K ring
             int pc = 0;                  // pieces so far
             bool ok = true;
@@ -248,27 +256,24 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc32_kernel(const AttnArgs a
                 ok = mbar_wait(bar(B_QFULL), pc & 1, ctl, a.status);
                 if (!ok) break;
                 for (int j = 0; j < nsteps; ++j, ++g) {
-                    const int b = g & 1, slot = g % kKSlots;
-                    ok = mbar_wait(bar(B_SFREE0 + b), ((g >> 1) & 1) ^ 1, ctl, a.status);
+                    const int slot = g % kKSlots;
+                    ok = mbar_wait(bar(B_SFREE), (g & 1) ^ 1, ctl, a.status);
                     if (ok) ok = mbar_wait(bar(B_KFULL0 + slot), (g / kKSlots) & 1, ctl, a.status);
                     if (!ok) break;
                     tc_fence_after();
                     const uint64_t dk = desc_kmajor(base + kOffK + (uint32_t)slot * kKSlot);
-                    const uint32_t t_s = tmem + kColS + 128u * (uint32_t)b;
 #pragma unroll
                     for (int kk = 0; kk < 8; ++kk) {          // 16 elements of d per MMA: Q_hi [K_hi; K_lo]^T, 128 columns
-                        const uint64_t qo = (uint64_t)(((kk >> 2) * kQPanel + (kk & 3) * 32) >> 4);
                         const uint64_t ko = (uint64_t)(((kk >> 2) * kKOperand + (kk & 3) * 32) >> 4);
-                        if (leader) tc_mma(t_s, dqh + qo, dk + ko, kIdescQK128, kk > 0);
+                        if (leader) tc_mma_ts(t_s, q_hi + kk * 8, dk + ko, kIdescQK128, kk > 0);
                     }
 #pragma unroll
                     for (int kk = 0; kk < 8; ++kk) {          // Q_lo K_hi^T onto columns 0-63
-                        const uint64_t qo = (uint64_t)(((kk >> 2) * kQPanel + (kk & 3) * 32) >> 4);
                         const uint64_t ko = (uint64_t)(((kk >> 2) * kKOperand + (kk & 3) * 32) >> 4);
-                        if (leader) tc_mma(t_s, dql + qo, dk + ko, kIdescQK64, 1);
+                        if (leader) tc_mma_ts(t_s, q_lo + kk * 8, dk + ko, kIdescQK64, 1);
                     }
                     if (!leader) continue;
-                    tc_commit(bar(B_SFULL0 + b));
+                    tc_commit(bar(B_SFULL));
                     if (kPair) tc_commit_pair(bar(B_KEMPTY0 + slot));     // the partner's converters write my slot too
                     else tc_commit(bar(B_KEMPTY0 + slot));
                 }
@@ -281,7 +286,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc32_kernel(const AttnArgs a
                 tc_commit(bar(B_DRAIN0));
                 mbar_wait_drain(bar(B_DRAIN0), 0, a.status);
             }
-        } else if (warp == 13) {
+        } else if (warp == 17) {
             // ------------------------------------------------------------------ issuer of the output MMAs
             int g = 0;                   // steps so far, all pieces = load number of the V ring
             bool ok = true;
@@ -310,6 +315,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc32_kernel(const AttnArgs a
                         if (leader) tc_mma_ts(t_o, p_hi + kk * 8, dvh + (uint64_t)((kk * 2048) >> 4), kIdescPV, 1);
                     if (!leader) continue;
                     tc_commit(bar(B_OFULL));
+                    tc_commit(bar(B_PFREE0 + b));
                     if (kPair) tc_commit_pair(bar(B_VEMPTY0 + slot));
                     else tc_commit(bar(B_VEMPTY0 + slot));
                 }
@@ -319,58 +325,38 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc32_kernel(const AttnArgs a
                 mbar_wait_drain(bar(B_DRAIN0 + 1), 0, a.status);
             }
         }
-    } else if (warp >= 4) {
+    } else if (warp >= 8) {
         // ------------------------------------------------------------------ converters: fp32 rows -> fp16 hi / lo tiles
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 104;");
-        const bool is_v = warp >= 8;
-        const int w4 = (warp - 4) & 3;                       // warp within its converter group
-        const int w8 = warp - 4;                             // warp among all converters (Q tile)
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
+        const bool is_v = warp >= 12;
+        const int w4 = warp & 3;                             // warp within its converter group
         const float *plane = reinterpret_cast<const float *>(is_v ? a.v_plane : a.k_plane);
-        const float *q_rot = reinterpret_cast<const float *>(a.q_rot);
         const int nslots = is_v ? kVSlots : kKSlots;
         const uint32_t ring = is_v ? kOffV : kOffK;
         uint8_t *smem = smem_raw + (base - smem_u32(smem_raw));        // the 1024-byte aligned tile area
         const int b_full = is_v ? B_VFULL0 : B_KFULL0, b_empty = is_v ? B_VEMPTY0 : B_KEMPTY0;
-        int lc = 0, pc = 0;                                  // ring loads and pieces so far
+        int lc = 0;                                          // ring loads so far
         bool ok = true;
         int kt0, ntiles, nsteps;
         for (int kvh = kvh_first; ok && piece(kvh, kt0, ntiles, nsteps); ++kvh) {
             if (nsteps <= 0) continue;
-            {
-                // the piece's Q tile: 16 rows per converter warp, row = token * G + head-in-group
-                float4 x[16];
-#pragma unroll
-                for (int i = 0; i < 16; ++i) {
-                    const int R = row0 + w8 * 16 + i, tok = R / G, gi = R % G;
-                    x[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-                    if (tok < n && gi < Gq) x[i] = *reinterpret_cast<const float4 *>(q_rot + ((int64_t)tok * a.H + kvh * Gq + gi) * kD + lane * 4);
-                }
-                if (pc > 0) ok = mbar_wait(bar(B_QEMPTY), (pc - 1) & 1, ctl, a.status);
-                ok = __all_sync(0xffffffffu, ok);
-                if (!ok) break;
-#pragma unroll
-                for (int i = 0; i < 16; ++i) {
-                    store_split4(smem + kOffQ, smem + kOffQ + kQPart, kQPanel, w8 * 16 + i, lane, x[i]);
-                }
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the MMAs read through the async proxy
-                __syncwarp();
-                if (lane == 0) mbar_arrive(bar(B_QFULL));
-                ++pc;
-            }
             const float *head = plane + (int64_t)kvh * a.capacity * kD;
             // rows of a step this warp converts: 16 of the 64, or 8 of this CTA's 32 in the paired variant
-            constexpr int NR = kPair ? 8 : 16;
+            constexpr int NR = 8, rows = kPair ? 8 : 16;         // (eight rows in flight: registers)
             const int r0 = kPair ? (int)rank * 32 + w4 * 8 : w4 * 16;
             for (int s = 0; s < nsteps; ++s, ++lc) {
                 const int64_t key0 = step_key0(kt0, s);
                 // rows past the end of the cache are not content (and may hold anything): they count as zero
                 float4 x[NR];
+                auto fetch = [&](int i0) {
 #pragma unroll
-                for (int i = 0; i < NR; ++i) {
-                    const int64_t key = key0 + r0 + i;
-                    x[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-                    if (key < L) x[i] = *reinterpret_cast<const float4 *>(head + key * kD + lane * 4);
-                }
+                    for (int i = 0; i < NR; ++i) {
+                        const int64_t key = key0 + r0 + i0 + i;
+                        x[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+                        if (key < L) x[i] = *reinterpret_cast<const float4 *>(head + key * kD + lane * 4);
+                    }
+                };
+                fetch(0);
                 const int slot = lc % nslots;
                 ok = mbar_wait(bar(b_empty + slot), ((lc / nslots) & 1) ^ 1, ctl, a.status);
                 ok = __all_sync(0xffffffffu, ok);
@@ -380,7 +366,11 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc32_kernel(const AttnArgs a
                 uint8_t *dst_lo = dst + (is_v ? kKPart : kKPanel);
                 const uint32_t panel = is_v ? kKPanel : kKOperand;
 #pragma unroll
-                for (int i = 0; i < NR; ++i) store_split4(dst, dst_lo, panel, r0 + i, lane, x[i]);
+                for (int i0 = 0; i0 < rows; i0 += NR) {
+                    if (i0 > 0) fetch(i0);
+#pragma unroll
+                    for (int i = 0; i < NR; ++i) store_split4(dst, dst_lo, panel, r0 + i0 + i, lane, x[i]);
+                }
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the MMAs (and the copies below) read through the async proxy
                 __syncwarp();
                 if (lane == 0) {
@@ -406,21 +396,20 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc32_kernel(const AttnArgs a
                 }
             }
         }
-    } else {
-        // ------------------------------------------------------------------ softmax and output rows, one thread per row
-        asm volatile("setmaxnreg.inc.sync.aligned.u32 248;");
-        const int r = warp * 32 + lane;                  // row of the CTA = TMEM lane
-        const uint32_t lane_addr = (uint32_t)(warp * 32) << 16;
+    } else if (warp >= 4) {
+        // ------------------------------------------------------------------ output rows, one thread per row
+        // The running output row, unnormalised, in round-to-nearest fp32: o = o * alpha + (P V of the step), alpha the factor by
+        // which the softmax moved the row's reference at that step.  What the softmax has to say about a row comes through
+        // shared memory, a float per row: alpha of step g in slot g % 3, and behind a piece's last step its sum and
+        // reference in the other two.
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 168;");
+        const int r = (warp & 3) * 32 + lane;            // row of the CTA = TMEM lane
         const int R = row0 + r, tok = R / G, gi = R % G;
-        const bool valid = tok < n && gi < Gq;       // (gi >= Gq: padding of a group that is no power of two)
-        // keys below `limit` are visible; a row past the chunk's end is never written, and each
-        // row of S, P and O depends on that row alone, so such rows are left unmasked
-        const int64_t limit = valid ? P + (tok + 1) * a.self_rows : ((int64_t)1 << 62);
-        const float sl2 = a.scale_log2;
+        const bool valid = tok < n && gi < Gq;
         const int64_t nG = (int64_t)n * G;
-        const uint32_t t_o = tmem + lane_addr + kColO;
-
-        int g = 0;                     // steps so far, all pieces
+        const uint32_t t_o = tmem + ((uint32_t)((warp & 3) * 32) << 16) + kColO;
+        const float *row_slot = reinterpret_cast<const float *>(smem_raw + (base - smem_u32(smem_raw)) + kOffRow) + r;
+        int g = 0, pc = 0;             // steps and pieces so far
         bool ok = true;
         int kt0, ntiles, nsteps;
         for (int kvh = kvh_first; ok && piece(kvh, kt0, ntiles, nsteps); ++kvh) {
@@ -435,21 +424,26 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc32_kernel(const AttnArgs a
                 }
                 continue;
             }
-            float m_ref = -INFINITY;   // reference maximum (raw score units) the probabilities are scaled by
-            float l = 0.f;
-            float o[kD];               // the running output row, unnormalised, in round-to-nearest fp32
+            float o[kD];
 #pragma unroll
             for (int c = 0; c < kD; ++c) o[c] = 0.f;
-            float alpha = 1.f;         // factor the reference moved by at the current step: owed to the P V of the step before
-
-            // adds the finished P V of the step before (computed under the old reference) and applies alpha
-            auto add_pv = [&](float scale) -> bool {
-                bool got = mbar_wait(bar(B_OFULL), (g - 1) & 1, ctl, a.status);
-                got = __all_sync(0xffffffffu, got);
-                if (!got) return false;
+            float l = 0.f, m_ref = 0.f;
+            for (int j = 0; j < nsteps; ++j, ++g) {
+                // (the probabilities' barrier as well: alpha was written ahead of them)
+                ok = mbar_wait(bar(B_PFULL0 + (g & 1)), (g >> 1) & 1, ctl, a.status) && mbar_wait(bar(B_OFULL), g & 1, ctl, a.status);
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) break;
                 tc_fence_after();
-                const bool rescale = __any_sync(0xffffffffu, scale != 1.f);      // rare: the reference moved at this step
-                const float2 sv = make_float2(scale, scale);
+                const float alpha = j > 0 ? row_slot[g % kRowSlots * kRows] : 1.f;
+                if (__any_sync(0xffffffffu, alpha != 1.f)) {          // rare: the reference moved at this step
+                    const float2 av = make_float2(alpha, alpha);
+#pragma unroll
+                    for (int c = 0; c < kD; c += 2) {
+                        const float2 v = __fmul2_rn(make_float2(o[c], o[c + 1]), av);
+                        o[c] = v.x;
+                        o[c + 1] = v.y;
+                    }
+                }
 #pragma unroll
                 for (int c0 = 0; c0 < kD; c0 += 32) {
                     uint32_t t[32];
@@ -457,34 +451,107 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc32_kernel(const AttnArgs a
                     tmem_wait_ld();
 #pragma unroll
                     for (int c = 0; c < 32; c += 2) {
-                        float2 v = __fadd2_rn(make_float2(o[c0 + c], o[c0 + c + 1]), make_float2(__uint_as_float(t[c]), __uint_as_float(t[c + 1])));
-                        if (rescale) v = __fmul2_rn(v, sv);
+                        const float2 v = __fadd2_rn(make_float2(o[c0 + c], o[c0 + c + 1]), make_float2(__uint_as_float(t[c]), __uint_as_float(t[c + 1])));
                         o[c0 + c] = v.x;
                         o[c0 + c + 1] = v.y;
                     }
                 }
+                if (j == nsteps - 1) {
+                    // (ahead of this step's arrival: the next piece's softmax writes the slots once that has come)
+                    ok = mbar_wait(bar(B_ROWDONE), pc & 1, ctl, a.status);
+                    ok = __all_sync(0xffffffffu, ok);
+                    if (!ok) break;
+                    l = row_slot[(g + 1) % kRowSlots * kRows];
+                    m_ref = row_slot[(g + 2) % kRowSlots * kRows];
+                }
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(bar(B_OFREE));
-                return true;
-            };
+            }
+            if (!ok) break;
+            ++pc;
+            const float inv = l > 0.f ? 1.f / l : 0.f;
+            const float lse2 = l > 0.f ? m_ref * a.scale_log2 + log2f(l) : -INFINITY;
+            if (valid) {
+                const int64_t row = (int64_t)tok * a.H + kvh * Gq + gi;
+                float4 *dst = direct ? reinterpret_cast<float4 *>(reinterpret_cast<float *>(a.out) + row * kD)
+                                     : reinterpret_cast<float4 *>(a.part_o + prow * kD);
+#pragma unroll
+                for (int c = 0; c < kD / 4; ++c)
+                    dst[c] = make_float4(o[4 * c] * inv, o[4 * c + 1] * inv, o[4 * c + 2] * inv, o[4 * c + 3] * inv);
+                if (!direct) a.part_lse[prow] = lse2;
+                else if (a.lse) a.lse[row] = lse2 * 0.6931471805599453f;
+            }
+        }
+    } else {
+        // ------------------------------------------------------------------ softmax, one thread per row
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 128;");
+        const int r = warp * 32 + lane;                  // row of the CTA = TMEM lane
+        const uint32_t lane_addr = (uint32_t)(warp * 32) << 16;
+        const int R = row0 + r, tok = R / G, gi = R % G;
+        const bool valid = tok < n && gi < Gq;       // (gi >= Gq: padding of a group that is no power of two)
+        // keys below `limit` are visible; a row past the chunk's end is never written, and each
+        // row of S, P and O depends on that row alone, so such rows are left unmasked
+        const int64_t limit = valid ? P + (tok + 1) * a.self_rows : ((int64_t)1 << 62);
+        const float sl2 = a.scale_log2;
+        float *row_slot = reinterpret_cast<float *>(smem_raw + (base - smem_u32(smem_raw)) + kOffRow) + r;
 
-            for (int j = 0; j < nsteps; ++j, ++g) {
-                const int b = g & 1;
-                const uint32_t t_s = tmem + lane_addr + kColS + 128u * (uint32_t)b;     // 64 scores, then their 64 small terms
-                const uint32_t t_p = tmem + lane_addr + kColP + 64u * (uint32_t)b;
-                ok = mbar_wait(bar(B_SFULL0 + b), (g >> 1) & 1, ctl, a.status);
+        int g = 0, pc = 0;             // steps and pieces so far
+        bool ok = true;
+        int kt0, ntiles, nsteps;
+        for (int kvh = kvh_first; ok && piece(kvh, kt0, ntiles, nsteps); ++kvh) {
+            if (nsteps <= 0) continue;
+            if (pc > 0) {
+                // the output warps have read what the piece before left in the rows' slots
+                ok = mbar_wait(bar(B_OFREE), (g - 1) & 1, ctl, a.status);
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) break;
+            }
+            // the piece's query row, split into tensor memory, two elements to a column
+            if (pc > 0) {
+                ok = mbar_wait(bar(B_QEMPTY), (pc - 1) & 1, ctl, a.status);
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
                 tc_fence_after();
+            }
+            const float4 *q_row = reinterpret_cast<const float4 *>(reinterpret_cast<const float *>(a.q_rot) + ((int64_t)tok * a.H + kvh * Gq + gi) * kD);
+#pragma unroll
+            for (int c0 = 0; c0 < kD / 4; c0 += 16) {
+                uint32_t hi[32], lo[32];
+#pragma unroll
+                for (int c = 0; c < 16; ++c) {
+                    const float4 x = valid ? q_row[c0 + c] : make_float4(0.f, 0.f, 0.f, 0.f);
+                    split2(x.x, x.y, hi[2 * c], lo[2 * c]);
+                    split2(x.z, x.w, hi[2 * c + 1], lo[2 * c + 1]);
+                }
+                KVF_TMEM_ST32(hi, 0, tmem + lane_addr + kColQ + 2 * c0);
+                KVF_TMEM_ST32(lo, 0, tmem + lane_addr + kColQ + 64 + 2 * c0);
+            }
+            tmem_wait_st();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar(B_QFULL));
+            float m_ref = -INFINITY;   // reference maximum (raw score units) the probabilities are scaled by
+            float l = 0.f;
+            for (int j = 0; j < nsteps; ++j, ++g) {
+                const int b = g & 1;
+                const uint32_t t_s = tmem + lane_addr + kColS;                          // 64 scores, then their 64 small terms
+                const uint32_t t_p = tmem + lane_addr + kColP + 64u * (uint32_t)b;
+                // (what needs no scores comes ahead of the wait for them: this thread's chain is what the kernel waits for)
                 const int64_t key0 = step_key0(kt0, j);
                 const int nvis = (int)max((int64_t)0, min((int64_t)kKeys, limit - key0));
                 // a step that starts before the window holds hidden columns (the sink tile, the window's first)
                 const bool masked = __any_sync(0xffffffffu, nvis < kKeys) || (kWindow && key0 < a.win_lo);
                 const int lo_c = kWindow ? (int)max((int64_t)0, min((int64_t)kKeys, a.win_lo - key0)) : 0;
                 const int sink_c = kWindow ? (int)max((int64_t)0, min((int64_t)kKeys, (int64_t)a.n_sink - key0)) : 0;
+                ok = mbar_wait(bar(B_SFULL), g & 1, ctl, a.status);
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) break;
+                tc_fence_after();
+                // (the P V that read this buffer two steps ago: asked ahead of the arithmetic, every phase is waited for)
+                uint32_t buffer_free = 1;
+                if (g > 1) buffer_free = mbar_test(bar(B_PFREE0 + b), ((g >> 1) - 1) & 1);
 
-                // first reading of the scores: the row maximum
                 // the step's 64 scores (columns c and 64 + c added up) into registers, and the row maximum
                 float v[64];
 #pragma unroll
@@ -504,7 +571,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc32_kernel(const AttnArgs a
                 // the scores are in registers: the issuer may overwrite them with the step after next
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(bar(B_SFREE0 + b));
+                if (lane == 0) mbar_arrive(bar(B_SFREE));
                 if (masked) {
 #pragma unroll
                     for (int c = 0; c < 64; ++c) v[c] = (c < nvis && (c >= lo_c || c < sink_c)) ? v[c] : -INFINITY;
@@ -520,7 +587,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc32_kernel(const AttnArgs a
                 // move the reference only when the maximum grew by more than the threshold: the
                 // probabilities then stay below 2^threshold and the output row is rarely rescaled
                 const bool grow = (m_tile - m_ref) * sl2 > kRescaleThreshold;   // also true when m_ref = -inf < m_tile
-                alpha = 1.f;
+                float alpha = 1.f;
                 if (grow) {
                     alpha = ex2((m_ref - m_tile) * sl2);                         // m_ref = -inf -> 0
                     l *= alpha;
@@ -529,57 +596,52 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc32_kernel(const AttnArgs a
                 const float m_safe = m_ref == -INFINITY ? 0.f : m_ref;
                 const float neg = -m_safe * sl2;
 
+                if (!__all_sync(0xffffffffu, buffer_free)) {
+                    ok = mbar_wait(bar(B_PFREE0 + b), ((g >> 1) - 1) & 1, ctl, a.status);
+                    ok = __all_sync(0xffffffffu, ok);
+                    if (!ok) break;
+                }
+                tc_fence_after();
+                // (that P V was issued once the output warps had added the one before: they have read this slot's alpha)
+                if (j > 0) row_slot[g % kRowSlots * kRows] = alpha;
                 // probabilities, split into fp16 hi / lo, written 16 keys at a time
                 float2 acc = make_float2(0.f, 0.f);
                 const float2 sl2v = make_float2(sl2, sl2), negv = make_float2(neg, neg);
 #pragma unroll
-                for (int h = 0; h < 4; ++h) {
-                    uint32_t ph[8], pl[8];
+                for (int h = 0; h < 2; ++h) {
+                    uint32_t ph[16], pl[16];
 #pragma unroll
-                    for (int c = 0; c < 8; ++c) {
-                        const float2 x = __ffma2_rn(make_float2(v[16 * h + 2 * c], v[16 * h + 2 * c + 1]), sl2v, negv);
+                    for (int c = 0; c < 16; ++c) {
+                        const float2 x = __ffma2_rn(make_float2(v[32 * h + 2 * c], v[32 * h + 2 * c + 1]), sl2v, negv);
                         float2 e;
                         e.x = ex2(x.x);
                         e.y = ex2(x.y);
                         acc = __fadd2_rn(acc, e);
                         const __half2 hh = __floats2half2_rn(e.x, e.y);
                         const float2 back = __half22float2(hh);
-                        const float2 rest = __fadd2_rn(e, make_float2(-back.x, -back.y));
+                        const float2 rest = __ffma2_rn(back, make_float2(-1.f, -1.f), e);        // e - back
                         ph[c] = half2_bits(hh);
                         pl[c] = half2_bits(__floats2half2_rn(rest.x, rest.y));
                     }
-                    KVF_TMEM_ST8(ph, 0, t_p + 8 * h);
-                    KVF_TMEM_ST8(pl, 0, t_p + 32 + 8 * h);
+                    KVF_TMEM_ST16(ph, 0, t_p + 16 * h);
+                    KVF_TMEM_ST16(pl, 0, t_p + 32 + 16 * h);
                 }
                 l += acc.x + acc.y;
                 tmem_wait_st();
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(bar(B_PFULL0 + b));
-
-                // the P V of the step before has had this step's softmax to finish in
-                if (j > 0) {                  // (first step of a piece: nothing accumulated yet, o is zero)
-                    ok = add_pv(alpha);
-                    if (!ok) break;
-                }
             }
             if (!ok) break;
-            // the last step's P V (g was advanced past it)
-            ok = add_pv(1.f);
+            // The last P V has run: the output warps have added the one before, and read the slots up to its step.
+            ok = mbar_wait(bar(B_PFREE0 + ((g - 1) & 1)), ((g - 1) >> 1) & 1, ctl, a.status);
+            ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
-
-            const float inv = l > 0.f ? 1.f / l : 0.f;
-            const float lse2 = l > 0.f ? m_ref * sl2 + log2f(l) : -INFINITY;
-            if (valid) {
-                const int64_t row = (int64_t)tok * a.H + kvh * Gq + gi;
-                float4 *dst = direct ? reinterpret_cast<float4 *>(reinterpret_cast<float *>(a.out) + row * kD)
-                                     : reinterpret_cast<float4 *>(a.part_o + prow * kD);
-#pragma unroll
-                for (int c = 0; c < kD / 4; ++c)
-                    dst[c] = make_float4(o[4 * c] * inv, o[4 * c + 1] * inv, o[4 * c + 2] * inv, o[4 * c + 3] * inv);
-                if (!direct) a.part_lse[prow] = lse2;
-                else if (a.lse) a.lse[row] = lse2 * 0.6931471805599453f;
-            }
+            row_slot[g % kRowSlots * kRows] = l;
+            row_slot[(g + 1) % kRowSlots * kRows] = m_ref;
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar(B_ROWDONE));
+            ++pc;
         }
     }
 
@@ -587,7 +649,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc32_kernel(const AttnArgs a
     __syncthreads();
     // (paired variant: neither CTA leaves while the partner may still send tiles or commits its way)
     if (kPair) cluster_sync_all();
-    if (warp == 12) {
+    if (warp == 16) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
     }
