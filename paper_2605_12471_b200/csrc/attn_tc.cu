@@ -881,10 +881,10 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
                 const uint32_t stage = base + offP + (uint32_t)warp * 4096u;
                 const int R1 = row0 + i * kRows + (warp & 3) * 32 + (lane >> 3), lg = __ffs(G) - 1;      // first of the rows I write out
                 // (partial rows lie one after the other; G is a power of two: with a divide per row and line the
-                // index arithmetic took as long as the stores.  The pointers cost bf16 rows 16 - 20 bytes of spills, 60 - 68 of
-                // loads, pairs of CTAs 168 and 280 with those of their registers; without them - one base and row pitch for both
-                // kinds of rows, denominators written first - 128 steps under a window 2991 -> 3015 us, 65 536 tokens of int8 in 256s
-                // 42.2 -> 42.9 ms)
+                // index arithmetic took as long as the stores.  The loops over the columns are not unrolled: the code runs
+                // once or twice a launch, steps of 256 - 512 tokens behind short prefixes take 1 - 2 % less, others the same, and bf16
+                // rows no longer spill.  Pairs of CTAs spill 108 bytes; one base and row pitch for both kinds of rows instead of
+                // two pointers: 65 536 tokens of int8 in 256s 42.2 -> 42.9 ms)
                 char *part = reinterpret_cast<char *>(a.part_o + (prow - R + R1) * kD) + (lane & 7) * 16;
                 char *fin = reinterpret_cast<char *>(a.out) + (lane & 7) * 16;
                 const int fin_row = kD * (a.out_f32 ? 4 : 2);
@@ -908,7 +908,7 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
                     }
                 };
                 if (!direct || a.out_f32) {
-#pragma unroll
+#pragma unroll 1
                     for (int c0 = 0; c0 < 128; c0 += 32) {
                         uint32_t w[32];
                         KVF_TMEM_LD32(w, 0, t_o + c0);
@@ -918,7 +918,7 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
                         emit(w, c0 * 4);
                     }
                 } else {
-#pragma unroll
+#pragma unroll 1
                     for (int c0 = 0; c0 < 128; c0 += 64) {
                         uint32_t o[64], w[32];
                         KVF_TMEM_LD32(o, 0, t_o + c0);
