@@ -340,7 +340,8 @@ float *kvf_cache_v_scales(const kvf_cache *c);
  *   plan[1] parts the key range of one KV head is cut into (1 = none).  CUDA-core kernel: equal
  *           splits.  Tensor-core kernel: the (KV head, key tile) pairs are cut into plan[2] /
  *           (row blocks: 256-row pairs in bf16, 128-row blocks in fp32) contiguous ranges that
- *           need not end at KV-head boundaries; this is their number per KV head, rounded up
+ *           need not end at KV-head boundaries; this is their number per KV head, rounded up.  Small
+ *           bf16 steps under a window: streams of key tiles of a 128-row tile (two to a CTA)
  *   plan[2] CTAs of the attention kernel
  *   plan[3] kernels launched by the step (3 = a combine kernel merges partial results; chunks of
  *           at most 128 / (H / Hkv) tokens always take that route on the tensor-core path; 1 = a small

@@ -70,6 +70,12 @@
 // with its own accumulator, K/V ring of three slots and partial result, so the overlap of one
 // stream's softmax with the other's MMAs survives and the step runs at HBM speed.
 //
+// Small steps under a window (kRanks).  Their key tiles are few, and what a step waited for were 128 KiB of partial results per CTA
+// (3.3 us), a third launch and its hand-overs.  Here a CTA has one row tile, its key tiles in two streams, the two accumulators
+// are merged in the CTA (both lie in the tensor-memory lanes of the same rows) and those of a cluster's CTAs by stores into each
+// other's shared memory.  Steps of 256 tokens under a window of 1020 22.8 -> 19.6 us, of 64 tokens 21.4 -> 14.7
+// (attn_tc_row_ranks has more); 128 steps of 256 tokens 2922 -> 2534 us.
+//
 // Every wait on an mbarrier is bounded (about one second): on expiry the thread raises the
 // CTA's abort flag and records the wait in the device status word, all roles leave their loops,
 // copies and MMAs still in flight are waited for (bounded again), tensor memory is released and
@@ -131,6 +137,7 @@ constexpr int kRingBars = 6;                  // 2 x 3 slots of the per-stream r
 enum { B_QFULL = 0, B_QEMPTY = 1, B_FULL0 = 2, B_EMPTY0 = B_FULL0 + kRingBars, B_SFULL0 = B_EMPTY0 + kRingBars,
        B_PA0 = B_SFULL0 + 2, B_PB0 = B_PA0 + 2, B_PVDONE0 = B_PB0 + 2, B_TURN0 = B_PVDONE0 + 2,
        B_DRAIN0 = B_TURN0 + 8, B_RAWFULL0 = B_DRAIN0 + 2, B_RAWEMPTY0 = B_RAWFULL0 + kRawSlotsPair,
+       B_READY = B_RAWFULL0, B_LANDED = B_RAWFULL0 + 1,       // (kRanks; the raw ring is quantised storage's)
        B_COUNT = B_RAWEMPTY0 + kRawSlotsPair };
 
 struct Ctl {
@@ -213,7 +220,9 @@ __device__ __forceinline__ void exp_half(const uint32_t *v, uint32_t *p, float2 
 // when every row pair has two row tiles (a chunk of a multiple of 512 / G tokens).
 // kEarly (bf16 rows, chunks of two row tiles): Q K^T of the next key tile is issued under the softmax of the
 // current one, see the issuer.
-template <bool kWindow, int kQuant, bool kPair, bool kEarly>
+// kRanks (bf16 rows, two streams): a cluster of that many CTAs has one row tile of one KV head, each an equal share of its key
+// tiles, and writes the output: no partial results, no merge kernel.  See the end of the kernel.
+template <bool kWindow, int kQuant, bool kPair, bool kEarly, int kRanks = 0>
 __global__ void __launch_bounds__(kQuant ? kThreadsQ8 : kThreads, 1)
 attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                const __grid_constant__ CUtensorMap map_v) {
@@ -236,10 +245,11 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
     // Ranges first, row pairs from the last to the first: the row pairs that see most keys start first and the shortest
     // fill the tail.  Both in x, which has no limit a chunk could reach (y ends at 65 535: 262 140 tokens of 64 query heads
     // per KV head).  (kPair: clusters along x, so x = row pair, y = range.)
+    // (kRanks: row tiles in the place of row pairs; a KV head's ranges are its cluster)
     const int pairs = kPair ? (int)gridDim.x : (int)gridDim.x / a.ngroups;
     const int qpair = kPair ? (int)blockIdx.x : pairs - 1 - (int)blockIdx.x / a.ngroups;
     const int group = kPair ? (int)blockIdx.y : (int)blockIdx.x % a.ngroups;
-    const uint32_t rank = kPair ? cluster_cta_rank() : 0u;     // which half of a tile's key rows this CTA expands
+    const uint32_t rank = kPair || kRanks > 1 ? cluster_cta_rank() : 0u;     // which half of a tile's key rows this CTA expands; which range it takes
     const int cb = blockIdx.z;     // cache of a batch (0 when there is one cache)
     const int G = a.Gp;     // rows per token in the row layout (a power of two >= a.G, the query heads per KV head)
     // (a ragged batch keeps its members' row counts in device memory, written by an earlier kernel
@@ -247,7 +257,8 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
     if (a.prefixes) pdl_wait();
     // tokens this cache folds; a.n is the longest chunk of the launch and the stride of the caches' blocks
     const int n = a.ns ? (int)a.ns[cb] : a.n, nmax = a.n;
-    if (qpair * 2 * kRows >= n * G) return;          // a shorter member of a batch: no row of this row pair exists
+    constexpr int kCtaRows = kRanks ? kRows : 2 * kRows;
+    if (qpair * kCtaRows >= n * G) return;           // a shorter member of a batch: no row of this row pair exists
     const int64_t P = a.prefixes ? a.prefixes[cb] : a.prefix, L = P + n * a.self_rows;
     // streams == 2 (chunks of at most 128 / G tokens, i.e. one row tile): the two tile slots work on
     // the SAME 128 rows and take alternate key tiles, so that one stream's softmax still runs under
@@ -258,13 +269,13 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
 
     // key tiles: this row pair needs tiles below nt_need; the group's share of the
     // (KV head, tile) line is [lin0, lin1)
-    const int row0 = qpair * 2 * kRows;
+    const int row0 = qpair * kCtaRows;
     // short chunks (at most 128 / G tokens in this row pair) leave the second row tile without a
     // valid row: its issuer and softmax warps then sit the kernel out
     const int tiles = (streams == 2 || row0 + kRows < n * G) ? 2 : 1;
     // (paired variant: both CTAs of a cluster walk the key tiles the later row pair needs; the earlier one
     // finds nothing visible in the last of them, and its rows' limits mask that tile out)
-    const int tok_last = min(n - 1, ((kPair ? (qpair | 1) * 2 * kRows : row0) + 2 * kRows - 1) / G);
+    const int tok_last = min(n - 1, ((kPair ? (qpair | 1) * 2 * kRows : row0) + kCtaRows - 1) / G);
     // (virtual key tiles: without a window they are the key tiles themselves)
     const WindowTiles wt(kWindow ? a.win_lo : 0, kWindow ? a.n_sink : 0, kRows);
     const int nt_need = (int)((P + (tok_last + 1) * a.self_rows + kRows - 1) / kRows) - wt.skip;
@@ -274,9 +285,14 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
     const int pcost = a.piece_cost, ntv = nt_all + pcost;
     const int64_t line = (int64_t)a.Hkv * ntv;
     const int64_t lin0 = group * line / a.ngroups, lin1 = (group + 1) * line / a.ngroups;
-    const int kvh_first = (int)(lin0 / ntv);
+    const int kvh_first = kRanks ? group / kRanks : (int)(lin0 / ntv);
     // piece k of this CTA: KV head kvh_first + k, tiles [kt0, kt0 + ntiles)
     auto piece = [&](int kvh, int &kt0, int &ntiles) -> bool {
+        if (kRanks) {
+            kt0 = (int)rank * nt_need / (kRanks ? kRanks : 1);
+            ntiles = ((int)rank + 1) * nt_need / (kRanks ? kRanks : 1) - kt0;
+            return kvh == kvh_first;
+        }
         const int64_t b = (int64_t)kvh * ntv;
         if (kvh >= a.Hkv || b >= lin1) return false;
         kt0 = max((int)(max(lin0, b) - b) - pcost, 0);
@@ -289,6 +305,10 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
         mbar_init(bar(B_QFULL), 1);
         mbar_init(bar(B_QEMPTY), tiles);                                  // both issuers read Q
         for (int s = 0; s < kRingBars; ++s) { mbar_init(bar(B_FULL0 + s), kQuant ? 4 : 1); mbar_init(bar(B_EMPTY0 + s), kPair ? 2 * tiles : streams == 2 ? 1 : tiles); }   // consumers of a K/V tile
+        if (kRanks > 1) {
+            mbar_init(bar(B_READY), kRanks - 1);
+            mbar_init(bar(B_LANDED), 1);
+        }
         if (kQuant)
             for (int s = 0; s < rawSlots; ++s) { mbar_init(bar(B_RAWFULL0 + s), 1); mbar_init(bar(B_RAWEMPTY0 + s), 4); }
         for (int i = 0; i < 2; ++i) {
@@ -310,7 +330,7 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
     pdl_launch_dependents();
     tc_fence_before();
     __syncthreads();
-    if (kPair) cluster_sync_all();      // the partner's barriers exist before anything is sent to them
+    if (kPair || kRanks > 1) cluster_sync_all();      // the partners' barriers exist before anything is sent to them
     tc_fence_after();
     pdl_wait();   // nothing above reads what an earlier kernel wrote; from here on the rotated chunk is read
     const uint32_t tmem = *reinterpret_cast<volatile uint32_t *>(&ctl->tmem_base);
@@ -723,9 +743,14 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
                 turn_base += nturns;
                 return true;
             };
+            // (kRanks) log2 reference and sum of my stream's row, where its first K/V slot was
+            auto leave_stats = [&](float m, float sum) {
+                asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(slot_addr(i * SR) + (uint32_t)r * 8u), "f"(m), "f"(sum) : "memory");
+            };
             if (ntiles <= j0) {
+                if (kRanks) leave_stats(-INFINITY, 0.f);
                 // no visible key for these rows in this range: an empty partial
-                if (!direct && valid) {
+                if (!kRanks && !direct && valid) {
                     float4 *po = reinterpret_cast<float4 *>(a.part_o + prow * kD);
 #pragma unroll 4
                     for (int c = 0; c < kD / 4; ++c) po[c] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -869,6 +894,10 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
             if (!ok) break;
             ++oc;
             tc_fence_after();
+            if (kRanks) {
+                leave_stats(m_ref == -INFINITY ? m_ref : m_ref * sl2, l);
+                continue;
+            }
             if (!warp_live) continue;
             const float inv = l > 0.f ? 1.f / l : 0.f;
             const float lse2 = l > 0.f ? m_ref * sl2 + log2f(l) : -INFINITY;
@@ -977,6 +1006,128 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
     __syncthreads();
     // (paired variant: neither CTA leaves while the partner may still send tiles or commits its way)
     if (kPair) cluster_sync_all();
+    if constexpr (kRanks > 0) {
+        // The two streams' results of a row are merged here, and those of the cluster's CTAs with them.  Thread (stream i, row r)
+        // takes columns 64 i .. + 63 of the row from both accumulators (a warp reaches its quarter of the lanes in either); of those each
+        // CTA finishes its share, 64 / kRanks, and sends the others theirs: into their K/V slots, once they have said that nothing
+        // uses those any more.  (Stores that complete on the receiver's barrier: with the values left in place, a cluster barrier
+        // ahead of the partner's loads and one behind them, this took 6 us.)
+        constexpr int W = 64 / kRanks;
+        constexpr uint32_t kFromRank = 2u * kRows * W * 4u;              // what a CTA sends another: its columns of 2 x 128 half rows ...
+        const uint32_t landing = base + kOffKV + kTileBytes, land_stats = base + kOffKV + 4096u;     // ... and a float2 per row, by sender
+        if (kRanks > 1 && threadIdx.x == 0) {
+            mbar_expect_tx(bar(B_LANDED), (kRanks - 1) * (kFromRank + kRows * 8u));
+            for (uint32_t s = 0; s < kRanks; ++s)
+                if (s != rank) mbar_arrive_cluster(peer_smem(bar(B_READY), s));
+        }
+        if (warp < 8) {
+            tc_fence_after();
+            const int lg = __ffs(G) - 1;                                 // (G is a power of two)
+            const int i = warp >> 2, r = (warp & 3) * 32 + lane, R = row0 + r, tok = R >> lg, gi = R & (G - 1), kvh = kvh_first;
+            float m[2], l[2];
+#pragma unroll
+            for (int s = 0; s < 2; ++s)
+                asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(m[s]), "=f"(l[s]) : "r"(slot_addr(s * SR) + (uint32_t)r * 8u) : "memory");
+            float M = fmaxf(m[0], m[1]);
+            const float M0 = M == -INFINITY ? 0.f : M, w0 = ex2(m[0] - M0), w1 = ex2(m[1] - M0);
+            float L = w0 * l[0] + w1 * l[1];
+            const bool seen0 = l[0] > 0.f, seen1 = l[1] > 0.f;           // (an accumulator that nothing was added to holds anything)
+            const uint32_t t_row = tmem + ((uint32_t)((warp & 3) * 32) << 16) + 256 + i * 64;
+            constexpr int C = W < 32 ? W : 32;                           // columns at a time
+            float v[C];
+            auto mix = [&](int c0) {                                     // C columns of my 64 from c0 on
+                uint32_t x[C], y[C];
+                if constexpr (C == 32) {
+                    KVF_TMEM_LD32(x, 0, t_row + c0);
+                    KVF_TMEM_LD32(y, 0, t_row + 128 + c0);
+                } else {
+                    KVF_TMEM_LD16(x, 0, t_row + c0);
+                    KVF_TMEM_LD16(y, 0, t_row + 128 + c0);
+                }
+                tmem_wait_ld();
+#pragma unroll
+                for (int c = 0; c < C; ++c) v[c] = (seen0 ? w0 * __uint_as_float(x[c]) : 0.f) + (seen1 ? w1 * __uint_as_float(y[c]) : 0.f);
+            };
+            // where column 4 q of a share lands: rows of W floats, their 16-byte pieces swizzled
+            auto place = [&](int from, int q) {
+                return landing + (uint32_t)from * kFromRank + (uint32_t)(i * kRows + r) * (W * 4u) + (uint32_t)((q ^ (r & (W / 4 - 1))) << 4);
+            };
+            float weight[kRanks];
+            weight[0] = 1.f;
+            bool ok = true;
+            if constexpr (kRanks > 1) {
+#pragma unroll 1
+                for (int t = 1; ok && t < kRanks; ++t) {
+                    const int s = ((int)rank + t) % kRanks;
+                    mix(s * W);
+                    if (t == 1) ok = mbar_wait(bar(B_READY), 0, ctl, a.status);
+                    ok = __all_sync(0xffffffffu, ok);
+                    if (!ok) break;
+                    const uint32_t landed = peer_smem(bar(B_LANDED), (uint32_t)s);
+#pragma unroll
+                    for (int c = 0; c < W; c += 4) peer_store4(peer_smem(place((int)rank, c >> 2), (uint32_t)s), make_float4(v[c], v[c + 1], v[c + 2], v[c + 3]), landed);
+                    if (i == 0) peer_store2(peer_smem(land_stats + ((uint32_t)rank * kRows + (uint32_t)r) * 8u, (uint32_t)s), make_float2(M, L), landed);
+                }
+            }
+#pragma unroll
+            for (int c0 = 0; c0 < W; c0 += C) {
+                mix((int)rank * W + c0);
+                if constexpr (kRanks > 1) {
+                    if (ok) ok = mbar_wait(bar(B_LANDED), 0, ctl, a.status);
+                    float2 st[kRanks];
+                    float most = M;
+#pragma unroll
+                    for (int s = 0; s < kRanks; ++s) {
+                        st[s] = make_float2(M, L);
+                        if (s != (int)rank)
+                            asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(st[s].x), "=f"(st[s].y) : "r"(land_stats + ((uint32_t)s * kRows + (uint32_t)r) * 8u) : "memory");
+                        most = fmaxf(most, st[s].x);
+                    }
+                    const float most0 = most == -INFINITY ? 0.f : most, mine = ex2(M - most0);
+                    L = 0.f;
+#pragma unroll
+                    for (int s = 0; s < kRanks; ++s) {
+                        weight[s] = ex2(st[s].x - most0);
+                        L += weight[s] * st[s].y;
+                    }
+                    M = most;
+#pragma unroll
+                    for (int c = 0; c < W; ++c) v[c] *= mine;
+#pragma unroll
+                    for (int s = 0; s < kRanks; ++s) {
+                        if (s == (int)rank) continue;
+#pragma unroll
+                        for (int c = 0; c < W; c += 4) {
+                            float4 o;
+                            asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(o.x), "=f"(o.y), "=f"(o.z), "=f"(o.w) : "r"(place(s, c >> 2)) : "memory");
+                            v[c] = fmaf(weight[s], o.x, v[c]); v[c + 1] = fmaf(weight[s], o.y, v[c + 1]);
+                            v[c + 2] = fmaf(weight[s], o.z, v[c + 2]); v[c + 3] = fmaf(weight[s], o.w, v[c + 3]);
+                        }
+                    }
+                }
+                if (tok >= n || gi >= a.G) continue;
+                // (a thread's 64 to 128 bytes of its row as they are: turned round in shared memory and written as whole pieces of rows
+                // by neighbouring threads, steps took 0.1 us less without a cluster, 0.4 us more with)
+                const float inv = L > 0.f ? 1.f / L : 0.f;
+                const int64_t row = ((int64_t)cb * nmax + tok) * a.H + kvh * a.G + gi, at = row * kD + i * 64 + (int)rank * W + c0;
+                if (a.out_f32) {
+#pragma unroll
+                    for (int c = 0; c < C; c += 4)
+                        *reinterpret_cast<float4 *>(reinterpret_cast<float *>(a.out) + at + c) =
+                            make_float4(v[c] * inv, v[c + 1] * inv, v[c + 2] * inv, v[c + 3] * inv);
+                } else {
+#pragma unroll
+                    for (int c = 0; c < C; c += 8)
+                        *reinterpret_cast<uint4 *>(reinterpret_cast<__nv_bfloat16 *>(a.out) + at + c) =
+                            make_uint4(pack_bf16(v[c] * inv, v[c + 1] * inv), pack_bf16(v[c + 2] * inv, v[c + 3] * inv),
+                                       pack_bf16(v[c + 4] * inv, v[c + 5] * inv), pack_bf16(v[c + 6] * inv, v[c + 7] * inv));
+                }
+                if (c0 == 0 && i == 0 && rank == 0 && a.lse) a.lse[row] = (L > 0.f ? M + log2f(L) : -INFINITY) * 0.6931471805599453f;
+            }
+        }
+        tc_fence_before();
+        __syncthreads();
+    }
     if (warp == 9) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
@@ -1244,6 +1395,53 @@ static bool pair_clusters_fit(const void *kernel, uint32_t smem) {
     return fit;
 }
 
+// Clusters of that many CTAs of one row tile that the device holds at once (queried once per device).
+template <int kRanks>
+static int ranks_at_once() {
+    static std::mutex mu;
+    static std::vector<std::pair<int, int>> seen;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+    std::lock_guard<std::mutex> lock(mu);
+    for (auto &d : seen)
+        if (d.first == dev) return d.second;
+    auto kernel = attn_tc_kernel<true, 0, false, false, kRanks>;
+    int clusters = 0;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(kRanks, 1, 1);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = kSmemBytes;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = kRanks; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (raise_smem_limit_once(reinterpret_cast<const void *>(kernel), (int)kSmemBytes) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&clusters, kernel, &cfg) != cudaSuccess) {
+        cudaGetLastError();
+        clusters = 0;
+    }
+    seen.push_back({dev, clusters});
+    return clusters;
+}
+
+// CTAs per row tile of a step under a window (units: row tiles of all KV heads).  us per step replayed in a graph, 256-row CTAs with
+// partial results and a merge kernel / one, two, four CTAs to a row tile (32 / 8 heads unless said otherwise):
+//   64 tokens, 16 units, 4 key tiles 19.7 / 15.4, 13.4, 12.9; 10 tiles 21.4 / 21.3, 16.6, 14.7; 33 tiles 25.4 / 44.6, 27.9, 20.7
+//   100 tokens, 32 units, 4 tiles 18.6 / 16.4, 13.9, 14.6; 10 tiles 21.0 / 22.2, 17.3, 15.9; 34 tiles 26.9 / 45.2, 28.5, 21.7
+//   256 tokens, 64 units, 5 tiles 19.8 / 17.5, 15.9; 11 tiles 22.8 / 23.4, 19.6; 35 tiles 32.1 / 47.3, 31.5; four: a second wave
+//   300 tokens of 28 / 4 heads, 76 units, 6 tiles 21.9 / 19.2; 12 tiles 25.4 / 24.7; 35 tiles 36.2 / 47.4; two: a second wave
+//   400 tokens, 104 units, 13 tiles 29.2 / 26.4; 20 tiles 34.9 / 34.0; 36 tiles 45.2 / 49.4
+//   512 tokens, 128 units, 13 tiles 30.8 / 27.2; 21 tiles 37.3 / 35.2; 37 tiles 49.4 / 51.2
+//   64 tokens of 16 / 16 heads, 16 units, 4 tiles 14.0 / 15.1, 13.1, 13.0; 33 tiles 21.7 / 43.7, 27.2, 20.6
+// So as many as the device holds at once, four only where the key tiles are more than two for each of two CTAs' streams; alone, a CTA
+// has all key tiles of 128 rows where a CTA of the other kind has a share of them for 256, and keeps ahead up to the line below.
+int attn_tc_row_ranks(int units, int sms, int64_t key_tiles) {
+    if (key_tiles > 8 && units <= ranks_at_once<4>()) return 4;
+    if (units <= ranks_at_once<2>()) return 2;
+    return units <= sms && key_tiles <= 46 * (int64_t)units / sms - 10 ? 1 : 0;
+}
+
 cudaError_t launch_attn_tc(const AttnArgs &a, const TcMaps &maps, cudaStream_t s) {
     static_assert(sizeof(Ctl) <= 512, "control block");
     static_assert(kSmemBytes <= 232448, "shared memory budget of one CTA");
@@ -1255,13 +1453,21 @@ cudaError_t launch_attn_tc(const AttnArgs &a, const TcMaps &maps, cudaStream_t s
                                     : a.streams == 1      ? (a.win_lo > 0 ? attn_tc_kernel<true, 0, false, true> : attn_tc_kernel<false, 0, false, true>)
                                     : (a.win_lo > 0 ? attn_tc_kernel<true, 0, false, false> : attn_tc_kernel<false, 0, false, false>);
     const uint32_t smem = quant ? kSmemBytesQ8 : kSmemBytes;
+    if (a.ranks) {
+        auto ranked = a.ranks == 4 ? attn_tc_kernel<true, 0, false, false, 4> : a.ranks == 2 ? attn_tc_kernel<true, 0, false, false, 2>
+                                                                                             : attn_tc_kernel<true, 0, false, false, 1>;
+        cudaError_t e = raise_smem_limit_once(reinterpret_cast<const void *>(ranked), (int)kSmemBytes);
+        if (e != cudaSuccess) return e;
+        const dim3 grid((a.n * a.Gp + kRows - 1) / kRows * a.ngroups, 1, a.batch);
+        return launch_pdl_cluster(a.ranks, ranked, grid, dim3(kThreads), kSmemBytes, s, a, maps.q, maps.k, maps.v);
+    }
     dim3 grid(attn_tc_row_pairs(a.n, a.Gp), a.ngroups, a.batch);
     if (pair_launch_ok(a)) {
         auto paired = a.quant_bits == 8 ? attn_tc_kernel<false, 8, true, true> : attn_tc_kernel<false, 4, true, true>;
         cudaError_t e = raise_smem_limit_once(reinterpret_cast<const void *>(paired), (int)kSmemBytesPair);
         if (e != cudaSuccess) return e;
         if (pair_clusters_fit(reinterpret_cast<const void *>(paired), kSmemBytesPair))
-            return launch_pdl_cluster2(paired, grid, dim3(kThreadsQ8), kSmemBytesPair, s, a, maps.q, maps.k_half, maps.v_half);
+            return launch_pdl_cluster(2, paired, grid, dim3(kThreadsQ8), kSmemBytesPair, s, a, maps.q, maps.k_half, maps.v_half);
     }
     cudaError_t e = raise_smem_limit_once(reinterpret_cast<const void *>(kernel), (int)smem);
     if (e != cudaSuccess) return e;

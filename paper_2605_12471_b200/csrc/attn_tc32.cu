@@ -139,19 +139,6 @@ __device__ __forceinline__ void store_split4(uint8_t *part_hi, uint8_t *part_lo,
     *reinterpret_cast<uint2 *>(part_lo + off) = make_uint2(l0, l1);
 }
 
-// 16 columns x (32-bit) of this thread's TMEM lane <-> registers
-#define KVF_TMEM_LD16(a, o, taddr)                                                              \
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 "                                      \
-                 "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];" \
-                 : "=r"(a[o + 0]), "=r"(a[o + 1]), "=r"(a[o + 2]), "=r"(a[o + 3]), "=r"(a[o + 4]), "=r"(a[o + 5]), "=r"(a[o + 6]), "=r"(a[o + 7]), \
-                   "=r"(a[o + 8]), "=r"(a[o + 9]), "=r"(a[o + 10]), "=r"(a[o + 11]), "=r"(a[o + 12]), "=r"(a[o + 13]), "=r"(a[o + 14]), "=r"(a[o + 15]) \
-                 : "r"(taddr) : "memory")
-#define KVF_TMEM_ST16(a, o, taddr)                                                              \
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%16], {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15};" \
-                 ::"r"(a[o + 0]), "r"(a[o + 1]), "r"(a[o + 2]), "r"(a[o + 3]), "r"(a[o + 4]), "r"(a[o + 5]), "r"(a[o + 6]), "r"(a[o + 7]), \
-                   "r"(a[o + 8]), "r"(a[o + 9]), "r"(a[o + 10]), "r"(a[o + 11]), "r"(a[o + 12]), "r"(a[o + 13]), "r"(a[o + 14]), "r"(a[o + 15]), \
-                   "r"(taddr) : "memory")
-
 // kPair: the CTAs of row blocks 2k and 2k + 1 form a cluster of two that walks the same 64-key steps.  Each
 // converts 32 of a step's 64 key rows (K and V) into its own slot and, with bulk copies that complete on the
 // partner's FULL barrier, into the partner's; a slot is free once the issuers of BOTH CTAs have committed their
@@ -705,7 +692,7 @@ cudaError_t launch_attn_tc32(const AttnArgs &a, cudaStream_t s) {
         cudaError_t e = raise_smem_limit_once(reinterpret_cast<const void *>(paired), (int)kSmemBytes);
         if (e != cudaSuccess) return e;
         if (pair_clusters_fit32(reinterpret_cast<const void *>(paired)))
-            return launch_pdl_cluster2(paired, grid, dim3(kThreads), kSmemBytes, s, a);
+            return launch_pdl_cluster(2, paired, grid, dim3(kThreads), kSmemBytes, s, a);
     }
     auto kernel = a.win_lo > 0 ? attn_tc32_kernel<true> : attn_tc32_kernel<false>;
     cudaError_t e = raise_smem_limit_once(reinterpret_cast<const void *>(kernel), (int)kSmemBytes);

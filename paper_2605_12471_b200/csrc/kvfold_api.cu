@@ -309,6 +309,7 @@ struct Plan {
     int splits;    // CUDA-core path: splits of the key range; tensor-core path: ranges per KV head (rounded up)
     int ngroups;   // tensor-core path: ranges of the (KV head, key tile) line
     int ctas, kernels;
+    int ranks;     // windowed steps: CTAs of a cluster that share a row tile (AttnArgs::ranks), else 0
     FoldSmallCut cut;   // of a small step
 };
 
@@ -326,7 +327,7 @@ Plan make_plan(const kvf_cache *c, int n, int64_t prefix, int batch = 1, int64_t
     Plan p;
     p.qdec = p.small = false;
     p.tc = c->tc || c->tc32;
-    p.ngroups = 0;
+    p.ngroups = p.ranks = 0;
     const int64_t L = prefix + n;
     const int Hkv = c->cfg.n_kv_heads;
     if ((c->quant || c->tc) && c->window <= 0 && n * c->G <= attn_q8_decode_max_rows()) {
@@ -354,6 +355,19 @@ Plan make_plan(const kvf_cache *c, int n, int64_t prefix, int batch = 1, int64_t
         // (row blocks of a KV head: 256-row pairs in the bf16 kernel, 128-row blocks in the fp32 one)
         const int pairs = c->tc32 ? attn_tc32_row_blocks(n, c->Gp) : attn_tc_row_pairs(n, c->Gp);
         const int streams = c->tc32 ? 1 : attn_tc_streams(n, c->Gp);
+        if (c->tc && !c->quant && c->force_splits <= 0 && window_lo(c, prefix) > 0) {
+            // Under a window the key tiles are few, whatever the prefix: a row tile's ranges are merged within a cluster (attn_tc.cu).
+            const int row_tiles = (int)(((int64_t)n * c->Gp + kKvTile - 1) / kKvTile);
+            const int64_t units = (int64_t)row_tiles * Hkv * batch;
+            p.ranks = units <= c->sm_count ? attn_tc_row_ranks((int)units, c->sm_count, nt) : 0;      // (else as without a window)
+            if (p.ranks) {
+                p.ngroups = Hkv * p.ranks;
+                p.splits = 2 * p.ranks;             // (each CTA's key tiles go to two streams)
+                p.ctas = row_tiles * p.ngroups * batch;
+                p.kernels = 2;
+                return p;
+            }
+        }
         const int64_t slots_cap = part_rows_cap / ((int64_t)n * c->Gp) / streams;   // slots = streams * (groups + Hkv - 1)
         int64_t groups = Hkv;
         if (c->force_splits > 0) {
@@ -697,6 +711,7 @@ kvf_status step_impl(kvf_cache *c, const void *q, const void *k_new, const void 
     aa.splits = plan.tc ? 1 : plan.splits;
     aa.ngroups = plan.ngroups;
     aa.streams = (c->tc && !plan.qdec) ? attn_tc_streams(n, c->Gp) : 1;
+    aa.ranks = plan.ranks;
     aa.out_f32 = (f.dtype == KVF_F32 || (f.flags & KVF_OUT_F32)) ? 1 : 0;
     aa.scale_log2 = c->scale_log2;
     aa.range_valid = 0;
@@ -1387,6 +1402,7 @@ kvf_status batch_step(kvf_batch *b, const void *q, const void *k_new, const void
     aa.splits = 1;
     aa.ngroups = plan.ngroups;
     aa.streams = plan.qdec ? 1 : attn_tc_streams(n, c0->Gp);
+    aa.ranks = plan.ranks;
     aa.out_f32 = (f.flags & KVF_OUT_F32) ? 1 : 0;
     aa.scale_log2 = c0->scale_log2;
     aa.range_valid = 0;

@@ -45,9 +45,9 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
-// The same with the grid's CTAs grouped into clusters of two along x.
+// The same with the grid's CTAs grouped into clusters of `ctas` along x.
 template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl_cluster2(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args &&...args) {
+cudaError_t launch_pdl_cluster(int ctas, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args &&...args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
@@ -57,7 +57,7 @@ cudaError_t launch_pdl_cluster2(void (*kernel)(KArgs...), dim3 grid, dim3 block,
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = g_pdl_allowed ? 1 : 0;
     attr[1].id = cudaLaunchAttributeClusterDimension;
-    attr[1].val.clusterDim.x = 2;
+    attr[1].val.clusterDim.x = (unsigned)ctas;
     attr[1].val.clusterDim.y = 1;
     attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
@@ -176,6 +176,8 @@ struct AttnArgs {
     int32_t splits;                  // CUDA-core path: equal splits of the key range
     int32_t ngroups;                 // tensor-core path: contiguous ranges of the (KV head, key tile) line
     int32_t streams;                 // tensor-core path: 2 = one row tile, its key tiles dealt to two streams
+    int32_t ranks;                   // bf16 rows: CTAs of a cluster that share one row tile's key tiles, each in two streams, and write
+                                     // the output themselves (0: not so)
     int32_t piece_cost;              // tensor-core path: the line the groups cut holds, in front of every KV head's key
                                      // tiles, this many virtual tiles that stand for what a second piece costs a CTA
                                      // (another Q load, another drain and set of partial rows): a CTA whose range
@@ -264,6 +266,7 @@ bool attn_tc_supported(int dtype, int d, int G);
 int attn_tc_padded_group(int G);       // G rounded up to a power of two: rows a token takes in the tcgen05 kernels' row layout
 int attn_tc_row_pairs(int n, int G);   // 256-row pairs per KV head (G: the padded group, as below)
 int attn_tc_streams(int n, int G);     // 2 when the chunk fits one 128-row tile
+int attn_tc_row_ranks(int units, int sms, int64_t key_tiles);        // AttnArgs::ranks for `units` row tiles of all KV heads, or 0
 cudaError_t launch_attn_tc(const AttnArgs &a, const TcMaps &maps, cudaStream_t s);   // grid (ngroups x row pairs); pairs of CTAs: (row pairs, ngroups)
 cudaError_t launch_combine_groups(const AttnArgs &a, int sms, cudaStream_t s);                // needed when ngroups != Hkv
 

@@ -1,0 +1,60 @@
+"""Small bf16 steps under a window (clusters of one, two or four CTAs per 128-row tile merge their key ranges): against the
+CUDA-core kernel on the same rows.
+
+Both read the same bf16 cache.  What the tensor-core kernel rounds are the probabilities, to bf16: an output element moves by at most
+2^-8 of sum p |v|, which the CUDA-core kernel gives when it is run on |v|.  Scores differ by fp32 sums of 128 products, up to ~60
+in the growing case (5e-4, as in test_early_issue_gpu.py): the same for a log-sum-exp, twice that of sum p |v| for an output.
+bf16 outputs are rounded by both, 2^-8 of the element each."""
+import pytest
+import torch
+
+from paper_2605_12471_b200 import binding
+
+pytestmark = pytest.mark.gpu
+
+
+def _run(h, kv, prefix, n, sinks, window, growing, out_f32, gen):
+    rows = prefix + n
+    q, k, v = (torch.randn(rows, heads, 128, generator=gen, device="cuda") for heads in (h, kv, kv))
+    if growing:
+        k *= torch.linspace(0.1, 12.0, rows, device="cuda")[:, None, None]
+    q, k, v = (x.bfloat16() for x in (q, k, v))
+
+    def fold(flags, values):
+        c = binding.Cache(binding.make_config(h, kv, 128, "bf16", rows, rows, rope_base=10000.0, flags=flags))
+        c.storage.zero_()
+        c.fold_step(q[:prefix].contiguous(), k[:prefix].contiguous(), values[:prefix].contiguous())
+        c.set_window(sinks, window)
+        lse = torch.empty(n, h, device="cuda")
+        before = c.launch_count()
+        out = c.fold_step(q[prefix:].contiguous(), k[prefix:].contiguous(), values[prefix:].contiguous(), lse=lse)
+        assert c.status() == binding.KVF_OK
+        return out.float(), lse, c.launch_count() - before, c.plan(n, prefix)
+
+    kind = binding.KVF_OUT_F32 if out_f32 else 0
+    a, la, launches, plan = fold(kind, v)
+    b, lb, _, _ = fold(kind | binding.KVF_FORCE_SIMT, v)
+    weight = fold(binding.KVF_OUT_F32 | binding.KVF_FORCE_SIMT, v.abs())[0]
+    bound = (2.0 ** -8 + 2 * 5e-4) * weight + (0.0 if out_f32 else 2 * 2.0 ** -8) * torch.maximum(a.abs(), b.abs())
+    assert ((a - b).abs() <= bound).all()
+    assert (la - lb).abs().max().item() <= 5e-4
+    assert launches == plan[3]
+    return plan
+
+
+# rows at the edges of a 128-row tile; one key tile (fewer than the CTAs of a cluster), a window inside it, many; padded groups
+@pytest.mark.parametrize("out_f32", [False, True], ids=["bf16", "f32"])
+@pytest.mark.parametrize("h,kv", [(8, 2), (7, 1), (3, 3)])
+@pytest.mark.parametrize("prefix,sinks,window", [(130, 1, 3), (300, 4, 20), (600, 0, 129), (900, 64, 300), (1500, 4, 1300)])
+def test_small_windowed_steps_against_the_cuda_core_kernel(h, kv, prefix, sinks, window, out_f32):
+    gen = torch.Generator(device="cuda").manual_seed(prefix + h)
+    for n in (17, 31, 32, 33, 65, 190):
+        _run(h, kv, prefix, n, sinks, window, n & 1, out_f32, gen)
+
+
+# clusters of four, two and one CTA (two streams each), and the 256-row CTAs beyond
+@pytest.mark.parametrize("n,window,parts", [(64, 1020, 8), (256, 1020, 4), (400, 500, 2), (700, 500, None)])
+def test_one_two_and_four_ctas_per_row_tile(n, window, parts):
+    plan = _run(32, 8, 2000, n, 4, window, False, False, torch.Generator(device="cuda").manual_seed(n))
+    if parts and torch.cuda.get_device_properties(0).multi_processor_count == 148:
+        assert plan[1] == parts and plan[3] == 2
