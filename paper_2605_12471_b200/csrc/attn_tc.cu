@@ -330,7 +330,8 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
     pdl_launch_dependents();
     tc_fence_before();
     __syncthreads();
-    if (kPair || kRanks > 1) cluster_sync_all();      // the partners' barriers exist before anything is sent to them
+    if (kPair) cluster_sync_all();      // the partner's barriers exist before anything is sent to them
+    if (kRanks > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");      // (waited for at the end, ahead of what is sent)
     tc_fence_after();
     pdl_wait();   // nothing above reads what an earlier kernel wrote; from here on the rotated chunk is read
     const uint32_t tmem = *reinterpret_cast<volatile uint32_t *>(&ctl->tmem_base);
@@ -1015,6 +1016,7 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
         constexpr int W = 64 / kRanks;
         constexpr uint32_t kFromRank = 2u * kRows * W * 4u;              // what a CTA sends another: its columns of 2 x 128 half rows ...
         const uint32_t landing = base + kOffKV + kTileBytes, land_stats = base + kOffKV + 4096u;     // ... and a float2 per row, by sender
+        if (kRanks > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
         if (kRanks > 1 && threadIdx.x == 0) {
             mbar_expect_tx(bar(B_LANDED), (kRanks - 1) * (kFromRank + kRows * 8u));
             for (uint32_t s = 0; s < kRanks; ++s)

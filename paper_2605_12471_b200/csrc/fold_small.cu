@@ -20,6 +20,7 @@
 // 0.34, half of the stall cycles on them), so slices are as short as the device has room for.  Tried: 4 x 4 blocks
 // per thread on half the threads (a third less shared-memory traffic, fewer warps: 6.3 us a tile).
 #include "kvfold_internal.h"
+#include "sm100_ptx.cuh"
 
 namespace kvf {
 namespace {
@@ -31,12 +32,16 @@ constexpr int kMaxRanks = 1 << (kFoldSmallWidths - 1);     // slices of the key 
 
 struct Smem {
     float q[BM * QS];
-    float k[kMaxBN * QS];                // behind the last key tile: this CTA's unnormalised output [BM][D]
+    float k[kMaxBN * QS];
     float v[kMaxBN * D];
     float p[BM * QS];
     float2 cs_q[BM][HALF];           // (cos, sin) per (token of the row tile, pair)
     float2 cs_k[kMaxBN][HALF];           // ... per (key of the tile that belongs to the chunk, pair)
-    float m[BM], l[BM];
+    // what the CTAs of the cluster send for this one's BM / ranks rows, by sender: unnormalised outputs, (maximum, sum)
+    float landed_o[BM * D];
+    float2 landed_ml[BM];
+    unsigned long long landed;       // the barrier they complete on
+    int abort;
 };
 
 __device__ __forceinline__ void unpack(const uint4 &w, float (&x)[4]) {
@@ -100,26 +105,6 @@ __device__ __forceinline__ void to_shared(float *dst, const float (&x)[N]) {
     for (int e = 0; e < N; e += 4) *reinterpret_cast<float4 *>(dst + e) = make_float4(x[e], x[e + 1], x[e + 2], x[e + 3]);
 }
 
-__device__ __forceinline__ uint32_t in_rank(const void *p, uint32_t rank) {
-    uint32_t r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
-    return r;
-}
-__device__ __forceinline__ float remote(uint32_t addr) {
-    float x;
-    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(x) : "r"(addr) : "memory");
-    return x;
-}
-__device__ __forceinline__ float4 remote4(uint32_t addr) {
-    float4 x;
-    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x.x), "=f"(x.y), "=f"(x.z), "=f"(x.w) : "r"(addr) : "memory");
-    return x;
-}
-__device__ __forceinline__ void cluster_sync() {
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-
 // BN = keys of a tile: 64, or 32 (see fold_small_cut).
 template <typename T, bool INTERLEAVED, int BN>
 __global__ void __launch_bounds__(kThreads, 2) fold_small_kernel(const __grid_constant__ RopeAppendArgs r, const __grid_constant__ AttnArgs a) {
@@ -146,6 +131,17 @@ __global__ void __launch_bounds__(kThreads, 2) fold_small_kernel(const __grid_co
     const int kt_begin = (int)((int64_t)rank * nt / ranks), kt_end = (int)((int64_t)(rank + 1) * nt / ranks);
 
     pdl_launch_dependents();
+    const uint32_t landed = smem_u32(&sm.landed);
+    if (ranks > 1) {
+        // (the partners' barriers exist once everybody has been here: waited for ahead of the first store to them)
+        if (tid == 0) {
+            mbar_init(landed, 1);
+            sm.abort = 0;
+            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+            mbar_expect_tx(landed, BM * (D * 4u + 8u));
+        }
+        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    }
     auto table = [&](float2 *cs, int64_t token, int j) {
         const double theta = (double)(r.pos0 + token) * r.table.inv_freq[j];
         double sn, cn;
@@ -336,28 +332,35 @@ __global__ void __launch_bounds__(kThreads, 2) fold_small_kernel(const __grid_co
         __syncwarp();                                     // (the next tile's probabilities overwrite these)
     }
 
-    // every slice's maximum, sum and unnormalised output, merged in slice order
-    __syncthreads();
+    // Every slice's maximum, sum and unnormalised output go to the CTA that finishes the row, which merges them in slice order.
+    // (Stores that complete on the receiver's barrier, instead of loads between two cluster barriers.)
+    const int rows = BM / ranks;                          // (ranks is a power of two)
+    if (ranks > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 #pragma unroll
     for (int i = 0; i < TR; ++i) {
-        *reinterpret_cast<float4 *>(sm.k + (TR * ty + i) * D + tx * 4) = make_float4(acc[i][0].x, acc[i][0].y, acc[i][1].x, acc[i][1].y);
-        if (tx == 0) {
-            sm.m[TR * ty + i] = m[i];
-            sm.l[TR * ty + i] = l[i];
+        const int row = TR * ty + i, at = rank * rows + row % rows;
+        const float4 o = make_float4(acc[i][0].x, acc[i][0].y, acc[i][1].x, acc[i][1].y);
+        if (ranks > 1) {
+            const uint32_t to = (uint32_t)(row / rows), done = peer_smem(landed, to);
+            peer_store4(peer_smem(smem_u32(&sm.landed_o[at * D + tx * 4]), to), o, done);
+            if (tx == 0) peer_store2(peer_smem(smem_u32(&sm.landed_ml[at]), to), make_float2(m[i], l[i]), done);
+        } else {
+            *reinterpret_cast<float4 *>(&sm.landed_o[at * D + tx * 4]) = o;
+            if (tx == 0) sm.landed_ml[at] = make_float2(m[i], l[i]);
         }
     }
-    if (ranks > 1) cluster_sync();
-    else __syncthreads();
-    const int rows = BM / ranks;                          // (ranks is a power of two)
+    if (ranks == 1) __syncthreads();
+    else if (!mbar_wait(landed, 0, &sm, a.status)) return;
     for (int i = tid; i < rows * (D / 4); i += kThreads) {
-        const int row = rank * rows + i / (D / 4), c = i % (D / 4);
+        const int own = i / (D / 4), row = rank * rows + own, c = i % (D / 4);
         const int R = row0 + row, tok = R / G, gi = R % G;
         if (tok >= n) continue;
-        float ms[kMaxRanks], M = -INFINITY;
+        float2 ml[kMaxRanks];
+        float M = -INFINITY;
 #pragma unroll
         for (int s = 0; s < kMaxRanks; ++s) {
-            ms[s] = s < ranks ? remote(in_rank(&sm.m[row], (uint32_t)s)) : -INFINITY;
-            M = fmaxf(M, ms[s]);
+            ml[s] = s < ranks ? sm.landed_ml[s * rows + own] : make_float2(-INFINITY, 0.f);
+            M = fmaxf(M, ml[s].x);
         }
         const float M0 = M == -INFINITY ? 0.f : M;
         float den = 0.f;
@@ -365,9 +368,9 @@ __global__ void __launch_bounds__(kThreads, 2) fold_small_kernel(const __grid_co
 #pragma unroll
         for (int s = 0; s < kMaxRanks; ++s) {
             if (s >= ranks) break;
-            const float w = exp2f(ms[s] - M0);
-            const float4 x = remote4(in_rank(&sm.k[row * D + c * 4], (uint32_t)s));
-            den = fmaf(w, remote(in_rank(&sm.l[row], (uint32_t)s)), den);
+            const float w = exp2f(ml[s].x - M0);
+            const float4 x = *reinterpret_cast<const float4 *>(&sm.landed_o[(s * rows + own) * D + c * 4]);
+            den = fmaf(w, ml[s].y, den);
             o.x = fmaf(w, x.x, o.x); o.y = fmaf(w, x.y, o.y); o.z = fmaf(w, x.z, o.z); o.w = fmaf(w, x.w, o.w);
         }
         const float inv = den > 0.f ? 1.f / den : 0.f;
@@ -384,7 +387,7 @@ __global__ void __launch_bounds__(kThreads, 2) fold_small_kernel(const __grid_co
         }
         if (c == 0 && a.lse) a.lse[at] = (den > 0.f ? M + log2f(den) : -INFINITY) * 0.6931471805599453f;
     }
-    if (ranks > 1) cluster_sync();                        // nobody leaves while a partner reads its shared memory
+    // (what others send has landed, and what this CTA sends needs it no more: nobody waits to leave)
 }
 
 // Once per kernel and device: shared-memory limit, clusters of 16 CTAs (beyond the portable eight), and how many clusters
