@@ -125,14 +125,15 @@ struct kvf_cache {
     const int32_t *page_table = nullptr;   // paged cache: device table, one page number per 128 tokens
     int64_t page_elems = 0;                // paged cache: elements per page
     int32_t n_pool_pages = 0;
-    // KVF_HOST_UPLOAD_AHEAD: the library's upload stream, "upload done" and "staging set read" events
-    cudaStream_t up_stream = nullptr;
-    cudaEvent_t ev_up[2] = {nullptr, nullptr}, ev_read[2] = {nullptr, nullptr};
+    // KVF_HOST_UPLOAD_AHEAD: the library's upload streams (queries; keys and values), "upload done" (by staging set and stream) and
+    // "staging set read" events
+    cudaStream_t up_stream[2] = {nullptr, nullptr};
+    cudaEvent_t ev_up[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}}, ev_read[2] = {nullptr, nullptr};
     bool ev_read_set[2] = {false, false};
     uint64_t host_steps = 0;
-    // KVF_HOST_DOWNLOAD_BEHIND: the library's download stream, "step done" (caller's stream) and "results
-    // copied" (download stream) events of the two result staging sets
-    cudaStream_t down_stream = nullptr;
+    // KVF_HOST_DOWNLOAD_BEHIND: the library's download streams, "step done" (caller's stream) and "results
+    // copied" (download stream) events, of the two result staging sets
+    cudaStream_t down_stream[2] = {nullptr, nullptr};
     cudaEvent_t ev_step[2] = {nullptr, nullptr}, ev_down[2] = {nullptr, nullptr};
     bool ev_down_set[2] = {false, false};
     uint64_t host_down_steps = 0;
@@ -1008,23 +1009,33 @@ kvf_status kvf_fold_step_host(kvf_cache *c, const void *q_host, const void *k_ho
         // upload on the library's stream into the staging set the step before last used: it runs
         // while the previous step computes, and starts once that set's last reader (the rotate +
         // append kernel of two steps ago, marked by ev_read) is done
-        if (!c->up_stream) {
-            e = cudaStreamCreateWithFlags(&c->up_stream, cudaStreamNonBlocking);
+        // (Copies of one stream follow one another with a gap, and a copy that has the other direction beside it is slower
+        // than the two together need be: 64 times 2 + 1/2 + 1/2 MB up and 2 MB down take 5.83 ms on one stream each way, 5.56 with two up,
+        // 4.90 with two each way; 4.42 without those down.  16 384 tokens in chunks of 256, whose two staging sets hold the copies back,
+        // 6.12 -> 5.99 ms, in chunks of 1024 5.19 -> 5.09; with two streams one way only no faster.)
+        if (!c->up_stream[1]) {
             for (int i = 0; i < 2 && e == cudaSuccess; ++i) {
-                e = cudaEventCreateWithFlags(&c->ev_up[i], cudaEventDisableTiming);
-                if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_read[i], cudaEventDisableTiming);
+                if (!c->up_stream[i]) e = cudaStreamCreateWithFlags(&c->up_stream[i], cudaStreamNonBlocking);
+                for (int k = 0; k < 2 && e == cudaSuccess; ++k)
+                    if (!c->ev_up[i][k]) e = cudaEventCreateWithFlags(&c->ev_up[i][k], cudaEventDisableTiming);
+                if (e == cudaSuccess && !c->ev_read[i]) e = cudaEventCreateWithFlags(&c->ev_read[i], cudaEventDisableTiming);
             }
-            if (e != cudaSuccess) return cuda_fail(e, "upload stream setup");
+            if (e != cudaSuccess) {
+                if (c->up_stream[1]) { cudaStreamDestroy(c->up_stream[1]); c->up_stream[1] = nullptr; }      // (asked again by the next call)
+                return cuda_fail(e, "upload stream setup");
+            }
         }
         set = (int)(c->host_steps & 1);
         if (set) { oq = c->lay.st_q2; ok_ = c->lay.st_k2; ov = c->lay.st_v2; }
-        cudaStream_t up = c->up_stream;
-        if (c->ev_read_set[set]) e = cudaStreamWaitEvent(up, c->ev_read[set], 0);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(w + oq, q_host, qb, cudaMemcpyHostToDevice, up);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(w + ok_, k_host, kb, cudaMemcpyHostToDevice, up);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(w + ov, v_host, kb, cudaMemcpyHostToDevice, up);
-        if (e == cudaSuccess) e = cudaEventRecord(c->ev_up[set], up);
-        if (e == cudaSuccess) e = cudaStreamWaitEvent(st, c->ev_up[set], 0);
+        for (int k = 0; k < 2; ++k)
+            if (c->ev_read_set[set] && e == cudaSuccess) e = cudaStreamWaitEvent(c->up_stream[k], c->ev_read[set], 0);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(w + oq, q_host, qb, cudaMemcpyHostToDevice, c->up_stream[0]);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(w + ok_, k_host, kb, cudaMemcpyHostToDevice, c->up_stream[1]);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(w + ov, v_host, kb, cudaMemcpyHostToDevice, c->up_stream[1]);
+        for (int k = 0; k < 2 && e == cudaSuccess; ++k) {
+            e = cudaEventRecord(c->ev_up[set][k], c->up_stream[k]);
+            if (e == cudaSuccess) e = cudaStreamWaitEvent(st, c->ev_up[set][k], 0);
+        }
     } else {
         e = cudaMemcpyAsync(w + oq, q_host, qb, cudaMemcpyHostToDevice, st);
         if (e == cudaSuccess) e = cudaMemcpyAsync(w + ok_, k_host, kb, cudaMemcpyHostToDevice, st);
@@ -1035,13 +1046,16 @@ kvf_status kvf_fold_step_host(kvf_cache *c, const void *q_host, const void *k_ho
     int oset = 0;
     size_t o_out = c->lay.st_out, o_lse = c->lay.st_lse;
     if (behind) {
-        if (!c->down_stream) {
-            e = cudaStreamCreateWithFlags(&c->down_stream, cudaStreamNonBlocking);
+        if (!c->down_stream[1]) {
             for (int i = 0; i < 2 && e == cudaSuccess; ++i) {
-                e = cudaEventCreateWithFlags(&c->ev_step[i], cudaEventDisableTiming);
-                if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_down[i], cudaEventDisableTiming);
+                if (!c->down_stream[i]) e = cudaStreamCreateWithFlags(&c->down_stream[i], cudaStreamNonBlocking);
+                if (e == cudaSuccess && !c->ev_step[i]) e = cudaEventCreateWithFlags(&c->ev_step[i], cudaEventDisableTiming);
+                if (e == cudaSuccess && !c->ev_down[i]) e = cudaEventCreateWithFlags(&c->ev_down[i], cudaEventDisableTiming);
             }
-            if (e != cudaSuccess) return cuda_fail(e, "download stream setup");
+            if (e != cudaSuccess) {
+                if (c->down_stream[1]) { cudaStreamDestroy(c->down_stream[1]); c->down_stream[1] = nullptr; }
+                return cuda_fail(e, "download stream setup");
+            }
         }
         oset = (int)(c->host_down_steps & 1);
         if (oset) { o_out = c->lay.st_out2; o_lse = c->lay.st_lse2; }
@@ -1060,7 +1074,7 @@ kvf_status kvf_fold_step_host(kvf_cache *c, const void *q_host, const void *k_ho
         c->ev_read_set[set] = true;
         c->host_steps++;
     }
-    cudaStream_t ds = behind ? c->down_stream : st;
+    cudaStream_t ds = behind ? c->down_stream[oset] : st;
     if (behind) {
         // the copies of this step's results run on the library's stream, behind the step, while the caller's
         // stream goes on with the next step
@@ -1212,15 +1226,18 @@ void kvf_cache_destroy(kvf_cache *c) {
     for (ProfRec &r : c->recs) { cudaEventDestroy(r.a); cudaEventDestroy(r.b); }
     for (cudaEvent_t e : c->pool) cudaEventDestroy(e);
     for (int i = 0; i < 2; ++i) {
-        if (c->ev_up[i]) cudaEventDestroy(c->ev_up[i]);
+        for (int k = 0; k < 2; ++k)
+            if (c->ev_up[i][k]) cudaEventDestroy(c->ev_up[i][k]);
         if (c->ev_read[i]) cudaEventDestroy(c->ev_read[i]);
     }
-    if (c->up_stream) cudaStreamDestroy(c->up_stream);
+    for (cudaStream_t up : c->up_stream)
+        if (up) cudaStreamDestroy(up);
     for (int i = 0; i < 2; ++i) {
         if (c->ev_step[i]) cudaEventDestroy(c->ev_step[i]);
         if (c->ev_down[i]) cudaEventDestroy(c->ev_down[i]);
     }
-    if (c->down_stream) cudaStreamDestroy(c->down_stream);
+    for (cudaStream_t down : c->down_stream)
+        if (down) cudaStreamDestroy(down);
     if (c->ev_attn) cudaEventDestroy(c->ev_attn);
     if (c->ev_comb) cudaEventDestroy(c->ev_comb);
     if (c->comb_stream) cudaStreamDestroy(c->comb_stream);
