@@ -85,6 +85,23 @@ __global__ void __launch_bounds__(kThreads, kResident) rope_append_q8_kernel(con
         sincos(theta, &sn, &cn);
         cs[t][j] = make_float2((float)cn, (float)sn);
     }
+    const int64_t qoff = (int64_t)b * a.n * a.H * d, koff = (int64_t)b * a.n * a.Hkv * d;
+    const __nv_bfloat16 *q = reinterpret_cast<const __nv_bfloat16 *>(a.q) + qoff;
+    const __nv_bfloat16 *k = reinterpret_cast<const __nv_bfloat16 *>(a.k_new) + koff;
+    const __nv_bfloat16 *v = reinterpret_cast<const __nv_bfloat16 *>(a.v_new) + koff;
+    __nv_bfloat16 *qr = reinterpret_cast<__nv_bfloat16 *>(a.q_rot) + qoff;
+    const int heads = a.H + (a.k_new ? 2 * a.Hkv : 0);     // query rows, key rows, value rows (queries only: kvf_attend)
+    // (the inputs' lines are called into L2 while the kernel before still finishes, as in rope_append.cu: two lines to a row, a warp's
+    // first four rows)
+    if (lane < 8) {
+        const int hh = warp + (lane >> 1) * (kThreads / 32);
+        const bool is_q = hh < a.H, is_v = hh >= a.H + a.Hkv;
+        const int g = is_q ? hh : is_v ? hh - a.H - a.Hkv : hh - a.H, row_heads = is_q ? a.H : a.Hkv;
+        const __nv_bfloat16 *row = (is_q ? q : is_v ? v : k) + ((int64_t)tok0 * row_heads + g) * d + (lane & 1) * half;
+#pragma unroll
+        for (int u = 0; u < kTok; ++u)
+            if (hh < heads && u < ntok) asm volatile("prefetch.global.L2 [%0];" ::"l"(row + (int64_t)u * row_heads * d));
+    }
     __syncthreads();
     pdl_wait();   // the table above needs nothing from earlier kernels; the writes below do
 
@@ -97,12 +114,6 @@ __global__ void __launch_bounds__(kThreads, kResident) rope_append_q8_kernel(con
             qp.v_scales[scale_idx(i / zero_rows, prefix + n + i % zero_rows)] = 0.f;
     }
 
-    const int64_t qoff = (int64_t)b * a.n * a.H * d, koff = (int64_t)b * a.n * a.Hkv * d;
-    const __nv_bfloat16 *q = reinterpret_cast<const __nv_bfloat16 *>(a.q) + qoff;
-    const __nv_bfloat16 *k = reinterpret_cast<const __nv_bfloat16 *>(a.k_new) + koff;
-    const __nv_bfloat16 *v = reinterpret_cast<const __nv_bfloat16 *>(a.v_new) + koff;
-    __nv_bfloat16 *qr = reinterpret_cast<__nv_bfloat16 *>(a.q_rot) + qoff;
-    const int heads = a.H + (a.k_new ? 2 * a.Hkv : 0);     // query rows, key rows, value rows (queries only: kvf_attend)
     for (int hh = warp; hh < heads; hh += kThreads / 32) {
         const bool is_q = hh < a.H, is_v = hh >= a.H + a.Hkv;
         const int g = is_q ? hh : is_v ? hh - a.H - a.Hkv : hh - a.H;        // query head, or KV head

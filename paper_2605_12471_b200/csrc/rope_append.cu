@@ -105,9 +105,6 @@ __global__ void __launch_bounds__(kThreads, kResident) rope_append_kernel(const 
         sincos(theta, &sn, &cn);
         cs[t][j] = make_float2((float)cn, (float)sn);
     }
-    __syncthreads();
-    pdl_wait();   // the table above needs nothing from earlier kernels; the writes below do
-
     const int64_t qoff = (int64_t)b * a.n * a.H * d, koff = (int64_t)b * a.n * a.Hkv * d;
     const T *q = reinterpret_cast<const T *>(a.q) + qoff;
     const T *k = reinterpret_cast<const T *>(a.k_new) + koff;
@@ -123,17 +120,47 @@ __global__ void __launch_bounds__(kThreads, kResident) rope_append_kernel(const 
     const int rot_items = heads * rot_chunks;
     const int v_chunks = d / VEC;
     const int items = rot_items + (a.v_new ? a.Hkv * v_chunks : 0);
+    struct Item {
+        bool value, query;
+        int c, g, row_heads;                                   // vector in the row, query head or KV head, heads of a token
+        const T *src;                                          // the first token's
+    };
+    auto item = [&](int idx) {
+        Item m;
+        m.value = idx >= rot_items;
+        const int it = m.value ? idx - rot_items : idx, chunks = m.value ? v_chunks : rot_chunks;
+        m.c = it % chunks;
+        const int hh = it / chunks;
+        m.query = !m.value && hh < a.H;
+        m.g = m.value || m.query ? hh : hh - a.H;
+        m.row_heads = m.query ? a.H : a.Hkv;
+        m.src = (m.query ? q : m.value ? v : k) + ((int64_t)tok0 * m.row_heads + m.g) * d + m.c * VEC;
+        return m;
+    };
+    // The inputs' lines are called into L2 while the kernel before still finishes; they are read, as everything else, behind the wait.
+    // Cold inputs, us: 128 steps of 256 tokens under a window 2547 -> 2508, 15 077 tokens of 28 / 4 heads in chunks of 256 2613 -> 2568;
+    // eight steps of 2048 tokens the same.
+    if ((int)threadIdx.x < items) {
+        const Item m = item(threadIdx.x);
+#pragma unroll
+        for (int t = 0; t < kTok; ++t)
+            if (t < ntok) {
+                const T *line = m.src + (int64_t)t * m.row_heads * d;
+                asm volatile("prefetch.global.L2 [%0];" ::"l"(line));
+                if (!INTERLEAVED && !m.value) asm volatile("prefetch.global.L2 [%0];" ::"l"(line + half));
+            }
+    }
+    __syncthreads();
+    pdl_wait();   // the table above needs nothing from earlier kernels; the writes below do
+
     float amax = 0.f;               // largest magnitude written (tracked only under a range limit, fp32 caches)
     const bool ranged = sizeof(T) == 4 && a.range_limit > 0.f;
     for (int idx = threadIdx.x; idx < items; idx += kThreads) {
-        const bool value = idx >= rot_items;
-        const int it = value ? idx - rot_items : idx, chunks = value ? v_chunks : rot_chunks;
-        const int c = it % chunks, hh = it / chunks;
-        const bool query = !value && hh < a.H;
-        const int g = value || query ? hh : hh - a.H;           // query head, or KV head
-        const int row_heads = query ? a.H : a.Hkv;
-        const T *src = (query ? q : value ? v : k) + ((int64_t)tok0 * row_heads + g) * d + c * VEC;
-        const int64_t src_step = (int64_t)row_heads * d;
+        const Item m = item(idx);
+        const bool value = m.value, query = m.query;
+        const int c = m.c, g = m.g;
+        const T *src = m.src;
+        const int64_t src_step = (int64_t)m.row_heads * d;
         T *plane = value ? vp : kp;
         auto dst = [&](int t) { return (query ? qr + ((int64_t)(tok0 + t) * a.H + g) * d : plane + rows.offset(g, prefix + tok0 + t)) + c * VEC; };
         uint4 lo[kTok], hi[kTok];
