@@ -580,23 +580,18 @@ int piece_cost_of(const kvf_cache *c, const Plan &plan, int streams) {
     return KVF_PIECE_COST;
 }
 
-// A step whose attention kernel is long enough for a chain of such steps to run at the power cap: bf16 rows, full
-// row tiles on the tensor cores and at least KVF_PDL_MAX_TILES key tiles per CTA.
-#ifndef KVF_PDL_MAX_TILES
-#define KVF_PDL_MAX_TILES 32
-#endif
-bool long_step(const kvf_cache *c, const Plan &plan, int streams, int64_t L) {
-    // KVF_DEPENDENT_LAUNCH=always / never in the environment overrides the rule (read once; for measurements)
-    static const int forced = [] {
+// KVF_DEPENDENT_LAUNCH=never in the environment (read once; for measurements) launches every step's kernels plainly.  Dependent
+// launches are never slower now.  Long tensor-bound steps of bf16 rows (32 key tiles per CTA and more) used to be launched plainly: at
+// the power cap the gaps came back as clock, 148.3 against 150.1 ms for 131 072 tokens in chunks of 256.  Since the issuing warps' overhead
+// is gone the chain is at a lower clock and the gaps are gaps: plain / dependent, three runs in turn, that chain 131.8, 131.1, 131.9 / 130.9,
+// 130.5, 130.3 ms; 32 768 tokens 9.80 / 9.64; 65 536 of 28 / 4 heads 34.6 / 34.0; 16 384 in chunks of 2048 2.12 / 2.09; 30 000 of 16 / 16
+// heads in chunks of 1000 4.12 / 4.04; 65 536 in chunks of 512 and 2048 the same.
+bool dependent_launches() {
+    static const bool never = [] {
         const char *e = std::getenv("KVF_DEPENDENT_LAUNCH");
-        return !e ? 0 : std::strcmp(e, "always") == 0 ? 1 : std::strcmp(e, "never") == 0 ? 2 : 0;
+        return e && std::strcmp(e, "never") == 0;
     }();
-    if (forced) return forced == 2;
-    // (bf16 rows only: the quantised kernels are bound by issue slots and the fp32 kernel by its softmax thread,
-    // not by the power cap - measured, they keep 0.2 - 0.5 % with dependent launches)
-    if (!c->tc || c->quant || plan.qdec || streams != 1 || plan.ngroups <= 0 || c->window > 0) return false;
-    const int64_t nt = (L + kKvTile - 1) / kKvTile;
-    return nt * c->cfg.n_kv_heads >= (int64_t)KVF_PDL_MAX_TILES * plan.ngroups;
+    return !never;
 }
 
 // The groups that touch each KV head, worked out once on the host for the combine kernel.
@@ -721,8 +716,7 @@ kvf_status step_impl(kvf_cache *c, const void *q, const void *k_new, const void 
     if (plan.tc && plan.kernels > 2)
         fill_group_ranges(aa, (L + kKvTile - 1) / kKvTile - WindowTiles(aa.win_lo, aa.n_sink, kKvTile).skip + aa.piece_cost);
 
-    // plain launches for long tensor-bound steps, dependent launches for short ones (see g_pdl_allowed)
-    const PdlScope pdl(!long_step(c, plan, aa.streams, L));
+    const PdlScope pdl(dependent_launches());
     cudaError_t e;
     if (plan.small) {
         e = cudaSuccess;                   // (the attention launch rotates and appends)
@@ -1428,7 +1422,7 @@ kvf_status batch_step(kvf_batch *b, const void *q, const void *k_new, const void
     if (!ragged && plan.kernels > 2)
         fill_group_ranges(aa, (P + n + kKvTile - 1) / kKvTile - WindowTiles(aa.win_lo, aa.n_sink, kKvTile).skip + aa.piece_cost);
 
-    const PdlScope pdl(!long_step(c0, plan, aa.streams, P + n));
+    const PdlScope pdl(dependent_launches());
     cudaError_t e = c0->quant ? launch_rope_append_q8(ra, c0->qp, (f.flags & KVF_ROPE_INTERLEAVED) != 0, B, st)
                               : launch_rope_append(ra, f.dtype, (f.flags & KVF_ROPE_INTERLEAVED) != 0, B, st);
     if (e != cudaSuccess) return cuda_fail(e, "rope_append launch (batch)");

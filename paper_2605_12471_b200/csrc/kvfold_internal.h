@@ -19,11 +19,8 @@ namespace kvf {
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
-// Whether the launches of the calling thread ask for it.  Overlapping a kernel's set-up with the tail of the one
-// before pays where a step is short (decode-shaped steps, short prefixes, the sink + window chain: 1.5 - 5 %);
-// a long chain of long tensor-bound steps runs at the power cap, where the idle gap between plain launches comes
-// back as clock (measured on the 131 072-token chain: 148.3 ms with plain launches against 150.1 ms, the
-// attention kernels at 1.53 instead of 1.505 GHz).  The host layer sets this per step (PdlScope).
+// Whether the launches of the calling thread ask for it: overlapping a kernel's set-up with the tail of the one before (decode-shaped
+// steps, short prefixes, the sink + window chain: 1.5 - 5 %; long chains 0.5 - 2 %).  The host layer sets this per step (PdlScope).
 inline thread_local bool g_pdl_allowed = true;
 struct PdlScope {
     bool saved;
