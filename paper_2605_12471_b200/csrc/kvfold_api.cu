@@ -647,7 +647,7 @@ bool disjoint_step(const kvf_cache *c, const void *q, const void *k_new, const v
 }
 
 kvf_status step_impl(kvf_cache *c, const void *q, const void *k_new, const void *v_new, int32_t n,
-                     int64_t pos0, void *out, float *lse, cudaStream_t st) {
+                     int64_t pos0, void *out, float *lse, cudaStream_t st, cudaEvent_t inputs_read = nullptr) {
     const kvf_config &f = c->cfg;
     const int64_t P = c->len;
     // k_new == null: queries only (kvf_attend) - nothing is appended, every query row sees the P rows held
@@ -730,6 +730,9 @@ kvf_status step_impl(kvf_cache *c, const void *q, const void *k_new, const void 
     }
     if (e != cudaSuccess) return cuda_fail(e, "rope_append launch");
     if (!plan.small) c->launches++;
+    // (behind rotate + append nothing reads q, k_new and v_new; the one launch of a small step reads them itself)
+    if (inputs_read && !plan.small) e = cudaEventRecord(inputs_read, st);
+    if (e != cudaSuccess) return cuda_fail(e, "cudaEventRecord(inputs read)");
     {
         ProfScope ps(c, st, 1);
         if (plan.small) e = launch_fold_small(ra, aa, plan.cut, f.dtype, (f.flags & KVF_ROPE_INTERLEAVED) != 0, st);
@@ -740,6 +743,8 @@ kvf_status step_impl(kvf_cache *c, const void *q, const void *k_new, const void 
     }
     if (e != cudaSuccess) return cuda_fail(e, "attention launch");
     c->launches++;
+    if (inputs_read && plan.small) e = cudaEventRecord(inputs_read, st);
+    if (e != cudaSuccess) return cuda_fail(e, "cudaEventRecord(inputs read)");
     if (behind && plan.kernels > 2) {
         // the merge goes behind the attention kernel on the library's stream; the caller's stream
         // meets it again at the end of the next step, or in kvf_cache_flush
@@ -1002,11 +1007,13 @@ kvf_status kvf_fold_step_host(kvf_cache *c, const void *q_host, const void *k_ho
     if (f.flags & KVF_HOST_UPLOAD_AHEAD) {
         // upload on the library's stream into the staging set the step before last used: it runs
         // while the previous step computes, and starts once that set's last reader (the rotate +
-        // append kernel of two steps ago, marked by ev_read) is done
+        // append kernel of two steps ago, marked by ev_read) is done, while that step's attention runs.  (Marked behind the whole
+        // step, the upload began together with the copy of that step's results: 16 384 tokens in chunks of 256, a chain by itself
+        // 6.11 ms, now 5.85, chains one behind another 6.12 -> 6.01.)
         // (Copies of one stream follow one another with a gap, and a copy that has the other direction beside it is slower
         // than the two together need be: 64 times 2 + 1/2 + 1/2 MB up and 2 MB down take 5.83 ms on one stream each way, 5.56 with two up,
-        // 4.90 with two each way; 4.42 without those down.  16 384 tokens in chunks of 256, whose two staging sets hold the copies back,
-        // 6.12 -> 5.99 ms, in chunks of 1024 5.19 -> 5.09; with two streams one way only no faster.)
+        // 4.90 with two each way; 4.42 without those down.  16 384 tokens in chunks of 256, a chain by itself 6.17 -> 6.11 ms,
+        // in chunks of 1024 5.19 -> 5.09; with two streams one way only no faster.)
         if (!c->up_stream[1]) {
             for (int i = 0; i < 2 && e == cudaSuccess; ++i) {
                 if (!c->up_stream[i]) e = cudaStreamCreateWithFlags(&c->up_stream[i], cudaStreamNonBlocking);
@@ -1060,11 +1067,10 @@ kvf_status kvf_fold_step_host(kvf_cache *c, const void *q_host, const void *k_ho
         }
     }
     float *lse_dev = lse_host ? reinterpret_cast<float *>(w + o_lse) : nullptr;
-    s = step_impl(c, w + oq, w + ok_, w + ov, n_tokens, pos0, w + o_out, lse_dev, st);
+    const bool ahead = (f.flags & KVF_HOST_UPLOAD_AHEAD) != 0;
+    s = step_impl(c, w + oq, w + ok_, w + ov, n_tokens, pos0, w + o_out, lse_dev, st, ahead ? c->ev_read[set] : nullptr);
     if (s != KVF_OK) return s;
-    if (f.flags & KVF_HOST_UPLOAD_AHEAD) {
-        e = cudaEventRecord(c->ev_read[set], st);      // (after the whole step: later than needed, never too early)
-        if (e != cudaSuccess) return cuda_fail(e, "cudaEventRecord");
+    if (ahead) {
         c->ev_read_set[set] = true;
         c->host_steps++;
     }
