@@ -226,7 +226,7 @@ kvf_status kvf_fold_step(kvf_cache *c, const void *q, const void *k_new, const v
 /*
  * The same step with HOST buffers (pinned memory recommended): copies q/k/v to the workspace
  * staging area, runs the step, copies `out` (and lse if not NULL) back, all on `cuda_stream`
- * (with KVF_HOST_UPLOAD_AHEAD the three uploads run on an internal stream that `cuda_stream` then
+ * (with KVF_HOST_UPLOAD_AHEAD the three uploads run on two internal streams that `cuda_stream` then
  * waits for; with KVF_HOST_DOWNLOAD_BEHIND the results are copied back on an internal stream, see
  * that flag for when they are there).  The host buffers must stay valid until the stream reaches
  * the end of the call (result buffers under KVF_HOST_DOWNLOAD_BEHIND: until the results are there).
