@@ -1476,6 +1476,8 @@ cudaError_t launch_attn_tc(const AttnArgs &a, const TcMaps &maps, cudaStream_t s
     return launch_pdl(kernel, dim3(grid.x * grid.y, 1, grid.z), dim3(quant ? kThreadsQ8 : kThreads), smem, s, a, maps.q, maps.k, maps.v);
 }
 
+bool attn_tc_merges_by_row(int parts, int64_t rows, int sms) { return parts > 8 && parts <= kRowMergeParts && rows <= 8 * (int64_t)sms; }
+
 cudaError_t launch_combine_groups(const AttnArgs &a, int sms, cudaStream_t s) {
     dim3 grid((a.n + kCombineTokens - 1) / kCombineTokens, a.Hkv, a.batch);
     // at most eight parts per KV head (two streams x four pieces, or eight pieces)?  The host knows when it
@@ -1496,7 +1498,7 @@ cudaError_t launch_combine_groups(const AttnArgs &a, int sms, cudaStream_t s) {
     // parts 1184: 6.1 / 4.6; 36 parts 1024: 9.8 / 5.3; 96 parts 64: 11.1 / 3.2, 1184: 20.7 / 9.1; groups of six to eight, whose tokens take
     // eight rows of a block, more: 12 / 2 heads, 74 parts, 48 rows 30.8 / 2.9, 768: 30.9 / 7.1.  More than 96 parts (one KV head on every
     // SM) would need more registers and shared memory.
-    if (known && !few && most <= kRowMergeParts && (int64_t)a.n * a.H * a.batch <= 8 * (int64_t)sms)
+    if (known && attn_tc_merges_by_row(most, (int64_t)a.n * a.H * a.batch, sms))
         return launch_pdl(combine_rows_kernel, dim3(a.n * a.G, a.Hkv, a.batch), dim3(256), (size_t)most * 512, s, a);
     if (few) return launch_pdl(combine_groups_kernel<true>, grid, dim3(256), 0, s, a);
     return launch_pdl(combine_groups_kernel<false>, grid, dim3(256), 0, s, a);

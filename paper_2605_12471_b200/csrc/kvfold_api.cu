@@ -393,9 +393,12 @@ Plan make_plan(const kvf_cache *c, int n, int64_t prefix, int batch = 1, int64_t
             // tile is no faster than one of two.  Fitted to 12 800 random steps timed under 2 to 18 cuts each (17 - 4096
             // tokens, seven head shapes, 64 - 60 K rows, windows, batches, all storages): rms 5 % of a step; the cut
             // chosen is 2.6 % above the best of them on average, where a fixed least of four tiles per CTA is 13 %.  (The fit is
-            // from before up to four parts, and nine and more of few rows, had merge kernels of their own, 1 - 5 us cheaper
-            // (launch_combine_groups has figures), and before pairs of CTAs on quantised rows issued Q K^T early; not
-            // fitted again since: more cuts than it chooses may pay.)
+            // from before up to four parts had a merge kernel of their own and pairs of CTAs on quantised rows issued Q K^T early.)
+            // Nine parts and more of few rows are merged a block per row, next to nothing a part: 7401 random steps timed
+            // under all their cuts (17 - 1250 tokens, eight head shapes, 64 - 40 K rows, all storages) take 1.2 % less than with those
+            // parts priced as the kernel for any number takes them, 3 in 10 000 more than 2 % longer (6 % at most), 1 in 100 over 23 %
+            // less: 45 tokens of 12 / 2 heads at prefix 7 K 8 ranges 26.5 us, 28 16.6; 21 of 32 / 4 at 6 K 26.4 / 17.2; the cut
+            // chosen is 1.7 % above the best.  (All constants fitted again: 1.4 %, but 1 in 100 over 2 % longer.)
             // us per step (ranges per head: time): 256 tokens of 32 / 8 heads, bf16, 4 key tiles 1: 17.4, 4: 18.1; 8 tiles
             // 1: 24.6, 2: 23.2, 4: 20.1; 64 tokens of 28 / 4 heads, 32 tiles 8: 22.2, 18: 31.2; 32 tokens of 12 / 2
             // heads, 126 tiles 31: 35.2, 72: 55.7; 48 tokens of 8 / 2 heads, int8, 43 tiles 10: 28.0, 24: 22.6.
@@ -403,6 +406,8 @@ Plan make_plan(const kvf_cache *c, int n, int64_t prefix, int batch = 1, int64_t
             const double rows = (double)n * c->cfg.n_q_heads * batch, launch = window_lo(c, prefix) > 0 ? -1.5 : 3.0;
             auto merge = [&](int64_t parts) {
                 if (parts <= 1) return 0.0;
+                if (Hkv <= kRangeHeads && attn_tc_merges_by_row((int)parts, (int64_t)n * c->cfg.n_q_heads * batch, c->sm_count))
+                    return launch + 1.0 + 0.11 * (double)parts + 1.2e-4 * rows * (double)parts;
                 return launch + 0.7 * std::max(c->Gp / 2, 2) * (double)((parts + 7) / 8) + (parts > 8 ? 2.0 : 0.0) + 1.2e-4 * rows * (double)parts;
             };
             const int64_t room = std::min<int64_t>(c->sm_count / (pairs * batch), slots_cap - (Hkv - 1));

@@ -263,6 +263,7 @@ bool attn_tc_supported(int dtype, int d, int G);
 int attn_tc_padded_group(int G);       // G rounded up to a power of two: rows a token takes in the tcgen05 kernels' row layout
 int attn_tc_row_pairs(int n, int G);   // 256-row pairs per KV head (G: the padded group, as below)
 int attn_tc_streams(int n, int G);     // 2 when the chunk fits one 128-row tile
+bool attn_tc_merges_by_row(int parts, int64_t rows, int sms);          // nine parts and more: a block per output row?
 int attn_tc_row_ranks(int units, int sms, int64_t key_tiles);        // AttnArgs::ranks for `units` row tiles of all KV heads, or 0
 cudaError_t launch_attn_tc(const AttnArgs &a, const TcMaps &maps, cudaStream_t s);   // grid (ngroups x row pairs); pairs of CTAs: (row pairs, ngroups)
 cudaError_t launch_combine_groups(const AttnArgs &a, int sms, cudaStream_t s);                // needed when ngroups != Hkv

@@ -42,3 +42,13 @@ def test_ranges_under_a_window():
                                                  (2048, 4000, binding.KVF_CACHE_INT8, 8)])        # 255 / 274 with 9
 def test_ranges_of_steps_that_fill_the_sms(n, rows, flags, groups):
     assert _plan(32, 8, n, rows, flags)[2] == groups * -(-n // 64)
+
+
+# few rows: a block per row merges any number of parts up to 96 in ~2 us, so the ranges are short
+@pytest.mark.parametrize("h,kv,n,rows,flags,lo,hi", [
+    (12, 2, 45, 7027, 0, 16, 48),                           # 16.6 us with 28, 26.5 with eight
+    (32, 4, 21, 6264, 0, 16, 37),                           # 17.2 with 25, 26.4 with eight
+    (12, 2, 18, 4663, binding.KVF_CACHE_INT4, 12, 48),      # 17.2 with 19, 26.0 with eight
+])
+def test_ranges_per_head_where_rows_are_merged_a_block_each(h, kv, n, rows, flags, lo, hi):
+    assert lo <= _plan(h, kv, n, rows, flags)[1] <= hi
