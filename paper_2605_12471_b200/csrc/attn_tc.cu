@@ -183,12 +183,14 @@ __device__ __forceinline__ bool mbar_try_wait4(const Phase (&w)[4]) {
           "r"(w[3].bar), "r"(w[3].parity), "r"(kSuspendHintNs) : "memory");
     return ok;
 }
-__device__ __forceinline__ bool mbar_wait4(const Phase (&w)[4], Ctl *ctl, int *status) {
-    if (mbar_try_wait4(w)) return true;
+__device__ __forceinline__ bool mbar_wait4_warp(const Phase (&w)[4], Ctl *ctl, int *status) {
+    bool ok = mbar_try_wait4(w);
+    if (!ok) {
+        ok = true;
 #pragma unroll
-    for (int k = 0; k < 4; ++k)
-        if (!mbar_wait(w[k].bar, w[k].parity, ctl, status)) return false;
-    return true;
+        for (int k = 0; k < 4; ++k) ok = ok && mbar_wait(w[k].bar, w[k].parity, ctl, status);
+    }
+    return __all_sync(0xffffffffu, ok);
 }
 
 // Instruction descriptor: D fp32, A and B bf16, M = 128, N = 128; bit 16 = B is MN-major.
@@ -562,6 +564,7 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
             // were what the kernel waited for.  Cycles of a CTA, 256 tokens in 131 072: 167 -> 152 million, deep chain 135.6 -> 131.5 ms;
             // 2048 tokens in 16 384: 1.76 -> 1.61 million, 1933 -> 1826 us; int8, 256 tokens in 65 536: 58.6 -> 53.0 million, 42.0 ->
             // 39.6 ms.  (Of it 3 % of the cycles of bf16 rows: what a tile waits for ahead of its first MMAs asked in one go.)
+            // (Every wait ends in a vote, see mbar_wait_warp.)
             const bool leader = elect_one();
             const int i = warp - 9;
             const uint32_t t_s = tmem + i * 128, t_o = tmem + 256 + i * 128;
@@ -608,7 +611,7 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
             int kt0, ntiles;
             for (int kvh = kvh_first; ok && piece(kvh, kt0, ntiles); ++kvh) {
                 if (ntiles <= 0) continue;
-                ok = mbar_wait(bar(B_QFULL), pc & 1, ctl, a.status);
+                ok = mbar_wait_warp(bar(B_QFULL), pc & 1, ctl, a.status);
                 if (!ok) break;
                 tc_fence_after();
                 // Per key tile: first half of P V (j - 1), second half, Q K^T (j).  The scores overwrite the
@@ -626,7 +629,7 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
                     uint32_t kpar = 0, vpar = 0;
                     if (more) ring(tk, kslot, kpar);
                     auto second_half = [&]() -> bool {
-                        if (!mbar_wait(bar(B_PB0 + i), (it - 1) & 1, ctl, a.status)) return false;
+                        if (!mbar_wait_warp(bar(B_PB0 + i), (it - 1) & 1, ctl, a.status)) return false;
                         tc_fence_after();
                         issue_pv_half(vslot, 1, true);
                         if ((kEarly || !more) && leader) tc_commit(bar(B_PVDONE0 + i));
@@ -641,7 +644,7 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
                         // (what is not there to be waited for is asked for twice; pairs of CTAs: a K tile is the last to come, and P V
                         // need not wait for it)
                         const Phase all[4] = {v_full, kEarly && !kPair && more ? Phase{bar(B_FULL0 + kslot), kpar} : v_full, p_half, my_turn};
-                        ok = mbar_wait4(all, ctl, a.status);
+                        ok = mbar_wait4_warp(all, ctl, a.status);
                         if (!ok) break;
                         tc_fence_after();
                         issue_pv_half(vslot, 0, jprev > j0);
@@ -650,7 +653,7 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
                     }
                     if (more) {
                         // (bf16 rows: waited for above, but for a piece's first)
-                        if (!kEarly || kPair || jprev < 0) ok = mbar_wait(bar(B_FULL0 + kslot), kpar, ctl, a.status);
+                        if (!kEarly || kPair || jprev < 0) ok = mbar_wait_warp(bar(B_FULL0 + kslot), kpar, ctl, a.status);
                         if (!ok) break;
                         tc_fence_after();
                         issue_qk(kslot);

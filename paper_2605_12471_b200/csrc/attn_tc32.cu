@@ -229,7 +229,8 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc32_kernel(const AttnArgs a
     if (warp >= 16) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");
         // (whole warps walk the issuers' loops and one thread issues: the descriptors stay in uniform registers.  In branches of one
-        // lane the chain of 65 536 tokens, 512 at a time, took 119.9 ms instead of 110.6, 176 million cycles of a CTA instead of 159)
+        // lane the chain of 65 536 tokens, 512 at a time, took 119.9 ms instead of 110.6, 176 million cycles of a CTA instead of 159.  Ahead of what the
+        // thread issues the lanes vote: all of them have then seen every phase it acts on, see mbar_wait_warp)
         const bool leader = elect_one();
         if (warp == 16) {
             // ------------------------------------------------------------------ issuer of the score MMAs
@@ -240,12 +241,12 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc32_kernel(const AttnArgs a
             int kt0, ntiles, nsteps;
             for (int kvh = kvh_first; ok && piece(kvh, kt0, ntiles, nsteps); ++kvh) {
                 if (nsteps <= 0) continue;
-                ok = mbar_wait(bar(B_QFULL), pc & 1, ctl, a.status);
+                ok = mbar_wait_warp(bar(B_QFULL), pc & 1, ctl, a.status);
                 if (!ok) break;
                 for (int j = 0; j < nsteps; ++j, ++g) {
                     const int slot = g % kKSlots;
-                    ok = mbar_wait(bar(B_SFREE), (g & 1) ^ 1, ctl, a.status);
-                    if (ok) ok = mbar_wait(bar(B_KFULL0 + slot), (g / kKSlots) & 1, ctl, a.status);
+                    ok = mbar_wait(bar(B_SFREE), (g & 1) ^ 1, ctl, a.status) && mbar_wait(bar(B_KFULL0 + slot), (g / kKSlots) & 1, ctl, a.status);
+                    ok = __all_sync(0xffffffffu, ok);
                     if (!ok) break;
                     tc_fence_after();
                     const uint64_t dk = desc_kmajor(base + kOffK + (uint32_t)slot * kKSlot);
@@ -281,9 +282,9 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc32_kernel(const AttnArgs a
             for (int kvh = kvh_first; ok && piece(kvh, kt0, ntiles, nsteps); ++kvh) {
                 for (int j = 0; j < nsteps; ++j, ++g) {
                     const int b = g & 1, slot = g % kVSlots;
-                    ok = mbar_wait(bar(B_VFULL0 + slot), (g / kVSlots) & 1, ctl, a.status);
-                    if (ok) ok = mbar_wait(bar(B_PFULL0 + b), (g >> 1) & 1, ctl, a.status);
+                    ok = mbar_wait(bar(B_VFULL0 + slot), (g / kVSlots) & 1, ctl, a.status) && mbar_wait(bar(B_PFULL0 + b), (g >> 1) & 1, ctl, a.status);
                     if (ok && g > 0) ok = mbar_wait(bar(B_OFREE), (g - 1) & 1, ctl, a.status);   // the previous P V has been added
+                    ok = __all_sync(0xffffffffu, ok);
                     if (!ok) break;
                     tc_fence_after();
                     const uint32_t v_hi = base + kOffV + (uint32_t)slot * kKSlot;

@@ -101,6 +101,14 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, Ctl *ct
     return mbar_wait_slow(bar, parity, ctl, status);
 }
 
+// The same for a warp of which one thread acts on what was waited for (an issuer).  The vote holds that thread back until every lane has
+// seen the phase: lanes that arrive nowhere are otherwise held by nothing, and a lane two phases behind misreads the parity and
+// waits until the limit.
+template <typename Ctl>
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, Ctl *ctl, int *status) {
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, ctl, status));
+}
+
 __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap *map, uint32_t bar, int c0, int c1, int c2) {
     asm volatile(
         "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"
