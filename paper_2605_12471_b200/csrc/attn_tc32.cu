@@ -196,7 +196,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc32_kernel(const AttnArgs a
         mbar_init(bar(B_SFREE), 4);
         for (int i = 0; i < 2; ++i) {
             mbar_init(bar(B_PFULL0 + i), 4);
-            mbar_init(bar(B_PFREE0 + i), 1);
+            mbar_init(bar(B_PFREE0 + i), 1 + 4);          // the P V that read the buffer, and the output warps, see there
         }
         mbar_init(bar(B_OFULL), 1);
         mbar_init(bar(B_OFREE), 4);
@@ -417,8 +417,14 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc32_kernel(const AttnArgs a
             for (int c = 0; c < kD; ++c) o[c] = 0.f;
             float l = 0.f, m_ref = 0.f;
             for (int j = 0; j < nsteps; ++j, ++g) {
-                // (the probabilities' barrier as well: alpha was written ahead of them)
-                ok = mbar_wait(bar(B_PFULL0 + (g & 1)), (g >> 1) & 1, ctl, a.status) && mbar_wait(bar(B_OFULL), g & 1, ctl, a.status);
+                // (The probabilities' barrier as well: alpha was written ahead of them.  The arrival says that it has been seen.  Without it the
+                // softmax, which runs ahead while a piece's rows are written out, could fill this buffer for step g + 2 first, and
+                // parity would no longer tell the phase of step g.)
+                ok = mbar_wait(bar(B_PFULL0 + (g & 1)), (g >> 1) & 1, ctl, a.status);
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) break;
+                if (lane == 0) mbar_arrive(bar(B_PFREE0 + (g & 1)));
+                ok = mbar_wait(bar(B_OFULL), g & 1, ctl, a.status);
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
                 tc_fence_after();
@@ -536,7 +542,8 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc32_kernel(const AttnArgs a
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
                 tc_fence_after();
-                // (the P V that read this buffer two steps ago: asked ahead of the arithmetic, every phase is waited for)
+                // (the P V that read this buffer two steps ago, and the output warps' word that they have seen that step's probabilities:
+                // asked ahead of the arithmetic, every phase is waited for)
                 uint32_t buffer_free = 1;
                 if (g > 1) buffer_free = mbar_test(bar(B_PFREE0 + b), ((g >> 1) - 1) & 1);
 
