@@ -344,6 +344,7 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
         ctl->clk0 = clock64();
         ctl->ns0 = global_ns();
     }
+    __syncwarp();     // (.aligned instructions want the warp together, here and below where threads have gone different ways)
     // K/V tile slots.  Two row tiles: one ring of 4 (quantised storage: 3) that both issuers walk in step.  Two streams:
     // each stream owns a ring of 3 (the sixth slot is the second Q tile, unused there), because a
     // parity wait is only sound for a thread that watches every use of its barrier in order.
@@ -877,6 +878,7 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
                                      "r"(p[4 * c]), "r"(p[4 * c + 1]), "r"(p[4 * c + 2]), "r"(p[4 * c + 3]) : "memory");
                     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the MMAs read through the async proxy
                 } else {
+                    __syncwarp();
                     KVF_TMEM_ST32(p, 0, t_s + 32);
                     tmem_wait_st();
                     tc_fence_before();
@@ -923,7 +925,6 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
                 const int fin_row = kD * (a.out_f32 ? 4 : 2);
                 const int64_t fin0 = (int64_t)cb * nmax * a.H + kvh * a.G;
                 auto emit = [&](const uint32_t (&w)[32], int byte0) {
-                    __syncwarp();                  // the segment before has been read
 #pragma unroll
                     for (int c = 0; c < 8; ++c)
                         asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(stage + (uint32_t)lane * 128u + (uint32_t)((c ^ (lane & 7)) << 4)),
@@ -944,6 +945,7 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
 #pragma unroll 1
                     for (int c0 = 0; c0 < 128; c0 += 32) {
                         uint32_t w[32];
+                        __syncwarp();              // the segment before has been read
                         KVF_TMEM_LD32(w, 0, t_o + c0);
                         tmem_wait_ld();
 #pragma unroll
@@ -954,6 +956,7 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
 #pragma unroll 1
                     for (int c0 = 0; c0 < 128; c0 += 64) {
                         uint32_t o[64], w[32];
+                        __syncwarp();
                         KVF_TMEM_LD32(o, 0, t_o + c0);
                         KVF_TMEM_LD32(o, 32, t_o + c0 + 32);
                         tmem_wait_ld();
@@ -969,6 +972,7 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
 #pragma unroll
             for (int c0 = 0; c0 < 128; c0 += 32) {
                 uint32_t o[32];
+                __syncwarp();
                 KVF_TMEM_LD32(o, 0, t_o + c0);
                 tmem_wait_ld();
                 if (!valid) continue;
@@ -1025,6 +1029,7 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
             for (uint32_t s = 0; s < kRanks; ++s)
                 if (s != rank) mbar_arrive_cluster(peer_smem(bar(B_READY), s));
         }
+        __syncwarp();
         if (warp < 8) {
             tc_fence_after();
             const int lg = __ffs(G) - 1;                                 // (G is a power of two)
@@ -1042,6 +1047,7 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
             float v[C];
             auto mix = [&](int c0) {                                     // C columns of my 64 from c0 on
                 uint32_t x[C], y[C];
+                __syncwarp();
                 if constexpr (C == 32) {
                     KVF_TMEM_LD32(x, 0, t_row + c0);
                     KVF_TMEM_LD32(y, 0, t_row + 128 + c0);

@@ -224,6 +224,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc32_kernel(const AttnArgs a
         ctl->clk0 = clock64();
         ctl->ns0 = global_ns();
     }
+    __syncwarp();     // (.aligned instructions want the warp together)
 
     // The shares of registers: softmax 128 x 128, output 128 x 168, converters 256 x 72, issuers 128 x 40 = the launch's 640 x 96.
     if (warp >= 16) {
@@ -518,6 +519,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc32_kernel(const AttnArgs a
                     split2(x.x, x.y, hi[2 * c], lo[2 * c]);
                     split2(x.z, x.w, hi[2 * c + 1], lo[2 * c + 1]);
                 }
+                __syncwarp();
                 KVF_TMEM_ST32(hi, 0, tmem + lane_addr + kColQ + 2 * c0);
                 KVF_TMEM_ST32(lo, 0, tmem + lane_addr + kColQ + 64 + 2 * c0);
             }

@@ -141,6 +141,7 @@ __global__ void __launch_bounds__(kThreads, 2) fold_small_kernel(const __grid_co
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
             mbar_expect_tx(landed, BM * (D * 4u + 8u));
         }
+        __syncwarp();                                     // (.aligned: the warp together)
         asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
     }
     auto table = [&](float2 *cs, int64_t token, int j) {
@@ -336,6 +337,7 @@ __global__ void __launch_bounds__(kThreads, 2) fold_small_kernel(const __grid_co
     // Every slice's maximum, sum and unnormalised output go to the CTA that finishes the row, which merges them in slice order.
     // (Stores that complete on the receiver's barrier, instead of loads between two cluster barriers.)
     const int rows = BM / ranks;                          // (ranks is a power of two)
+    __syncwarp();
     if (ranks > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 #pragma unroll
     for (int i = 0; i < TR; ++i) {

@@ -31,6 +31,25 @@ def test_waits_of_issuing_warps_end_in_a_vote(name, end):
             assert not any("leader" in line for line in lines[i:until])
 
 
+# .aligned instructions want all lanes of a warp together, which only a warp-wide instruction makes sure of behind a branch of some of
+# them.  Read down the text of a role; __syncthreads and votes count as much as __syncwarp.
+@pytest.mark.parametrize("name", ["attn_tc.cu", "attn_tc32.cu", "fold_small.cu"])
+def test_aligned_instructions_stand_behind_a_reconvergence(name):
+    apart = None
+    for number, line in enumerate(_source(name).splitlines(), 1):
+        code = line.split("//")[0]
+        if "// -----" in line or "tcgen05.alloc" in code or code.startswith(("__global__", "}")) or code.strip() == "continue;":
+            apart = None                         # (another role, warps that the branch before did not hold, a branch that ends here)
+        if re.search(r"KVF_TMEM_(LD|ST)\d+\(|\.aligned;|cluster_sync_all\(\)", code):
+            assert apart is None, f"{name}:{number}: behind the branch in line {apart}"
+        if re.search(r"\b(if|for) \(.*\b(lane == 0|tid == 0|threadIdx\.x == 0|clocked\)|valid\)|gi1? >= a\.G|i = tid;)", code):
+            apart = number
+        if re.search(r"__syncwarp|__syncthreads|_sync\(0xffffffffu|mbar_wait4?_warp\(", code):
+            apart = None
+    for kernel in ("attn_tc.cu", "attn_tc32.cu"):          # (the roles begin with setmaxnreg)
+        assert re.search(r"ns0 = global_ns\(\);\n    }\n    __syncwarp\(\);", _source(kernel))
+
+
 class _Overtaken(Exception):
     pass
 
