@@ -333,7 +333,7 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
     tc_fence_before();
     __syncthreads();
     if (kPair) cluster_sync_all();      // the partner's barriers exist before anything is sent to them
-    if (kRanks > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");      // (waited for at the end, ahead of what is sent)
+    if (kRanks > 1) cluster_arrive();      // (waited for at the end, ahead of what is sent)
     tc_fence_after();
     pdl_wait();   // nothing above reads what an earlier kernel wrote; from here on the rotated chunk is read
     const uint32_t tmem = *reinterpret_cast<volatile uint32_t *>(&ctl->tmem_base);
@@ -1023,8 +1023,11 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
         constexpr int W = 64 / kRanks;
         constexpr uint32_t kFromRank = 2u * kRows * W * 4u;              // what a CTA sends another: its columns of 2 x 128 half rows ...
         const uint32_t landing = base + kOffKV + kTileBytes, land_stats = base + kOffKV + 4096u;     // ... and a float2 per row, by sender
-        if (kRanks > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-        if (kRanks > 1 && threadIdx.x == 0) {
+        // (A CTA that has given up a wait asks for nothing, sends nothing and writes nothing.)
+        if (kRanks > 1) cluster_wait();
+        bool ok = __all_sync(0xffffffffu, *reinterpret_cast<volatile int *>(&ctl->abort) == 0);
+        const bool asked = kRanks > 1 && ok;
+        if (asked && threadIdx.x == 0) {
             mbar_expect_tx(bar(B_LANDED), (kRanks - 1) * (kFromRank + kRows * 8u));
             for (uint32_t s = 0; s < kRanks; ++s)
                 if (s != rank) mbar_arrive_cluster(peer_smem(bar(B_READY), s));
@@ -1065,7 +1068,6 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
             };
             float weight[kRanks];
             weight[0] = 1.f;
-            bool ok = true;
             if constexpr (kRanks > 1) {
 #pragma unroll 1
                 for (int t = 1; ok && t < kRanks; ++t) {
@@ -1079,12 +1081,14 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
                     for (int c = 0; c < W; c += 4) peer_store4(peer_smem(place((int)rank, c >> 2), (uint32_t)s), make_float4(v[c], v[c + 1], v[c + 2], v[c + 3]), landed);
                     if (i == 0) peer_store2(peer_smem(land_stats + ((uint32_t)rank * kRows + (uint32_t)r) * 8u, (uint32_t)s), make_float2(M, L), landed);
                 }
+                __syncwarp();
+                cluster_arrive_relaxed();          // (nothing goes to a partner any more, see the end)
             }
 #pragma unroll
             for (int c0 = 0; c0 < W; c0 += C) {
                 mix((int)rank * W + c0);
                 if constexpr (kRanks > 1) {
-                    if (ok) ok = mbar_wait(bar(B_LANDED), 0, ctl, a.status);
+                    ok = ok && mbar_wait(bar(B_LANDED), 0, ctl, a.status);
                     float2 st[kRanks];
                     float most = M;
 #pragma unroll
@@ -1116,7 +1120,7 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
                         }
                     }
                 }
-                if (tok >= n || gi >= a.G) continue;
+                if (!ok || tok >= n || gi >= a.G) continue;
                 // (a thread's 64 to 128 bytes of its row as they are: turned round in shared memory and written as whole pieces of rows
                 // by neighbouring threads, steps took 0.1 us less without a cluster, 0.4 us more with)
                 const float inv = L > 0.f ? 1.f / L : 0.f;
@@ -1135,9 +1139,21 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
                 }
                 if (c0 == 0 && i == 0 && rank == 0 && a.lse) a.lse[row] = (L > 0.f ? M + log2f(L) : -INFINITY) * 0.6931471805599453f;
             }
+        } else if (kRanks > 1) {
+            cluster_arrive_relaxed();
         }
         tc_fence_before();
         __syncthreads();
+        // Nobody leaves while a partner may still arrive or store here.  Where READY and LANDED have come nothing can; where a wait for them
+        // was given up the partners may have sent before they arrived, and that is waited for: one CTA's time-out must not become
+        // a fault of another.
+        if (kRanks > 1) {
+            cluster_wait();
+            if (!ok && threadIdx.x == 0) {
+                mbar_wait_drain(bar(B_READY), 0, a.status);
+                if (asked) mbar_wait_drain(bar(B_LANDED), 0, a.status);
+            }
+        }
     }
     if (warp == 9) {
         tc_fence_after();

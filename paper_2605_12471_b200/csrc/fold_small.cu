@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(kThreads, 2) fold_small_kernel(const __grid_co
             mbar_expect_tx(landed, BM * (D * 4u + 8u));
         }
         __syncwarp();                                     // (.aligned: the warp together)
-        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+        cluster_arrive();
     }
     auto table = [&](float2 *cs, int64_t token, int j) {
         const double theta = (double)(r.pos0 + token) * r.table.inv_freq[j];
@@ -338,7 +338,7 @@ __global__ void __launch_bounds__(kThreads, 2) fold_small_kernel(const __grid_co
     // (Stores that complete on the receiver's barrier, instead of loads between two cluster barriers.)
     const int rows = BM / ranks;                          // (ranks is a power of two)
     __syncwarp();
-    if (ranks > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    if (ranks > 1) cluster_wait();
 #pragma unroll
     for (int i = 0; i < TR; ++i) {
         const int row = TR * ty + i, at = rank * rows + row % rows;
@@ -352,9 +352,15 @@ __global__ void __launch_bounds__(kThreads, 2) fold_small_kernel(const __grid_co
             if (tx == 0) sm.landed_ml[at] = make_float2(m[i], l[i]);
         }
     }
-    if (ranks == 1) __syncthreads();
-    else if (!mbar_wait(landed, 0, &sm, a.status)) return;
-    for (int i = tid; i < rows * (D / 4); i += kThreads) {
+    bool ok = true;
+    if (ranks == 1) {
+        __syncthreads();
+    } else {
+        __syncwarp();
+        cluster_arrive_relaxed();                         // (nothing goes to a partner any more)
+        ok = mbar_wait(landed, 0, &sm, a.status);
+    }
+    for (int i = tid; ok && i < rows * (D / 4); i += kThreads) {
         const int own = i / (D / 4), row = rank * rows + own, c = i % (D / 4);
         const int R = row0 + row, tok = R / G, gi = R % G;
         if (tok >= n) continue;
@@ -390,7 +396,13 @@ __global__ void __launch_bounds__(kThreads, 2) fold_small_kernel(const __grid_co
         }
         if (c == 0 && a.lse) a.lse[at] = (den > 0.f ? M + log2f(den) : -INFINITY) * 0.6931471805599453f;
     }
-    // (what others send has landed, and what this CTA sends needs it no more: nobody waits to leave)
+    // Nobody leaves while a partner may still store here.  What others send has landed, so they have arrived and this is no wait; where the
+    // wait was given up, what they sent before they arrived is waited for: one CTA's time-out must not become a fault of another.
+    if (ranks > 1) {
+        __syncwarp();
+        cluster_wait();
+        if (!ok && tid == 0) mbar_wait_drain(landed, 0, a.status);
+    }
 }
 
 // Once per kernel and device: shared-memory limit, clusters of 16 CTAs (beyond the portable eight), and how many clusters

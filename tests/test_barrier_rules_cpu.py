@@ -134,3 +134,17 @@ def test_no_role_of_the_f32_kernel_falls_two_phases_behind(pieces):
     _explore(_f32_programs(pieces, arrives), counts)
     with pytest.raises(_Overtaken):              # what the output warps' arrival is for
         _explore(_f32_programs(pieces, False), {**counts, "PFREE": 1})
+
+
+# A cluster whose CTAs store into one another: each arrives once more behind its last store and waits for the others ahead of its end, on
+# every way out.
+@pytest.mark.parametrize("name,begin", [("attn_tc.cu", "if constexpr (kRanks > 0) {"), ("fold_small.cu", "if (ranks > 1) cluster_wait();")])
+def test_no_cta_leaves_a_cluster_that_may_still_store_into_it(name, begin):
+    text = re.sub(r"//.*", "", _source(name))
+    start = text.index(begin)
+    end = text.index("\n}\n", start)
+    merge = text[start:end]
+    last_store = merge.rindex("peer_store")
+    assert merge.index("cluster_wait()") < merge.index("peer_store")                # the partners' barriers exist
+    assert last_store < merge.index("cluster_arrive_relaxed()") < merge.rindex("cluster_wait()")
+    assert not re.search(r"\breturn;", merge)
