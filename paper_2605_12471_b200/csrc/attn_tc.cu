@@ -1044,7 +1044,8 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
             float M = fmaxf(m[0], m[1]);
             const float M0 = M == -INFINITY ? 0.f : M, w0 = ex2(m[0] - M0), w1 = ex2(m[1] - M0);
             float L = w0 * l[0] + w1 * l[1];
-            const bool seen0 = l[0] > 0.f, seen1 = l[1] > 0.f;           // (an accumulator that nothing was added to holds anything)
+            // (an accumulator that nothing was added to holds anything; the sum of a row that has met a NaN is one)
+            const bool seen0 = l[0] != 0.f, seen1 = l[1] != 0.f;
             const uint32_t t_row = tmem + ((uint32_t)((warp & 3) * 32) << 16) + 256 + i * 64;
             constexpr int C = W < 32 ? W : 32;                           // columns at a time
             float v[C];
@@ -1123,7 +1124,7 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
                 if (!ok || tok >= n || gi >= a.G) continue;
                 // (a thread's 64 to 128 bytes of its row as they are: turned round in shared memory and written as whole pieces of rows
                 // by neighbouring threads, steps took 0.1 us less without a cluster, 0.4 us more with)
-                const float inv = L > 0.f ? 1.f / L : 0.f;
+                const float inv = L == 0.f ? 0.f : 1.f / L;
                 const int64_t row = ((int64_t)cb * nmax + tok) * a.H + kvh * a.G + gi, at = row * kD + i * 64 + (int)rank * W + c0;
                 if (a.out_f32) {
 #pragma unroll

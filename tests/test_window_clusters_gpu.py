@@ -58,3 +58,44 @@ def test_one_two_and_four_ctas_per_row_tile(n, window, parts):
     plan = _run(32, 8, 2000, n, 4, window, False, False, torch.Generator(device="cuda").manual_seed(n))
     if parts and torch.cuda.get_device_properties(0).multi_processor_count == 148:
         assert plan[1] == parts and plan[3] == 2
+
+
+# A NaN, or an infinity that makes one, reaches the rows that see it and no others, as with the CUDA-core kernel.  `where`: a query
+# element, a key of the chunk (seen from its token on), a key of an earlier step inside the window, one outside (seen by nobody).
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")], ids=["nan", "inf"])
+@pytest.mark.parametrize("where", ["query", "own key", "earlier key", "hidden key"])
+@pytest.mark.parametrize("n,window", [(64, 1020), (256, 1020), (400, 500), (700, 500)])
+def test_not_a_number_reaches_the_rows_that_see_it(n, window, where, bad):
+    h, kv, prefix = 32, 8, 2000
+    rows, gen = prefix + n, torch.Generator(device="cuda").manual_seed(n)
+    q, k, v = (torch.randn(rows, heads, 128, generator=gen, device="cuda").bfloat16() for heads in (h, kv, kv))
+    q2, k2 = q.clone(), k.clone()
+    if where == "query":
+        q2[prefix + n // 2, 9, 77] = bad
+    else:
+        k2[{"own key": prefix + n // 3, "earlier key": prefix - 10, "hidden key": prefix - window - 300}[where], 2, 5] = bad
+
+    def fold(flags, q, k):
+        c = binding.Cache(binding.make_config(h, kv, 128, "bf16", rows, rows, rope_base=10000.0, flags=flags))
+        c.storage.zero_()
+        c.fold_step(q[:prefix].contiguous(), k[:prefix].contiguous(), v[:prefix].contiguous())
+        c.set_window(4, window)
+        if flags:
+            c.set_splits(1)          # (the CUDA-core kernel's merge leaves out a part whose sum is a NaN)
+        lse = torch.empty(n, h, device="cuda")
+        out = c.fold_step(q[prefix:].contiguous(), k[prefix:].contiguous(), v[prefix:].contiguous(), lse=lse)
+        assert c.status() == binding.KVF_OK
+        return out, lse
+
+    clean, clean_lse = fold(0, q, k)
+    out, lse = fold(0, q2, k2)
+    simt, _ = fold(binding.KVF_FORCE_SIMT, q2, k2)
+    assert torch.equal(out.isnan(), simt.isnan())
+    seen = torch.zeros(n, h, dtype=torch.bool, device="cuda")
+    if where == "query":
+        seen[n // 2, 9] = True
+    elif where != "hidden key":
+        seen[n // 3 if where == "own key" else 0:, 8:12] = True
+    assert torch.equal(out[~seen], clean[~seen]) and torch.equal(lse[~seen], clean_lse[~seen])
+    if bad != bad:
+        assert out[seen].isnan().all()
