@@ -58,18 +58,19 @@ enum {
     KVF_FORCE_SIMT = 8u,       /* use the CUDA-core attention kernel even where a tensor-core
                                   kernel applies (bisecting aid, and the path for fp32 caches whose
                                   values leave fp16's range; same results within tolerance)      */
-    KVF_HOST_UPLOAD_AHEAD = 32u, /* kvf_fold_step_host copies a step's q/k/v to the device on a stream of the
-                                  library's own, into one of two staging sets, so that the upload of step
+    KVF_HOST_UPLOAD_AHEAD = 32u, /* kvf_fold_step_host copies a step's q/k/v to the device on two streams of
+                                  the library's own, into one of two staging sets, so that the upload of step
                                   t+1 runs while step t computes (the call's stream waits for the upload;
                                   results and errors are as without the flag).  Needs a workspace that no
                                   other cache's host steps use at the same time */
-    KVF_HOST_DOWNLOAD_BEHIND = 128u, /* kvf_fold_step_host copies a step's results (out, lse) back on a stream of
-                                  the library's own, behind the step, from one of two result staging sets, so
+    KVF_HOST_DOWNLOAD_BEHIND = 128u, /* kvf_fold_step_host copies a step's results (out, lse) back on one of two
+                                  streams of the library's own, behind the step, from one of two result staging sets, so
                                   that the copy of step t runs while step t+1 computes instead of standing in
                                   front of it on the caller's stream.  The contract on the results relaxes:
                                   those of call t are in host memory once the caller's stream has passed the
                                   end of call t+1, or of a kvf_cache_host_flush made after call t - not
-                                  already at the end of call t.  Can be combined with KVF_HOST_UPLOAD_AHEAD;
+                                  already at the end of call t.  Where the result buffers of two calls overlap,
+                                  the later call's results are written last.  Can be combined with KVF_HOST_UPLOAD_AHEAD;
                                   needs a workspace that no other cache's host steps use at the same time */
     KVF_COMBINE_BEHIND = 256u, /* kvf_fold_step and kvf_fold_step_host launch the kernel that merges the key
                                   ranges' partial results (the last kernel of a step whose plan has three)
@@ -227,7 +228,7 @@ kvf_status kvf_fold_step(kvf_cache *c, const void *q, const void *k_new, const v
  * The same step with HOST buffers (pinned memory recommended): copies q/k/v to the workspace
  * staging area, runs the step, copies `out` (and lse if not NULL) back, all on `cuda_stream`
  * (with KVF_HOST_UPLOAD_AHEAD the three uploads run on two internal streams that `cuda_stream` then
- * waits for; with KVF_HOST_DOWNLOAD_BEHIND the results are copied back on an internal stream, see
+ * waits for; with KVF_HOST_DOWNLOAD_BEHIND the results are copied back on internal streams, see
  * that flag for when they are there).  The host buffers must stay valid until the stream reaches
  * the end of the call (result buffers under KVF_HOST_DOWNLOAD_BEHIND: until the results are there).
  */

@@ -137,6 +137,7 @@ struct kvf_cache {
     cudaEvent_t ev_step[2] = {nullptr, nullptr}, ev_down[2] = {nullptr, nullptr};
     bool ev_down_set[2] = {false, false};
     uint64_t host_down_steps = 0;
+    struct HostRange { uintptr_t begin, end; } down_to[2] = {{0, 0}, {0, 0}};   // where the last call's results (out, lse) go
     // KVF_COMBINE_BEHIND: the library's stream for the merge of the partial results, "attention launched"
     // (caller's stream) and "merged" (that stream) events, which capture, if any, the open merge belongs to,
     // and which of the two sets of partial results the next step with a merge writes
@@ -1087,6 +1088,18 @@ kvf_status kvf_fold_step_host(kvf_cache *c, const void *q_host, const void *k_ho
         if (e == cudaSuccess) e = cudaStreamWaitEvent(ds, c->ev_step[oset], 0);
         if (e == cudaSuccess && c->comb_pending) e = cudaStreamWaitEvent(ds, c->ev_comb, 0);   // the merge writes the results
         if (e != cudaSuccess) return cuda_fail(e, "download stream hand-over");
+        // the last call's copies run on the other stream: these go behind them where both write the same host memory (copies of the
+        // call before that are over, the caller's stream has passed them)
+        const kvf_cache::HostRange to[2] = {
+            {reinterpret_cast<uintptr_t>(out_host), reinterpret_cast<uintptr_t>(out_host) + ob},
+            {reinterpret_cast<uintptr_t>(lse_host), reinterpret_cast<uintptr_t>(lse_host) + (lse_host ? (size_t)n_tokens * f.n_q_heads * 4 : 0)}};
+        bool shared = false;
+        for (const kvf_cache::HostRange &x : to)
+            for (const kvf_cache::HostRange &y : c->down_to) shared = shared || (x.begin < y.end && y.begin < x.end);
+        if (shared && c->ev_down_set[oset ^ 1]) e = cudaStreamWaitEvent(ds, c->ev_down[oset ^ 1], 0);
+        if (e != cudaSuccess) return cuda_fail(e, "cudaStreamWaitEvent(last download)");
+        c->down_to[0] = to[0];
+        c->down_to[1] = to[1];
     } else if (kvf_status js = join_combine(c, st)) {
         return js;
     }
