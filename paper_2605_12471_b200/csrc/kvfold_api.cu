@@ -653,7 +653,7 @@ bool disjoint_step(const kvf_cache *c, const void *q, const void *k_new, const v
 }
 
 kvf_status step_impl(kvf_cache *c, const void *q, const void *k_new, const void *v_new, int32_t n,
-                     int64_t pos0, void *out, float *lse, cudaStream_t st, cudaEvent_t inputs_read = nullptr) {
+                     int64_t pos0, void *out, float *lse, cudaStream_t st, int staging_set = -1) {
     const kvf_config &f = c->cfg;
     const int64_t P = c->len;
     // k_new == null: queries only (kvf_attend) - nothing is appended, every query row sees the P rows held
@@ -736,8 +736,14 @@ kvf_status step_impl(kvf_cache *c, const void *q, const void *k_new, const void 
     }
     if (e != cudaSuccess) return cuda_fail(e, "rope_append launch");
     if (!plan.small) c->launches++;
-    // (behind rotate + append nothing reads q, k_new and v_new; the one launch of a small step reads them itself)
-    if (inputs_read && !plan.small) e = cudaEventRecord(inputs_read, st);
+    // Inputs in a staging set: the event behind their last reader, rotate + append or the one launch of a small step.  The next upload into
+    // the set waits for it, also if the rest of this step fails.
+    auto inputs_read = [&]() {
+        const cudaError_t r = cudaEventRecord(c->ev_read[staging_set], st);
+        if (r == cudaSuccess) c->ev_read_set[staging_set] = true;
+        return r;
+    };
+    if (staging_set >= 0 && !plan.small) e = inputs_read();
     if (e != cudaSuccess) return cuda_fail(e, "cudaEventRecord(inputs read)");
     {
         ProfScope ps(c, st, 1);
@@ -749,7 +755,7 @@ kvf_status step_impl(kvf_cache *c, const void *q, const void *k_new, const void 
     }
     if (e != cudaSuccess) return cuda_fail(e, "attention launch");
     c->launches++;
-    if (inputs_read && plan.small) e = cudaEventRecord(inputs_read, st);
+    if (staging_set >= 0 && plan.small) e = inputs_read();
     if (e != cudaSuccess) return cuda_fail(e, "cudaEventRecord(inputs read)");
     if (behind && plan.kernels > 2) {
         // the merge goes behind the attention kernel on the library's stream; the caller's stream
@@ -1074,12 +1080,9 @@ kvf_status kvf_fold_step_host(kvf_cache *c, const void *q_host, const void *k_ho
     }
     float *lse_dev = lse_host ? reinterpret_cast<float *>(w + o_lse) : nullptr;
     const bool ahead = (f.flags & KVF_HOST_UPLOAD_AHEAD) != 0;
-    s = step_impl(c, w + oq, w + ok_, w + ov, n_tokens, pos0, w + o_out, lse_dev, st, ahead ? c->ev_read[set] : nullptr);
+    s = step_impl(c, w + oq, w + ok_, w + ov, n_tokens, pos0, w + o_out, lse_dev, st, ahead ? set : -1);
     if (s != KVF_OK) return s;
-    if (ahead) {
-        c->ev_read_set[set] = true;
-        c->host_steps++;
-    }
+    if (ahead) c->host_steps++;
     cudaStream_t ds = behind ? c->down_stream[oset] : st;
     if (behind) {
         // the copies of this step's results run on the library's stream, behind the step, while the caller's

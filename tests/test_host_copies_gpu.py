@@ -90,3 +90,30 @@ def test_results_of_steps_that_share_a_buffer_come_in_order(flags, offset):
         torch.cuda.current_stream().synchronize()
         assert torch.equal(got.view(torch.int16), out.view(torch.int16)) and torch.equal(got_lse, lse)
     assert host.status() == binding.KVF_OK
+
+
+# Staging sets are written again as soon as their last reader is done: rotate + append, or the one launch of a small step.  Large and
+# small steps in turn, so that copies and kernels of several steps lie side by side in every order.
+@pytest.mark.parametrize("flags", [AHEAD, BEHIND, AHEAD | BEHIND, AHEAD | BEHIND | binding.KVF_COMBINE_BEHIND],
+                         ids=["ahead", "behind", "both", "both_and_merge_behind"])
+@pytest.mark.parametrize("shape,dtype,chunks", [
+    ((4, 1, 64), "f32", [64] * 6),                                   # one launch each
+    ((4, 1, 64), "bf16", [64, 2000, 1, 2000, 300, 64, 64, 1, 1]),    # one launch and three in turn
+    ((32, 8, 128), "bf16", [2048, 1, 32, 2048, 3, 2048, 2048, 64, 1, 1]),
+    ((32, 8, 128), "f32", [512, 1, 512, 32, 32, 512]),
+], ids=["small", "small_and_large", "bf16", "f32"])
+def test_host_steps_of_different_size_in_turn(shape, dtype, chunks, flags):
+    host, ins, want = _chain(shape, dtype, chunks, flags, 5)
+    got = [(torch.zeros_like(o).pin_memory(), torch.zeros_like(l).pin_memory()) for o, l in want]
+    for _ in range(5):
+        for o, l in got:
+            o.zero_()
+            l.zero_()
+        host.set_len(0)
+        for x, (o, l) in zip(ins, got):
+            host.fold_step_host(*x, o, lse=l)
+        host.flush()
+        torch.cuda.current_stream().synchronize()
+        for t, ((o, l), (wo, wl)) in enumerate(zip(got, want)):
+            assert torch.equal(o, wo) and torch.equal(l, wl), t
+    assert host.status() == binding.KVF_OK
