@@ -443,7 +443,8 @@ kvf_status kvf_batch_fold_step_varlen(kvf_batch *b, const void *q, const void *k
                                       const int32_t *n_tokens, int32_t max_tokens, const int64_t *pos0_or_null,
                                       void *out, float *lse_or_null, void *cuda_stream);
 
-/* kvf_cache_plan for a batch step; plan[2] counts the CTAs of all members. */
+/* kvf_cache_plan for a step of kvf_batch_fold_step; plan[2] counts the CTAs of all members.  (Steps of members that differ may be cut
+ * into fewer ranges: their partial results are merged by a kernel to which many parts cost more.) */
 kvf_status kvf_batch_plan(const kvf_batch *b, int32_t n_tokens, int64_t prefix_len, int32_t plan[4]);
 
 /* The batch's own device status word, encoded as kvf_cache_status_word (0 = no wait gave up). */

@@ -324,7 +324,8 @@ int64_t window_lo(const kvf_cache *c, int64_t prefix) {
     return lo <= c->n_sink ? 0 : lo;       // the window reaches the sinks: nothing is hidden
 }
 
-Plan make_plan(const kvf_cache *c, int n, int64_t prefix, int batch = 1, int64_t part_rows_cap = -1, bool one_launch = true) {
+// (`ragged`: the members' row counts are known on the device only, and with them which ranges a KV head has)
+Plan make_plan(const kvf_cache *c, int n, int64_t prefix, int batch = 1, int64_t part_rows_cap = -1, bool one_launch = true, bool ragged = false) {
     if (part_rows_cap < 0) part_rows_cap = c->part_rows_cap;
     Plan p;
     p.qdec = p.small = false;
@@ -407,7 +408,8 @@ Plan make_plan(const kvf_cache *c, int n, int64_t prefix, int batch = 1, int64_t
             const double rows = (double)n * c->cfg.n_q_heads * batch, launch = window_lo(c, prefix) > 0 ? -1.5 : 3.0;
             auto merge = [&](int64_t parts) {
                 if (parts <= 1) return 0.0;
-                if (Hkv <= kRangeHeads && attn_tc_merges_by_row((int)parts, (int64_t)n * c->cfg.n_q_heads * batch, c->sm_count))
+                // (the kernel that merges a block per row is told the ranges by the host, see launch_combine_groups)
+                if (!ragged && Hkv <= kRangeHeads && attn_tc_merges_by_row((int)parts, (int64_t)n * c->cfg.n_q_heads * batch, c->sm_count))
                     return launch + 1.0 + 0.11 * (double)parts + 1.2e-4 * rows * (double)parts;
                 return launch + 0.7 * std::max(c->Gp / 2, 2) * (double)((parts + 7) / 8) + (parts > 8 ? 2.0 : 0.0) + 1.2e-4 * rows * (double)parts;
             };
@@ -1376,7 +1378,7 @@ kvf_status batch_step(kvf_batch *b, const void *q, const void *k_new, const void
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     const kvf_config &f = c0->cfg;
     const int B = (int)b->caches.size();
-    const Plan plan = make_plan(c0, n, P, B, b->part_rows);
+    const Plan plan = make_plan(c0, n, P, B, b->part_rows, true, ragged);
     int64_t *dev_prefixes = reinterpret_cast<int64_t *>(b->workspace + b->off_lens);
     int64_t *dev_pos0s = dev_prefixes + B;
     int64_t *dev_ns = dev_pos0s + B;

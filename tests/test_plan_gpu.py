@@ -52,3 +52,31 @@ def test_ranges_of_steps_that_fill_the_sms(n, rows, flags, groups):
 ])
 def test_ranges_per_head_where_rows_are_merged_a_block_each(h, kv, n, rows, flags, lo, hi):
     assert lo <= _plan(h, kv, n, rows, flags)[1] <= hi
+
+
+def test_ranges_of_ragged_steps_are_priced_with_their_own_merge():
+    """The kernel that merges many parts of few rows needs the ranges from the host, which does not have them for members of different
+    length: those keep to ranges that one trip to memory merges, eight a head.  Told from the bits, as the order of the sums is the cut's."""
+    h, kv, n, prefix, pages = 12, 2, 45, 7027, 56
+    cfg = binding.make_config(h, kv, 128, "bf16", pages * 128, 1024, rope_base=10000.0, flags=binding.KVF_OUT_F32)
+    pool = torch.zeros(binding.paged_pool_bytes(cfg, 2 * pages), dtype=torch.uint8, device="cuda")
+    tables = torch.arange(2 * pages, dtype=torch.int32, device="cuda").view(2, pages)
+    caches = [binding.PagedCache(cfg, pool, 2 * pages, tables[i]) for i in range(2)]
+    gen = torch.Generator(device="cuda").manual_seed(8)
+    draw = lambda *lead: [torch.randn(*lead, heads, 128, generator=gen, device="cuda").bfloat16() for heads in (h, kv, kv)]
+    for c in caches:
+        for at in range(0, prefix, 1024):
+            c.fold_step(*draw(min(1024, prefix - at)))
+    batch, x = binding.Batch(caches), draw(2, n)
+
+    def step(splits):
+        for c in caches:
+            c.set_len(prefix)
+        caches[0].set_splits(splits)
+        return batch.fold_step(*x, ragged=True)
+
+    out, lock_step = step(0), batch.plan(n, prefix)[1]
+    if torch.cuda.get_device_properties(0).multi_processor_count == 148:
+        assert lock_step > 8                                # members that advance together
+        assert torch.equal(out, step(8)) and not torch.equal(out, step(lock_step))
+    assert batch.status_word() == 0
