@@ -312,8 +312,9 @@ kvf_status kvf_cache_set_len(kvf_cache *c, int64_t len);
 kvf_status kvf_cache_status(kvf_cache *c);
 
 /* The raw device status word behind kvf_cache_status (same synchronisation): 0, or for the first
- * bounded wait that gave up 5 + 256 * (index of the barrier in the kernel's control block)
- * + 65536 * (waiting warp) + 2^24 * (awaited parity) - what a bug report should quote.
+ * bounded wait that gave up 5 + 256 * (index of the barrier in the kernel's control block; of no
+ * meaning for the one-launch steps of head_dim 64, which have one barrier) + 65536 * (waiting warp)
+ * + 2^24 * (awaited parity) - what a bug report should quote.
  * -1 for a null handle or a failed copy. */
 int32_t kvf_cache_status_word(kvf_cache *c);
 

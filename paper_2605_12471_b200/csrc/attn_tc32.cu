@@ -565,7 +565,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc32_kernel(const AttnArgs a
                         v[32 * h + c + 1] = t.y;
                     }
                 }
-                // the scores are in registers: the issuer may overwrite them with the step after next
+                // the scores are in registers: the issuer may overwrite them with the next step's
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(bar(B_SFREE));

@@ -58,7 +58,8 @@ __device__ __forceinline__ void add_clock_counters(int *status, long long cycles
 
 // First timed-out wait of a launch leaves 5 (KVF_ERR_TIMEOUT) in the low byte of the status word,
 // the barrier's index in the control block in bits 8-15, the waiting warp in bits 16-23 and the
-// awaited parity in bit 24 (the barrier block is 1024-byte aligned, so the index is in the address).
+// awaited parity in bit 24 (the barrier block of the tcgen05 kernels is 1024-byte aligned, so the index is in the address; the
+// one barrier of fold_small.cu lies anywhere, and bits 8-15 mean nothing there).
 __device__ __forceinline__ void report_timeout(int *status, uint32_t bar, uint32_t parity) {
     atomicCAS(status, 0, (int)(5u | (((bar & 1023u) >> 3) << 8) | ((threadIdx.x >> 5) << 16) | ((parity & 1u) << 24)));
 }
