@@ -99,3 +99,45 @@ def test_not_a_number_reaches_the_rows_that_see_it(n, window, where, bad):
     assert torch.equal(out[~seen], clean[~seen]) and torch.equal(lse[~seen], clean_lse[~seen])
     if bad != bad:
         assert out[seen].isnan().all()
+
+
+# paged caches (pages in no order), alone and advancing together: clusters of four, two and one CTA
+@pytest.mark.parametrize("members,n,window,parts", [(1, 64, 1020, 8), (2, 64, 1020, 8), (3, 64, 1020, 4), (3, 100, 400, 2), (2, 33, 150, 4)])
+def test_paged_caches_and_batches_under_a_window(members, n, window, parts):
+    h, kv, prefix = 32, 8, 1500
+    rows, gen = prefix + n, torch.Generator(device="cuda").manual_seed(members + n)
+    cfg = lambda flags: binding.make_config(h, kv, 128, "bf16", rows, rows, rope_base=10000.0, flags=binding.KVF_OUT_F32 | flags)
+    pages = 4 * (-(-rows // 512))
+    tables = torch.randperm(members * pages, generator=gen, device="cuda").to(torch.int32).view(members, pages)
+    pool = torch.full((binding.paged_pool_bytes(cfg(0), members * pages) // 2,), 0x7FC0, dtype=torch.int16, device="cuda").view(torch.uint8)
+    caches = [binding.PagedCache(cfg(0), pool, members * pages, t) for t in tables]
+    x = [torch.randn(members, rows, heads, 128, generator=gen, device="cuda").bfloat16() for heads in (h, kv, kv)]
+    chunk = lambda y: y[:, prefix:].contiguous()
+    for i, c in enumerate(caches):
+        c.fold_step(*(y[i, :prefix].contiguous() for y in x))
+        c.set_window(4, window)
+    lse = torch.empty(members, n, h, device="cuda")
+    if members == 1:
+        plan = caches[0].plan(n, prefix)
+        out = caches[0].fold_step(*(chunk(y)[0] for y in x), lse=lse[0])[None]
+        assert caches[0].status() == binding.KVF_OK
+    else:
+        batch = binding.Batch(caches)
+        plan = batch.plan(n, prefix)
+        out = batch.fold_step(*(chunk(y) for y in x), lse=lse)
+        assert batch.status_word() == 0
+    if torch.cuda.get_device_properties(0).multi_processor_count == 148:
+        assert plan[1] == parts and plan[3] == 2
+    for i in range(members):
+        def simt(values):
+            c = binding.Cache(cfg(binding.KVF_FORCE_SIMT))
+            c.storage.zero_()
+            c.fold_step(*(y[i, :prefix].contiguous() for y in (x[0], x[1], values)))
+            c.set_window(4, window)
+            want_lse = torch.empty(n, h, device="cuda")
+            return c.fold_step(*(y[i, prefix:].contiguous() for y in (x[0], x[1], values)), lse=want_lse), want_lse
+
+        want, want_lse = simt(x[2])
+        weight, _ = simt(x[2].abs())
+        assert ((out[i] - want).abs() <= (2.0 ** -8 + 2 * 5e-4) * weight).all()
+        assert (lse[i] - want_lse).abs().max().item() <= 5e-4
