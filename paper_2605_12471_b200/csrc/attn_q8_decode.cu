@@ -76,7 +76,7 @@ struct Ctl {
 
 // NB = 8-row blocks of query rows (1: up to 8 rows, 2: up to 16).  A scheduler of the SM holds 16 K
 // registers: with 13 warps one of them has four (128 registers a thread, enough for one block of
-// rows), with 11 none has more than three (168, what two blocks need without spilling).
+// rows), with 11 none has more than three (168: two blocks of rows on codes keep all but 160 bytes in them).
 // BITS = 16 stands for a cache of plain bf16 rows: the same kernel without the expansion (a tile is then two
 // 128-byte-swizzled panels of 64 columns, 32 KiB; three stages of 64 KiB, six consumer warps).
 template <int BITS, int NB> struct Geo {

@@ -73,8 +73,8 @@
 // Small steps under a window (kRanks).  Their key tiles are few, and what a step waited for were 128 KiB of partial results per CTA
 // (3.3 us), a third launch and its hand-overs.  Here a CTA has one row tile, its key tiles in two streams, the two accumulators
 // are merged in the CTA (both lie in the tensor-memory lanes of the same rows) and those of a cluster's CTAs by stores into each
-// other's shared memory.  Steps of 256 tokens under a window of 1020 22.8 -> 19.6 us, of 64 tokens 21.4 -> 14.7
-// (attn_tc_row_ranks has more); 128 steps of 256 tokens 2922 -> 2534 us.
+// other's shared memory.  Steps of 256 tokens under a window of 1020 22.8 -> 19.4 us, of 64 tokens 21.4 -> 14.7
+// (attn_tc_row_ranks has more); 128 steps of 256 tokens 2922 -> 2526 us.
 //
 // Every wait on an mbarrier is bounded (about one second): on expiry the thread raises the
 // CTA's abort flag and records the wait in the device status word, all roles leave their loops,
@@ -917,8 +917,8 @@ attn_tc_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_q, cons
                 const int R1 = row0 + i * kRows + (warp & 3) * 32 + (lane >> 3), lg = __ffs(G) - 1;      // first of the rows I write out
                 // (partial rows lie one after the other; G is a power of two: with a divide per row and line the
                 // index arithmetic took as long as the stores.  The loops over the columns are not unrolled: the code runs
-                // once or twice a launch, steps of 256 - 512 tokens behind short prefixes take 1 - 2 % less, others the same, and bf16
-                // rows no longer spill.  Pairs of CTAs spill 108 bytes; one base and row pitch for both kinds of rows instead of
+                // once or twice a launch, steps of 256 - 512 tokens behind short prefixes take 1 - 2 % less, others the same, and this
+                // code spills nothing on bf16 rows.  Pairs of CTAs spill 108 bytes; one base and row pitch for both kinds of rows instead of
                 // two pointers: 65 536 tokens of int8 in 256s 42.2 -> 42.9 ms)
                 char *part = reinterpret_cast<char *>(a.part_o + (prow - R + R1) * kD) + (lane & 7) * 16;
                 char *fin = reinterpret_cast<char *>(a.out) + (lane & 7) * 16;
@@ -1453,17 +1453,13 @@ static int ranks_at_once() {
     return clusters;
 }
 
-// CTAs per row tile of a step under a window (units: row tiles of all KV heads).  us per step replayed in a graph, 256-row CTAs with
-// partial results and a merge kernel / one, two, four CTAs to a row tile (32 / 8 heads unless said otherwise):
-//   64 tokens, 16 units, 4 key tiles 19.7 / 15.4, 13.4, 12.9; 10 tiles 21.4 / 21.3, 16.6, 14.7; 33 tiles 25.4 / 44.6, 27.9, 20.7
-//   100 tokens, 32 units, 4 tiles 18.6 / 16.4, 13.9, 14.6; 10 tiles 21.0 / 22.2, 17.3, 15.9; 34 tiles 26.9 / 45.2, 28.5, 21.7
-//   256 tokens, 64 units, 5 tiles 19.8 / 17.5, 15.9; 11 tiles 22.8 / 23.4, 19.6; 35 tiles 32.1 / 47.3, 31.5; four: a second wave
-//   300 tokens of 28 / 4 heads, 76 units, 6 tiles 21.9 / 19.2; 12 tiles 25.4 / 24.7; 35 tiles 36.2 / 47.4; two: a second wave
-//   400 tokens, 104 units, 13 tiles 29.2 / 26.4; 20 tiles 34.9 / 34.0; 36 tiles 45.2 / 49.4
-//   512 tokens, 128 units, 13 tiles 30.8 / 27.2; 21 tiles 37.3 / 35.2; 37 tiles 49.4 / 51.2
-//   64 tokens of 16 / 16 heads, 16 units, 4 tiles 14.0 / 15.1, 13.1, 13.0; 33 tiles 21.7 / 43.7, 27.2, 20.6
-// So as many as the device holds at once, four only where the key tiles are more than two for each of two CTAs' streams; alone, a CTA
-// has all key tiles of 128 rows where a CTA of the other kind has a share of them for 256, and keeps ahead up to the line below.
+// CTAs per row tile of a step under a window (units: row tiles of all KV heads).  As many as the device holds at once, four only where
+// the key tiles are more than two for each of two CTAs' streams; alone, a CTA has all key tiles of 128 rows where a CTA of the other
+// kind has a share of them for 256, and keeps ahead up to the line below.  us per step, 256-row CTAs with partial results and a
+// merge kernel / one, two, four CTAs to a row tile, 32 / 8 heads:
+//   64 tokens, 16 units, 4 key tiles 19.7 / 15.4, 13.4, 12.9; 33 tiles 25.4 / 44.6, 27.9, 20.7
+//   100 tokens, 32 units, 4 tiles 18.6 / 16.4, 13.9, 14.6; 10 tiles 21.0 / 22.2, 17.3, 15.9
+//   400 tokens, 104 units, 20 tiles 34.9 / 34.0; 36 tiles 45.2 / 49.4 (two: a second wave)
 int attn_tc_row_ranks(int units, int sms, int64_t key_tiles) {
     if (key_tiles > 8 && units <= ranks_at_once<4>()) return 4;
     if (units <= ranks_at_once<2>()) return 2;

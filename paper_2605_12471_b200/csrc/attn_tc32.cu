@@ -53,7 +53,7 @@
 // the output rows had warps of their own and the queries lay in tensor memory, the softmax thread added P V as well
 // (800 cycles of its 2700) and the MMAs read Q from shared memory (64 KB a step more; with the output warps alone the MMAs
 // took that time instead: 159 -> 162 million cycles of a CTA).  65 536 tokens in chunks of 512: 159 -> 134 million cycles, 111 ->
-// 102 ms (1.48 -> 1.38 GHz).
+// 97 - 102 ms (1.48 -> 1.39 GHz).  (ptxas spills 112 - 160 bytes, 56 - 80 before the output warps; other shares of the registers: 138 million cycles.)
 //
 // Every wait on an mbarrier is bounded and reports through the status word, as in the bf16 kernel.
 #include "kvfold_internal.h"

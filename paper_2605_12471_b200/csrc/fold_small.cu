@@ -15,8 +15,8 @@
 // visible, rows of the chunk causally.
 //
 // Measured (fp32, 64 tokens of 4 / 1 heads at prefix 448, replayed back to back): 33.9 us per step through the three
-// kernels, 7.2 us here, 5.2 at prefix 0 (launch, one trip to memory, one key tile of 32, the merge).  With the merge as loads
-// between two cluster barriers it was 8.7 and 5.6; one token at prefix 500 6.7 -> 4.9.  A key
+// kernels, 7.1 us here, 5.0 at prefix 0 (launch, one trip to memory, one key tile of 32, the merge).  With the merge as loads
+// between two cluster barriers it was 8.7 and 5.6; one token at prefix 500 6.7 -> 4.8.  A key
 // tile more in a slice costs 3.7 - 5 us: latency of dependent shared-memory loads at two warps per scheduler (IPC
 // 0.34, half of the stall cycles on them), so slices are as short as the device has room for.  Tried: 4 x 4 blocks
 // per thread on half the threads (a third less shared-memory traffic, fewer warps: 6.3 us a tile).
@@ -492,12 +492,9 @@ int fold_small_ranks(int row_tiles, int64_t key_tiles, const FoldSmallFit &fit) 
 
 // The cut a small step runs with: as many slices as that or more, in tiles of 64 or 32 keys, by what the longest slice costs
 // (us per tile: 3.9 while a cluster's CTAs have an SM each, 6.6 where they share it; 32 keys 2.2).  More slices than whole
-// tiles fit into (the last ones empty) where that makes the longest one shorter: 64 tokens of 4 / 1 heads, three key tiles
-// in two slices 14.3 us, in four 7.8; five in four 14.5, in eight 8.6.  Tiles of 32 keys up to one CTA per SM: the same step in
-// eight slices 6.7, 64 tokens at prefix 0 7.0 -> 5.6, one token 5.8 -> 4.3 (bf16 6.1 -> 4.8).  (Those figures are from before the
-// merge by stores, which takes 0.5 - 2 us off each; since then 64 tokens at prefix 448, eight row tiles: 7.55 in eight slices of 64 keys,
-// 7.2 in sixteen of 32, where the larger merge used to cost more than that; 64 tokens of 8 / 2 heads at prefix 700 18.2 -> 16.2.)
-// (A window's first tile holds its sinks, up to 64: no tiles of 32.)
+// tiles fit into (the last ones empty) where that makes the longest one shorter: 64 tokens of 4 / 1 heads, five key tiles in four
+// slices 14.5 us, in eight 8.6.  Tiles of 32 keys up to one CTA per SM: 64 tokens at prefix 448 7.55 in eight slices of 64 keys, 7.2 in
+// sixteen of 32; 64 tokens of 8 / 2 heads at prefix 700 18.2 / 16.2.  (A window's first tile holds its sinks, up to 64: no tiles of 32.)
 FoldSmallCut fold_small_cut(int row_tiles, int64_t keys, bool window, const FoldSmallFit &fit) {
     auto cost = [&](const FoldSmallCut &c) {
         const int64_t tiles = (keys + c.keys - 1) / c.keys, slice = (tiles + c.ranks - 1) / c.ranks;

@@ -394,13 +394,11 @@ Plan make_plan(const kvf_cache *c, int n, int64_t prefix, int batch = 1, int64_t
             // tokens), beyond eight the merge kernel that holds any number, the parts written and read.  A range of one
             // tile is no faster than one of two.  Fitted to 12 800 random steps timed under 2 to 18 cuts each (17 - 4096
             // tokens, seven head shapes, 64 - 60 K rows, windows, batches, all storages): rms 5 % of a step; the cut
-            // chosen is 2.6 % above the best of them on average, where a fixed least of four tiles per CTA is 13 %.  (The fit is
-            // from before up to four parts had a merge kernel of their own and pairs of CTAs on quantised rows issued Q K^T early.)
+            // chosen is 2.6 % above the best of them on average, where a fixed least of four tiles per CTA is 13 %.  (The merge kernel
+            // for up to four parts and the early Q K^T on codes came later.)
             // Nine parts and more of few rows are merged a block per row, next to nothing a part: 7401 random steps timed
-            // under all their cuts (17 - 1250 tokens, eight head shapes, 64 - 40 K rows, all storages) take 1.2 % less than with those
-            // parts priced as the kernel for any number takes them, 3 in 10 000 more than 2 % longer (6 % at most), 1 in 100 over 23 %
-            // less: 45 tokens of 12 / 2 heads at prefix 7 K 8 ranges 26.5 us, 28 16.6; 21 of 32 / 4 at 6 K 26.4 / 17.2; the cut
-            // chosen is 1.7 % above the best.  (All constants fitted again: 1.4 %, but 1 in 100 over 2 % longer.)
+            // under all their cuts take 1.2 % less with those parts priced so, 3 in 10 000 more than 2 % longer, 1 in 100 over 23 %
+            // less (45 tokens of 12 / 2 heads at prefix 7 K: 8 ranges 26.5 us, 28 16.6); the cut chosen is 1.7 % above the best.
             // us per step (ranges per head: time): 256 tokens of 32 / 8 heads, bf16, 4 key tiles 1: 17.4, 4: 18.1; 8 tiles
             // 1: 24.6, 2: 23.2, 4: 20.1; 64 tokens of 28 / 4 heads, 32 tiles 8: 22.2, 18: 31.2; 32 tokens of 12 / 2
             // heads, 126 tiles 31: 35.2, 72: 55.7; 48 tokens of 8 / 2 heads, int8, 43 tiles 10: 28.0, 24: 22.6.
@@ -588,12 +586,9 @@ int piece_cost_of(const kvf_cache *c, const Plan &plan, int streams) {
     return KVF_PIECE_COST;
 }
 
-// KVF_DEPENDENT_LAUNCH=never in the environment (read once; for measurements) launches every step's kernels plainly.  Dependent
-// launches are never slower now.  Long tensor-bound steps of bf16 rows (32 key tiles per CTA and more) used to be launched plainly: at
-// the power cap the gaps came back as clock, 148.3 against 150.1 ms for 131 072 tokens in chunks of 256.  Since the issuing warps' overhead
-// is gone the chain is at a lower clock and the gaps are gaps: plain / dependent, three runs in turn, that chain 131.8, 131.1, 131.9 / 130.9,
-// 130.5, 130.3 ms; 32 768 tokens 9.80 / 9.64; 65 536 of 28 / 4 heads 34.6 / 34.0; 16 384 in chunks of 2048 2.12 / 2.09; 30 000 of 16 / 16
-// heads in chunks of 1000 4.12 / 4.04; 65 536 in chunks of 512 and 2048 the same.
+// KVF_DEPENDENT_LAUNCH=never in the environment (read once; for measurements) launches every step's kernels plainly.  Dependent launches
+// are never slower: plain / dependent 131.6 / 130.6 ms for 131 072 tokens in chunks of 256, 9.80 / 9.64 for 32 768, the same for
+// 65 536 in chunks of 512 and 2048, 1.5 - 5 % for short steps.
 bool dependent_launches() {
     static const bool never = [] {
         const char *e = std::getenv("KVF_DEPENDENT_LAUNCH");
@@ -1019,15 +1014,10 @@ kvf_status kvf_fold_step_host(kvf_cache *c, const void *q_host, const void *k_ho
     size_t oq = c->lay.st_q, ok_ = c->lay.st_k, ov = c->lay.st_v;
     int set = 0;
     if (f.flags & KVF_HOST_UPLOAD_AHEAD) {
-        // upload on the library's stream into the staging set the step before last used: it runs
-        // while the previous step computes, and starts once that set's last reader (the rotate +
-        // append kernel of two steps ago, marked by ev_read) is done, while that step's attention runs.  (Marked behind the whole
-        // step, the upload began together with the copy of that step's results: 16 384 tokens in chunks of 256, a chain by itself
-        // 6.11 ms, now 5.85, chains one behind another 6.12 -> 6.01.)
-        // (Copies of one stream follow one another with a gap, and a copy that has the other direction beside it is slower
-        // than the two together need be: 64 times 2 + 1/2 + 1/2 MB up and 2 MB down take 5.83 ms on one stream each way, 5.56 with two up,
-        // 4.90 with two each way; 4.42 without those down.  16 384 tokens in chunks of 256, a chain by itself 6.17 -> 6.11 ms,
-        // in chunks of 1024 5.19 -> 5.09; with two streams one way only no faster.)
+        // Upload on the library's streams into the staging set the step before last used, once that set's last reader (ev_read: its
+        // rotate + append) is done: it runs while the previous step computes.  Two streams, because copies of one follow one another
+        // with a gap: 64 times 3 MB up and 2 MB down take 5.83 ms on one stream each way, 4.90 on two.  16 384 tokens in chunks of
+        // 256, a chain by itself: 6.17 ms with one stream each way and the event behind the whole step, now 5.85.
         if (!c->up_stream[1]) {
             for (int i = 0; i < 2 && e == cudaSuccess; ++i) {
                 if (!c->up_stream[i]) e = cudaStreamCreateWithFlags(&c->up_stream[i], cudaStreamNonBlocking);
