@@ -115,3 +115,31 @@ def test_batches_append_the_bits_of_single_caches(flags):
             torch.cuda.synchronize()
             pools.append(pool)
         assert torch.equal(*pools)
+
+
+# Rotate + append calls its inputs' lines into L2, and every kernel sets itself up, while the kernel before still runs: inputs that this
+# kernel is writing are read as it leaves them, in buffers that hold the step before's until then.
+@pytest.mark.parametrize("dtype,flags,chunk", [("bf16", 0, 1), ("bf16", 0, 256), ("bf16", 0, 2048), ("bf16", binding.KVF_CACHE_INT8, 256),
+                                               ("bf16", binding.KVF_ROPE_INTERLEAVED, 300), ("f32", 0, 512)])
+def test_inputs_written_by_the_kernel_ahead_of_the_step(dtype, flags, chunk):
+    steps, kind = 8, torch.float32 if dtype == "f32" else torch.bfloat16
+    gen = torch.Generator(device="cuda").manual_seed(chunk)
+    ins = [[torch.randn(chunk, h, 128, generator=gen, device="cuda").to(kind) for h in (32, 8, 8)] for _ in range(steps)]
+    total = steps * chunk
+    outs = []
+    for own_buffers in (True, False):
+        cache = binding.Cache(binding.make_config(32, 8, 128, dtype, total, chunk, rope_base=10000.0, flags=flags))
+        cache.storage.zero_()
+        x, out = [torch.zeros_like(y) for y in ins[0]], []
+        torch.cuda.synchronize()
+        for y in ins:
+            if own_buffers:
+                out.append(cache.fold_step(*y))
+                torch.cuda.synchronize()
+            else:
+                torch._foreach_copy_(x, y)
+                out.append(cache.fold_step(*x))
+        torch.cuda.synchronize()
+        assert cache.status() == binding.KVF_OK
+        outs.append((out, cache.storage))
+    assert all(torch.equal(a, b) for a, b in zip(outs[0][0], outs[1][0])) and torch.equal(outs[0][1], outs[1][1])
